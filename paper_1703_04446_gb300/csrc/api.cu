@@ -12,15 +12,14 @@
 
 #include "lgnk_internal.h"
 
-cudaError_t launch_trace_2d(bool nonstat, int model, int mode, const TraceArgs& a, int nblocks, cudaStream_t s);
-cudaError_t launch_trace_3d(bool nonstat, int model, int mode, const TraceArgs& a, int nblocks, cudaStream_t s);
+cudaError_t launch_trace_2d(TimeMode tm, int model, int mode, const TraceArgs& a, cudaStream_t s);
+cudaError_t launch_trace_3d(TimeMode tm, int model, int mode, const TraceArgs& a, cudaStream_t s);
 
 cudaError_t launch_ell_2d(int mode, const EllArgs& a, cudaStream_t s);
 cudaError_t launch_ell_3d(int mode, const EllArgs& a, cudaStream_t s);
 
-cudaError_t launch_trace(int d, bool nonstat, int model, int mode, const TraceArgs& a, int nblocks, cudaStream_t s) {
-    return d == 3 ? launch_trace_3d(nonstat, model, mode, a, nblocks, s)
-                  : launch_trace_2d(nonstat, model, mode, a, nblocks, s);
+cudaError_t launch_trace(int d, TimeMode tm, int model, int mode, const TraceArgs& a, cudaStream_t s) {
+    return d == 3 ? launch_trace_3d(tm, model, mode, a, s) : launch_trace_2d(tm, model, mode, a, s);
 }
 
 cudaError_t launch_ell(int d, int mode, const EllArgs& a, cudaStream_t s) {
@@ -85,7 +84,10 @@ struct lgnk_ctx {
     size_t M = 0, Mv = 0, n = 0;  // image voxels, velocity nodes per block, unknowns
     size_t ipad = 0, vpad = 0;    // padded image elements, padded velocity nodes
     size_t vt_bytes = 0;          // bytes of one gradient-accumulator element
-    SliceTable slices{};          // stage-time slices of the velocity
+    SliceTable slices{};          // stage-time slices of the velocity (assembled rows and their products)
+    TimeMode tm = TM_STEADY;      // of the matrix-free kernels
+    bool gn_rows = false;         // transport: the Gauss-Newton product by rows (MODE_HROW)
+    SliceTable grads{};           // what their gradients are accumulated on: the slices, or the time nodes
     int tiles[3] = {1, 1, 1};
     int trace_blocks = 0;
     double cellvol = 0.0;         // image h^d (Eq. 10)
@@ -259,6 +261,7 @@ TraceArgs base_args(const lgnk_ctx* ctx) {
     const bool transport = ctx->prob.model == LGNK_TRANSPORT;
     // transport traces y(v, x_c, 1, 0) backward, continuity y(v, x_c, 0, 1) forward
     a.dt = (float)((transport ? -1.0 : 1.0) / ctx->N);
+    a.dt6 = a.dt / 6.0f;
     a.t0 = transport ? 1.0f : 0.0f;
     a.cellvol = (float)ctx->cellvol;
     for (int i = 0; i < 3; ++i) a.tiles[i] = ctx->tiles[i];
@@ -283,6 +286,10 @@ TraceArgs base_args(const lgnk_ctx* ctx) {
                                             (ctx->prob.image.hi[i] - ctx->prob.image.lo[i]))
                                   : 0.0f;
     a.slice_nodes = (long long)ctx->vpad;
+    for (int m = 0; m < ctx->slices.n; ++m) {
+        a.tj[m] = ctx->slices.j[m];
+        a.tth[m] = ctx->slices.th[m];
+    }
     a.V = ctx->Vp;
     a.dV = ctx->dVp;
     a.Tp = ctx->Tp;
@@ -311,7 +318,8 @@ int trace_blocks_for(const lgnk_ctx* ctx, int mode) {
 
 lgnk_status trace(lgnk_ctx* ctx, int mode, const TraceArgs& a) {
     if (ctx->prof) TRY(record_event(ctx));
-    KL(launch_trace(ctx->d, ctx->K > 1, ctx->prob.model, mode, a, ctx->trace_blocks, ctx->stream));
+    const TimeMode tm = mode == MODE_ASM && ctx->K > 1 ? TM_SLICES : ctx->tm;
+    KL(launch_trace(ctx->d, tm, ctx->prob.model, mode, a, ctx->stream));
     ctx->trace_launches++;
     if (ctx->prof) TRY(record_event(ctx));
     return LGNK_OK;
@@ -327,8 +335,8 @@ lgnk_status pack_T(lgnk_ctx* ctx, const float* T) {
     return LGNK_OK;
 }
 
-lgnk_status zero_G(lgnk_ctx* ctx) {
-    CK(cudaMemsetAsync(ctx->Gp, 0, ctx->vpad * ctx->slices.n * ctx->vt_bytes, ctx->stream));
+lgnk_status zero_G(lgnk_ctx* ctx, const SliceTable& tab) {
+    CK(cudaMemsetAsync(ctx->Gp, 0, ctx->vpad * tab.n * ctx->vt_bytes, ctx->stream));
     return LGNK_OK;
 }
 
@@ -415,7 +423,7 @@ lgnk_status objective_enqueue(lgnk_ctx* ctx, const float* v, const float* T, con
     int nred = trace_blocks_for(ctx, grad != nullptr ? MODE_OBJGRAD : MODE_FWD);
     if (ctx->prob.model == LGNK_TRANSPORT) {
         if (grad != nullptr) {
-            TRY(zero_G(ctx));
+            TRY(zero_G(ctx, ctx->grads));
             TRY(trace(ctx, MODE_OBJGRAD, a));
         } else {
             a.u1 = ctx->itmp;
@@ -432,7 +440,7 @@ lgnk_status objective_enqueue(lgnk_ctx* ctx, const float* v, const float* T, con
         KL(launch_residual(ctx->itmp, R, ctx->rp, ctx->ig, ctx->d, (float)ctx->cellvol, ctx->partial, nred,
                            ctx->stream));
         if (grad != nullptr) {
-            TRY(zero_G(ctx));
+            TRY(zero_G(ctx, ctx->grads));
             TraceArgs b = base_args(ctx);
             b.T = T;
             b.r = ctx->rp;
@@ -441,7 +449,7 @@ lgnk_status objective_enqueue(lgnk_ctx* ctx, const float* v, const float* T, con
     }
     KL(launch_reduce(ctx->partial, nred, ctx->dres + 0, ctx->stream));
     if (grad != nullptr) {
-        KL(launch_distribute_gradient(ctx->d, ctx->Gp, grad, ctx->vg, ctx->K, ctx->slices, 1.0f, ctx->stream));
+        KL(launch_distribute_gradient(ctx->d, ctx->Gp, grad, ctx->vg, ctx->K, ctx->grads, 1.0f, ctx->stream));
         TRY(reg_apply(ctx, v, grad, ctx->prob.alpha * ctx->wreg, 0.0, grad));
     }
     // S = 1/2 dt h_v^d v^T A_reg v
@@ -476,11 +484,11 @@ lgnk_status objective_packed(lgnk_ctx* ctx, const float* v, const float* T, cons
 // The data term of the Gauss-Newton product into the slice gradients Gp
 // (the first half of hessvec_packed).
 lgnk_status hessvec_accumulate(lgnk_ctx* ctx, const float* T, const float* dv) {
-    // packs the direction and zeroes the slice gradients in one pass
-    KL(launch_pack_velocity(ctx->d, dv, ctx->dVp, ctx->vg, ctx->K, ctx->slices, ctx->stream, ctx->Gp));
+    // packs the direction and zeroes the gradients in one pass
+    KL(launch_pack_velocity(ctx->d, dv, ctx->dVp, ctx->vg, ctx->K, ctx->slices, ctx->stream, ctx->Gp, ctx->grads.n));
     if (ctx->prob.model == LGNK_TRANSPORT) {
         TraceArgs a = base_args(ctx);
-        TRY(trace(ctx, MODE_HESS, a));
+        TRY(trace(ctx, ctx->gn_rows ? MODE_HROW : MODE_HESS, a));
     } else {
         TRY(zero_acc(ctx));
         TraceArgs a = base_args(ctx);
@@ -496,22 +504,22 @@ lgnk_status hessvec_accumulate(lgnk_ctx* ctx, const float* T, const float* dv) {
     return LGNK_OK;
 }
 
-// out = the distributed slice gradients + the regularizer's term of dv.
-lgnk_status hessvec_finish(lgnk_ctx* ctx, const float* dv, float* out) {
+// out = the distributed gradients (of the slices or nodes of tab) + the regularizer's term of dv.
+lgnk_status hessvec_finish(lgnk_ctx* ctx, const SliceTable& tab, const float* dv, float* out) {
     if (ctx->prob.regularizer == LGNK_DIFFUSION) {
         // the slice gradients' distribution, the Laplacian of dv and gamma dv in one pass
-        KL(launch_hess_finish(ctx->d, ctx->Gp, dv, out, ctx->vg, ctx->K, ctx->slices, 1.0f,
+        KL(launch_hess_finish(ctx->d, ctx->Gp, dv, out, ctx->vg, ctx->K, tab, 1.0f,
                               (float)(ctx->prob.alpha * ctx->wreg), (float)ctx->prob.gamma, nullptr, 0, nullptr,
                               nullptr, nullptr, ctx->stream));
         return LGNK_OK;
     }
-    KL(launch_distribute_gradient(ctx->d, ctx->Gp, out, ctx->vg, ctx->K, ctx->slices, 1.0f, ctx->stream));
+    KL(launch_distribute_gradient(ctx->d, ctx->Gp, out, ctx->vg, ctx->K, tab, 1.0f, ctx->stream));
     return reg_apply(ctx, dv, out, ctx->prob.alpha * ctx->wreg, ctx->prob.gamma, out);
 }
 
 lgnk_status hessvec_packed(lgnk_ctx* ctx, const float* T, const float* dv, float* out) {
     TRY(hessvec_accumulate(ctx, T, dv));
-    return hessvec_finish(ctx, dv, out);
+    return hessvec_finish(ctx, ctx->grads, dv, out);
 }
 
 EllArgs ell_args(const lgnk_ctx* ctx) {
@@ -571,7 +579,7 @@ lgnk_status assemble_enqueue(lgnk_ctx* ctx, const float* v = nullptr, const floa
     if (R != nullptr) {
         KL(launch_reduce(ctx->partial, ctx->trace_blocks, ctx->dres + 0, ctx->stream));
         // grad = J^T (h^d res) through the rows, then the regularizer
-        TRY(zero_G(ctx));
+        TRY(zero_G(ctx, ctx->slices));
         EllArgs e = ell_args(ctx);
         e.r = ctx->itmp;
         TRY(ell(ctx, ELL_JTVP, e));
@@ -622,13 +630,14 @@ lgnk_status assemble_packed(lgnk_ctx* ctx, const float* v = nullptr, const float
 }
 
 lgnk_status hessvec_assembled_accumulate(lgnk_ctx* ctx, const float* dv) {
-    KL(launch_pack_velocity(ctx->d, dv, ctx->dVp, ctx->vg, ctx->K, ctx->slices, ctx->stream, ctx->Gp));
+    KL(launch_pack_velocity(ctx->d, dv, ctx->dVp, ctx->vg, ctx->K, ctx->slices, ctx->stream, ctx->Gp,
+                            ctx->slices.n));
     return ell(ctx, ELL_HESS, ell_args(ctx));
 }
 
 lgnk_status hessvec_assembled_packed(lgnk_ctx* ctx, const float* dv, float* out) {
     TRY(hessvec_assembled_accumulate(ctx, dv));
-    return hessvec_finish(ctx, dv, out);
+    return hessvec_finish(ctx, ctx->slices, dv, out);
 }
 
 lgnk_status precond_apply(lgnk_ctx* ctx, const float* r, float* z) {
@@ -804,6 +813,16 @@ lgnk_status lgnk_create(const lgnk_problem* prob, void* stream, size_t mem_budge
     {
         const bool transport = prob->model == LGNK_TRANSPORT;
         make_slice_table(ctx->K, ctx->N, transport ? 1.0 : 0.0, (transport ? -1.0 : 1.0) / ctx->N, &ctx->slices);
+        // Gradients on the time nodes where a time cell spans at least one step
+        // (K - 1 <= N): then consecutive stages share their time cell.  With shorter
+        // time cells every stage time is in one of its own, and a slice takes half
+        // the reductions of two nodes.
+        ctx->tm = ctx->K == 1 ? TM_STEADY : (ctx->K - 1 <= ctx->N ? TM_NODES : TM_SLICES);
+        if (ctx->tm == TM_NODES) make_node_table(ctx->K, &ctx->grads);
+        else ctx->grads = ctx->slices;
+        // rows instead of a tangent sweep where they measured faster (RowScatter): 3D,
+        // stationary, and enough stages to outweigh the row's fixed cost
+        ctx->gn_rows = transport && d == 3 && ctx->K == 1 && ctx->N >= 4;
     }
     const size_t vbytes = ctx->vpad * ctx->slices.n * ctx->vt_bytes;
     const size_t pbytes = ctx->vpad * ctx->slices.n * velocity_pair_bytes(d);
@@ -939,7 +958,7 @@ lgnk_status lgnk_jtvp(lgnk_ctx* ctx, const float* v, const float* T, const float
     REQUIRE(v && T && r && gv, "v, T, r and gv must be non-NULL");
     REQUIRE(distinct(gv, {v, T, r}), "outputs must not alias inputs");
     TRY(pack_v(ctx, v, ctx->Vp));
-    TRY(zero_G(ctx));
+    TRY(zero_G(ctx, ctx->grads));
     TraceArgs a = base_args(ctx);
     if (ctx->prob.model == LGNK_TRANSPORT) {
         TRY(pack_T(ctx, T));
@@ -950,7 +969,7 @@ lgnk_status lgnk_jtvp(lgnk_ctx* ctx, const float* v, const float* T, const float
         a.r = ctx->rp;
     }
     TRY(trace(ctx, MODE_JTVP, a));
-    KL(launch_distribute_gradient(ctx->d, ctx->Gp, gv, ctx->vg, ctx->K, ctx->slices, 1.0f, ctx->stream));
+    KL(launch_distribute_gradient(ctx->d, ctx->Gp, gv, ctx->vg, ctx->K, ctx->grads, 1.0f, ctx->stream));
     return LGNK_OK;
 }
 
@@ -999,7 +1018,7 @@ lgnk_status lgnk_jtvp_assembled(lgnk_ctx* ctx, const float* r, float* gv) {
     CHECK_CTX();
     REQUIRE(r && gv && (const void*)r != (const void*)gv, "r and gv must be non-NULL and distinct");
     REQUIRE(ctx->asm_valid, "no assembled J on this context (call lgnk_assemble)");
-    TRY(zero_G(ctx));
+    TRY(zero_G(ctx, ctx->slices));
     EllArgs e = ell_args(ctx);
     e.r = r;
     TRY(ell(ctx, ELL_JTVP, e));
@@ -1158,11 +1177,11 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
         auto body = [&](bool readback) -> lgnk_status {
             TRY(use_asm ? hessvec_assembled_accumulate(ctx, p) : hessvec_accumulate(ctx, T, p));
             if (fused_finish) {
-                KL(launch_hess_finish(ctx->d, ctx->Gp, p, Hp, ctx->vg, ctx->K, ctx->slices, 1.0f,
+                KL(launch_hess_finish(ctx->d, ctx->Gp, p, Hp, ctx->vg, ctx->K, use_asm ? ctx->slices : ctx->grads, 1.0f,
                                       (float)(ctx->prob.alpha * ctx->wreg), (float)ctx->prob.gamma, ctx->partial, nb,
                                       ctx->dcounter, ctx->dres, ctx->fsc, s));
             } else {
-                TRY(hessvec_finish(ctx, p, Hp));
+                TRY(hessvec_finish(ctx, use_asm ? ctx->slices : ctx->grads, p, Hp));
                 KL(launch_dot_fused(p, Hp, nullptr, n, ctx->partial, nb, ctx->dcounter, ctx->dres, 2, 2, 0, ctx->fsc,
                                     s));
             }

@@ -40,17 +40,19 @@ __device__ __forceinline__ void split_xyz(unsigned i, unsigned nx, unsigned ny, 
 // t_m (linear in time between the K nodes) at the padded node and at its +x
 // neighbour, [v(node) | v(node + 1)], as 8 floats (3D: xyz + zero pad, twice;
 // 32 bytes) or 4 floats (2D).  One 256-bit (3D) or 128-bit (2D) load then
-// returns both x-corners of a cell row.  With Gz given, the slice gradients,
-// which share the [slice][padded node] index, are zeroed in the same pass.
+// returns both x-corners of a cell row.  With Gz given, the first nz slices of
+// the gradients, which share the [slice][padded node] index, are zeroed in the
+// same pass.
 template <int D>
 __global__ void pack_velocity_kernel(const float* __restrict__ v, float* __restrict__ Vp, DevGrid g, SliceTable tab,
-                                     void* Gz) {
+                                     void* Gz, int nz) {
     const size_t nodes = padded_size(g);
     const size_t total = nodes * tab.n;
+    const size_t zero = Gz != nullptr ? nodes * nz : 0;
     const size_t Mv = (size_t)g.m[0] * g.m[1] * g.m[2];
     constexpr int PS = (D == 3) ? 8 : 4;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        if (Gz != nullptr) {
+        if (i < zero) {
             if (D == 3) reinterpret_cast<float4*>(Gz)[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             else reinterpret_cast<float2*>(Gz)[i] = make_float2(0.0f, 0.0f);
         }
@@ -1095,11 +1097,12 @@ inline int grid_for(size_t count) {
 }  // namespace
 
 cudaError_t launch_pack_velocity(int d, const float* v, void* Vp, const DevGrid& g, int K, const SliceTable& t,
-                                 cudaStream_t s, void* Gz) {
+                                 cudaStream_t s, void* Gz, int nz) {
     (void)K;
+    if (nz > t.n) return cudaErrorInvalidValue;
     const size_t total = (size_t)g.mp[0] * g.mp[1] * g.mp[2] * t.n;
-    if (d == 3) pack_velocity_kernel<3><<<grid_for(total), kBlock, 0, s>>>(v, (float*)Vp, g, t, Gz);
-    else pack_velocity_kernel<2><<<grid_for(total), kBlock, 0, s>>>(v, (float*)Vp, g, t, Gz);
+    if (d == 3) pack_velocity_kernel<3><<<grid_for(total), kBlock, 0, s>>>(v, (float*)Vp, g, t, Gz, nz);
+    else pack_velocity_kernel<2><<<grid_for(total), kBlock, 0, s>>>(v, (float*)Vp, g, t, Gz, nz);
     return cudaGetLastError();
 }
 
@@ -1109,6 +1112,14 @@ cudaError_t launch_distribute_gradient(int d, const void* Gp, float* out, const 
     if (d == 3) distribute_gradient_kernel<3><<<grid_for(total), kBlock, 0, s>>>((const float*)Gp, out, g, K, t, scale);
     else distribute_gradient_kernel<2><<<grid_for(total), kBlock, 0, s>>>((const float*)Gp, out, g, K, t, scale);
     return cudaGetLastError();
+}
+
+void make_node_table(int K, SliceTable* t) {
+    t->n = K;
+    for (int m = 0; m < K; ++m) {
+        t->j[m] = m;
+        t->th[m] = 0.0f;
+    }
 }
 
 void make_slice_table(int K, int N, double t0, double dt, SliceTable* t) {

@@ -25,9 +25,15 @@ struct DevGrid {
     float inv_h[3];
 };
 
-enum TraceMode { MODE_FWD = 0, MODE_JVP = 1, MODE_JTVP = 2, MODE_HESS = 3, MODE_OBJGRAD = 4, MODE_ASM = 5 };
+enum TraceMode { MODE_FWD = 0, MODE_JVP = 1, MODE_JTVP = 2, MODE_HESS = 3, MODE_OBJGRAD = 4, MODE_ASM = 5, MODE_HROW = 6 };
 
-// Voxel tile of one 256-thread CTA of the tracing kernels (x, y, z).
+// Time dependence of a traced velocity.  TM_STEADY: one slice (K = 1).
+// TM_SLICES, TM_NODES: gathers read the velocity at the 2N + 1 stage times.
+// TM_SLICES also accumulates the gradient per stage time; TM_NODES accumulates
+// it on the K time nodes, each stage adding to both nodes of its time cell.
+enum TimeMode { TM_STEADY = 0, TM_SLICES = 1, TM_NODES = 2 };
+
+// Voxel tile of one CTA of the tracing kernels (x, y, z).
 inline void trace_tile_shape(int d, int* t) {
     if (d == 3) { t[0] = 8; t[1] = 8; t[2] = 4; }
     else { t[0] = 16; t[1] = 16; t[2] = 1; }
@@ -46,7 +52,7 @@ struct SliceTable {
 struct TraceArgs {
     DevGrid ig, vg;
     int K, N;
-    float dt, t0;
+    float dt, t0, dt6;        // step (negative backward in time), start time, dt / 6
     float cellvol;            // image cell volume h^d (SSD weight)
     int tiles[3];             // voxel tiles per axis (grid = product), set per launch
     // continuous velocity-grid index of the start point of voxel i along axis a:
@@ -55,8 +61,10 @@ struct TraceArgs {
     float vxi_af[3], vxi_bf[3];  // the same in FP32 (per-stage recomputation)
     float pic_rho[3];         // continuity PIC half-width in image cells per axis (0: width = cell)
     long long slice_nodes;    // padded velocity nodes per time slice
+    int tj[LGNK_MAX_SLICES];  // TM_NODES: time cell of stage time m, and the offset in it
+    float tth[LGNK_MAX_SLICES];
     const void* V;            // pair-packed velocity slices [m][zp][yp][xp] x [v(node) | v(node+1)]
-    const void* dV;           // pair-packed direction slices (JVP, HESS)
+    const void* dV;           // pair-packed direction slices (JVP, HESS, HROW)
     const float* Tp;          // padded template (gathers)
     const float* T;           // template, ABI layout (continuity particle masses)
     const float* R;           // reference, ABI layout (OBJGRAD, FWD with residual)
@@ -64,7 +72,7 @@ struct TraceArgs {
     float* u1;                // transport FWD output (ABI layout)
     float* yout;              // optional end points [d][M]
     float* acc;               // continuity splat accumulator (padded image)
-    void* G;                  // gradient accumulator slices [m][zp][yp][xp] of float4 (3D) / float2 (2D)
+    void* G;                  // gradient accumulator slices (TM_NODES: nodes) [m][zp][yp][xp] of float4 (3D) / float2 (2D)
     double* partial;          // per-block partial sums of res^2 (FP64)
     // MODE_ASM (transport): rows of the assembled J, entry-major [e][voxel]
     long long* ekey;          // element of the lower corner of the entry's cell in the slice gradient space
@@ -95,19 +103,20 @@ struct EllArgs {
 cudaError_t launch_ell(int d, int mode, const EllArgs& a, cudaStream_t s);
 
 // trace kernels (trace2d.cu / trace3d.cu)
-cudaError_t launch_trace(int d, bool nonstat, int model, int mode, const TraceArgs& a, int nblocks,
-                         cudaStream_t s);
+cudaError_t launch_trace(int d, TimeMode tm, int model, int mode, const TraceArgs& a, cudaStream_t s);
 
 // grid utilities (grid_ops.cu)
 // ABI velocity [K][d][z][y][x] -> pair-packed padded time slices
 // (velocity_pair_bytes(d) bytes per node and slice)
-// (and, when Gz is given, zero the slice gradients of the same slices and padding)
+// (and, when Gz is given, zero nz gradient slices, at most as many as t has)
 cudaError_t launch_pack_velocity(int d, const float* v, void* Vp, const DevGrid& g, int K, const SliceTable& t,
-                                 cudaStream_t s, void* Gz = nullptr);
+                                 cudaStream_t s, void* Gz = nullptr, int nz = 0);
 inline size_t velocity_pair_bytes(int d) { return d == 3 ? 32 : 16; }
 // slice gradients [m][padded nodes] -> ABI [K][d][z][y][x], out = scale * sum_m w_j(m) G_m
 cudaError_t launch_distribute_gradient(int d, const void* Gp, float* out, const DevGrid& g, int K,
                                        const SliceTable& t, float scale, cudaStream_t s);
+// the K time nodes as a table of slices (TM_NODES)
+void make_node_table(int K, SliceTable* t);
 // stage-time slices of a trace with N steps from t0 in steps dt, over K time nodes
 void make_slice_table(int K, int N, double t0, double dt, SliceTable* t);
 cudaError_t launch_pack_image(const float* T, float* Tp, const DevGrid& g, int d, float scale, cudaStream_t s);

@@ -133,6 +133,7 @@ extern "C" lgnk_status lgnk_forward_transport_static(const lgnk_problem* prob, c
     a.K = K;
     a.N = prob->rk4_steps;
     a.dt = (float)(-1.0 / prob->rk4_steps);
+    a.dt6 = a.dt / 6.0f;
     a.t0 = 1.0f;
     double cellvol = 1.0;
     for (int i = 0; i < 3; ++i) {
@@ -154,7 +155,7 @@ extern "C" lgnk_status lgnk_forward_transport_static(const lgnk_problem* prob, c
     a.R = R;
     a.u1 = u1;
     a.partial = R != nullptr ? partial : nullptr;
-    if (e == cudaSuccess) e = launch_trace(d, K > 1, LGNK_TRANSPORT, MODE_FWD, a, nblocks, s);
+    if (e == cudaSuccess) e = launch_trace(d, K > 1 ? TM_SLICES : TM_STEADY, LGNK_TRANSPORT, MODE_FWD, a, s);
     if (e == cudaSuccess && R != nullptr) {
         e = launch_reduce(partial, nblocks, sum, s);
         if (e == cudaSuccess) {

@@ -8,11 +8,15 @@
 //   JVP      trace with the forward-mode derivative of Alg. 1 applied to dv,
 //            then du = grad T(y) . dy (transport) or the splat of
 //            T(x_c) grad_y w . dy (continuity) (Sec. 3.2).
-//   JTVP     trace storing the step starts, seed the adjoint at the end point,
-//            sweep the RK4 steps backwards scattering into the gradient.
+//   JTVP     trace recording the stages, seed the adjoint at the end point,
+//            sweep the RK4 stages backwards scattering into the gradient.
 //   HESS     transport only: the Gauss-Newton product J^T h^d J dv fused per
 //            voxel (u1 at voxel i depends only on characteristic i, so the
 //            JVP value feeds that voxel's JTVP seed directly).
+//   HROW     the same product by rows (3D, stationary velocity): the adjoint
+//            sweep seeded with grad T(y_i) yields the row J_i as a few blocks of
+//            corner vectors; they are dotted with dv and scattered scaled by
+//            h^d J_i dv (RowScatter).
 //   OBJGRAD  transport only: u1, SSD partials and the JTVP of h^d res fused.
 //   ASM      transport only: the adjoint sweep seeded with grad T(y) yields
 //            row i of J = d_v u1 (Sec. 3.3 assembles J as a sparse matrix);
@@ -30,11 +34,19 @@
 // exact evaluation.
 //
 // Jacobian-free derivative products.  d_y I(v, y) enters only as J q (tangent)
-// and J^T mu (adjoint).  The interpolant is evaluated separably, one plane of
-// four corners at a time (x then y lerps, then z): the same lerps give the
-// value and the three axis derivatives, J q contracts them with q, and J^T mu
-// is the gradient of the scalar interpolant of v . mu (corners contracted with
-// mu first).  No d x d matrix lives in registers.
+// and J^T mu (adjoint), the gradient of the scalar interpolant of v . mu
+// (coefficients contracted with mu first).  No d x d matrix lives in registers.
+//
+// Cells in registers.  A stage evaluates the interpolant of its velocity cell
+// from registers and reads memory only when the cell or the stage's time slice
+// changes; the adjoint's contributions to a cell are summed in registers (in
+// moment form) and leave them only when the cell changes.
+//
+// What bounds these kernels: first the issue slots, now latency.  Paired FP32
+// instructions, the row form of the Gauss-Newton product and the floor without
+// conversions took the 128^3 product from 495M to 336M warp instructions (issue
+// slots 0.70 -> 0.58 busy) and from 554 to 466 us; what the warps wait for is
+// the cell's corners after a change (long scoreboard, at 16 warps per SM).
 //
 // Time slices.  Every RK4 stage time is t0 + m dt/2 (m = 0..2N), so the host
 // packs the velocity (and the direction) at those 2N + 1 times, linearly
@@ -43,13 +55,20 @@
 // a stationary one (K = 1: a single slice), and no time interpolation happens
 // in the kernels.
 //
-// Gradient scatter.  (d_v I)^T mu goes to the padded gradient accumulator of
-// the stage's slice with one vector reduction (red.global.add.v4.f32 / .v2)
-// per corner, executed by the L2 atomic units; consecutive stages in the same
-// cell and slice are combined first.  The host then distributes the slices
-// onto the K time nodes with the transposed time weights.  A shared-memory tile of the velocity grid was measured
-// slower: float atomics on shared memory retry under the heavy same-address
-// contention of neighbouring characteristics.
+// Gradient scatter.  (d_v I)^T mu goes to the padded gradient accumulator with
+// one vector reduction (red.global.add.v4.f32 / .v2) per corner of a finished
+// block, executed by the L2 atomic units.  With K - 1 <= N the accumulator has
+// the K time nodes (TM_NODES): a stage adds to the blocks of both nodes of its
+// time cell, which at least one whole step shares, and a node's block is
+// reduced once per cell.  Per stage time (TM_SLICES) it would be reduced at
+// every second stage; measured on the brain-scale J^T (K = 9, N = 16) 7.8 ms
+// with slices against 6.2 ms with nodes, and on the 128 x 150 x 128 product
+// with K = 2, N = 5 1058 against 870 us (both with the other changes here).
+// With shorter time cells (K - 1 > N) every stage time has two nodes of its own
+// and the slices take half the reductions; a streaming kernel then distributes
+// them onto the time nodes with the transposed time weights.  A shared-memory
+// tile of the velocity grid was measured slower: float atomics on shared memory
+// retry under the heavy same-address contention of neighbouring characteristics.
 #pragma once
 
 #include <type_traits>
@@ -58,6 +77,48 @@
 #include "lgnk_internal.h"
 
 namespace lgnk {
+
+// Paired FP32 arithmetic: two values in one 64-bit register, one instruction
+// for both (each half rounds as the scalar instruction does).  The tracing
+// kernels are bound by issue slots, not by the FP32 lanes, so a pair costs
+// half the slots of two scalars.  The pairs used below are the two x-corners
+// (or the two coefficients that differ by a factor f_x) of one component:
+// they leave poly_coeffs, the moment sums and poly_value as pairs and are
+// never repacked inside a stage; only f_y, f_z and mu are duplicated.
+using pair2 = unsigned long long;
+__device__ __forceinline__ pair2 pk(float lo, float hi) {
+    pair2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpk(pair2 p, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p));
+}
+__device__ __forceinline__ float lo2(pair2 p) {
+    float a, b;
+    unpk(p, a, b);
+    return a;
+}
+__device__ __forceinline__ float hi2(pair2 p) {
+    float a, b;
+    unpk(p, a, b);
+    return b;
+}
+__device__ __forceinline__ pair2 fma2(pair2 a, pair2 b, pair2 c) {
+    pair2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ pair2 mul2(pair2 a, pair2 b) {
+    pair2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ pair2 sub2(pair2 a, pair2 b) {
+    pair2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 
 template <int D> struct VecT;
 template <> struct VecT<2> { using type = float2; };
@@ -74,8 +135,7 @@ template <int D> struct TileShape;
 template <> struct TileShape<2> { static constexpr int X = 16, Y = 16, Z = 1; };
 template <> struct TileShape<3> { static constexpr int X = 8, Y = 8, Z = 4; };
 
-// Voxel handled by this thread (recomputed from the block and thread indices
-// where needed rather than held in registers).
+// Voxel handled by this thread.
 template <int D>
 __device__ __forceinline__ void voxel_index(const TraceArgs& A, int* idx) {
     using TS = TileShape<D>;
@@ -108,25 +168,64 @@ __device__ __forceinline__ void start_on_image(const int* idx, Start<D>& s) {
     }
 }
 
-// Start of this thread's characteristic on the velocity grid:
+// Floor of t as floor(t) + kFloorMagic: adding 1.5 2^23 rounded down leaves
+// the integer in the low mantissa bits (|t| < 2^22; grids have at most 2^20
+// cells per axis), on the FP32 pipe, where floorf and the conversion to an
+// integer take two instructions of the quarter-rate conversion unit.
+constexpr float kFloorMagic = 12582912.0f;
+constexpr int kFloorMagicBits = 0x4B400000;
+
+// This thread's characteristic on the velocity grid, held for the whole trace:
+// the fraction F0 of its start's continuous index, the clamps of the offset
+// t = F0 + u / h (to [-2 - I0, m - I0 + 1/2], which keeps the lower corner in
+// [-2, m]) and the constant of the linear cell index.
+template <int D>
+struct VelocityStart {
+    float F0[D], lo[D], hi[D];
+    unsigned c;
+};
+
 // (x_c - lo_v) / h_v - 1/2 = vxi_a + (i + 1/2) vxi_b, evaluated in FP32 (one
 // rounding, below 1e-5 cells for grids up to 2^7 cells).
 template <int D>
-__device__ __forceinline__ void start_on_velocity(const TraceArgs& A, Start<D>& s) {
-    int idx[3];
-    voxel_index<D>(A, idx);
+__device__ __forceinline__ void start_on_velocity(const TraceArgs& A, const int* idx, VelocityStart<D>& s) {
+    unsigned st = 1;
+    s.c = 0;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
         const float xi = fmaf((float)idx[a] + 0.5f, A.vxi_bf[a], A.vxi_af[a]);
         const int i0 = min(max((int)floorf(xi), -2), A.vg.m[a]);
-        s.I0[a] = i0;
         s.F0[a] = xi - (float)i0;
+        s.lo[a] = (float)(-2 - i0);
+        s.hi[a] = (float)(A.vg.m[a] - i0) + 0.5f;
+        s.c += st * (unsigned)(i0 + LGNK_PAD - kFloorMagicBits);
+        st *= (unsigned)A.vg.mp[a];
     }
 }
 
-// Cell of the point at displacement u from the start: per-axis padded index p
-// of the lower corner and fractional offsets f in [0, 1].  NaN maps to the
-// lowest clamp, so any point addresses padded storage.
+// Cell of the point at displacement u from the start, on the velocity grid:
+// its linear padded index, and the fractional offsets f in [0, 1].  NaN maps
+// to the lowest clamp, so any point addresses padded storage.  (The index
+// arithmetic wraps: the magic's bits cancel against s.c.)
+template <int D>
+__device__ __forceinline__ int locate_velocity(const DevGrid& g, const VelocityStart<D>& s, const float* u, float* f) {
+    unsigned b = 0;
+    unsigned k[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        float t = fmaf(u[a], g.inv_h[a], s.F0[a]);
+        t = fminf(fmaxf(t, s.lo[a]), s.hi[a]);
+        const float r = __fadd_rd(t, kFloorMagic);
+        f[a] = t - (r - kFloorMagic);
+        k[a] = __float_as_uint(r);
+    }
+    if (D == 3) b = k[0] + (unsigned)g.mp[0] * (k[1] + (unsigned)g.mp[1] * k[D - 1]);
+    else b = k[0] + (unsigned)g.mp[0] * k[1];
+    return (int)(b + s.c);
+}
+
+// Cell of a point on a grid from the start's split index (the image at the
+// end of the trace): per-axis padded index p of the lower corner, offsets f.
 template <int D>
 __device__ __forceinline__ void locate(const DevGrid& g, const Start<D>& s, const float* u, int* p, float* f) {
 #pragma unroll
@@ -193,8 +292,6 @@ __device__ __forceinline__ void pair_value(const float* __restrict__ V, size_t e
     }
 }
 
-__device__ __forceinline__ float lerp(float a, float b, float t) { return fmaf(t, b - a, a); }
-
 // Element of corner (0, cy, cz) of the cell with lower corner `base` in the
 // slice starting at element `s0`.
 template <int D>
@@ -204,99 +301,6 @@ __device__ __forceinline__ size_t corner_elem(const DevGrid& g, size_t s0, int b
     return s0 + (size_t)o;
 }
 
-// One plane (fixed z corner) of the cell: bilinear value and the unscaled
-// derivatives along the fractional x and y offsets, per component.
-template <int D, bool GRAD>
-__device__ __forceinline__ void plane(const DevGrid& g, const float* __restrict__ V, size_t s0, int base, int cz,
-                                      const float* f, float* val, float* dx, float* dy) {
-    float c00[3], c10[3], c01[3], c11[3];
-    pair_value<D>(V, corner_elem<D>(g, s0, base, 0, 0, cz), c00, c10);
-    pair_value<D>(V, corner_elem<D>(g, s0, base, 0, 1, cz), c01, c11);
-#pragma unroll
-    for (int q = 0; q < D; ++q) {
-        const float a0 = lerp(c00[q], c10[q], f[0]);
-        const float a1 = lerp(c01[q], c11[q], f[0]);
-        val[q] = lerp(a0, a1, f[1]);
-        if (GRAD) {
-            dx[q] = lerp(c10[q] - c00[q], c11[q] - c01[q], f[1]);
-            dy[q] = a1 - a0;
-        }
-    }
-}
-
-// Scalar version: corner values contracted with mu first (s_c = v_c . mu).
-template <int D>
-__device__ __forceinline__ void plane_dot(const DevGrid& g, const float* __restrict__ V, size_t s0, int base, int cz,
-                                          const float* f, const float* mu, float& val, float& dx, float& dy) {
-    float c[4];
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        float a[3], b[3];
-        pair_value<D>(V, corner_elem<D>(g, s0, base, 0, r, cz), a, b);
-        float sa = 0.0f, sb = 0.0f;
-#pragma unroll
-        for (int q = 0; q < D; ++q) {
-            sa = fmaf(a[q], mu[q], sa);
-            sb = fmaf(b[q], mu[q], sb);
-        }
-        c[2 * r] = sa;
-        c[2 * r + 1] = sb;
-    }
-    const float a0 = lerp(c[0], c[1], f[0]);
-    const float a1 = lerp(c[2], c[3], f[0]);
-    val = lerp(a0, a1, f[1]);
-    dx = lerp(c[1] - c[0], c[3] - c[2], f[1]);
-    dy = a1 - a0;
-}
-
-// val = I(v, y, t) at the slice of t (Sec. 3.1, Step 1: multilinear in space,
-// linear in time through the slice).
-template <int D>
-__device__ __forceinline__ void stage_value(const DevGrid& g, const float* __restrict__ V, size_t s0, const int* p,
-                                            const float* f, float* val) {
-    const int base = linear<D>(g, p);
-    plane<D, false>(g, V, s0, base, 0, f, val, nullptr, nullptr);
-    if (D == 3) {
-        float v1[D];
-        plane<D, false>(g, V, s0, base, 1, f, v1, nullptr, nullptr);
-#pragma unroll
-        for (int q = 0; q < D; ++q) val[q] = lerp(val[q], v1[q], f[D - 1]);
-    }
-}
-
-// Tangent stage: val = I(v, y, t), Jq = d_y I(v, y, t) q, dval = I(dv, y, t).
-template <int D>
-__device__ __forceinline__ void stage_tangent(const DevGrid& g, const float* __restrict__ V,
-                                              const float* __restrict__ dV, size_t s0, const int* p, const float* f,
-                                              const float* qv, float* val, float* Jq, float* dval) {
-    const int base = linear<D>(g, p);
-    float qs[D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) qs[a] = qv[a] * g.inv_h[a];
-    float dx[D], dy[D];
-    plane<D, true>(g, V, s0, base, 0, f, val, dx, dy);
-    if (D == 3) {
-        float v1[D], dx1[D], dy1[D];
-        plane<D, true>(g, V, s0, base, 1, f, v1, dx1, dy1);
-#pragma unroll
-        for (int q = 0; q < D; ++q) {
-            const float dz = v1[q] - val[q];
-            Jq[q] = dz * qs[D - 1];
-            val[q] = lerp(val[q], v1[q], f[D - 1]);
-            dx[q] = lerp(dx[q], dx1[q], f[D - 1]);
-            dy[q] = lerp(dy[q], dy1[q], f[D - 1]);
-        }
-    } else {
-#pragma unroll
-        for (int q = 0; q < D; ++q) Jq[q] = 0.0f;
-    }
-#pragma unroll
-    for (int q = 0; q < D; ++q) Jq[q] = fmaf(dx[q], qs[0], fmaf(dy[q], qs[1], Jq[q]));
-    stage_value<D>(g, dV, s0, p, f, dval);
-}
-
-// Destination of the adjoint scatter (d_v I)^T mu: the padded gradient
-// accumulator of each slice, with a one-entry write-combining slot.
 // A pending cell block in moment form.  The block's corner vectors are
 // sum_stages w_c(f) mu with w_c = prod_a (c_a ? f_a : 1 - f_a); expanding the
 // product, they follow from the moments m_k = sum_stages phi_k(f) mu, phi_k =
@@ -306,156 +310,261 @@ __device__ __forceinline__ void stage_tangent(const DevGrid& g, const float* __r
 // products of offsets, D adds and (2^d - 1) D FMAs (3D: 4 FMUL, 3 FADD, 21
 // FFMA) instead of the corner weights and (2^d) D FMAs (12 FMUL, 3 FADD, 24
 // FFMA); the conversion (12 FADD per component in 3D) is paid once per block.
-// Blocks are flat, m[k D + q].
+// Blocks are held as pairs over the x axis, m[q][j] = (m_2j, m_2j+1) of
+// component q.
 template <int D>
-__device__ __forceinline__ void moments_add(float* m, const float* f, const float* mu) {
-    float phi[1 << D];
-    phi[1] = f[0];
-    phi[2] = f[1];
-    phi[3] = f[0] * f[1];
-    if (D == 3) {
-        phi[4] = f[D - 1];
-        phi[5] = f[0] * f[D - 1];
-        phi[6] = f[1] * f[D - 1];
-        phi[7] = phi[3] * f[D - 1];
-    }
-#pragma unroll
-    for (int q = 0; q < D; ++q) m[q] += mu[q];
-#pragma unroll
-    for (int k = 1; k < (1 << D); ++k)
-#pragma unroll
-        for (int q = 0; q < D; ++q) m[k * D + q] = fmaf(phi[k], mu[q], m[k * D + q]);
-}
-
-// Moments to corner vectors, in place.
-template <int D>
-__device__ __forceinline__ void moments_to_corners(float* m) {
-#pragma unroll
-    for (int b = 1; b < (1 << D); b <<= 1)
-#pragma unroll
-        for (int k = 0; k < (1 << D); ++k)
-            if (!(k & b)) {
-#pragma unroll
-                for (int q = 0; q < D; ++q) m[k * D + q] -= m[(k | b) * D + q];
-            }
-}
-
-template <int D>
-__device__ __forceinline__ void block_zero(float* m) {
-#pragma unroll
-    for (int k = 0; k < (1 << D) * D; ++k) m[k] = 0.0f;
-}
-
-// Consecutive adjoint stages of a characteristic usually fall in the same
-// velocity cell and slice; their contributions w_c(f) mu are then summed per
-// corner and sent as one vector reduction instead of two.
-template <int D>
-struct Scatter {
-    typename VecT<D>::type* G;
-    size_t s0;      // slice of the pending contribution
-    int base;       // its cell, -1 if none
-    float f[D];
-    float mu[D];
+struct Block {
+    static constexpr int NP = 1 << (D - 1);     // pairs per component
+    pair2 m[D][NP];
 };
 
 template <int D>
-__device__ __forceinline__ void scatter_flush(const DevGrid& g, Scatter<D>& S, bool two, const float* f2,
-                                              const float* mu2) {
+__device__ __forceinline__ void moments_add(Block<D>& B, const float* f, const float* mu) {
+    constexpr int NP = Block<D>::NP;
+    pair2 phi[NP];
+    phi[0] = pk(1.0f, f[0]);
+    phi[1] = mul2(pk(f[1], f[1]), phi[0]);
+    if (D == 3) {
+        const pair2 fz = pk(f[D - 1], f[D - 1]);
+        phi[NP / 2] = mul2(fz, phi[0]);
+        phi[NP - 1] = mul2(fz, phi[1]);
+    }
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+        const pair2 w = pk(mu[q], mu[q]);
+#pragma unroll
+        for (int k = 0; k < NP; ++k) B.m[q][k] = fma2(phi[k], w, B.m[q][k]);
+    }
+}
+
+// Moments to corner vectors, in place: afterwards m[q][j] holds corners
+// (0, cy, cz) and (1, cy, cz), j = cy + 2 cz.
+template <int D>
+__device__ __forceinline__ void moments_to_corners(Block<D>& B) {
+    constexpr int NP = Block<D>::NP;
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            float a, b;
+            unpk(B.m[q][k], a, b);
+            B.m[q][k] = pk(a - b, b);
+        }
+#pragma unroll
+        for (int b = 1; b < NP; b <<= 1)
+#pragma unroll
+            for (int k = 0; k < NP; ++k)
+                if (!(k & b)) B.m[q][k] = sub2(B.m[q][k], B.m[q][k | b]);
+    }
+}
+
+template <int D>
+__device__ __forceinline__ void block_zero(Block<D>& B) {
+#pragma unroll
+    for (int q = 0; q < D; ++q)
+#pragma unroll
+        for (int k = 0; k < Block<D>::NP; ++k) B.m[q][k] = 0;
+}
+
+// Corner c of a block of corner vectors.
+template <int D>
+__device__ __forceinline__ void block_corner(const Block<D>& B, int c, float* x) {
+#pragma unroll
+    for (int q = 0; q < D; ++q) x[q] = (c & 1) ? hi2(B.m[q][c >> 1]) : lo2(B.m[q][c >> 1]);
+}
+
+// Adds w times a block of corner vectors at cell `key` to the gradients.
+template <int D>
+__device__ __forceinline__ void block_red(const DevGrid& g, typename VecT<D>::type* G, int key, const Block<D>& B,
+                                          float w) {
 #pragma unroll
     for (int c = 0; c < (1 << D); ++c) {
-        float w = (c & 1 ? S.f[0] : 1.0f - S.f[0]) * ((c >> 1) & 1 ? S.f[1] : 1.0f - S.f[1]);
-        if (D == 3) w *= ((c >> 2) & 1) ? S.f[D - 1] : 1.0f - S.f[D - 1];
-        float w2 = 0.0f;
-        if (two) {
-            w2 = (c & 1 ? f2[0] : 1.0f - f2[0]) * ((c >> 1) & 1 ? f2[1] : 1.0f - f2[1]);
-            if (D == 3) w2 *= ((c >> 2) & 1) ? f2[D - 1] : 1.0f - f2[D - 1];
-        }
-        const size_t e = corner_elem<D>(g, S.s0, S.base, c & 1, (c >> 1) & 1, (c >> 2) & 1);
         float x[D];
-#pragma unroll
-        for (int q = 0; q < D; ++q) x[q] = fmaf(w2, two ? mu2[q] : 0.0f, w * S.mu[q]);
-        red_vec(S.G + e, x, 1.0f);
-    }
-    S.base = -1;
-}
-
-// Add the contribution w_c(f) mu at cell `base` of slice `s0`.
-template <int D>
-__device__ __forceinline__ void scatter_add(const DevGrid& g, Scatter<D>& S, size_t s0, int base, const float* f,
-                                            const float* mu) {
-    if (S.base == base && S.s0 == s0) {
-        scatter_flush<D>(g, S, true, f, mu);
-        return;
-    }
-    if (S.base >= 0) scatter_flush<D>(g, S, false, f, mu);
-    S.base = base;
-    S.s0 = s0;
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        S.f[a] = f[a];
-        S.mu[a] = mu[a];
+        block_corner<D>(B, c, x);
+        red_vec(G + corner_elem<D>(g, (size_t)key, 0, c & 1, (c >> 1) & 1, (c >> 2) & 1), x, w);
     }
 }
 
-template <int D>
-__device__ __forceinline__ void scatter_init(Scatter<D>& S, void* G) {
-    S.G = static_cast<typename VecT<D>::type*>(G);
-    S.base = -1;
-    S.s0 = 0;
-}
+// Destinations of the adjoint contributions w_c(f) mu.  The pending cell stays
+// in registers (in moment form) and leaves them only when a stage falls in
+// another cell (`emit`).  In time-node mode (NB = 2) a stage contributes to
+// both nodes of its time cell, (1 - th) w_c mu to the block of node j and th w_c
+// mu to that of node j + 1; node j's block is blk[j mod 2], so that when the
+// sweep moves on to the next time cell one node is finished and the other's
+// block stays where it is.  All keys are 32-bit element offsets (the packed
+// velocity has fewer than 2^31 elements: checked when the context is created).
 
-template <int D>
-__device__ __forceinline__ void scatter_finish(const DevGrid& g, Scatter<D>& S) {
-    if (S.base >= 0) scatter_flush<D>(g, S, false, S.f, S.mu);
-}
-
-// Destination of the adjoint scatter with the whole pending cell in
-// registers: the contributions w_c(f) mu of consecutive stages in one cell and
-// slice are accumulated (in moment form) and sent as 2^d vector reductions
-// only when the cell or slice changes (the transport matvec, where
-// consecutive stages mostly share a cell).  The block is zeroed inside the
-// flush, so that a stage's update is the same FMAs whether it opens a block or
-// not: written as "fresh ? w mu : w mu + blk", the compiler evaluated both and
-// selected, 24 FMULs and 24 selects per stage (the 128^3 matvec kernel went
-// 0.630 -> 0.586 ms with both changes, the assembly 0.653 -> 0.627 ms).
-template <int D>
+// Gradients and J^T r: the block's corners go to the slice (node) gradients
+// with one vector reduction each.
+template <int D, int NB>
 struct BlockScatter {
     typename VecT<D>::type* G;
-    int key;                  // s0 + base of the pending cell, -1 if none (the packed velocity has
-                              // fewer than 2^31 elements: checked when the context is created)
-    float blk[(1 << D) * D];
+    int key, odd, sn;         // cell of the pending block(s) at its (earlier) node, -1 if none; NB = 2: that
+                              // node's parity; elements per node
+    Block<D> blk[NB];
 };
 
-template <int D>
-__device__ __forceinline__ void scatter_init(BlockScatter<D>& S, void* G) {
-    S.G = static_cast<typename VecT<D>::type*>(G);
-    S.key = -1;
-    block_zero<D>(S.blk);
+template <int D, int NB>
+__device__ __forceinline__ void scatter_emit(const DevGrid& g, BlockScatter<D, NB>& S, int b, int key) {
+    moments_to_corners<D>(S.blk[b]);
+    block_red<D>(g, S.G, key, S.blk[b], 1.0f);
 }
 
+// The fused Gauss-Newton product by rows (MODE_HROW).  Row i of J is the adjoint
+// sweep seeded with grad T(y_i), so one sweep yields both J_i dv (the blocks
+// dotted with the direction's corners) and, scaled by h^d J_i dv, the row's
+// contribution to J^T h^d J dv.  The blocks are kept until the dot product is
+// known: the last in registers, the earlier ones (a trajectory leaves its
+// velocity cell 0.4 times on average on the 128^3 workload) in a per-thread
+// local array.  A row with more than CAP earlier blocks is swept a second time
+// (`direct`) with the scaled seed and then scatters as the gradient does.
+// Against a tangent sweep for J dv (MODE_HESS) this drops the direction's
+// interpolation and the products d_y I q at every stage, 390 instead of 615
+// FP32 operations per voxel-step, and adds the blocks' way through local
+// memory once per row: at 128^3 0.447 against 0.513 ms with N = 8, 0.279 against
+// 0.293 ms with N = 4, but 0.200 against 0.190 ms with N = 2 (64 x 60 x 62:
+// 61 / 70, 39 / 43, 30.5 / 28.6 us).  It stays with the tangent sweep in 2D (cheap
+// stages: 10 to 20% slower by rows) and for K > 1 (a block per time node and
+// cell: 5 to 40% slower).
+template <int D, int NB>
+struct RowScatter {
+    static constexpr int CAP = 6;
+    static constexpr int NV = (1 << D) * D / 4;      // float4s of a block
+    typename VecT<D>::type* G;
+    int key, odd, sn, n;
+    bool direct;
+    float du;                 // of the blocks that were not kept
+    const float* dV;
+    float4* st;               // [CAP][NV], moments
+    int* stkey;               // [CAP]
+    Block<D> blk[NB];
+};
+
+// The block of corner vectors . the direction at cell `key`
 template <int D>
-__device__ __forceinline__ void block_flush(const DevGrid& g, BlockScatter<D>& S) {
-    moments_to_corners<D>(S.blk);
+__device__ __forceinline__ float block_dot(const DevGrid& g, const float* __restrict__ dV, int key,
+                                           const Block<D>& B) {
+    float s = 0.0f;
 #pragma unroll
-    for (int c = 0; c < (1 << D); ++c)
-        red_vec(S.G + corner_elem<D>(g, (size_t)S.key, 0, c & 1, (c >> 1) & 1, (c >> 2) & 1), S.blk + c * D, 1.0f);
-    block_zero<D>(S.blk);
-}
-
-template <int D>
-__device__ __forceinline__ void scatter_finish(const DevGrid& g, BlockScatter<D>& S) {
-    if (S.key >= 0) block_flush<D>(g, S);
-}
-
-template <int D>
-__device__ __forceinline__ void scatter_add(const DevGrid& g, BlockScatter<D>& S, size_t s0, int base, const float* f,
-                                            const float* mu) {
-    const int key = (int)s0 + base;
-    if (key != S.key) {
-        if (S.key >= 0) block_flush<D>(g, S);
-        S.key = key;
+    for (int j = 0; j < Block<D>::NP; ++j) {
+        float lo[3], hi[3];
+        pair_value<D>(dV, corner_elem<D>(g, (size_t)key, 0, 0, j & 1, j >> 1), lo, hi);
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+            float a, b;
+            unpk(B.m[q][j], a, b);
+            s = fmaf(a, lo[q], s);
+            s = fmaf(b, hi[q], s);
+        }
     }
-    moments_add<D>(S.blk, f, mu);
+    return s;
+}
+
+template <int D>
+__device__ __forceinline__ void block_store(float4* dst, const Block<D>& B) {
+    constexpr int NP = Block<D>::NP, NV = (1 << D) * D / 4;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        float a[4];
+        unpk(B.m[(2 * v) / NP][(2 * v) % NP], a[0], a[1]);
+        unpk(B.m[(2 * v + 1) / NP][(2 * v + 1) % NP], a[2], a[3]);
+        dst[v] = make_float4(a[0], a[1], a[2], a[3]);
+    }
+}
+
+template <int D>
+__device__ __forceinline__ void block_load(const float4* src, Block<D>& B) {
+    constexpr int NP = Block<D>::NP, NV = (1 << D) * D / 4;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        const float4 t = src[v];
+        B.m[(2 * v) / NP][(2 * v) % NP] = pk(t.x, t.y);
+        B.m[(2 * v + 1) / NP][(2 * v + 1) % NP] = pk(t.z, t.w);
+    }
+}
+
+template <int D, int NB>
+__device__ __forceinline__ void scatter_emit(const DevGrid& g, RowScatter<D, NB>& S, int b, int key) {
+    if (S.direct) {
+        moments_to_corners<D>(S.blk[b]);
+        block_red<D>(g, S.G, key, S.blk[b], 1.0f);
+    } else {
+        if (S.n < RowScatter<D, NB>::CAP) {
+            // converted and dotted after the sweep, where the warp's lanes are together again
+            block_store<D>(S.st + S.n * RowScatter<D, NB>::NV, S.blk[b]);
+            S.stkey[S.n] = key;
+        } else {
+            moments_to_corners<D>(S.blk[b]);
+            S.du += block_dot<D>(g, S.dV, key, S.blk[b]);
+        }
+        S.n++;
+    }
+}
+
+template <int D, int NB, template <int, int> class SC>
+__device__ __forceinline__ void scatter_init(SC<D, NB>& S, void* G, int sn) {
+    S.G = static_cast<typename VecT<D>::type*>(G);
+    S.sn = sn;
+    S.key = -1;
+    S.odd = 0;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) block_zero<D>(S.blk[b]);
+}
+
+// Element of the cell whose pending contributions blk[b] holds.
+template <int D, int NB, template <int, int> class SC>
+__device__ __forceinline__ int block_key(const SC<D, NB>& S, int b) {
+    return NB == 2 && b != S.odd ? S.key + S.sn : S.key;
+}
+
+template <int D, int NB, template <int, int> class SC>
+__device__ __forceinline__ void block_out(const DevGrid& g, SC<D, NB>& S, int b) {
+    scatter_emit(g, S, b, block_key(S, b));
+    block_zero<D>(S.blk[b]);
+}
+
+// Every pending block out.
+template <int D, int NB, template <int, int> class SC>
+__device__ __forceinline__ void scatter_finish(const DevGrid& g, SC<D, NB>& S) {
+    if (S.key < 0) return;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) block_out(g, S, b);
+}
+
+template <int D, int NB, template <int, int> class SC>
+__device__ __forceinline__ void scatter_cell(const DevGrid& g, SC<D, NB>& S, int key, int odd) {
+    if (key == S.key) return;
+    if (S.key >= 0) {
+        // the finished nodes: one of the two if only the time cell moved on by one
+        const bool later = key == S.key + S.sn, earlier = key == S.key - S.sn;
+        if (NB == 1 || !later || S.odd != 0)
+            if (NB == 1 || !earlier || S.odd == 0) block_out(g, S, NB - 1);
+        if (NB == 2)
+            if ((!later || S.odd == 0) && (!earlier || S.odd != 0)) block_out(g, S, 0);
+    }
+    S.key = key;
+    S.odd = odd;
+}
+
+// Add the contribution w_c(f) mu at cell `key` (NB = 2: of the earlier node,
+// whose parity is odd, with the time offset th).
+template <int D, int NB, template <int, int> class SC>
+__device__ __forceinline__ void scatter_add(const DevGrid& g, SC<D, NB>& S, int key, int odd, float th, const float* f,
+                                            const float* mu) {
+    scatter_cell(g, S, key, odd);
+    if (NB == 1) {
+        moments_add<D>(S.blk[0], f, mu);
+    } else {
+        const float t1 = odd ? 1.0f - th : th;      // weight of the odd node
+        float m1[D], m0[D];
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+            m1[q] = t1 * mu[q];
+            m0[q] = mu[q] - m1[q];
+        }
+        moments_add<D>(S.blk[0], f, m0);
+        moments_add<D>(S.blk[NB - 1], f, m1);
+    }
 }
 
 // Destination of the adjoint contributions when a row of J is assembled: the
@@ -473,35 +582,31 @@ struct AsmTable {
     bool overflow;
 };
 
-// The block of the current cell is kept in registers (pblk) until the cell
-// changes; it is then committed to the row (kept in the table's local array
-// it was placed in local memory: 1.23 ms for the 128^3 assembly, 0.79 ms apart).
-template <int D>
+// The block of the current cell is kept in registers until the cell changes;
+// it is then committed to the row (kept in the table's local array it was
+// placed in local memory: 1.23 ms for the 128^3 assembly, 0.79 ms apart).
+template <int D, int NB>
 struct AsmRow {
-    static constexpr int CAP = AsmTable<D>::CAP;
     static constexpr int B = (1 << D) * D;
+    typename VecT<D>::type* G;
     AsmTable<D>* tab;
-    float* blk;               // entry 0 of this voxel's blocks in the ELL array
+    float* row;               // entry 0 of this voxel's blocks in the ELL array
     size_t stride;            // floats from entry j to entry j + 1 of one voxel
-    long long pkey;
-    float pblk[B];
+    int key, odd, sn;
+    Block<D> blk[NB];
 };
 
-template <int D>
-__device__ __forceinline__ void scatter_init(AsmRow<D>& S, void*) {
-    S.pkey = -1;
-    block_zero<D>(S.pblk);
-}
-
-// The pending block's corner vectors into the row (asm_commit).
-template <int D>
-__device__ __forceinline__ void asm_store(AsmRow<D>& S) {
-    constexpr int B = AsmRow<D>::B;
+// Adds the pending block to the row's entry of its cell (a new entry if the
+// row has none yet).
+template <int D, int NB>
+__device__ __forceinline__ void scatter_emit(const DevGrid&, AsmRow<D, NB>& S, int b, int key) {
+    constexpr int B = AsmRow<D, NB>::B;
     AsmTable<D>& T = *S.tab;
+    moments_to_corners<D>(S.blk[b]);
     int j = T.n - 1;
 #pragma unroll 1
     for (; j >= 0; --j)       // newest first: a trajectory revisits the cell it just left
-        if (T.key[j] == S.pkey) break;
+        if (T.key[j] == key) break;
     const bool fresh = j < 0;
     if (fresh) {
         if (T.n == AsmTable<D>::CAP) {
@@ -509,220 +614,208 @@ __device__ __forceinline__ void asm_store(AsmRow<D>& S) {
             return;
         }
         j = T.n++;
-        T.key[j] = S.pkey;
+        T.key[j] = key;
     }
-    float4* dst = reinterpret_cast<float4*>(S.blk + (size_t)j * S.stride);
+    float x[B];               // [corner][component]
+#pragma unroll
+    for (int c = 0; c < (1 << D); ++c) block_corner<D>(S.blk[b], c, x + c * D);
+    float4* dst = reinterpret_cast<float4*>(S.row + (size_t)j * S.stride);
 #pragma unroll
     for (int k = 0; k < B / 4; ++k) {
-        float4 b = make_float4(S.pblk[4 * k], S.pblk[4 * k + 1], S.pblk[4 * k + 2], S.pblk[4 * k + 3]);
+        float4 w = make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
         if (!fresh) {
             const float4 o = dst[k];
-            b.x += o.x;
-            b.y += o.y;
-            b.z += o.z;
-            b.w += o.w;
+            w.x += o.x;
+            w.y += o.y;
+            w.z += o.z;
+            w.w += o.w;
         }
-        dst[k] = b;
+        dst[k] = w;
     }
 }
 
-// Add the pending block (moments, converted here to corner vectors) to the
-// row's entry of its cell (a new entry if the row has none yet), and zero it.
-template <int D>
-__device__ __forceinline__ void asm_commit(AsmRow<D>& S) {
-    moments_to_corners<D>(S.pblk);
-    asm_store<D>(S);
-    block_zero<D>(S.pblk);
+// Stage time of stage st (0..3) of step k: slice 2k, 2k + 1, 2k + 1, 2k + 2.
+template <int TM>
+__device__ __forceinline__ int stage_slice(int k, int st) {
+    return TM == TM_STEADY ? 0 : 2 * k + ((st + 1) >> 1);
 }
 
-template <int D>
-__device__ __forceinline__ void scatter_finish(const DevGrid&, AsmRow<D>& S) {
-    if (S.pkey >= 0) asm_commit<D>(S);
-    S.pkey = -1;
-}
-
-template <int D>
-__device__ __forceinline__ void scatter_add(const DevGrid& g, AsmRow<D>& S, size_t s0, int base, const float* f,
-                                            const float* mu) {
-    (void)g;
-    const long long key = (long long)s0 + base;
-    if (key != S.pkey) {
-        if (S.pkey >= 0) asm_commit<D>(S);
-        S.pkey = key;
-    }
-    moments_add<D>(S.pblk, f, mu);
-}
-
-// Adjoint stage: scatter w_c mu into the slice's gradient and return
-// nu = d_y I(v, y, t)^T mu = grad_y (v . mu) of the interpolant.
-template <int D, class SC>
-__device__ __forceinline__ void stage_adjoint(const DevGrid& g, const float* __restrict__ V, SC& S,
-                                              size_t s0, int base, const float* f, const float* mu, float* nu) {
-    float s_0, dx, dy;
-    plane_dot<D>(g, V, s0, base, 0, f, mu, s_0, dx, dy);
-    if (D == 3) {
-        float s_1, dx1, dy1;
-        plane_dot<D>(g, V, s0, base, 1, f, mu, s_1, dx1, dy1);
-        nu[D - 1] = (s_1 - s_0) * g.inv_h[D - 1];
-        dx = lerp(dx, dx1, f[D - 1]);
-        dy = lerp(dy, dy1, f[D - 1]);
-    }
-    nu[0] = dx * g.inv_h[0];
-    nu[1] = dy * g.inv_h[1];
-    scatter_add<D>(g, S, s0, base, f, mu);
-}
-
-// The velocity cell last met (and the direction's, when DV), kept in
-// registers as the coefficients of its multilinear interpolant, per component
+// The multilinear interpolant of a cell in polynomial form, per component
 //   3D: v(f) = a0 + a1 fx + a2 fy + a3 fz + a4 fx fy + a5 fx fz + a6 fy fz + a7 fx fy fz
 //   2D: v(f) = a0 + a1 fx + a2 fy + a3 fx fy
-// with f the fractional offsets in the cell.  Consecutive RK4 stages mostly
-// fall in the same cell and slice (stages 2 and 3 share their time and nearly
-// their position, stage 4 of a step is stage 1 of the next), so a stage
-// recomputes the coefficients only when its cell or slice changes.  From the
-// coefficients the value and the d derivatives of a component cost 11 FMAs
-// in 3D and the value alone 7 (the lerps of the corner values took about 23
-// and 14 operations); the interpolant is the same multilinear function.
-template <int D, bool DV>
-struct CellCache {
-    static constexpr int NC = 1 << D;
-    int key;                  // s0 + base of the cached cell, -1 when empty (32 bits: see BlockScatter)
-    float a[D][NC];           // coefficients of v, per component
-    float b[DV ? D : 1][DV ? NC : 1];   // of dv
-};
-
-// Coefficients of one component from its corner values c[cx + 2 cy + 4 cz].
+// with f the fractional offsets in the cell, held as pairs over the x axis:
+//   3D: (a0, a1), (a2, a4), (a3, a5), (a6, a7)     2D: (a0, a1), (a2, a3)
+// so that fixing f_y (and f_z) is one paired FMA for both halves and f_x is
+// applied last.  Coefficients of one component from its corner values, c[j] =
+// corners (0, cy, cz) and (1, cy, cz), j = cy + 2 cz.
 template <int D>
-__device__ __forceinline__ void poly_coeffs(const float* c, float* a) {
-    a[0] = c[0];
-    a[1] = c[1] - c[0];
-    a[2] = c[2] - c[0];
-    if (D == 2) {
-        a[3] = (c[3] - c[2]) - a[1];
-    } else {
-        a[3] = c[4] - c[0];
-        a[4] = (c[3] - c[2]) - a[1];
-        a[5] = (c[5] - c[4]) - a[1];
-        a[6] = (c[6] - c[4]) - a[2];
-        a[7] = ((c[7] - c[6]) - (c[5] - c[4])) - a[4];
+__device__ __forceinline__ void poly_coeffs(const pair2* c, pair2* a) {
+    constexpr int NP = 1 << (D - 1);
+    pair2 e[NP];              // (value, x difference) of every row of the cell
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+        float lo, hi;
+        unpk(c[j], lo, hi);
+        e[j] = pk(lo, hi - lo);
+    }
+    a[0] = e[0];
+    a[1] = sub2(e[1], e[0]);
+    if (D == 3) {
+        a[NP / 2] = sub2(e[NP / 2], e[0]);
+        a[NP - 1] = sub2(sub2(e[NP - 1], e[NP / 2]), a[1]);
     }
 }
 
-template <int D, bool DV>
-__device__ __forceinline__ void cache_cell(const DevGrid& g, const float* __restrict__ V, const float* __restrict__ dV,
-                                           size_t s0, int base, CellCache<D, DV>& C) {
-    const int key = (int)s0 + base;
-    if (key == C.key) return;
-    C.key = key;
-    float cv[1 << D][D], cd[DV ? (1 << D) : 1][D];
-#pragma unroll
-    for (int r = 0; r < (1 << (D - 1)); ++r) {
-        pair_value<D>(V, corner_elem<D>(g, s0, base, 0, r & 1, r >> 1), cv[2 * r], cv[2 * r + 1]);
-        if (DV) pair_value<D>(dV, corner_elem<D>(g, s0, base, 0, r & 1, r >> 1), cd[2 * r], cd[2 * r + 1]);
+// The interpolant with f_y (and f_z) applied: (value at f_x = 0, x slope).
+// The order of the sums is fixed (f_y, then f_z, then f_x): the positions of
+// every kernel that traces the same velocity agree bit for bit.
+template <int D>
+__device__ __forceinline__ pair2 poly_row(const pair2* a, const pair2* fd) {
+    constexpr int NP = 1 << (D - 1);
+    if (D == 2) return fma2(fd[0], a[1], a[0]);
+    const pair2 t = fma2(fd[D - 2], a[NP - 1], a[1]);
+    return fma2(fd[D - 2], a[NP / 2], fma2(fd[0], t, a[0]));
+}
+
+// f_y (and f_z) duplicated into pairs
+template <int D>
+__device__ __forceinline__ void dup_offsets(const float* f, pair2* fd) {
+    fd[0] = pk(f[1], f[1]);
+    if (D == 3) fd[D - 2] = pk(f[D - 1], f[D - 1]);
+}
+
+template <int D>
+__device__ __forceinline__ float row_value(pair2 row, const float* f) {
+    float v, gx;
+    unpk(row, v, gx);
+    return fmaf(f[0], gx, v);
+}
+
+// Derivatives along the fractional offsets (per cell width); the constant
+// coefficient is not read.
+template <int D>
+__device__ __forceinline__ void poly_grad(const pair2* a, const float* f, const pair2* fd, float* gr) {
+    constexpr int NP = 1 << (D - 1);
+    float t0, t1;
+    if (D == 2) {
+        unpk(a[1], t0, t1);
+        gr[0] = fmaf(f[1], t1, hi2(a[0]));
+        gr[1] = fmaf(f[0], t1, t0);
+        return;
     }
+    unpk(fma2(fd[D - 2], a[NP - 1], a[1]), t0, t1);
+    gr[0] = fmaf(f[D - 1], hi2(a[NP / 2]), fmaf(f[1], t1, hi2(a[0])));
+    gr[1] = fmaf(f[0], t1, t0);
+    unpk(fma2(fd[0], a[NP - 1], a[NP / 2]), t0, t1);
+    gr[D - 1] = fmaf(f[0], t1, t0);
+}
+
+// The same interpolant as nested linear interpolations (x, then y, then z) of
+// the corner values; c[j] = the two values along the last axis, j = cx (+ 2 cy
+// in 3D), so that all but the last axis are paired.
+template <int D>
+__device__ __forceinline__ float lerp_value(const pair2* c, const float* f, const pair2* fx) {
+    pair2 r;
+    if (D == 2) {
+        r = fma2(fx[0], sub2(c[1], c[0]), c[0]);
+    } else {
+        const pair2 a0 = fma2(fx[0], sub2(c[1], c[0]), c[0]);
+        const pair2 a1 = fma2(fx[0], sub2(c[D], c[2]), c[2]);
+        r = fma2(fx[D - 2], sub2(a1, a0), a0);
+    }
+    float lo, hi;
+    unpk(r, lo, hi);
+    return fmaf(f[D - 1], hi - lo, lo);
+}
+
+// ... with its product with qs (a direction in cell widths).
+template <int D>
+__device__ __forceinline__ float lerp_value_dot(const pair2* c, const float* f, const pair2* fx, const float* qs,
+                                                float& dot) {
+    float lo, hi, l0, l1;
+    if (D == 2) {
+        const pair2 d = sub2(c[1], c[0]);
+        unpk(fma2(fx[0], d, c[0]), lo, hi);
+        unpk(d, l0, l1);
+        const float dl = hi - lo;
+        dot = fmaf(fmaf(f[1], l1 - l0, l0), qs[0], dl * qs[1]);
+        return fmaf(f[1], dl, lo);
+    }
+    const pair2 d0 = sub2(c[1], c[0]), d1 = sub2(c[D], c[2]);
+    const pair2 a0 = fma2(fx[0], d0, c[0]);
+    const pair2 dy = sub2(fma2(fx[0], d1, c[2]), a0);
+    unpk(fma2(fx[D - 2], dy, a0), lo, hi);
+    const float dl = hi - lo;
+    // x and y slopes share the remaining interpolation: dot them first
+    const pair2 dx = fma2(fx[D - 2], sub2(d1, d0), d0);
+    unpk(fma2(dx, pk(qs[0], qs[0]), mul2(dy, pk(qs[1], qs[1]))), l0, l1);
+    dot = fmaf(dl, qs[D - 1], fmaf(f[D - 1], l1 - l0, l0));
+    return fmaf(f[D - 1], dl, lo);
+}
+
+// f_x (and f_y in 3D) duplicated into pairs, for the lerp forms
+template <int D>
+__device__ __forceinline__ void dup_offsets_x(const float* f, pair2* fx) {
+    fx[0] = pk(f[0], f[0]);
+    if (D == 3) fx[D - 2] = pk(f[1], f[1]);
+}
+
+// The corner values of a cell as pairs: over the x axis, c[q][cy + 2 cz], or,
+// with LAST, over the last axis, c[q][cx (+ 2 cy)].
+template <int D, bool LAST>
+__device__ __forceinline__ void load_corners(const DevGrid& g, const float* __restrict__ V, int key,
+                                             pair2 (&c)[D][1 << (D - 1)]) {
+    constexpr int NP = 1 << (D - 1);
+    float lo[NP][3], hi[NP][3];
+#pragma unroll
+    for (int j = 0; j < NP; ++j)
+        pair_value<D>(V, corner_elem<D>(g, (size_t)key, 0, 0, j & 1, j >> 1), lo[j], hi[j]);
 #pragma unroll
     for (int q = 0; q < D; ++q) {
-        float c[1 << D];
+        if (!LAST) {
 #pragma unroll
-        for (int k = 0; k < (1 << D); ++k) c[k] = cv[k][q];
-        poly_coeffs<D>(c, C.a[q]);
-        if (DV) {
-#pragma unroll
-            for (int k = 0; k < (1 << D); ++k) c[k] = cd[k][q];
-            poly_coeffs<D>(c, C.b[DV ? q : 0]);
+            for (int j = 0; j < NP; ++j) c[q][j] = pk(lo[j][q], hi[j][q]);
+        } else if (D == 2) {
+            c[q][0] = pk(lo[0][q], lo[1][q]);
+            c[q][1] = pk(hi[0][q], hi[1][q]);
+        } else {
+            c[q][0] = pk(lo[0][q], lo[NP / 2][q]);
+            c[q][1] = pk(hi[0][q], hi[NP / 2][q]);
+            c[q][NP / 2] = pk(lo[1][q], lo[NP - 1][q]);
+            c[q][NP - 1] = pk(hi[1][q], hi[NP - 1][q]);
         }
     }
 }
 
-// Value of the interpolant with coefficients a at f.
-template <int D>
-__device__ __forceinline__ float poly_value(const float* a, const float* f) {
-    if (D == 2) return fmaf(f[0], fmaf(f[1], a[3], a[1]), fmaf(f[1], a[2], a[0]));
-    const float gx = fmaf(f[2], a[5], fmaf(f[1], fmaf(f[2], a[7], a[4]), a[1]));
-    const float u = fmaf(f[2], a[3], fmaf(f[1], fmaf(f[2], a[6], a[2]), a[0]));
-    return fmaf(f[0], gx, u);
-}
+// The velocity cell a sweep last met, kept in registers: consecutive stages
+// mostly fall in the same cell and slice (stages 2 and 3 share their time and
+// nearly their position, stage 4 of a step is stage 1 of the next), so a stage
+// reads memory only when its cell or slice changes.  FORM: the polynomial
+// coefficients, or the corner values for the nested interpolation.  The
+// forward sweep of the transport model evaluates coefficients, that of the
+// mass-preserving model corner values: the form fixes the rounding of the
+// positions, and with it on which side of a cell face a characteristic ends.
+enum CellForm { POLY = 0, CORNERS = 1 };
+template <int D, int FORM>
+struct Cell {
+    static constexpr int NP = 1 << (D - 1);
+    int key;                  // element of the cached cell, -1 when empty (32 bits: the packed velocity has
+                              // fewer than 2^31 elements, checked when the context is created)
+    pair2 e[D][NP];
+};
 
-// Value and derivatives along the fractional offsets (per cell width).
-template <int D>
-__device__ __forceinline__ float poly_value_grad(const float* a, const float* f, float* gr) {
-    if (D == 2) {
-        gr[0] = fmaf(f[1], a[3], a[1]);
-        gr[1] = fmaf(f[0], a[3], a[2]);
-        return fmaf(f[0], gr[0], fmaf(f[1], a[2], a[0]));
+template <int D, int FORM>
+__device__ __forceinline__ void cell_at(const DevGrid& g, const float* __restrict__ V, int key, Cell<D, FORM>& C) {
+    if (key == C.key) return;
+    C.key = key;
+    if constexpr (FORM == CORNERS) {
+        load_corners<D, true>(g, V, key, C.e);
+    } else {
+        pair2 c[D][1 << (D - 1)];
+        load_corners<D, false>(g, V, key, c);
+#pragma unroll
+        for (int q = 0; q < D; ++q) poly_coeffs<D>(c[q], C.e[q]);
     }
-    const float t1 = fmaf(f[2], a[7], a[4]);
-    const float t4 = fmaf(f[2], a[6], a[2]);
-    gr[0] = fmaf(f[2], a[5], fmaf(f[1], t1, a[1]));
-    gr[1] = fmaf(f[0], t1, t4);
-    gr[2] = fmaf(f[1], fmaf(f[0], a[7], a[6]), fmaf(f[0], a[5], a[3]));
-    return fmaf(f[0], gr[0], fmaf(f[2], a[3], fmaf(f[1], t4, a[0])));
-}
-
-// Derivatives only (the constant coefficient is not read).
-template <int D>
-__device__ __forceinline__ void poly_grad(const float* a, const float* f, float* gr) {
-    if (D == 2) {
-        gr[0] = fmaf(f[1], a[3], a[1]);
-        gr[1] = fmaf(f[0], a[3], a[2]);
-        return;
-    }
-    const float t1 = fmaf(f[2], a[7], a[4]);
-    gr[0] = fmaf(f[2], a[5], fmaf(f[1], t1, a[1]));
-    gr[1] = fmaf(f[0], t1, fmaf(f[2], a[6], a[2]));
-    gr[2] = fmaf(f[1], fmaf(f[0], a[7], a[6]), fmaf(f[0], a[5], a[3]));
-}
-
-// The cached-cell forms of stage_tangent, stage_adjoint and stage_value.
-template <int D>
-__device__ __forceinline__ void stage_tangent_cached(const DevGrid& g, const float* __restrict__ V,
-                                                     const float* __restrict__ dV, size_t s0, const int* p,
-                                                     const float* f, const float* qv, CellCache<D, true>& C,
-                                                     float* val, float* Jq, float* dval) {
-    cache_cell<D, true>(g, V, dV, s0, linear<D>(g, p), C);
-    float qs[D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) qs[a] = qv[a] * g.inv_h[a];
-#pragma unroll
-    for (int q = 0; q < D; ++q) {
-        float gr[D];
-        val[q] = poly_value_grad<D>(C.a[q], f, gr);
-        float jq = gr[D - 1] * qs[D - 1];
-#pragma unroll
-        for (int a = D - 2; a >= 0; --a) jq = fmaf(gr[a], qs[a], jq);
-        Jq[q] = jq;
-        dval[q] = poly_value<D>(C.b[q], f);
-    }
-}
-
-template <int D, class SC>
-__device__ __forceinline__ void stage_adjoint_cached(const DevGrid& g, const float* __restrict__ V, SC& S,
-                                                     CellCache<D, false>& C, size_t s0, int base, const float* f,
-                                                     const float* mu, float* nu) {
-    cache_cell<D, false>(g, V, nullptr, s0, base, C);
-    // coefficients of the scalar interpolant of v . mu (its constant is not needed)
-    float sc[1 << D];
-#pragma unroll
-    for (int i = 1; i < (1 << D); ++i) {
-        float t = C.a[0][i] * mu[0];
-#pragma unroll
-        for (int q = 1; q < D; ++q) t = fmaf(C.a[q][i], mu[q], t);
-        sc[i] = t;
-    }
-    sc[0] = 0.0f;
-    float gr[D];
-    poly_grad<D>(sc, f, gr);
-#pragma unroll
-    for (int a = 0; a < D; ++a) nu[a] = gr[a] * g.inv_h[a];
-    scatter_add<D>(g, S, s0, base, f, mu);
-}
-
-template <int D>
-__device__ __forceinline__ void stage_value_cached(const DevGrid& g, const float* __restrict__ V, size_t s0,
-                                                   const int* p, const float* f, CellCache<D, false>& C, float* val) {
-    cache_cell<D, false>(g, V, nullptr, s0, linear<D>(g, p), C);
-#pragma unroll
-    for (int q = 0; q < D; ++q) val[q] = poly_value<D>(C.a[q], f);
 }
 
 // T(y) and optionally grad T(y) from the padded image, y at displacement u.
@@ -946,8 +1039,8 @@ __device__ __noinline__ void pic_hat(const DevGrid& g, const int* I0, const floa
 // offsets in it, as one 16-byte word (f0, f1, f2 or 0, base).  The adjoint
 // then needs no second lookup of the stage position.
 template <int D>
-__device__ __forceinline__ float4 stage_word(const DevGrid& g, const int* p, const float* f) {
-    return make_float4(f[0], f[1], D == 3 ? f[D - 1] : 0.0f, __int_as_float(linear<D>(g, p)));
+__device__ __forceinline__ float4 stage_word(int base, const float* f) {
+    return make_float4(f[0], f[1], D == 3 ? f[D - 1] : 0.0f, __int_as_float(base));
 }
 
 template <int D>
@@ -958,246 +1051,230 @@ __device__ __forceinline__ int stage_from_word(const float4 w, float* f) {
     return __float_as_int(w.w);
 }
 
-// Slices of the stages of step k: t_k (2k), t_k + dt/2 (2k + 1, stages 2 and
-// 3), t_k + dt (2k + 2); a stationary field has the single slice 0.
-template <bool NS>
-__device__ __forceinline__ void step_slices(const TraceArgs& A, int k, size_t& s1, size_t& s2, size_t& s4) {
-    if (NS) {
-        s1 = (size_t)(2 * k) * A.slice_nodes;
-        s2 = s1 + A.slice_nodes;
-        s4 = s2 + A.slice_nodes;
-    } else {
-        s1 = s2 = s4 = 0;
-    }
-}
-
-// What the forward and tangent sweeps record of each stage for an adjoint
-// sweep (RM): 0 nothing; 1 the stage positions (u, u2, u3, u4 into pos[0 ..
-// 4d)), from which the adjoint looks the cells up again; 2 each stage's cell
-// and offsets (one 16-byte word per stage into cells[0..3]), so the adjoint
-// needs no lookup.  Transport records cells (the 128^3 matvec 0.706 -> 0.630
-// ms); the mass-preserving kernels record positions, whose record is a
-// quarter smaller: their local-memory traffic is what reaches DRAM, and the
-// brain-scale J^T measured 8.43 ms with positions against 8.87 ms with cells.
-enum RecordMode { REC_NONE = 0, REC_POS = 1, REC_CELL = 2 };
-
-// One RK4 step of the characteristic (Alg. 1 without the derivative), on the
-// displacement u, recording its stages as RM says.
-template <int D, bool NS, int RM, bool CACHE>
-__device__ __forceinline__ void rk4_step(const TraceArgs& A, const float* V, float* u, int k, float* pos,
-                                         float4* rec, CellCache<D, false>& C) {
-    size_t s1, s2, s4;
-    step_slices<NS>(A, k, s1, s2, s4);
-    Start<D> sv;
-    start_on_velocity<D>(A, sv);
+// The forward sweep: RK4 on the displacement u (Alg. 1 without the
+// derivative).  With REC, each stage's cell and offsets are recorded for the
+// adjoint sweep (the trajectory is not stored in global memory: the record is
+// a per-thread local array).
+template <int D, int TM, int FORM, bool REC>
+__device__ __forceinline__ void value_sweep(const TraceArgs& A, const VelocityStart<D>& sv, const float* V, float* u,
+                                            float4* rec) {
+    Cell<D, FORM> C;
+    C.key = -1;
     const float dt = A.dt, hdt = 0.5f * A.dt;
-    int p[D];
-    float f[D], vs[D], us[D], acc[D];
-    if (RM == REC_POS) {
+#pragma unroll 1
+    for (int k = 0; k < A.N; ++k) {
+        float us[D], acc[D];
 #pragma unroll
-        for (int a = 0; a < D; ++a) pos[a] = u[a];
+        for (int a = 0; a < D; ++a) us[a] = u[a];
+#pragma unroll
+        for (int st = 0; st < 4; ++st) {
+            float f[D];
+            const int base = locate_velocity<D>(A.vg, sv, us, f);
+            if (REC) rec[4 * k + st] = stage_word<D>(base, f);
+            const int m = stage_slice<TM>(k, st), key = m * (int)A.slice_nodes + base;
+            cell_at<D, FORM>(A.vg, V, key, C);
+            pair2 fd[D - 1];
+            if (FORM == CORNERS) dup_offsets_x<D>(f, fd);
+            else dup_offsets<D>(f, fd);
+#pragma unroll
+            for (int q = 0; q < D; ++q) {
+                const float v = FORM == CORNERS ? lerp_value<D>(C.e[q], f, fd) : row_value<D>(poly_row<D>(C.e[q], fd), f);
+                acc[q] = st == 0 ? v : (st == 3 ? acc[q] + v : fmaf(2.0f, v, acc[q]));
+                if (st < 3) us[q] = fmaf(st == 2 ? dt : hdt, v, u[q]);
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < D; ++a) u[a] = fmaf(A.dt6, acc[a], u[a]);
     }
-    locate<D>(A.vg, sv, u, p, f);
-    if (RM == REC_CELL) rec[0] = stage_word<D>(A.vg, p, f);
-    if constexpr (CACHE) stage_value_cached<D>(A.vg, V, s1, p, f, C, vs);
-    else stage_value<D>(A.vg, V, s1, p, f, vs);
-#pragma unroll
-    for (int a = 0; a < D; ++a) { acc[a] = vs[a]; us[a] = fmaf(hdt, vs[a], u[a]); }
-    if (RM == REC_POS) {
-#pragma unroll
-        for (int a = 0; a < D; ++a) pos[D + a] = us[a];
-    }
-    locate<D>(A.vg, sv, us, p, f);
-    if (RM == REC_CELL) rec[1] = stage_word<D>(A.vg, p, f);
-    if constexpr (CACHE) stage_value_cached<D>(A.vg, V, s2, p, f, C, vs);
-    else stage_value<D>(A.vg, V, s2, p, f, vs);
-#pragma unroll
-    for (int a = 0; a < D; ++a) { acc[a] = fmaf(2.0f, vs[a], acc[a]); us[a] = fmaf(hdt, vs[a], u[a]); }
-    if (RM == REC_POS) {
-#pragma unroll
-        for (int a = 0; a < D; ++a) pos[2 * D + a] = us[a];
-    }
-    locate<D>(A.vg, sv, us, p, f);
-    if (RM == REC_CELL) rec[2] = stage_word<D>(A.vg, p, f);
-    if constexpr (CACHE) stage_value_cached<D>(A.vg, V, s2, p, f, C, vs);
-    else stage_value<D>(A.vg, V, s2, p, f, vs);
-#pragma unroll
-    for (int a = 0; a < D; ++a) { acc[a] = fmaf(2.0f, vs[a], acc[a]); us[a] = fmaf(dt, vs[a], u[a]); }
-    if (RM == REC_POS) {
-#pragma unroll
-        for (int a = 0; a < D; ++a) pos[3 * D + a] = us[a];
-    }
-    locate<D>(A.vg, sv, us, p, f);
-    if (RM == REC_CELL) rec[3] = stage_word<D>(A.vg, p, f);
-    if constexpr (CACHE) stage_value_cached<D>(A.vg, V, s4, p, f, C, vs);
-    else stage_value<D>(A.vg, V, s4, p, f, vs);
-    const float s6 = dt / 6.0f;
-#pragma unroll
-    for (int a = 0; a < D; ++a) u[a] = fmaf(s6, acc[a] + vs[a], u[a]);
 }
 
-// One RK4 step with the derivative recursion of Alg. 1 applied to dv:
+// The forward sweep with the derivative recursion of Alg. 1 applied to dv:
 // D_s = I(dv, y_s, t_s) + d_y I(v, y_s, t_s) (dy + c_s dt D_{s-1}).
-template <int D, bool NS, int RM, bool CACHE>
-__device__ __forceinline__ void rk4_tangent_step(const TraceArgs& A, const float* V, const float* dV, float* u,
-                                                 float* dy, int k, float* pos, float4* rec, CellCache<D, true>& C) {
-    size_t s1, s2, s4;
-    step_slices<NS>(A, k, s1, s2, s4);
-    Start<D> sv;
-    start_on_velocity<D>(A, sv);
+template <int D, int TM, int FORM, bool REC>
+__device__ __forceinline__ void tangent_sweep(const TraceArgs& A, const VelocityStart<D>& sv, const float* V,
+                                              const float* dV, float* u, float* dy, float4* rec) {
+    Cell<D, FORM> C;
+    Cell<D, POLY> B;
+    C.key = -1;           // of both cells
     const float dt = A.dt, hdt = 0.5f * A.dt;
-    int p[D];
-    float f[D], us[D], q[D], vs[D], Jq[D], dvs[D], sv_acc[D], sd_acc[D], Ds;
-    // stage 1 at y, offset dy
-    if (RM == REC_POS) {
+#pragma unroll 1
+    for (int k = 0; k < A.N; ++k) {
+        float us[D], q[D], acc[D], dacc[D];
 #pragma unroll
-        for (int a = 0; a < D; ++a) pos[a] = u[a];
-    }
-    locate<D>(A.vg, sv, u, p, f);
-    if (RM == REC_CELL) rec[0] = stage_word<D>(A.vg, p, f);
-    if constexpr (CACHE) stage_tangent_cached<D>(A.vg, V, dV, s1, p, f, dy, C, vs, Jq, dvs);
-    else stage_tangent<D>(A.vg, V, dV, s1, p, f, dy, vs, Jq, dvs);
+        for (int a = 0; a < D; ++a) {
+            us[a] = u[a];
+            q[a] = dy[a];
+        }
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-        Ds = dvs[a] + Jq[a];
-        sv_acc[a] = vs[a];
-        sd_acc[a] = Ds;
-        us[a] = fmaf(hdt, vs[a], u[a]);
-        q[a] = fmaf(hdt, Ds, dy[a]);
-    }
-    // stage 2
-    if (RM == REC_POS) {
+        for (int st = 0; st < 4; ++st) {
+            float f[D], vs[D], ds[D], qs[D];
+            const int base = locate_velocity<D>(A.vg, sv, us, f);
+            if (REC) rec[4 * k + st] = stage_word<D>(base, f);
+            const int m = stage_slice<TM>(k, st), key = m * (int)A.slice_nodes + base;
+            if (key != C.key) {       // both fields' loads in flight together
+                C.key = key;
+                pair2 c[D][1 << (D - 1)], b[D][1 << (D - 1)];
+                load_corners<D, FORM == CORNERS>(A.vg, V, key, c);
+                load_corners<D, false>(A.vg, dV, key, b);
 #pragma unroll
-        for (int a = 0; a < D; ++a) pos[D + a] = us[a];
-    }
-    locate<D>(A.vg, sv, us, p, f);
-    if (RM == REC_CELL) rec[1] = stage_word<D>(A.vg, p, f);
-    if constexpr (CACHE) stage_tangent_cached<D>(A.vg, V, dV, s2, p, f, q, C, vs, Jq, dvs);
-    else stage_tangent<D>(A.vg, V, dV, s2, p, f, q, vs, Jq, dvs);
+                for (int a = 0; a < D; ++a) {
+                    if (FORM == CORNERS) {
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-        Ds = dvs[a] + Jq[a];
-        sv_acc[a] = fmaf(2.0f, vs[a], sv_acc[a]);
-        sd_acc[a] = fmaf(2.0f, Ds, sd_acc[a]);
-        us[a] = fmaf(hdt, vs[a], u[a]);
-        q[a] = fmaf(hdt, Ds, dy[a]);
-    }
-    // stage 3
-    if (RM == REC_POS) {
+                        for (int j = 0; j < (1 << (D - 1)); ++j) C.e[a][j] = c[a][j];
+                    } else {
+                        poly_coeffs<D>(c[a], C.e[a]);
+                    }
+                    poly_coeffs<D>(b[a], B.e[a]);
+                }
+            }
 #pragma unroll
-        for (int a = 0; a < D; ++a) pos[2 * D + a] = us[a];
-    }
-    locate<D>(A.vg, sv, us, p, f);
-    if (RM == REC_CELL) rec[2] = stage_word<D>(A.vg, p, f);
-    if constexpr (CACHE) stage_tangent_cached<D>(A.vg, V, dV, s2, p, f, q, C, vs, Jq, dvs);
-    else stage_tangent<D>(A.vg, V, dV, s2, p, f, q, vs, Jq, dvs);
+            for (int a = 0; a < D; ++a) qs[a] = q[a] * A.vg.inv_h[a];
+            pair2 fd[D - 1];
+            dup_offsets<D>(f, fd);
+            if constexpr (FORM == CORNERS) {
+                pair2 fx[D - 1];
+                dup_offsets_x<D>(f, fx);
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-        Ds = dvs[a] + Jq[a];
-        sv_acc[a] = fmaf(2.0f, vs[a], sv_acc[a]);
-        sd_acc[a] = fmaf(2.0f, Ds, sd_acc[a]);
-        us[a] = fmaf(dt, vs[a], u[a]);
-        q[a] = fmaf(dt, Ds, dy[a]);
-    }
-    // stage 4
-    if (RM == REC_POS) {
+                for (int a = 0; a < D; ++a) vs[a] = lerp_value_dot<D>(C.e[a], f, fx, qs, ds[a]);
+            } else {
 #pragma unroll
-        for (int a = 0; a < D; ++a) pos[3 * D + a] = us[a];
-    }
-    locate<D>(A.vg, sv, us, p, f);
-    if (RM == REC_CELL) rec[3] = stage_word<D>(A.vg, p, f);
-    if constexpr (CACHE) stage_tangent_cached<D>(A.vg, V, dV, s4, p, f, q, C, vs, Jq, dvs);
-    else stage_tangent<D>(A.vg, V, dV, s4, p, f, q, vs, Jq, dvs);
-    const float s6 = dt / 6.0f;
+                for (int a = 0; a < D; ++a) {
+                    float gr[D];
+                    vs[a] = row_value<D>(poly_row<D>(C.e[a], fd), f);
+                    poly_grad<D>(C.e[a], f, fd, gr);
+                    float jq = gr[D - 1] * qs[D - 1];
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-        dy[a] = fmaf(s6, sd_acc[a] + dvs[a] + Jq[a], dy[a]);
-        u[a] = fmaf(s6, sv_acc[a] + vs[a], u[a]);
+                    for (int b = D - 2; b >= 0; --b) jq = fmaf(gr[b], qs[b], jq);
+                    ds[a] = jq;
+                }
+            }
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+                const float d = row_value<D>(poly_row<D>(B.e[a], fd), f) + ds[a];
+                acc[a] = st == 0 ? vs[a] : (st == 3 ? acc[a] + vs[a] : fmaf(2.0f, vs[a], acc[a]));
+                dacc[a] = st == 0 ? d : (st == 3 ? dacc[a] + d : fmaf(2.0f, d, dacc[a]));
+                if (st < 3) {
+                    us[a] = fmaf(st == 2 ? dt : hdt, vs[a], u[a]);
+                    q[a] = fmaf(st == 2 ? dt : hdt, d, dy[a]);
+                }
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            u[a] = fmaf(A.dt6, acc[a], u[a]);
+            dy[a] = fmaf(A.dt6, dacc[a], dy[a]);
+        }
     }
 }
 
-// Transpose of one tangent step from recorded stage positions (RM = 1): the
-// same as rk4_adjoint_step below, with each stage's cell looked up again.
-template <int D, bool NS, class SC, bool CACHE>
-__device__ __forceinline__ void rk4_adjoint_step_pos(const TraceArgs& A, const float* V, SC& S, const float* rec,
-                                                     float* lam, int k, CellCache<D, false>& C) {
-    size_t s1, s2, s4;
-    step_slices<NS>(A, k, s1, s2, s4);
-    Start<D> sv;
-    start_on_velocity<D>(A, sv);
-    const float dt = A.dt, hdt = 0.5f * A.dt;
-    int p[D];
-    float f[D], us[D];
-    float mu[D], nu[D], acc[D];
-    const float c16 = dt / 6.0f, c13 = dt / 3.0f;
-    // stage 4
+// The adjoint sweep: from lam, the adjoint of the end point, scatter every
+// stage's contribution and leave in lam the adjoint of the start.  Stages in
+// reverse, D_s = I(dv, y_s) + J_s (dy + c_s dt D_{s-1}):
+//   mu_4 = dt/6 lam, mu_3 = dt/3 lam + dt nu_4, mu_2 = dt/3 lam + dt/2 nu_3,
+//   mu_1 = dt/6 lam + dt/2 nu_2, nu_s = J_s^T mu_s, lam += nu_1 + .. + nu_4
+// with J_s^T mu the gradient of the scalar interpolant of v . mu.  The records
+// are read one stage ahead of their use: they come from L2 more often than
+// from L1 (the records of the resident threads exceed the L1), and the load is
+// then in flight during a stage's arithmetic.
+template <int D, int TM, int NB, template <int, int> class SC>
+__device__ __forceinline__ void adjoint_sweep(const TraceArgs& A, const float* V, SC<D, NB>& S, const float4* rec,
+                                              float* lam, Cell<D, POLY>& C) {
+    constexpr int NP = 1 << (D - 1);
+    const float dt = A.dt, hdt = 0.5f * A.dt, c16 = A.dt6, c13 = 2.0f * A.dt6;
+    float4 word = rec[4 * A.N - 1];
+#pragma unroll 1
+    for (int k = A.N - 1; k >= 0; --k) {
+        float nu[D], acc[D];
 #pragma unroll
-    for (int a = 0; a < D; ++a) { mu[a] = c16 * lam[a]; us[a] = rec[3 * D + a]; }
-    locate<D>(A.vg, sv, us, p, f);
-    if constexpr (CACHE) stage_adjoint_cached<D, SC>(A.vg, V, S, C, s4, linear<D>(A.vg, p), f, mu, nu);
-    else stage_adjoint<D, SC>(A.vg, V, S, s4, linear<D>(A.vg, p), f, mu, nu);
-    // stage 3
+        for (int st = 3; st >= 0; --st) {
+            float f[D], mu[D];
+            const int base = stage_from_word<D>(word, f);
+            word = rec[st > 0 ? 4 * k + st - 1 : max(4 * k - 1, 0)];
 #pragma unroll
-    for (int a = 0; a < D; ++a) { acc[a] = nu[a]; mu[a] = fmaf(c13, lam[a], dt * nu[a]); us[a] = rec[2 * D + a]; }
-    locate<D>(A.vg, sv, us, p, f);
-    if constexpr (CACHE) stage_adjoint_cached<D, SC>(A.vg, V, S, C, s2, linear<D>(A.vg, p), f, mu, nu);
-    else stage_adjoint<D, SC>(A.vg, V, S, s2, linear<D>(A.vg, p), f, mu, nu);
-    // stage 2
+            for (int a = 0; a < D; ++a) {
+                const float c = (st == 1 || st == 2) ? c13 : c16;
+                mu[a] = st == 3 ? c * lam[a] : fmaf(c, lam[a], (st == 2 ? dt : hdt) * nu[a]);
+            }
+            const int m = stage_slice<TM>(k, st);
+            cell_at<D, POLY>(A.vg, V, m * (int)A.slice_nodes + base, C);
+            pair2 sc[NP];         // coefficients of the scalar interpolant of v . mu
 #pragma unroll
-    for (int a = 0; a < D; ++a) { acc[a] += nu[a]; mu[a] = fmaf(c13, lam[a], hdt * nu[a]); us[a] = rec[D + a]; }
-    locate<D>(A.vg, sv, us, p, f);
-    if constexpr (CACHE) stage_adjoint_cached<D, SC>(A.vg, V, S, C, s2, linear<D>(A.vg, p), f, mu, nu);
-    else stage_adjoint<D, SC>(A.vg, V, S, s2, linear<D>(A.vg, p), f, mu, nu);
-    // stage 1
+            for (int q = 0; q < D; ++q) {
+                const pair2 w = pk(mu[q], mu[q]);
 #pragma unroll
-    for (int a = 0; a < D; ++a) { acc[a] += nu[a]; mu[a] = fmaf(c16, lam[a], hdt * nu[a]); us[a] = rec[a]; }
-    locate<D>(A.vg, sv, us, p, f);
-    if constexpr (CACHE) stage_adjoint_cached<D, SC>(A.vg, V, S, C, s1, linear<D>(A.vg, p), f, mu, nu);
-    else stage_adjoint<D, SC>(A.vg, V, S, s1, linear<D>(A.vg, p), f, mu, nu);
+                for (int j = 0; j < NP; ++j) sc[j] = q == 0 ? mul2(C.e[0][j], w) : fma2(C.e[q][j], w, sc[j]);
+            }
+            pair2 fd[D - 1];
+            dup_offsets<D>(f, fd);
+            float gr[D];
+            poly_grad<D>(sc, f, fd, gr);
 #pragma unroll
-    for (int a = 0; a < D; ++a) lam[a] += acc[a] + nu[a];
+            for (int a = 0; a < D; ++a) {
+                nu[a] = gr[a] * A.vg.inv_h[a];
+                acc[a] = st == 3 ? nu[a] : acc[a] + nu[a];
+            }
+            if (NB == 2) scatter_add(A.vg, S, A.tj[m] * (int)A.slice_nodes + base, A.tj[m] & 1, A.tth[m], f, mu);
+            else scatter_add(A.vg, S, m * (int)A.slice_nodes + base, 0, 0.0f, f, mu);
+        }
+#pragma unroll
+        for (int a = 0; a < D; ++a) lam[a] += acc[a];
+    }
 }
 
-// Transpose of one tangent step: given lam (adjoint of the step's end point),
-// scatter the step's contribution into the gradient and return the adjoint of
-// its start.  The cells and offsets of the stages were recorded by the
-// forward sweep (rec[0..3]); each stage's J^T mu and scatter share one pass.
-template <int D, bool NS, class SC, bool CACHE>
-__device__ __forceinline__ void rk4_adjoint_step(const TraceArgs& A, const float* V, SC& S, const float4* rec,
-                                                 float* lam, int k, CellCache<D, false>& C) {
-    size_t s1, s2, s4;
-    step_slices<NS>(A, k, s1, s2, s4);
-    const float dt = A.dt, hdt = 0.5f * A.dt;
-    float f[D];
-    float mu[D], nu[D], acc[D];
-    const float c16 = dt / 6.0f, c13 = dt / 3.0f;
-    int base;
-    // stage 4: D4 = I(dv, y4) + J4 (dy + dt D3)
+// The fused Gauss-Newton product of one voxel (RowScatter): the row's sweep,
+// then its blocks dotted with the direction and, scaled by h^d J_i dv, into
+// the gradients; a row whose blocks did not fit is swept again with the scaled
+// seed.
+template <int D, int TM, int NB>
+__device__ __forceinline__ void gauss_newton_row(const TraceArgs& A, const float* V, RowScatter<D, NB>& S,
+                                                 const float4* rec, const float* gT, Cell<D, POLY>& C) {
+    constexpr int NV = RowScatter<D, NB>::NV, CAP = RowScatter<D, NB>::CAP;
+    S.direct = false;
+    S.n = 0;
+    S.du = 0.0f;
+    float lam[D];
 #pragma unroll
-    for (int a = 0; a < D; ++a) mu[a] = c16 * lam[a];
-    base = stage_from_word<D>(rec[3], f);
-    if constexpr (CACHE) stage_adjoint_cached<D, SC>(A.vg, V, S, C, s4, base, f, mu, nu);
-    else stage_adjoint<D, SC>(A.vg, V, S, s4, base, f, mu, nu);
-    // stage 3: D3 = I(dv, y3) + J3 (dy + dt/2 D2)
+    for (int a = 0; a < D; ++a) lam[a] = gT[a];
+#pragma unroll 1
+    for (;;) {
+        adjoint_sweep<D, TM>(A, V, S, rec, lam, C);
+        if (S.direct) {
+            scatter_finish(A.vg, S);
+            return;
+        }
+        float du = S.du;
 #pragma unroll
-    for (int a = 0; a < D; ++a) { acc[a] = nu[a]; mu[a] = fmaf(c13, lam[a], dt * nu[a]); }
-    base = stage_from_word<D>(rec[2], f);
-    if constexpr (CACHE) stage_adjoint_cached<D, SC>(A.vg, V, S, C, s2, base, f, mu, nu);
-    else stage_adjoint<D, SC>(A.vg, V, S, s2, base, f, mu, nu);
-    // stage 2: D2 = I(dv, y2) + J2 (dy + dt/2 D1)
+        for (int b = 0; b < NB; ++b) {
+            moments_to_corners<D>(S.blk[b]);
+            du += block_dot<D>(A.vg, S.dV, block_key(S, b), S.blk[b]);
+        }
+        const int kept = min(S.n, CAP);
+        Block<D> B;
+#pragma unroll 1
+        for (int j = 0; j < kept; ++j) {
+            block_load<D>(S.st + j * NV, B);
+            moments_to_corners<D>(B);
+            du += block_dot<D>(A.vg, S.dV, S.stkey[j], B);
+            block_store<D>(S.st + j * NV, B);
+        }
+        const float s = A.cellvol * du;
+        if (S.n <= CAP) {
 #pragma unroll
-    for (int a = 0; a < D; ++a) { acc[a] += nu[a]; mu[a] = fmaf(c13, lam[a], hdt * nu[a]); }
-    base = stage_from_word<D>(rec[1], f);
-    if constexpr (CACHE) stage_adjoint_cached<D, SC>(A.vg, V, S, C, s2, base, f, mu, nu);
-    else stage_adjoint<D, SC>(A.vg, V, S, s2, base, f, mu, nu);
-    // stage 1: D1 = I(dv, y) + J1 dy
+            for (int b = 0; b < NB; ++b) block_red<D>(A.vg, S.G, block_key(S, b), S.blk[b], s);
+#pragma unroll 1
+            for (int j = 0; j < S.n; ++j) {
+                block_load<D>(S.st + j * NV, B);
+                block_red<D>(A.vg, S.G, S.stkey[j], B, s);
+            }
+            return;
+        }
+        S.direct = true;
+        S.key = -1;
 #pragma unroll
-    for (int a = 0; a < D; ++a) { acc[a] += nu[a]; mu[a] = fmaf(c16, lam[a], hdt * nu[a]); }
-    base = stage_from_word<D>(rec[0], f);
-    if constexpr (CACHE) stage_adjoint_cached<D, SC>(A.vg, V, S, C, s1, base, f, mu, nu);
-    else stage_adjoint<D, SC>(A.vg, V, S, s1, base, f, mu, nu);
+        for (int b = 0; b < NB; ++b) block_zero<D>(S.blk[b]);
 #pragma unroll
-    for (int a = 0; a < D; ++a) lam[a] += acc[a] + nu[a];
+        for (int a = 0; a < D; ++a) lam[a] = s * gT[a];
+    }
 }
 
 // Finish one assembled row: its keys at [e][voxel] (the blocks are already
@@ -1386,58 +1463,34 @@ static cudaError_t launch_ell_dim(int mode, const EllArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// 256 threads; FWD at 64 registers (4 CTAs per SM; 80 registers, 3 CTAs, for
-// the 3D transport sweep with its value cell cache: 0.256 -> 0.226 ms on the
-// 128^3 image against the uncached sweep at 4 CTAs), the other derivative
-// modes at 80 (3 CTAs): measured fastest among 64/80/128-register and
-// 256/512-thread configurations on the 128^3 matvec.
-template <int D, int MODEL, int MODE>
+// CTAs per SM the register budget of a kernel is set for (256 threads).  The
+// 3D kernels hold a cell's coefficients and a pending block (24 registers each,
+// 48 for the two nodes of a time cell) and run at 128 registers; the forward
+// sweep holds the coefficients only and runs at 80.
+template <int D, int TM, int MODEL, int MODE>
 struct TraceOccupancy {
-    // CTAs per SM the register budget is set for: the 3D transport modes hold
-    // cached cells (v and dv corners) and the pending scatter block and run at
-    // 128 registers (measured on the 128^3 matvec: 1.42 ms at 3 CTAs without
-    // either, 1.50 ms with the cache at 80 registers, 1.31 ms with it at 128,
-    // 0.82 ms with the scatter block as well; the assembly 1.23 -> 0.79 ms
-    // from 3 to 2 CTAs with its pending block in registers)
-    static constexpr int value =
-        MODE == MODE_FWD ? ((D == 3 && MODEL == LGNK_TRANSPORT) ? 3 : 4) : ((D == 3 && MODEL == LGNK_TRANSPORT) ? 2 : 3);
+    static constexpr int value = D == 3 ? (MODE == MODE_FWD ? 3 : 2) : (MODE == MODE_FWD ? 4 : 3);
 };
 
-template <int D, bool NS, int MODEL, int MODE>
-__global__ void __launch_bounds__(LGNK_BLOCK, (TraceOccupancy<D, MODEL, MODE>::value)) trace_kernel(const TraceArgs A) {
-    using VT = typename VecT<D>::type;
-    constexpr bool TANGENT = (MODE == MODE_JVP || MODE == MODE_HESS);
-    constexpr bool ADJOINT = (MODE == MODE_JTVP || MODE == MODE_HESS || MODE == MODE_OBJGRAD || MODE == MODE_ASM);
-    using SC = typename std::conditional<
-        MODE == MODE_ASM, AsmRow<D>,
-        typename std::conditional<(MODE == MODE_HESS || MODE == MODE_JTVP || MODE == MODE_OBJGRAD) && MODEL == LGNK_TRANSPORT, BlockScatter<D>, Scatter<D>>::type>::type;
-    // cached velocity cells and whole-cell scatter blocks for transport; the
-    // continuity kernels (many time slices, longer trajectories) were measured
-    // faster without either
-    constexpr bool CACHE = MODEL == LGNK_TRANSPORT;
+template <int D, int TM, int MODEL, int MODE>
+__global__ void __launch_bounds__(LGNK_BLOCK, (TraceOccupancy<D, TM, MODEL, MODE>::value)) trace_kernel(const TraceArgs A) {
+    constexpr bool TRANSPORT = MODEL == LGNK_TRANSPORT;
+    constexpr int FORM = TRANSPORT ? POLY : CORNERS;
+    constexpr bool ROWS = MODE == MODE_HROW;
+    constexpr bool TANGENT = MODE == MODE_JVP || MODE == MODE_HESS;
+    constexpr bool ADJOINT = MODE != MODE_FWD && MODE != MODE_JVP;
+    constexpr int NB = TM == TM_NODES ? 2 : 1;
+    using SC = typename std::conditional<MODE == MODE_ASM, AsmRow<D, NB>,
+                                         typename std::conditional<ROWS, RowScatter<D, NB>, BlockScatter<D, NB>>::type>::type;
     const float* V = static_cast<const float*>(A.V);
     const float* dV = static_cast<const float*>(A.dV);
+    lsum ssd = lsum_zero();  // res^2 of this thread's voxel (FWD with R, OBJGRAD, ASM with R)
+    int entries = 0;         // MODE_ASM: blocks of this thread's row
 
     int idx[3];
     voxel_index<D>(A, idx);
     const bool active = idx[0] < A.ig.m[0] && idx[1] < A.ig.m[1] && (D == 2 || idx[2] < A.ig.m[2]);
-    lsum ssd = lsum_zero();  // res^2 of this thread's voxel (FWD with R, OBJGRAD, ASM with R)
-    int entries = 0;           // MODE_ASM: blocks of this thread's row
-
-    SC S;
-    scatter_init<D>(S, A.G);
-    AsmTable<D> row_table;        // MODE_ASM: the keys of the row being assembled
-    if constexpr (MODE == MODE_ASM) {
-        row_table.n = 0;
-        row_table.overflow = false;
-        S.tab = &row_table;
-        const size_t Mi = (size_t)A.ig.m[0] * A.ig.m[1] * (D == 3 ? A.ig.m[2] : 1);
-        const int vx = idx[0] + A.ig.m[0] * (idx[1] + A.ig.m[1] * (D == 3 ? idx[2] : 0));
-        S.stride = Mi * AsmRow<D>::B;
-        S.blk = A.eblk + (size_t)vx * AsmRow<D>::B;
-    }
-
-    int sp[D];                    // continuity FWD / JVP: the end cell, offsets, mass and dy of the splat
+    int sp[D];                // continuity FWD / JVP: the end cell, offsets, mass and dy of the splat
     float sf[D], sdy[D], smass = 0.0f;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
@@ -1453,32 +1506,15 @@ __global__ void __launch_bounds__(LGNK_BLOCK, (TraceOccupancy<D, MODEL, MODE>::v
             u[a] = 0.0f;
             dy[a] = 0.0f;
         }
-        CellCache<D, true> tcache;
-        tcache.key = -1;
-        CellCache<D, false> vcache;   // v corners for the forward and adjoint sweeps
-        vcache.key = -1;
-        // the stages of every step, recorded for the adjoint sweep (RecordMode)
-        // in a per-thread local array as 16-byte words.  Kept
-        // in shared memory instead, the full record (2 CTAs x 96 KB on the
-        // 128^3 matvec) shrank the L1 that the gathers use and measured slower
-        // (0.828 against 0.814 ms); keeping only each step's start there and
-        // recomputing the other positions in the adjoint sweep measured 0.974
-        // ms, and on the brain-scale mass-preserving J^T 9.56 against 8.47 ms.
-        constexpr int RM = !ADJOINT ? REC_NONE : (MODEL == LGNK_TRANSPORT ? REC_CELL : REC_POS);
-        constexpr int WPS = RM == REC_CELL ? 4 : D;     // 16-byte words per step
-        float4 lrec[ADJOINT ? LGNK_MAX_STEPS * WPS : 1];
-
-#pragma unroll 1
-        for (int k = 0; k < A.N; ++k) {
-            float4* rec = lrec + (ADJOINT ? WPS * k : 0);
-            float pos[4 * D];
-            if (TANGENT) rk4_tangent_step<D, NS, RM, CACHE>(A, V, dV, u, dy, k, pos, rec, tcache);
-            else rk4_step<D, NS, RM, CACHE>(A, V, u, k, pos, rec, vcache);
-            if constexpr (RM == REC_POS) {
-#pragma unroll
-                for (int w = 0; w < D; ++w) rec[w] = make_float4(pos[4 * w], pos[4 * w + 1], pos[4 * w + 2], pos[4 * w + 3]);
-            }
-        }
+        VelocityStart<D> sv;
+        start_on_velocity<D>(A, idx, sv);
+        // the stages, recorded for the adjoint sweep in a per-thread local
+        // array.  Kept in shared memory instead, the record shrank the L1
+        // that the gathers use and measured slower (0.828 against 0.814 ms
+        // for an earlier 128^3 product).
+        float4 rec[ADJOINT ? 4 * LGNK_MAX_STEPS : 1];
+        if constexpr (TANGENT) tangent_sweep<D, TM, FORM, ADJOINT>(A, sv, V, dV, u, dy, rec);
+        else value_sweep<D, TM, FORM, ADJOINT>(A, sv, V, u, rec);
         if (A.yout != nullptr) {
             const int M = A.ig.m[0] * A.ig.m[1] * (D == 3 ? A.ig.m[2] : 1);
 #pragma unroll
@@ -1491,48 +1527,35 @@ __global__ void __launch_bounds__(LGNK_BLOCK, (TraceOccupancy<D, MODEL, MODE>::v
         float lam[D];
         Start<D> si;
         start_on_image<D>(idx, si);
-        if (MODEL == LGNK_TRANSPORT) {
-            float gT[D];
-            if (MODE == MODE_FWD) {
+        if constexpr (TRANSPORT) {
+            if constexpr (MODE == MODE_FWD) {
                 const float val = sample_image<D, false>(A.ig, si, A.Tp, u, nullptr);
                 A.u1[vox] = val;
                 if (A.R != nullptr) lsum_add_sqdiff(ssd, val, A.R[vox]);
-            } else if (MODE == MODE_JVP) {
-                sample_image<D, true>(A.ig, si, A.Tp, u, gT);
-                float du = 0.0f;
-#pragma unroll
-                for (int a = 0; a < D; ++a) du = fmaf(gT[a], dy[a], du);
-                A.u1[vox] = du;
-            } else if (MODE == MODE_JTVP) {
-                sample_image<D, true>(A.ig, si, A.Tp, u, gT);
-                const float r = A.r[vox];
-#pragma unroll
-                for (int a = 0; a < D; ++a) lam[a] = r * gT[a];
-            } else if (MODE == MODE_HESS) {
-                sample_image<D, true>(A.ig, si, A.Tp, u, gT);
-                float du = 0.0f;
-#pragma unroll
-                for (int a = 0; a < D; ++a) du = fmaf(gT[a], dy[a], du);
-                const float s = A.cellvol * du;
-#pragma unroll
-                for (int a = 0; a < D; ++a) lam[a] = s * gT[a];
-            } else if (MODE == MODE_ASM) {
+            } else {
+                float gT[D];
                 const float val = sample_image<D, true>(A.ig, si, A.Tp, u, gT);
+                if constexpr (TANGENT) {
+                    float du = 0.0f;
 #pragma unroll
-                for (int a = 0; a < D; ++a) lam[a] = gT[a];
-                if (A.R != nullptr) {     // with the objective: SSD and the gradient's weights h^d res
-                    const float Rv = A.R[vox];
-                    lsum_add_sqdiff(ssd, val, Rv);
-                    A.u1[vox] = A.cellvol * (val - Rv);
+                    for (int a = 0; a < D; ++a) du = fmaf(gT[a], dy[a], du);
+                    if (MODE == MODE_JVP) A.u1[vox] = du;
+                    const float s = A.cellvol * du;      // MODE_HESS: the seed h^d J dv
+#pragma unroll
+                    for (int a = 0; a < D; ++a) lam[a] = s * gT[a];
+                } else {
+                    float s = 1.0f;                      // MODE_HROW and MODE_ASM: the row of J
+                    if (MODE == MODE_JTVP) s = A.r[vox];
+                    if (MODE == MODE_OBJGRAD || (MODE == MODE_ASM && A.R != nullptr)) {
+                        const float Rv = A.R[vox];
+                        lsum_add_sqdiff(ssd, val, Rv);
+                        const float w = A.cellvol * (val - Rv);
+                        if (MODE == MODE_ASM) A.u1[vox] = w;     // the gradient's weights h^d res
+                        else s = w;
+                    }
+#pragma unroll
+                    for (int a = 0; a < D; ++a) lam[a] = s * gT[a];
                 }
-            } else {  // MODE_OBJGRAD
-                const float val = sample_image<D, true>(A.ig, si, A.Tp, u, gT);
-                if (A.u1 != nullptr) A.u1[vox] = val;
-                const float Rv = A.R[vox];
-                lsum_add_sqdiff(ssd, val, Rv);
-                const float s = A.cellvol * (val - Rv);
-#pragma unroll
-                for (int a = 0; a < D; ++a) lam[a] = s * gT[a];
             }
         } else {
             const float mass = __ldg(A.T + vox);
@@ -1548,7 +1571,7 @@ __global__ void __launch_bounds__(LGNK_BLOCK, (TraceOccupancy<D, MODEL, MODE>::v
                     for (int a = 0; a < D; ++a) lam[a] = mass * gr[a];
                 }
             } else if (MODE == MODE_FWD || MODE == MODE_JVP) {
-                locate<D>(A.ig, si, u, sp, sf);   // splat after the loop, with the whole CTA
+                locate<D>(A.ig, si, u, sp, sf);   // splat after the trace, with the whole CTA
                 smass = mass;
 #pragma unroll
                 for (int a = 0; a < D; ++a) sdy[a] = dy[a];
@@ -1560,80 +1583,100 @@ __global__ void __launch_bounds__(LGNK_BLOCK, (TraceOccupancy<D, MODEL, MODE>::v
             }
         }
 
-        if (ADJOINT) {
-#pragma unroll 1
-            for (int k = A.N - 1; k >= 0; --k) {
-                if constexpr (RM == REC_CELL) {
-                    rk4_adjoint_step<D, NS, SC, CACHE>(A, V, S, lrec + WPS * k, lam, k, vcache);
-                } else {
-                    float pos[4 * D];
-#pragma unroll
-                    for (int w = 0; w < D; ++w) {
-                        const float4 word = lrec[WPS * k + w];
-                        pos[4 * w] = word.x;
-                        pos[4 * w + 1] = word.y;
-                        pos[4 * w + 2] = word.z;
-                        pos[4 * w + 3] = word.w;
-                    }
-                    rk4_adjoint_step_pos<D, NS, SC, CACHE>(A, V, S, pos, lam, k, vcache);
-                }
-            }
-            scatter_finish<D>(A.vg, S);
-            if constexpr (MODE == MODE_ASM) {
-                write_row<D>(A, *S.tab, vox);
-                entries = S.tab->n;
+        if constexpr (ADJOINT) {
+            Cell<D, POLY> C;
+            C.key = -1;
+            SC S;
+            scatter_init(S, A.G, (int)A.slice_nodes);
+            if constexpr (ROWS) {
+                float4 rowst[RowScatter<D, NB>::CAP * RowScatter<D, NB>::NV];
+                int rowkey[RowScatter<D, NB>::CAP];
+                S.dV = dV;
+                S.st = rowst;
+                S.stkey = rowkey;
+                gauss_newton_row<D, TM>(A, V, S, rec, lam, C);
+            } else if constexpr (MODE == MODE_ASM) {
+                AsmTable<D> row_table;        // the keys of the row being assembled
+                row_table.n = 0;
+                row_table.overflow = false;
+                S.tab = &row_table;
+                const size_t Mi = (size_t)A.ig.m[0] * A.ig.m[1] * (D == 3 ? A.ig.m[2] : 1);
+                S.stride = Mi * AsmRow<D, NB>::B;
+                S.row = A.eblk + (size_t)vox * AsmRow<D, NB>::B;
+                adjoint_sweep<D, TM>(A, V, S, rec, lam, C);
+                scatter_finish(A.vg, S);
+                write_row<D>(A, row_table, vox);
+                entries = row_table.n;
+            } else {
+                adjoint_sweep<D, TM>(A, V, S, rec, lam, C);
+                scatter_finish(A.vg, S);
             }
         }
     }
-
-    if constexpr (MODEL == LGNK_CONTINUITY && (MODE == MODE_FWD || MODE == MODE_JVP)) {
+    if constexpr (!TRANSPORT && (MODE == MODE_FWD || MODE == MODE_JVP)) {
         if (A.pic_rho[0] <= 0.0f) splat_tiled<D, MODE == MODE_JVP>(A.ig, A.acc, active, sp, sf, smass, sdy);
     }
-    if (MODE == MODE_OBJGRAD || MODE == MODE_FWD || MODE == MODE_ASM) {
+
+    if constexpr (TRANSPORT && (MODE == MODE_OBJGRAD || MODE == MODE_FWD || MODE == MODE_ASM)) {
         if (A.partial != nullptr) {
             const lsum s = lsum_block_sum(ssd);
             if (threadIdx.x == 0) A.partial[blockIdx.x] = lsum_value(s);
         }
     }
-    if (MODE == MODE_ASM && A.cpartial != nullptr) {
-        __syncthreads();      // lsum_block_sum's shared slots are reused
-        lsum c = lsum_zero();
-        lsum_add(c, (float)entries);
-        c = lsum_block_sum(c);   // exact: at most 256 x 16 blocks
-        if (threadIdx.x == 0) A.cpartial[blockIdx.x] = lsum_value(c);
+    if constexpr (MODE == MODE_ASM) {
+        if (A.cpartial != nullptr) {
+            __syncthreads();      // lsum_block_sum's shared slots are reused
+            lsum c = lsum_zero();
+            lsum_add(c, (float)entries);
+            c = lsum_block_sum(c);   // exact: at most 256 x 16 blocks
+            if (threadIdx.x == 0) A.cpartial[blockIdx.x] = lsum_value(c);
+        }
     }
 }
 
-template <int D, bool NS, int MODEL, int MODE>
-static cudaError_t launch_one(const TraceArgs& a0, int nblocks, cudaStream_t s) {
-    (void)nblocks;
+template <int D, int TM, int MODEL, int MODE>
+static cudaError_t launch_one(const TraceArgs& a0, cudaStream_t s) {
     TraceArgs a = a0;
     int ts[3];
     trace_tile_shape(D, ts);
     for (int i = 0; i < 3; ++i) a.tiles[i] = (a.ig.m[i] + ts[i] - 1) / ts[i];
     const int blocks = a.tiles[0] * a.tiles[1] * a.tiles[2];
-    const int threads = ts[0] * ts[1] * ts[2];
-    trace_kernel<D, NS, MODEL, MODE><<<blocks, threads, 0, s>>>(a);
+    trace_kernel<D, TM, MODEL, MODE><<<blocks, LGNK_BLOCK, 0, s>>>(a);
     return cudaGetLastError();
 }
 
-template <int D, bool NS>
-static cudaError_t launch_dim(int model, int mode, const TraceArgs& a, int nblocks, cudaStream_t s) {
+template <int D, int TM>
+static cudaError_t launch_dim(int model, int mode, const TraceArgs& a, cudaStream_t s) {
     if (model == LGNK_TRANSPORT) {
         switch (mode) {
-            case MODE_FWD: return launch_one<D, NS, LGNK_TRANSPORT, MODE_FWD>(a, nblocks, s);
-            case MODE_JVP: return launch_one<D, NS, LGNK_TRANSPORT, MODE_JVP>(a, nblocks, s);
-            case MODE_JTVP: return launch_one<D, NS, LGNK_TRANSPORT, MODE_JTVP>(a, nblocks, s);
-            case MODE_HESS: return launch_one<D, NS, LGNK_TRANSPORT, MODE_HESS>(a, nblocks, s);
-            case MODE_OBJGRAD: return launch_one<D, NS, LGNK_TRANSPORT, MODE_OBJGRAD>(a, nblocks, s);
-            case MODE_ASM: return launch_one<D, NS, LGNK_TRANSPORT, MODE_ASM>(a, nblocks, s);
+            case MODE_FWD: return launch_one<D, TM, LGNK_TRANSPORT, MODE_FWD>(a, s);
+            case MODE_JVP: return launch_one<D, TM, LGNK_TRANSPORT, MODE_JVP>(a, s);
+            case MODE_JTVP: return launch_one<D, TM, LGNK_TRANSPORT, MODE_JTVP>(a, s);
+            case MODE_HESS: return launch_one<D, TM, LGNK_TRANSPORT, MODE_HESS>(a, s);
+            case MODE_HROW:
+                if constexpr (D == 3 && TM == TM_STEADY) return launch_one<D, TM, LGNK_TRANSPORT, MODE_HROW>(a, s);
+                break;
+            case MODE_OBJGRAD: return launch_one<D, TM, LGNK_TRANSPORT, MODE_OBJGRAD>(a, s);
+            case MODE_ASM:      // rows are kept per (slice, cell)
+                if constexpr (TM != TM_NODES) return launch_one<D, TM, LGNK_TRANSPORT, MODE_ASM>(a, s);
+                break;
         }
     } else {
         switch (mode) {
-            case MODE_FWD: return launch_one<D, NS, LGNK_CONTINUITY, MODE_FWD>(a, nblocks, s);
-            case MODE_JVP: return launch_one<D, NS, LGNK_CONTINUITY, MODE_JVP>(a, nblocks, s);
-            case MODE_JTVP: return launch_one<D, NS, LGNK_CONTINUITY, MODE_JTVP>(a, nblocks, s);
+            case MODE_FWD: return launch_one<D, TM, LGNK_CONTINUITY, MODE_FWD>(a, s);
+            case MODE_JVP: return launch_one<D, TM, LGNK_CONTINUITY, MODE_JVP>(a, s);
+            case MODE_JTVP: return launch_one<D, TM, LGNK_CONTINUITY, MODE_JTVP>(a, s);
         }
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <int D>
+static cudaError_t launch_trace_dim(TimeMode tm, int model, int mode, const TraceArgs& a, cudaStream_t s) {
+    switch (tm) {
+        case TM_STEADY: return launch_dim<D, TM_STEADY>(model, mode, a, s);
+        case TM_SLICES: return launch_dim<D, TM_SLICES>(model, mode, a, s);
+        case TM_NODES: return launch_dim<D, TM_NODES>(model, mode, a, s);
     }
     return cudaErrorInvalidValue;
 }
