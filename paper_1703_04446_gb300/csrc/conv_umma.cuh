@@ -1,11 +1,11 @@
 // Tensor-core convolutions of the warm-start network: every 3x3 convolution
 // and both of its gradients as an implicit GEMM on the 5th-generation tensor
 // cores (tcgen05.mma, kind::f16: bf16 operands, FP32 accumulation in tensor
-// memory).
+// memory), with the operands brought to shared memory by TMA.
 //
-//   forward       D[pixel][co]      = sum_(ci,tap) x_eff[pixel + tap][ci] W[co][ci][tap]
-//   data gradient D[in pixel][ci]   = sum_(co,tap,up) dz[pixel - tap][co] W[co][ci][tap]
-//   weight grad.  D[co][(ci,tap)]   = sum_pixel dz[pixel][co] x_eff[pixel + tap][ci]
+//   forward       D[pixel][co]       = sum_(tap,ci) x_eff[pixel + tap][ci] W[co][ci][tap]
+//   data gradient D[in pixel][ci]    = sum_(tap,up,co) dz[pixel - tap][co] W[co][ci][tap]
+//   weight grad.  D[(tap,ci)][co]    = sum_pixel x_eff[pixel + tap][ci] dz[pixel][co]
 //
 // The network's FP32 activations and gradients enter as sums of three bf16
 // planes, x = hi + mid + lo with hi = bf16(x), mid = bf16(x - hi), lo =
@@ -18,33 +18,45 @@
 // exponents reach 2^-16 of the leading one are formed (the three dropped
 // ones are below FP32 resolution).
 //
-// One CTA of 128 threads computes a 128 x BN tile of D.  Per K chunk of 64,
-// the threads gather the operands (the im2col addressing of the convolution)
-// and write them to shared memory in the K-major canonical layout of the
-// tensor cores without swizzle: core matrices of 8 rows x 16 bytes, the 8
-// core matrices of a row group along K at 128-byte steps (leading byte
-// offset 128), row groups at 1024-byte steps (stride byte offset 1024).  One
-// elected thread issues the MMAs (K = 16 each) and commits them to the
-// stage's mbarrier; with two stages the gather of chunk c + 1 overlaps the
-// MMAs of chunk c, with one the next gather waits for them (and two CTAs fit
-// on an SM instead, overlapping each other).  The epilogue reads the accumulator from
-// tensor memory (tcgen05.ld, each warp its 32 lanes) and applies bias, ReLU,
-// skip connection and scale, or writes gradients / weight-gradient partials.
-// Every mbarrier wait is bounded; a wait that runs out sets an error flag,
-// waits once more for the MMAs in flight, skips the epilogue and frees the
-// tensor memory.
+// Operands.  The planes of a tensor are one NHWC array [3][B][h][h][cp] (cp:
+// channels padded to a multiple of 16), described to TMA as a 5D tensor.  A
+// box of spatial positions x `kb` channels x 3 planes of it is a whole operand
+// tile in the tensor cores' swizzled layout: a row of shared memory is one
+// pixel's channels.  A convolution's tap is a shift of the box (zero fill
+// outside the image is the padding), a stride of two is a traversal stride of
+// the tensor map, and what has no such form is cut into the four parities of
+// the finer grid (`phases`): an upsampled input, and the data gradient of a
+// stride-2 layer, whose pixels of one parity meet the same subset of the taps.
+// The forward and data-gradient GEMMs read the tile K-major (K = channels of
+// one tap), the weight gradient MN-major (K = pixels).
+//
+// A CTA is persistent (one per SM) and has a TMA warp, an MMA warp and four
+// epilogue warps.  Tiles of 128 rows x bn columns (x a slice of K) are handed
+// out in turn; operand stages form a ring with full / empty mbarriers, and two
+// accumulators in tensor memory let the epilogue of one tile run under the
+// MMAs of the next.  K runs in the order (tap, channel), 16 at a time with the
+// plane products innermost, in one accumulator.
+//
+// The per-thread gather this replaces (cp.async of 16-byte chunks, one operand
+// stage per CTA) waited on its copies: 0.40 ms for the 128 -> 64 channel
+// upsampled layer at batch 32 (tensor pipe 7% active), and the weight
+// gradient, which split FP32 elements on the fly, 1.7 ms.
+//
+// Every mbarrier wait is bounded; a wait that runs out sets an error flag and
+// a flag that ends the CTA's other roles, the CTA then waits (bounded) for its
+// copies and MMAs in flight and frees the tensor memory.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
 
 namespace umma {
 
 constexpr int BM = 128;
-constexpr int BK = 64;
-constexpr int kThreads = 128;
-constexpr int kMaxStages = 2;
-constexpr int kTileBytes = BM * BK * 2;     // one bf16 plane of a 128 x 64 operand tile
+constexpr int BK = 64;                      // K per chunk (the unit of the K split)
+constexpr int kThreads = 192;               // TMA warp, MMA warp, four epilogue warps
+constexpr int kMaxStages = 6;
 constexpr long kWaitLimit = 1L << 22;       // mbarrier polls before giving up
 
 enum Kind { FWD = 0, BWD_DATA = 1, BWD_WEIGHT = 2 };
@@ -52,20 +64,27 @@ enum Kind { FWD = 0, BWD_DATA = 1, BWD_WEIGHT = 2 };
 struct ConvGemm {
     int kind;
     int ci, co, stride, up, hin, hout, batch;   // the layer and the batch
-    int cp;                   // FWD: input channels padded to 8; BWD_DATA: output channels padded to 8
-    int M, N, K;              // GEMM sizes
-    int bn;                   // N per CTA: multiple of 16, <= 256 (<= 128 for BWD_WEIGHT)
-    int chunks_per_split;     // K chunks per CTA along grid.z (split K; every chunk when grid.z = 1)
-    float* part;              // FWD, BWD_DATA with grid.z > 1: raw partial tiles [z][N][M], finished by
-                              // finish_split_kernel
-    int stages;               // operand buffers in shared memory (1 or 2)
-    const float* a;           // BWD_WEIGHT: output gradient dz
-    const __nv_bfloat16* planes;  // FWD: the input's planes; BWD_DATA: dz's planes ([3][B][h][h][cp], see split_planes)
-    size_t plane_elems;       // elements of one plane
-    const float* x;           // BWD_WEIGHT: layer input x (the B operand)
-    const __nv_bfloat16* w;   // FWD, BWD_DATA: weight matrix [rows >= N rounded to bn][wld], zero padded
-    int wld;                  // its row length (K rounded up to 64)
-    float* out;               // FWD: layer output; BWD_DATA: input gradient; BWD_WEIGHT: partials [z][co][ci*9]
+    int cp;                   // channels of the A planes (padded): FWD and BWD_WEIGHT the input's, BWD_DATA dz's
+    int kb;                   // channels per row of the A tile (64, 32 or 16: its swizzle)
+    int kz;                   // BWD_WEIGHT: the same for the dz tile
+    int N;                    // columns of D
+    int bn;                   // columns per tile: a multiple of 16, <= 256 (<= 128 for BWD_WEIGHT)
+    int ntn;                  // column tiles
+    int grid;                 // side of the grid of positions that is tiled
+    int phases;               // 1, or 4 parities of the finer grid
+    int bx, by, bb;           // box of positions (powers of two): 128, or 64 for BWD_WEIGHT (its K chunk)
+    int tx, ty, tb;           // boxes per axis
+    int mtiles;               // BWD_WEIGHT: tiles of 128 rows (tap, ci); else unused
+    int chunks, chunks_per_split, splits;   // K chunks, and how they are split over tiles
+    int items;                // tiles in all
+    int stages, stage_bytes, a_bytes;
+    int ncols;                // tensor-memory columns of one accumulator
+    long long M;              // FWD, BWD_DATA: rows of D (pixels of the batch)
+    float* part;              // FWD, BWD_DATA with splits > 1: raw partial tiles [split][N][M], finished by
+                              // finish_split_kernel; BWD_WEIGHT: [split][co][9 cp]
+    float* out;               // FWD: layer output (may be NULL); BWD_DATA: input gradient
+    __nv_bfloat16* nplanes;   // FWD: the output's planes, the next layer's input (may be NULL)
+    int ncp;                  // their channels (co padded to 16)
     float* r;                 // FWD: activation before the skip add (may be NULL)
     const float* add;         // FWD: skip tensor (may be NULL)
     const float* bias;        // FWD
@@ -77,19 +96,23 @@ struct ConvGemm {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Shared-memory matrix descriptor, K-major without swizzle (leading byte
-// offset: core matrices along K; stride byte offset: 8-row groups).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+// Shared-memory matrix descriptor of a swizzled tile whose rows are 2 kb bytes
+// (leading byte offset: MN blocks of an MN-major tile; stride byte offset:
+// 8-row groups; swizzle of 128, 64 or 32 bytes).
+__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo, int kb) {
     uint64_t d = (uint64_t)((addr >> 4) & 0x3FFFu);
     d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
     d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
     d |= (uint64_t)1 << 46;   // descriptor version of this architecture
+    d |= (uint64_t)(kb == 64 ? 2 : (kb == 32 ? 4 : 6)) << 61;
     return d;
 }
 
-// Instruction descriptor of kind::f16: D FP32, A and B bf16, both K-major, M x N.
-__host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// Instruction descriptor of kind::f16: D FP32, A and B bf16, M x N; mn: both
+// operands MN-major instead of K-major.
+__device__ __forceinline__ uint32_t instr_desc(int M, int N, bool mn) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? (1u << 15) | (1u << 16) : 0u) | ((uint32_t)(N >> 3) << 17) |
+           ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
@@ -99,19 +122,56 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
         "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
+__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)));
+}
+
+__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity));
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
     return ok != 0;
 }
 
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-    for (long i = 0; i < kWaitLimit; ++i)
+// Waits for the phase; false when the polls run out or another role gave up.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* dead) {
+    for (long i = 0; i < kWaitLimit; ++i) {
         if (mbar_try(bar, parity)) return true;
+        if ((i & 255) == 255 && *dead) return false;
+    }
+    *dead = 1;
     return false;
+}
+
+__device__ __forceinline__ void tma_5d(uint32_t dst, const CUtensorMap* map, uint64_t* bar, int c, int x, int y, int b) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], "
+        "[%2];" ::"r"(dst),
+        "l"(map), "r"(smem_u32(bar)), "r"(c), "r"(x), "r"(y), "r"(b), "r"(0)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap* map, uint64_t* bar, int k, int row) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
+            dst),
+        "l"(map), "r"(smem_u32(bar)), "r"(k), "r"(row)
+        : "memory");
 }
 
 // x = hi + mid + lo exactly (see the file comment)
@@ -122,339 +182,386 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16& h, __nv_bfloat16&
     l = __float2bfloat16_rn(r1 - __bfloat162float(m));
 }
 
-// Byte offset of the 16-byte chunk (row, k group) in a canonical tile.
-__device__ __forceinline__ uint32_t chunk_off(int row, int kg) {
-    return (uint32_t)(((row >> 3) * 8 + kg) * 128 + (row & 7) * 16);
+// The planes of 8 channels of one pixel, at element e of planes of pe elements.
+__device__ __forceinline__ void store_planes8(__nv_bfloat16* planes, size_t pe, size_t e, const float* v) {
+    __align__(16) __nv_bfloat16 h[8], m[8], l[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) split3(v[j], h[j], m[j], l[j]);
+    *reinterpret_cast<uint4*>(planes + e) = *reinterpret_cast<const uint4*>(h);
+    *reinterpret_cast<uint4*>(planes + pe + e) = *reinterpret_cast<const uint4*>(m);
+    *reinterpret_cast<uint4*>(planes + 2 * pe + e) = *reinterpret_cast<const uint4*>(l);
 }
 
-// Input value at effective position (y, x) of an (optionally upsampled) input
-// of side hin; zero outside.
-__device__ __forceinline__ float in_eff(const float* __restrict__ in, int hin, int up, int y, int x) {
-    const int he = up ? 2 * hin : hin;
-    if (y < 0 || x < 0 || y >= he || x >= he) return 0.0f;
-    if (up) {
-        y >>= 1;
-        x >>= 1;
-    }
-    return __ldg(in + (size_t)y * hin + x);
-}
-
-// Element (row, k) of the A operand of BWD_WEIGHT: row = output channel, k
-// = pixel of the batch (zero outside the GEMM).
-__device__ __forceinline__ float a_elem(const ConvGemm& g, int row, int k) {
-    if (row >= g.M || k >= g.K) return 0.0f;
-    const int P = g.hout * g.hout;
-    const int b = k / P, o = k - b * P;
-    return __ldg(g.a + ((size_t)b * g.co + row) * P + o);
-}
-
-// The row of A a thread gathers for FWD and BWD_DATA, decomposed once: its
-// image and pixel coordinates (rows past M are marked invalid).
-struct RowCtx {
-    bool valid;
-    int b, y, x;     // FWD: output pixel (oy, ox); BWD_DATA: input pixel (iy, ix)
+// One tile of work.  FWD, BWD_DATA: a box of 128 positions of one parity, a
+// column tile and a slice of K.  BWD_WEIGHT: 128 rows (tap, ci), a column tile
+// and a slice of the pixel chunks.
+struct Item {
+    int nt, sp, ph, x0, y0, b0, mt;
 };
 
-__device__ __forceinline__ RowCtx row_ctx(const ConvGemm& g, int row) {
-    RowCtx r;
-    r.valid = row < g.M;
-    const int h = g.kind == FWD ? g.hout : g.hin;
-    const int P = h * h;
-    r.b = row / P;
-    const int p = row - r.b * P;
-    r.y = p / h;
-    r.x = p - r.y * h;
-    return r;
+__device__ __forceinline__ void box_origin(const ConvGemm& g, int tile, int& x0, int& y0, int& b0) {
+    x0 = (tile % g.tx) * g.bx;
+    tile /= g.tx;
+    y0 = (tile % g.ty) * g.by;
+    b0 = (tile / g.ty) * g.bb;
 }
 
-// The source of the 16-byte chunks (three planes) of A at the thread's row
-// for the K position `pos` (tap, or tap and up position) and channels c0 ..
-// c0 + 7, for FWD and BWD_DATA: K runs over (pos, channel) with the channel
-// fastest, so a chunk is 8 channels of one source pixel of the NHWC planes.
-// Returns false where the tap falls outside (the chunk is zero); e receives
-// the element offset of the chunk in one plane.
-__device__ __forceinline__ bool a_chunk_src(const ConvGemm& g, const RowCtx& r, int pos, int c0, size_t* e) {
-    if (!r.valid || pos >= (g.up && g.kind == BWD_DATA ? 36 : 9)) return false;
-    int y, x, h;
-    if (g.kind == FWD) {
-        const int ky = pos / 3, kx = pos - ky * 3;
-        const int ey = r.y * g.stride + ky - 1, ex = r.x * g.stride + kx - 1;
-        const int he = g.up ? 2 * g.hin : g.hin;
-        if (ey < 0 || ex < 0 || ey >= he || ex >= he) return false;
-        y = g.up ? ey >> 1 : ey;
-        x = g.up ? ex >> 1 : ex;
-        h = g.hin;
-    } else {   // BWD_DATA: pos = tap * R + up position
-        const int R = g.up ? 4 : 1;
-        const int t = pos / R, dd = pos - t * R;
-        const int ky = t / 3, kx = t - ky * 3;
-        const int ey = g.up ? 2 * r.y + (dd >> 1) : r.y, ex = g.up ? 2 * r.x + (dd & 1) : r.x;
-        const int ny = ey + 1 - ky, nx = ex + 1 - kx;
-        if (ny < 0 || nx < 0) return false;
-        if (g.stride == 2 && ((ny | nx) & 1)) return false;
-        y = ny / g.stride;
-        x = nx / g.stride;
-        if (y >= g.hout || x >= g.hout) return false;
-        h = g.hout;
+__device__ __forceinline__ Item item_at(const ConvGemm& g, int i) {
+    Item t;
+    t.nt = i % g.ntn;
+    i /= g.ntn;
+    t.ph = t.x0 = t.y0 = t.b0 = t.mt = 0;
+    if (g.kind == BWD_WEIGHT) {
+        t.mt = i % g.mtiles;
+        t.sp = i / g.mtiles;
+        return t;
     }
-    *e = (((size_t)r.b * h + y) * h + x) * g.cp + c0;
+    t.sp = i % g.splits;
+    i /= g.splits;
+    t.ph = i % g.phases;
+    box_origin(g, i / g.phases, t.x0, t.y0, t.b0);
+    return t;
+}
+
+// FWD, BWD_DATA: the K units (kb channels of one position pos: a tap, or a
+// tap and an up position) of a tile's slice of K.
+__device__ __forceinline__ void unit_range(const ConvGemm& g, int sp, int& u0, int& u1) {
+    const int upc = BK / g.kb, npos = g.kind == BWD_DATA && g.up ? 36 : 9;
+    u0 = sp * g.chunks_per_split * upc;
+    u1 = min((sp + 1) * g.chunks_per_split * upc, npos * (g.cp / g.kb));
+}
+
+// Start of the source box along one axis for tap coordinate k (0..2), up
+// position d, parity p and tile origin o; false when this parity does not
+// meet the tap (stride-2 data gradient).
+__device__ __forceinline__ bool axis_start(const ConvGemm& g, int o, int k, int d, int p, int& s) {
+    if (g.kind == BWD_DATA) {
+        if (g.up) {
+            s = 2 * o + d + 1 - k;
+        } else if (g.stride == 2) {
+            if ((p + 1 - k) & 1) return false;
+            s = o + (p + 1 - k) / 2;
+        } else {
+            s = o + 1 - k;
+        }
+    } else {
+        s = g.up ? o + ((p + k - 1) >> 1) : g.stride * o + k - 1;
+    }
     return true;
 }
 
-// 16 bytes global -> shared without passing through registers; with
-// valid == false the 16 shared bytes are zero-filled and nothing is read.
-__device__ __forceinline__ void cp_async16(uint8_t* dst, const void* src, bool valid) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0));
+__device__ __forceinline__ bool unit_source(const ConvGemm& g, const Item& t, int u, int& c0, int& x, int& y) {
+    const int upp = g.cp / g.kb, pos = u / upp;
+    c0 = (u - pos * upp) * g.kb;
+    const int R = g.kind == BWD_DATA && g.up ? 4 : 1, tap = pos / R, dd = pos - tap * R;
+    const int ky = tap / 3, kx = tap - ky * 3;
+    return axis_start(g, t.y0, ky, dd >> 1, t.ph >> 1, y) && axis_start(g, t.x0, kx, dd & 1, t.ph & 1, x);
 }
 
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Three bf16 planes of an FP32 tensor [B][C][h][h] (NCHW) in NHWC order with
-// the channels padded to cp (a multiple of 8) by zeros: plane q, element
-// ((b h + y) h + x) cp + c.  One thread per 8 channels of one pixel.
-__global__ void split_planes_kernel(const float* __restrict__ src, __nv_bfloat16* planes, int B, int C, int h,
-                                    int cp) {
-    const size_t P = (size_t)h * h;
-    const size_t n = (size_t)B * P * (cp / 8);
-    const size_t pe = (size_t)B * P * cp;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t pix = i % (B * P);            // consecutive threads: consecutive pixels (coalesced reads)
-        const int c0 = (int)(i / (B * P)) * 8;
-        const size_t b = pix / P, o = pix % P;
-        __align__(16) __nv_bfloat16 hv[8], mv[8], lv[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int c = c0 + j;
-            const float v = c < C ? __ldg(src + (b * C + c) * P + o) : 0.0f;
-            split3(v, hv[j], mv[j], lv[j]);
-        }
-        const size_t e = pix * cp + c0;
-        *reinterpret_cast<uint4*>(planes + e) = *reinterpret_cast<const uint4*>(hv);
-        *reinterpret_cast<uint4*>(planes + pe + e) = *reinterpret_cast<const uint4*>(mv);
-        *reinterpret_cast<uint4*>(planes + 2 * pe + e) = *reinterpret_cast<const uint4*>(lv);
-    }
-}
-
-// Element (row, k) of the B operand of BWD_WEIGHT: row = (ci, tap), k = pixel.
-__device__ __forceinline__ float bw_elem(const ConvGemm& g, int row, int k) {
-    if (row >= g.N || k >= g.K) return 0.0f;
-    const int P = g.hout * g.hout;
-    const int b = k / P, o = k - b * P;
-    const int oy = o / g.hout, ox = o - oy * g.hout;
-    const int c = row / 9, t = row - c * 9;
-    const int ky = t / 3, kx = t - ky * 3;
-    const float* in = g.x + ((size_t)b * g.ci + c) * g.hin * g.hin;
-    return in_eff(in, g.hin, g.up, oy * g.stride + ky - 1, ox * g.stride + kx - 1);
-}
-
-// Gather 8 FP32 values (row, k0 .. k0 + 7) and store their three bf16 planes
-// at chunk offset `off` of the plane tiles starting at `planes` (kTileBytes
-// apart for A, bn * 128 apart for B).
-template <bool IS_A>
-__device__ __forceinline__ void gather_split(const ConvGemm& g, int row, int k0, uint8_t* planes, uint32_t pstride,
-                                             uint32_t off) {
-    __align__(16) __nv_bfloat16 h[8], m[8], l[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const float v = IS_A ? a_elem(g, row, k0 + j) : bw_elem(g, row, k0 + j);
-        split3(v, h[j], m[j], l[j]);
-    }
-    *reinterpret_cast<uint4*>(planes + off) = *reinterpret_cast<const uint4*>(h);
-    *reinterpret_cast<uint4*>(planes + pstride + off) = *reinterpret_cast<const uint4*>(m);
-    *reinterpret_cast<uint4*>(planes + 2 * pstride + off) = *reinterpret_cast<const uint4*>(l);
-}
-
-__host__ __device__ inline size_t stage_bytes(int kind, int bn) {
-    return (size_t)3 * kTileBytes + (size_t)(kind == BWD_WEIGHT ? 3 : 1) * bn * BK * 2;
-}
-
-__global__ void __launch_bounds__(kThreads, 1) conv_gemm_kernel(const ConvGemm g) {
-    extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ __align__(8) uint64_t bar[kMaxStages];
+__global__ void __launch_bounds__(kThreads, 1)
+    conv_gemm_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
+                     const ConvGemm g) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], accf[2], acce[2];
     __shared__ uint32_t tmem_base;
+    __shared__ int dead;
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool bw = g.kind == BWD_WEIGHT;
-    const int pb = bw ? 3 : 1;                    // B planes
-    const uint32_t bplane = (uint32_t)g.bn * BK * 2;
-    const size_t sbytes = stage_bytes(g.kind, g.bn);
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * g.bn;
-    const int nchunks_all = (g.K + BK - 1) / BK;
-    const int c_begin = blockIdx.z * g.chunks_per_split;
-    const int c_end = min(nchunks_all, c_begin + g.chunks_per_split);
-    const bool split = !bw && gridDim.z > 1;
-    const uint32_t ncols = g.bn <= 32 ? 32u : (g.bn <= 64 ? 64u : (g.bn <= 128 ? 128u : 256u));
+    const uint32_t alloc_cols = 2u * (uint32_t)g.ncols;
 
-    if (warp == 0) {
+    if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(ncols));
+                     "r"(alloc_cols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        for (int s = 0; s < kMaxStages; ++s)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bar[s])), "r"(1));
+        dead = 0;
+        for (int s = 0; s < kMaxStages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(&accf[s], 1);
+            mbar_init(&acce[s], 4);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_base;
-    const uint32_t idesc = instr_desc(BM, g.bn);
+    const uint32_t smem0 = smem_u32(smem);
+    const int S = g.stages;
+    const uint32_t arow = 2u * (uint32_t)g.kb;                  // bytes of a row of the A tile
+    const uint32_t zrow = 2u * (uint32_t)g.kz;                  // of the dz tile (BWD_WEIGHT)
 
-    const RowCtx rc = row_ctx(g, m0 + tid);    // FWD, BWD_DATA: this thread's A row
-    bool failed = false;
-    int issued = 0;
-    int last = -1;      // index (from c_begin) of the last chunk whose MMAs were committed
-    for (int c = c_begin; c < c_end; ++c) {
-        const int S = g.stages, i = c - c_begin, s = i % S;
-        uint8_t* sa = smem + s * sbytes;
-        uint8_t* sb = sa + 3 * kTileBytes;
-        if (i >= S) {   // the MMAs of chunk i - S read this stage (its use i / S - 1): one thread polls
-            const bool ok = tid != 0 || mbar_wait(&bar[s], (uint32_t)((i / S - 1) & 1));
-            if (__syncthreads_or(!ok)) {
-                failed = true;
-                break;
-            }
-        }
-        const int k0 = c * BK;
-        // A: 128 rows x 8 k groups
-        if (g.kind == BWD_WEIGHT) {
-            for (int it = tid; it < BM * 8; it += kThreads) {    // lanes along k: contiguous pixels
-                const int row = it >> 3, kg = it & 7;
-                gather_split<true>(g, m0 + row, k0 + kg * 8, sa, kTileBytes, chunk_off(row, kg));
-            }
-        } else {
-            // lanes along rows: neighbouring pixels; (pos, c0) of k0 + 8 kg stepped, not divided.
-            // The 24 copies of a thread are all in flight before the wait below.
-            int pos = k0 / g.cp, c0 = k0 - pos * g.cp;
-#pragma unroll
-            for (int kg = 0; kg < 8; ++kg) {
-                size_t e = 0;
-                const bool ok = a_chunk_src(g, rc, pos, c0, &e);
-                const uint32_t off = chunk_off(tid, kg);
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    cp_async16(sa + q * kTileBytes + off, g.planes + q * g.plane_elems + (ok ? e : 0), ok);
-                c0 += 8;
-                if (c0 == g.cp) {
-                    c0 = 0;
-                    ++pos;
-                }
-            }
-        }
-        // B: bn rows x 8 k groups
-        if (bw) {
-            for (int it = tid; it < g.bn * 8; it += kThreads) {
-                const int row = it >> 3, kg = it & 7;
-                gather_split<false>(g, n0 + row, k0 + kg * 8, sb, bplane, chunk_off(row, kg));
-            }
-        } else {
-            for (int it = tid; it < g.bn * 8; it += kThreads) {
-                const int row = it >> 3, kg = it & 7;
-                cp_async16(sb + chunk_off(row, kg), g.w + (size_t)(n0 + row) * g.wld + k0 + kg * 8, true);
-            }
-            cp_async_wait_all();
-        }
-        asm volatile("fence.proxy.async.shared::cta;");
-        __syncthreads();
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            const uint32_t a0 = smem_u32(sa), b0 = smem_u32(sb);
-#pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk) {
-                // plane pairs (pa, pb) with pa + pb <= 2
-#pragma unroll
-                for (int pa = 0; pa < 3; ++pa) {
-                    for (int q = 0; q < pb && pa + q <= 2; ++q) {
-                        const uint64_t ad = smem_desc(a0 + pa * kTileBytes + kk * 256, 128, 1024);
-                        const uint64_t bd = smem_desc(b0 + q * bplane + kk * 256, 128, 1024);
-                        mma_bf16(tmem, ad, bd, idesc, (issued > 0) ? 1u : 0u);
-                        ++issued;
+    if (warp == 0) {
+        // ---- TMA: one elected thread
+        if (lane == 0) {
+            int n = 0;                                          // stages filled so far
+            bool ok = true;
+            for (int it = blockIdx.x; ok && it < g.items; it += gridDim.x) {
+                const Item t = item_at(g, it);
+                if (!bw) {
+                    int u0, u1;
+                    unit_range(g, t.sp, u0, u1);
+                    for (int u = u0; u < u1; ++u) {
+                        int c0, x, y;
+                        if (!unit_source(g, t, u, c0, x, y)) continue;
+                        const int s = n % S;
+                        if (n >= S && !(ok = mbar_wait(&empty[s], (uint32_t)((n / S - 1) & 1), &dead))) break;
+                        const uint32_t sa = smem0 + (uint32_t)s * (uint32_t)g.stage_bytes;
+                        mbar_expect(&full[s], 3u * BM * arow + (uint32_t)g.bn * arow);
+                        tma_5d(sa, &amap, &full[s], c0, x, y, t.b0);
+                        tma_2d(sa + (uint32_t)g.a_bytes, &bmap, &full[s], u * g.kb, t.nt * g.bn);
+                        ++n;
+                    }
+                } else {
+                    const int nblk = 9 * g.cp / g.kb, per = BM / g.kb, bpt = g.cp / g.kb;
+                    const int b_lo = t.mt * per, b_hi = min(nblk, b_lo + per);
+                    const int tiles = g.tx * g.ty * g.tb;
+                    const int c_hi = min(g.chunks, (t.sp + 1) * g.chunks_per_split);
+                    for (int c = t.sp * g.chunks_per_split; c < c_hi; ++c) {
+                        const int ph = c / tiles;
+                        int x0, y0, b0;
+                        box_origin(g, c - ph * tiles, x0, y0, b0);
+                        const int s = n % S;
+                        if (n >= S && !(ok = mbar_wait(&empty[s], (uint32_t)((n / S - 1) & 1), &dead))) break;
+                        const uint32_t sa = smem0 + (uint32_t)s * (uint32_t)g.stage_bytes;
+                        const uint32_t ablk = 3u * BK * arow, zblk = 3u * BK * zrow;
+                        mbar_expect(&full[s], (uint32_t)(b_hi - b_lo) * ablk + (uint32_t)(g.bn / g.kz) * zblk);
+                        for (int b = b_lo; b < b_hi; ++b) {
+                            const int tap = b / bpt, ky = tap / 3, kx = tap - ky * 3;
+                            int x, y;
+                            axis_start(g, y0, ky, 0, ph >> 1, y);
+                            axis_start(g, x0, kx, 0, ph & 1, x);
+                            tma_5d(sa + (uint32_t)(b - b_lo) * ablk, &amap, &full[s], (b - tap * bpt) * g.kb, x, y, b0);
+                        }
+                        for (int j = 0; j < g.bn / g.kz; ++j)
+                            tma_5d(sa + (uint32_t)g.a_bytes + (uint32_t)j * zblk, &bmap, &full[s],
+                                   t.nt * g.bn + j * g.kz, g.up ? 2 * x0 + (ph & 1) : x0,
+                                   g.up ? 2 * y0 + (ph >> 1) : y0, b0);
+                        ++n;
                     }
                 }
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_u32(&bar[s])));
-        }
-        last = i;   // a later chunk reusing this stage waits for these MMAs first (above)
-    }
-    if (!failed && last >= 0) {
-        // the last commit covers every MMA issued before it
-        const bool ok = tid != 0 || mbar_wait(&bar[last % g.stages], (uint32_t)((last / g.stages) & 1));
-        failed = __syncthreads_or(!ok);
-    }
-    if (failed) {
-        if (tid == 0) atomicExch(g.err, 1);
-        // once more, bounded, for whatever is still in flight
-        if (tid == 0 && last >= 0) mbar_wait(&bar[last % g.stages], (uint32_t)((last / g.stages) & 1));
-    } else if (last >= 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const int row = m0 + warp * 32 + lane;     // this thread's accumulator row (TMEM lane)
-        for (int c0 = 0; c0 < g.bn; c0 += 16) {
-            uint32_t v[16];
-            const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                : "r"(ta));
-            asm volatile("tcgen05.wait::ld.sync.aligned;");
-            if (row >= g.M) continue;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int n = n0 + c0 + j;
-                if (n >= g.N) break;
-                const float acc = __uint_as_float(v[j]);
-                if (split) {
-                    g.part[((size_t)blockIdx.z * g.N + n) * g.M + row] = acc;
-                } else if (g.kind == FWD) {
-                    const int P = g.hout * g.hout;
-                    const int b = row / P, o = row - b * P;
-                    const size_t oi = ((size_t)b * g.co + n) * P + o;
-                    float z = acc + g.bias[n];
-                    if (g.relu) z = fmaxf(z, 0.0f);
-                    if (g.r != nullptr) g.r[oi] = z;
-                    if (g.add != nullptr) z += g.add[oi];
-                    g.out[oi] = g.scale * z;
-                } else if (g.kind == BWD_DATA) {
-                    const int P = g.hin * g.hin;
-                    const int b = row / P, p = row - b * P;
-                    float* o = g.out + ((size_t)b * g.ci + n) * P + p;
-                    *o = g.accumulate ? *o + acc : acc;
-                } else {
-                    g.out[((size_t)blockIdx.z * g.co + row) * g.N + n] = acc;
+            // the copies still in flight land before the CTA may end (bounded)
+            for (int k = max(0, n - S); !ok && k < n; ++k) {
+                for (long i = 0; i < kWaitLimit && !mbar_try(&full[k % S], (uint32_t)((k / S) & 1)); ++i) {
                 }
             }
+        }
+    } else if (warp == 1) {
+        // ---- MMA: one elected thread
+        if (lane == 0) {
+            const uint32_t idesc = instr_desc(BM, g.bn, bw);
+            int n = 0, a = 0;                                   // stages consumed, tiles begun
+            bool ok = true;
+            for (int it = blockIdx.x; ok && it < g.items; it += gridDim.x, ++a) {
+                const Item t = item_at(g, it);
+                const int ab = a & 1;
+                if (a >= 2 && !(ok = mbar_wait(&acce[ab], (uint32_t)((a / 2 - 1) & 1), &dead))) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t d = tmem + (uint32_t)(ab * g.ncols);
+                uint32_t issued = 0;
+                int u0, u1;
+                if (bw) {
+                    u0 = t.sp * g.chunks_per_split;
+                    u1 = min(g.chunks, u0 + g.chunks_per_split);
+                } else {
+                    unit_range(g, t.sp, u0, u1);
+                }
+                for (int u = u0; u < u1; ++u) {
+                    int c0, x, y;
+                    if (!bw && !unit_source(g, t, u, c0, x, y)) continue;
+                    const int s = n % S;
+                    if (!(ok = mbar_wait(&full[s], (uint32_t)((n / S) & 1), &dead))) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t sa = smem0 + (uint32_t)s * (uint32_t)g.stage_bytes, sb = sa + (uint32_t)g.a_bytes;
+                    if (!bw) {
+                        for (int kk = 0; kk < g.kb / 16; ++kk) {
+                            const uint64_t bd = smem_desc(sb + kk * 32, 16, 8 * arow, g.kb);
+#pragma unroll
+                            for (int p = 0; p < 3; ++p) {
+                                mma_bf16(d, smem_desc(sa + p * BM * arow + kk * 32, 16, 8 * arow, g.kb), bd, idesc, issued);
+                                issued = 1;
+                            }
+                        }
+                    } else {
+                        // 16 pixels at a time; plane pairs (dz, x) with pz + px <= 2
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+#pragma unroll
+                            for (int pz = 0; pz < 3; ++pz) {
+                                const uint64_t bd =
+                                    smem_desc(sb + pz * BK * zrow + kk * 16 * zrow, 3u * BK * zrow, 8 * zrow, g.kz);
+#pragma unroll
+                                for (int px = 0; px + pz <= 2; ++px) {
+                                    mma_bf16(d, smem_desc(sa + px * BK * arow + kk * 16 * arow, 3u * BK * arow, 8 * arow, g.kb),
+                                             bd, idesc, issued);
+                                    issued = 1;
+                                }
+                            }
+                        }
+                    }
+                    mma_commit(&empty[s]);
+                    ++n;
+                }
+                if (!ok) break;
+                if (issued) mma_commit(&accf[ab]);
+                else mbar_arrive(&accf[ab]);                    // an empty slice of K
+            }
+            // bounded wait for the MMAs still in flight
+            if (!ok && n > 0) {
+                for (long i = 0; i < kWaitLimit && !mbar_try(&empty[(n - 1) % S], (uint32_t)(((n - 1) / S) & 1)); ++i) {
+                }
+            }
+        }
+    } else {
+        // ---- epilogue: warp w reads the tensor-memory lanes 32 (w mod 4) ..
+        const int quad = warp & 3, row = quad * 32 + lane;
+        const int fine = g.phases == 4 && !bw ? 2 : 1;          // output positions per tiled position
+        const int ho = g.kind == FWD ? g.hout : g.hin;          // side of the output
+        int a = 0;
+        bool ok = true;
+        for (int it = blockIdx.x; ok && it < g.items; it += gridDim.x, ++a) {
+            const Item t = item_at(g, it);
+            const int ab = a & 1;
+            ok = mbar_wait(&accf[ab], (uint32_t)((a / 2) & 1), &dead);
+            if (__any_sync(0xffffffffu, !ok)) {
+                ok = false;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            bool empty_k = false;
+            if (!bw && g.kind == BWD_DATA && g.splits > 1) {    // a slice whose taps this parity never meets
+                int u0, u1, c0, x, y;
+                unit_range(g, t.sp, u0, u1);
+                empty_k = true;
+                for (int u = u0; empty_k && u < u1; ++u) empty_k = !unit_source(g, t, u, c0, x, y);
+            }
+            // where this row goes
+            bool valid;
+            size_t P = (size_t)ho * ho, o = 0;
+            int b = 0;
+            if (bw) {
+                o = (size_t)t.mt * BM + row;
+                valid = o < (size_t)9 * g.cp;
+            } else {
+                const int px = t.x0 + row % g.bx, py = t.y0 + (row / g.bx) % g.by;
+                b = t.b0 + row / (g.bx * g.by);
+                valid = px < g.grid && py < g.grid && b < g.batch;
+                o = (size_t)(py * fine + (fine == 2 ? t.ph >> 1 : 0)) * ho + px * fine + (fine == 2 ? t.ph & 1 : 0);
+            }
+            for (int c0 = 0; c0 < g.bn; c0 += 16) {
+                uint32_t v[16];
+                const uint32_t ta = tmem + (uint32_t)(ab * g.ncols) + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+                    : "r"(ta));
+                asm volatile("tcgen05.wait::ld.sync.aligned;");
+                if (!valid) continue;
+                const int n0 = t.nt * g.bn + c0;
+                if (bw || g.splits > 1) {
+                    const size_t rows = bw ? (size_t)9 * g.cp : (size_t)g.M;
+                    float* p = g.part + ((size_t)t.sp * g.N + n0) * rows + (bw ? o : (size_t)b * P + o);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (n0 + j < g.N) p[j * rows] = empty_k ? 0.0f : __uint_as_float(v[j]);
+                } else if (g.kind == FWD) {
+                    // the loads of a group of columns are all in flight before its stores
+                    float z[16];
+                    const size_t oi = ((size_t)b * g.co + n0) * P + o;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) z[j] = g.add != nullptr && n0 + j < g.N ? __ldg(g.add + oi + j * P) : 0.0f;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const bool in = n0 + j < g.N;
+                        float t1 = __uint_as_float(v[j]) + (in ? __ldg(g.bias + n0 + j) : 0.0f);
+                        if (g.relu) t1 = fmaxf(t1, 0.0f);
+                        if (g.r != nullptr && in) g.r[oi + j * P] = t1;
+                        if (g.add != nullptr) t1 += z[j];
+                        z[j] = in ? g.scale * t1 : 0.0f;
+                        if (g.out != nullptr && in) g.out[oi + j * P] = z[j];
+                    }
+                    if (g.nplanes != nullptr && n0 < g.ncp) {
+                        const size_t pe = (size_t)g.batch * P * g.ncp, e = ((size_t)b * P + o) * g.ncp + n0;
+                        store_planes8(g.nplanes, pe, e, z);
+                        store_planes8(g.nplanes, pe, e + 8, z + 8);
+                    }
+                } else {
+                    float* p = g.out + ((size_t)b * g.ci + n0) * P + o;
+                    float z[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) z[j] = g.accumulate && n0 + j < g.N ? p[j * P] : 0.0f;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (n0 + j < g.N) p[j * P] = z[j] + __uint_as_float(v[j]);
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acce[ab]);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
+    if (tid == 0 && dead) atomicExch(g.err, 1);
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(alloc_cols));
 }
 
-// The end of a split-K FWD or BWD_DATA GEMM: the partial tiles summed over z
-// in increasing order (deterministic), then the epilogue of the unsplit
-// kernel.  One thread per (n, row), rows fastest.
+// The end of a split-K FWD or BWD_DATA GEMM: the partial tiles summed over the
+// splits in increasing order (deterministic), then the epilogue of the unsplit
+// kernel.  One thread per 8 columns of a row, rows fastest.
 __global__ void finish_split_kernel(const ConvGemm g, int splits) {
-    const size_t total = (size_t)g.M * g.N;
+    const size_t M = (size_t)g.M, total = M * ((g.N + 7) / 8);
+    const int h = g.kind == FWD ? g.hout : g.hin, C = g.kind == FWD ? g.co : g.ci;
+    const size_t P = (size_t)h * h;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int n = (int)(i / g.M), row = (int)(i - (size_t)n * g.M);
-        float acc = 0.0f;
-        for (int z = 0; z < splits; ++z) acc += g.part[((size_t)z * g.N + n) * g.M + row];
-        if (g.kind == FWD) {
-            const int P = g.hout * g.hout;
-            const int b = row / P, o = row - b * P;
-            const size_t oi = ((size_t)b * g.co + n) * P + o;
-            float z = acc + g.bias[n];
-            if (g.relu) z = fmaxf(z, 0.0f);
-            if (g.r != nullptr) g.r[oi] = z;
-            if (g.add != nullptr) z += g.add[oi];
-            g.out[oi] = g.scale * z;
-        } else {
-            const int P = g.hin * g.hin;
-            const int b = row / P, p = row - b * P;
-            float* o = g.out + ((size_t)b * g.ci + n) * P + p;
-            *o = g.accumulate ? *o + acc : acc;
+        const int n0 = (int)(i / M) * 8;
+        const size_t row = i - (size_t)(n0 / 8) * M, b = row / P, o = row - b * P;
+        float acc[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
+        for (int z = 0; z < splits; ++z) {
+            const float* p = g.part + ((size_t)z * g.N + n0) * M + row;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (n0 + j < g.N) acc[j] += p[j * M];
         }
+        const size_t oi = (b * C + n0) * P + o;
+        if (g.kind == FWD) {
+            float z[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) z[j] = g.add != nullptr && n0 + j < g.N ? __ldg(g.add + oi + j * P) : 0.0f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const bool in = n0 + j < g.N;
+                float t = acc[j] + (in ? __ldg(g.bias + n0 + j) : 0.0f);
+                if (g.relu) t = fmaxf(t, 0.0f);
+                if (g.r != nullptr && in) g.r[oi + j * P] = t;
+                if (g.add != nullptr) t += z[j];
+                z[j] = in ? g.scale * t : 0.0f;
+                if (g.out != nullptr && in) g.out[oi + j * P] = z[j];
+            }
+            if (g.nplanes != nullptr) store_planes8(g.nplanes, M * g.ncp, row * g.ncp + n0, z);
+        } else {
+            float z[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) z[j] = g.accumulate && n0 + j < g.N ? g.out[oi + j * P] : 0.0f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (n0 + j < g.N) g.out[oi + j * P] = z[j] + acc[j];
+        }
+    }
+    // channels of the planes past the last column group
+    if (g.kind == FWD && g.nplanes != nullptr && (g.N + 7) / 8 * 8 < g.ncp) {
+        const float zero[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        for (size_t row = blockIdx.x * (size_t)blockDim.x + threadIdx.x; row < M; row += (size_t)gridDim.x * blockDim.x)
+            store_planes8(g.nplanes, M * g.ncp, row * g.ncp + g.ncp - 8, zero);
     }
 }
 

@@ -16,9 +16,11 @@
 // FP32 master weights after every Adam step); activations, gradients and
 // accumulation are FP32.  Loss 1/2 mean((v - target)^2) / scale^2.
 //
-// Every convolution, its data gradient and its weight gradient run as implicit
-// GEMMs on the tensor cores (conv_umma.cuh); bias gradients, the loss, the
-// ReLU masks and Adam are elementwise kernels here.
+// The convolutions, their data gradients and their weight gradients run as
+// implicit GEMMs on the tensor cores (conv_umma.cuh), each reading the bf16
+// planes that the kernel before it wrote; the first layer (two input channels,
+// 18 products a value) and its weight gradient are direct FP32 kernels here, as
+// are the ReLU masks, the loss and Adam.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -42,16 +44,22 @@ struct Layer {
     size_t woff, boff;        // offsets of W and b in the parameter vector
     // bf16 weight matrices of the tensor-core GEMMs, zero padded, K ordered
     // as the operand planes are (channel fastest):
-    // forward wf[co][tap * cpi + ci] (cpi = ci rounded up to 8; rows to a
+    // forward wf[co][tap * cpi + ci] (cpi = ci rounded up to 16; rows to a
     // multiple of bnf, rows of ldf), data gradient
-    // wd[ci][(tap * R + up position) * cpo + co] (cpo = co rounded up to 8, R = 4 when up)
+    // wd[ci][(tap * R + up position) * cpo + co] (cpo = co rounded up to 16, R = 4 when up)
     int cpi, cpo, bnf, ldf, rowsf, bnd, ldd, rowsd;
     __nv_bfloat16 *wf, *wd;
 };
 
-#ifndef LGNK_CONV_STAGES
-#define LGNK_CONV_STAGES 1    // operand buffers per CTA (1: two CTAs per SM)
-#endif
+// The launch of one GEMM of a layer at one batch size: everything but the
+// tensors of the call.  Kept per layer and kind for the last batch size.
+struct Plan {
+    int batch = 0;
+    umma::ConvGemm g;
+    CUtensorMap a, b;
+    int grid = 0;
+    size_t smem = 0;
+};
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -77,41 +85,185 @@ __global__ void pack_wmats_kernel(const float* __restrict__ p, Layer L) {
     }
 }
 
-// dW[i] = sum_s part[s][i], s in increasing order.
-__global__ void sum_slices_kernel(const float* __restrict__ part, float* dW, size_t n, int slices) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+// The end of a layer's weight and bias gradients, partials summed in increasing
+// order: dW[co][ci][tap] = sum_s part[s][co][tap cp + ci], and behind it
+// db[co] = sum_s bpart[s][co].
+__global__ void sum_slices_kernel(const float* __restrict__ part, const float* __restrict__ bpart, float* dW, int co,
+                                  int ci, int cp, int slices, int bslices) {
+    const int nw = co * ci * 9, rows = 9 * cp;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nw + co; i += gridDim.x * blockDim.x) {
         float s = 0.0f;
-        for (int k = 0; k < slices; ++k) s += part[(size_t)k * n + i];
+        if (i < nw) {
+            const int n = i / (ci * 9), r = i - n * ci * 9, c = r / 9, t = r - c * 9;
+            const float* p = part + (size_t)n * rows + t * cp + c;
+            for (int k = 0; k < slices; ++k) s += p[(size_t)k * co * rows];
+        } else {
+            for (int k = 0; k < bslices; ++k) s += bpart[(size_t)k * co + i - nw];
+        }
         dW[i] = s;
     }
 }
 
-// db[co] = sum_{b, o} dz[b][co][o]
-__global__ void bias_grad_kernel(const float* __restrict__ dz, float* db, int C, size_t P, int B) {
-    const int co = blockIdx.x;
-    float s = 0.0f;
-    for (size_t q = threadIdx.x; q < P * B; q += blockDim.x) s += dz[((q / P) * C + co) * P + q % P];
-    __shared__ float red[kT];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = kT / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
+// The output gradient of a layer, dz = g (m > 0) (m: the ReLU's output, as FP32
+// mr or as planes mp of cp channels; none: dz = g), as planes and as partial
+// bias gradients bpart[s][co] (the sums over the pixels of block column s).
+// One pass over g instead of a masking pass, a splitting pass and a bias pass
+// (0.11 + 0.19 + 0.20 ms of a 128^2 batch-32 training step).  A thread handles 8
+// channels of one pixel at a time; a warp covers 4 (2) neighbouring channel
+// groups of 8 (16) pixels, so that reads (channel rows) and writes (pixels)
+// both touch whole sectors.
+constexpr int kBiasSlices = 64;
+__global__ void __launch_bounds__(kT) mask_split_kernel(const float* __restrict__ g, const float* __restrict__ mr,
+                                                        const __nv_bfloat16* __restrict__ mp, __nv_bfloat16* planes,
+                                                        float* bpart, int C, int cp, int P, int B, int gs) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pw = 32 / gs;      // pixels per warp
+    const int c0 = (blockIdx.y * gs + lane / pw) * 8;
+    const size_t n = (size_t)P * B, pe = n * cp;
+    float sum[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sum[j] = 0.0f;
+    const size_t step = (size_t)gridDim.x * (kT / 32) * pw;
+    for (size_t pix = ((size_t)blockIdx.x * (kT / 32) + warp) * pw + lane % pw; pix < n; pix += step) {
+        const size_t b = pix / P, o = pix - b * P, e = pix * cp + c0;
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = c0 + j < C ? __ldg(g + (b * C + c0 + j) * P + o) : 0.0f;
+        if (mr != nullptr) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (c0 + j < C && !(__ldg(mr + (b * C + c0 + j) * P + o) > 0.0f)) v[j] = 0.0f;
+        } else if (mp != nullptr) {
+            __align__(16) __nv_bfloat16 m[8];
+            *reinterpret_cast<uint4*>(m) = __ldg(reinterpret_cast<const uint4*>(mp + e));
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (!(__bfloat162float(m[j]) > 0.0f)) v[j] = 0.0f;
+        }
+        umma::store_planes8(planes, pe, e, v);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) sum[j] += v[j];
     }
-    if (threadIdx.x == 0) db[co] = red[0];
+    __shared__ float red[kT / 32][4][8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        for (int w = pw / 2; w > 0; w >>= 1) sum[j] += __shfl_down_sync(0xffffffffu, sum[j], w, pw);
+    if (lane % pw == 0) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) red[warp][lane / pw][j] = sum[j];
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < gs * 8) {
+        const int gi = threadIdx.x / 8, j = threadIdx.x % 8, c = (blockIdx.y * gs + gi) * 8 + j;
+        float s = 0.0f;
+        for (int w = 0; w < kT / 32; ++w) s += red[w][gi][j];
+        if (c < C) bpart[(size_t)blockIdx.x * C + c] = s;
+    }
 }
 
-// g *= (r > 0): gradient through a relu whose output is r.
-__global__ void relu_mask_kernel(float* g, const float* __restrict__ r, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        if (r[i] <= 0.0f) g[i] = 0.0f;
+// The first layer, e0 = relu(conv(x = [T, R]) + b), written as the next layer's
+// planes.  Two input channels make K = 18: as an implicit GEMM its operand rows
+// are 32 bytes of mostly padding (0.19 ms at batch 32, 128^2, against 0.10 ms for
+// a gather kernel); here a thread holds the 18 inputs of a pixel and makes
+// kFirstCh channels, bound by the 6 bytes a value it writes.
+constexpr int kFirstCh = 16;
+__global__ void __launch_bounds__(kT) conv_first_kernel(const float* __restrict__ T, const float* __restrict__ R,
+                                                        const float* __restrict__ W, const float* __restrict__ bias,
+                                                        __nv_bfloat16* planes, int C, int cp, int m, int B) {
+    __shared__ float w[kFirstCh][18], bs[kFirstCh];
+    const int c0 = blockIdx.y * kFirstCh;
+    for (int i = threadIdx.x; i < kFirstCh * 18; i += kT) {
+        const int c = i / 18, k = i % 18, tap = k >> 1, ci = k & 1;       // order (tap, ci)
+        w[c][k] = c0 + c < C ? __bfloat162float(__float2bfloat16_rn(W[((size_t)(c0 + c) * 2 + ci) * 9 + tap])) : 0.0f;
+    }
+    if (threadIdx.x < kFirstCh) bs[threadIdx.x] = c0 + (int)threadIdx.x < C ? bias[c0 + threadIdx.x] : 0.0f;
+    __syncthreads();
+    const size_t P = (size_t)m * m, n = P * B;
+    for (size_t i = blockIdx.x * (size_t)kT + threadIdx.x; i < n; i += (size_t)gridDim.x * kT) {
+        const size_t b = i / P;
+        const int o = (int)(i - b * P), y = o / m, x = o - y * m;
+        float in[18];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
+            const bool ok = yy >= 0 && yy < m && xx >= 0 && xx < m;
+            const size_t e = b * P + (size_t)(ok ? yy * m + xx : 0);
+            in[2 * t] = ok ? __ldg(T + e) : 0.0f;
+            in[2 * t + 1] = ok ? __ldg(R + e) : 0.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < kFirstCh; q += 8) {
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                float a = 0.0f;
+#pragma unroll
+                for (int k = 0; k < 18; ++k) a = fmaf(in[k], w[q + j][k], a);
+                v[j] = c0 + q + j < C ? fmaxf(a + bs[q + j], 0.0f) : 0.0f;
+            }
+            umma::store_planes8(planes, n * cp, i * cp + c0 + q, v);
+        }
+    }
 }
 
-__global__ void stack_input_kernel(const float* __restrict__ T, const float* __restrict__ R, float* x, size_t n, int B) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n * B; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t b = i / n, p = i % n;
-        x[(b * 2) * n + p] = T[i];
-        x[(b * 2 + 1) * n + p] = R[i];
+// Partial weight and bias gradients of the first layer from the gradient g of
+// e0 (masked here by e0 > 0, its planes): part[s][co][(tap, ci)] and bpart[s][co]
+// over the pixels of block column s.  A thread accumulates 18 x kFirstW products
+// over its pixels; a block sums them once.
+constexpr int kFirstW = 4;
+__global__ void __launch_bounds__(kT) conv_first_wgrad_kernel(const float* __restrict__ T, const float* __restrict__ R,
+                                                              const float* __restrict__ g,
+                                                              const __nv_bfloat16* __restrict__ e0, float* part,
+                                                              float* bpart, int C, int cp, int m, int B) {
+    const int c0 = blockIdx.y * kFirstW, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t P = (size_t)m * m, n = P * B;
+    float acc[kFirstW][19];
+#pragma unroll
+    for (int j = 0; j < kFirstW; ++j)
+#pragma unroll
+        for (int k = 0; k < 19; ++k) acc[j][k] = 0.0f;
+    for (size_t i = blockIdx.x * (size_t)kT + threadIdx.x; i < n; i += (size_t)gridDim.x * kT) {
+        const size_t b = i / P;
+        const int o = (int)(i - b * P), y = o / m, x = o - y * m;
+        __align__(8) __nv_bfloat16 h[kFirstW];
+        *reinterpret_cast<uint2*>(h) = __ldg(reinterpret_cast<const uint2*>(e0 + i * cp + c0));
+        float z[kFirstW];
+#pragma unroll
+        for (int j = 0; j < kFirstW; ++j) {
+            z[j] = c0 + j < C ? __ldg(g + (b * C + c0 + j) * P + o) : 0.0f;
+            if (!(__bfloat162float(h[j]) > 0.0f)) z[j] = 0.0f;
+            acc[j][18] += z[j];
+        }
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
+            const bool ok = yy >= 0 && yy < m && xx >= 0 && xx < m;
+            const size_t e = b * P + (size_t)(ok ? yy * m + xx : 0);
+            const float a = ok ? __ldg(T + e) : 0.0f, r = ok ? __ldg(R + e) : 0.0f;
+#pragma unroll
+            for (int j = 0; j < kFirstW; ++j) {
+                acc[j][2 * t] = fmaf(a, z[j], acc[j][2 * t]);
+                acc[j][2 * t + 1] = fmaf(r, z[j], acc[j][2 * t + 1]);
+            }
+        }
+    }
+    __shared__ float red[kT / 32][kFirstW * 19];
+#pragma unroll
+    for (int j = 0; j < kFirstW; ++j)
+#pragma unroll
+        for (int k = 0; k < 19; ++k) {
+            float s = acc[j][k];
+#pragma unroll
+            for (int w = 16; w > 0; w >>= 1) s += __shfl_down_sync(0xffffffffu, s, w);
+            if (lane == 0) red[warp][j * 19 + k] = s;
+        }
+    __syncthreads();
+    for (int q = threadIdx.x; q < kFirstW * 19; q += kT) {
+        const int j = q / 19, k = q % 19;
+        float s = 0.0f;
+        for (int w = 0; w < kT / 32; ++w) s += red[w][q];
+        if (c0 + j >= C) continue;
+        if (k < 18) part[((size_t)blockIdx.x * C + c0 + j) * 18 + k] = s;
+        else bpart[(size_t)blockIdx.x * C + c0 + j] = s;
     }
 }
 
@@ -161,11 +313,14 @@ struct lgnk_ws {
     std::vector<Layer> L;
     size_t nparams;
     float *p, *g, *am, *as;     // master weights, gradients, Adam moments
-    float *x, *e0, *e1, *e2, *e3, *r4, *d2, *r5, *d1, *z6;   // activations
-    float *ga, *gb, *gc;        // gradient scratch (largest activation each)
+    float *e1, *e2, *r4, *r5, *z6;   // activations that are read as FP32
+    float *ga, *gb, *gc;        // gradients of e1 (and d1), e2 (and d2), and the others in turn
     float* wpart;               // per-slice weight-gradient partials
-    __nv_bfloat16* planes;      // bf16 planes of a GEMM operand (umma::split_planes_kernel)
-    size_t planes_cap;          // elements of one plane it holds
+    float* bpart;               // per-slice bias-gradient partials
+    __nv_bfloat16* planes[7];   // bf16 planes of the input of layer 1..6
+    __nv_bfloat16* zplanes;     // of the output gradient at hand
+    Plan plans[7][3];           // [layer][umma::Kind]
+    int sms, smem_max;          // of the device: SMs, dynamic shared memory of the GEMM kernel
     float* gpart;               // split-K partial tiles of the FWD and BWD_DATA GEMMs
     size_t gpart_cap;           // floats it holds
     int* derr;                  // set by a tensor-core kernel whose wait ran out
@@ -198,20 +353,11 @@ lgnk_status ws_alloc_n(lgnk_ws* w, size_t n, T** out) {
 
 size_t act_size(const lgnk_ws* w, int layer_out_c, int side, int B) { return (size_t)B * layer_out_c * side * side; }
 
-// planes of src [B][C][h][h] into w->planes (channels padded to cp)
-cudaError_t split_planes(lgnk_ws* w, const float* src, int B, int C, int h, int cp, size_t* plane_elems) {
-    *plane_elems = (size_t)B * h * h * cp;
-    if (*plane_elems > w->planes_cap) return cudaErrorInvalidValue;
-    const size_t n = (size_t)B * h * h * (cp / 8);
-    umma::split_planes_kernel<<<blocks_for(n), kT, 0, w->stream>>>(src, w->planes, B, C, h, cp);
-    return cudaGetLastError();
-}
-
-// CTAs a GEMM launch should reach: two per SM
+// Tiles a split GEMM should reach: two per SM
 constexpr int kGemmCtas = 2 * 152;
 
 // K slices of a FWD / BWD_DATA GEMM with `tiles` output tiles and `chunks` K
-// chunks: enough slices to give about two CTAs per SM, each at least two
+// chunks: enough slices to give about two tiles per SM, each at least two
 // chunks (1 when the tiles alone fill the GPU)
 inline int split_slices(int tiles, int chunks) {
     if (tiles >= kGemmCtas) return 1;
@@ -220,42 +366,31 @@ inline int split_slices(int tiles, int chunks) {
     return (chunks + cps - 1) / cps;
 }
 
-cudaError_t launch_gemm(lgnk_ws* w, umma::ConvGemm& g, int grid_x, int grid_y, int grid_z) {
-    g.stages = LGNK_CONV_STAGES;
-    const size_t smem = (size_t)g.stages * umma::stage_bytes(g.kind, g.bn);
-    int dev = 0, optin = 0;
-    cudaFuncAttributes fa{};
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, umma::conv_gemm_kernel);
-    if (e == cudaSuccess && smem + fa.sharedSizeBytes > (size_t)optin) e = cudaErrorInvalidValue;
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(umma::conv_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 optin - (int)fa.sharedSizeBytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return e;
-    }
-    g.err = w->derr;
-    umma::conv_gemm_kernel<<<dim3(grid_x, grid_y, grid_z), umma::kThreads, smem, w->stream>>>(g);
-    return cudaGetLastError();
+// channels per row of an operand tile whose planes have cp channels
+inline int row_channels(int cp) { return cp % 64 == 0 ? 64 : (cp % 32 == 0 ? 32 : 16); }
+
+// The box of `total` positions (powers of two per axis) that covers a batch of
+// side x side grids with the fewest boxes; among equals the widest, so that
+// where the side divides, the boxes follow the pixels' linear order.
+void choose_box(int side, int batch, int total, umma::ConvGemm* g) {
+    long long best = -1;
+    for (int bx = total; bx >= 1; bx /= 2)
+        for (int by = total / bx; by >= 1; by /= 2) {
+            const int bb = total / (bx * by);
+            const long long n = (long long)((side + bx - 1) / bx) * ((side + by - 1) / by) * ((batch + bb - 1) / bb);
+            if (best >= 0 && n >= best) continue;
+            best = n;
+            g->bx = bx;
+            g->by = by;
+            g->bb = bb;
+        }
+    g->tx = (side + g->bx - 1) / g->bx;
+    g->ty = (side + g->by - 1) / g->by;
+    g->tb = (batch + g->bb - 1) / g->bb;
 }
 
-// a FWD or BWD_DATA GEMM, split along K when its tiles do not fill the GPU
-cudaError_t launch_gemm_split(lgnk_ws* w, umma::ConvGemm& g, int grid_y) {
-    const int gx = (g.M + umma::BM - 1) / umma::BM;
-    const int chunks = (g.K + umma::BK - 1) / umma::BK;
-    const int splits = split_slices(gx * grid_y, chunks);
-    g.chunks_per_split = (chunks + splits - 1) / splits;
-    g.part = w->gpart;
-    if (splits > 1 && (size_t)splits * g.M * g.N > w->gpart_cap) return cudaErrorInvalidValue;
-    cudaError_t e = launch_gemm(w, g, gx, grid_y, splits);
-    if (e != cudaSuccess || splits == 1) return e;
-    umma::finish_split_kernel<<<blocks_for((size_t)g.M * g.N), kT, 0, w->stream>>>(g, splits);
-    return cudaGetLastError();
-}
-
-umma::ConvGemm gemm_base(const Layer& L, int kind, int B) {
+// Everything of a layer's GEMM but its tensors, maps and stages.
+umma::ConvGemm gemm_shape(const Layer& L, int kind, int B) {
     umma::ConvGemm g{};
     g.kind = kind;
     g.ci = L.ci;
@@ -265,80 +400,186 @@ umma::ConvGemm gemm_base(const Layer& L, int kind, int B) {
     g.hin = L.hin;
     g.hout = L.hout;
     g.batch = B;
+    g.cp = kind == umma::BWD_DATA ? L.cpo : L.cpi;
+    g.kb = row_channels(g.cp);
+    g.phases = (kind != umma::BWD_DATA && L.up) || (kind == umma::BWD_DATA && L.stride == 2) ? 4 : 1;
+    if (kind == umma::BWD_WEIGHT) {
+        g.N = L.co;
+        g.kz = row_channels(L.cpo);
+        g.bn = std::min(128, L.cpo);
+        g.bn = round_up(g.bn, g.kz);
+        g.ntn = (L.cpo + g.bn - 1) / g.bn;
+        g.grid = L.up ? L.hin : L.hout;
+        choose_box(g.grid, B, umma::BK, &g);
+        g.mtiles = (9 * g.cp + umma::BM - 1) / umma::BM;
+        g.chunks = g.phases * g.tx * g.ty * g.tb;
+        const int tiles = g.mtiles * g.ntn;
+        const int s = std::min(kMaxSlices, std::min(g.chunks, std::max(1, (kGemmCtas + tiles - 1) / tiles)));
+        g.chunks_per_split = (g.chunks + s - 1) / s;
+        g.splits = (g.chunks + g.chunks_per_split - 1) / g.chunks_per_split;
+        g.items = tiles * g.splits;
+        g.a_bytes = 3 * umma::BK * umma::BM * 2;
+        g.stage_bytes = round_up(g.a_bytes + 3 * umma::BK * g.bn * 2, 1024);
+    } else {
+        const bool f = kind == umma::FWD;
+        const int ho = f ? L.hout : L.hin;
+        g.N = f ? L.co : L.ci;
+        g.bn = f ? L.bnf : L.bnd;
+        g.ntn = (f ? L.rowsf : L.rowsd) / g.bn;
+        g.grid = g.phases == 4 ? ho / 2 : ho;
+        choose_box(g.grid, B, umma::BM, &g);
+        const int tiles = g.phases * g.tx * g.ty * g.tb * g.ntn;
+        g.chunks = (9 * (!f && L.up ? 4 : 1) * g.cp + umma::BK - 1) / umma::BK;
+        const int s = split_slices(tiles, g.chunks);
+        g.chunks_per_split = (g.chunks + s - 1) / s;
+        g.splits = (g.chunks + g.chunks_per_split - 1) / g.chunks_per_split;
+        g.items = tiles * g.splits;
+        g.M = (long long)B * ho * ho;
+        g.a_bytes = 3 * umma::BM * 2 * g.kb;
+        g.stage_bytes = round_up(g.a_bytes + g.bn * 2 * g.kb, 1024);
+    }
+    g.ncols = g.bn <= 32 ? 32 : (g.bn <= 64 ? 64 : (g.bn <= 128 ? 128 : 256));
     return g;
 }
 
-// out = scale (act(conv(in) + b) + add), r = act(conv(in) + b) (tensor-core GEMM)
-cudaError_t conv_fwd(lgnk_ws* w, int l, const float* in, float* out, float* r, const float* add, int relu, float scale,
-                     int B) {
+typedef CUresult (*EncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeTiled encode_tiled() {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q{};
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return reinterpret_cast<EncodeTiled>(fn);
+}
+
+inline CUtensorMapSwizzle swizzle_of(int kb) {
+    return kb == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : (kb == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+}
+
+// Planes [3][B][h][h][cp] in boxes of 3 planes x (bb, by, bx) positions, `step`
+// apart, x kb channels.
+bool planes_map(EncodeTiled enc, CUtensorMap* m, __nv_bfloat16* p, int cp, int h, int B, int kb,
+                const umma::ConvGemm& g, int step) {
+    const cuuint64_t row = 2ull * cp, dims[5] = {(cuuint64_t)cp, (cuuint64_t)h, (cuuint64_t)h, (cuuint64_t)B, 3};
+    const cuuint64_t strides[4] = {row, row * h, row * h * h, row * h * h * B};
+    const cuuint32_t box[5] = {(cuuint32_t)kb, (cuuint32_t)(g.bx * step), (cuuint32_t)(g.by * step), (cuuint32_t)g.bb, 3};
+    const cuuint32_t steps[5] = {1, (cuuint32_t)step, (cuuint32_t)step, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, p, dims, strides, box, steps, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               swizzle_of(kb), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool weights_map(EncodeTiled enc, CUtensorMap* m, __nv_bfloat16* p, int ld, int rows, int kb, int bn) {
+    const cuuint64_t dims[2] = {(cuuint64_t)ld, (cuuint64_t)rows}, strides[1] = {2ull * ld};
+    const cuuint32_t box[2] = {(cuuint32_t)kb, (cuuint32_t)bn}, steps[2] = {1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p, dims, strides, box, steps, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               swizzle_of(kb), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The plan of layer l's GEMM at batch B, made on first use and when the batch
+// size changes.
+cudaError_t gemm_plan(lgnk_ws* w, int l, int kind, int B, Plan** out) {
+    Plan& p = w->plans[l][kind];
+    *out = &p;
+    if (p.batch == B) return cudaSuccess;
+    p.batch = 0;
     const Layer& L = w->L[l];
-    umma::ConvGemm g = gemm_base(L, umma::FWD, B);
-    g.M = B * L.hout * L.hout;
-    g.N = L.co;
-    g.K = 9 * L.cpi;
-    g.cp = L.cpi;
-    g.bn = L.bnf;
-    cudaError_t e = split_planes(w, in, B, L.ci, L.hin, L.cpi, &g.plane_elems);
+    p.g = gemm_shape(L, kind, B);
+    umma::ConvGemm& g = p.g;
+    const EncodeTiled enc = encode_tiled();
+    if (enc == nullptr) return cudaErrorNotSupported;
+    bool ok;
+    if (kind == umma::FWD) {
+        ok = planes_map(enc, &p.a, w->planes[l], g.cp, L.hin, B, g.kb, g, L.stride) &&
+             weights_map(enc, &p.b, L.wf, L.ldf, L.rowsf, g.kb, g.bn);
+    } else if (kind == umma::BWD_DATA) {
+        ok = planes_map(enc, &p.a, w->zplanes, g.cp, L.hout, B, g.kb, g, L.up ? 2 : 1) &&
+             weights_map(enc, &p.b, L.wd, L.ldd, L.rowsd, g.kb, g.bn);
+    } else {
+        ok = planes_map(enc, &p.a, w->planes[l], g.cp, L.hin, B, g.kb, g, L.stride) &&
+             planes_map(enc, &p.b, w->zplanes, L.cpo, L.hout, B, g.kz, g, L.up ? 2 : 1);
+    }
+    if (!ok) return cudaErrorInvalidValue;
+    g.stages = std::min(umma::kMaxStages, (w->smem_max - 1024) / g.stage_bytes);
+    if (g.stages < 1) return cudaErrorInvalidValue;
+    p.smem = (size_t)g.stages * g.stage_bytes + 1024;
+    p.grid = std::min(g.items, w->sms);
+    g.err = w->derr;
+    if (kind == umma::BWD_WEIGHT) g.part = w->wpart;
+    else {
+        g.part = w->gpart;
+        if (g.splits > 1 && (size_t)g.splits * g.M * g.N > w->gpart_cap) return cudaErrorInvalidValue;
+    }
+    p.batch = B;
+    return cudaSuccess;
+}
+
+cudaError_t launch_gemm(lgnk_ws* w, const Plan& p, const umma::ConvGemm& g) {
+    umma::conv_gemm_kernel<<<p.grid, umma::kThreads, p.smem, w->stream>>>(p.a, p.b, g);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || g.kind == umma::BWD_WEIGHT || g.splits == 1) return e;
+    umma::finish_split_kernel<<<blocks_for((size_t)g.M * g.N), kT, 0, w->stream>>>(g, g.splits);
+    return cudaGetLastError();
+}
+
+// Layer l >= 1 from the planes of its input: out = scale (act(conv + b) + add)
+// (FP32, may be NULL), r = act(conv + b) (may be NULL), and the next layer's
+// planes if there is one.
+cudaError_t conv_fwd(lgnk_ws* w, int l, float* out, float* r, const float* add, int relu, float scale, int B) {
+    const Layer& L = w->L[l];
+    Plan* p = nullptr;
+    cudaError_t e = gemm_plan(w, l, umma::FWD, B, &p);
     if (e != cudaSuccess) return e;
-    g.planes = w->planes;
-    g.w = L.wf;
-    g.wld = L.ldf;
+    umma::ConvGemm g = p->g;
     g.out = out;
     g.r = r;
     g.add = add;
     g.bias = w->p + L.boff;
     g.relu = relu;
     g.scale = scale;
-    return launch_gemm_split(w, g, L.rowsf / L.bnf);
+    g.nplanes = l < 6 ? w->planes[l + 1] : nullptr;
+    g.ncp = l < 6 ? w->L[l + 1].cpi : 0;
+    return launch_gemm(w, *p, g);
 }
 
-// weight and bias gradients of layer l from its input `in` and output gradient
-// dz; with din, also the input gradient (added to din when accumulate)
-cudaError_t conv_bwd(lgnk_ws* w, int l, const float* in, const float* dz, float* din, int accumulate, int B) {
+cudaError_t sum_slices(lgnk_ws* w, const Layer& L, int cp, int slices, int bslices) {
+    const size_t n = (size_t)L.co * L.ci * 9 + L.co;
+    sum_slices_kernel<<<blocks_for(n), kT, 0, w->stream>>>(w->wpart, w->bpart, w->g + L.woff, L.co, L.ci, cp, slices,
+                                                           bslices);
+    return cudaGetLastError();
+}
+
+// Backward of layer l >= 1 from the gradient gz of its ReLU's output (masked by
+// that output, mr or mp; neither: gz is the gradient of the convolution): weight
+// and bias gradients, and the input gradient into din (added when accumulate).
+cudaError_t conv_bwd(lgnk_ws* w, int l, const float* gz, const float* mr, const __nv_bfloat16* mp, float* din,
+                     int accumulate, int B) {
     const Layer& L = w->L[l];
-    // weight gradient: D[co][(ci, tap)] over the batch's pixels, K split into slices
-    umma::ConvGemm g = gemm_base(L, umma::BWD_WEIGHT, B);
-    g.M = L.co;
-    g.N = L.ci * 9;
-    g.K = B * L.hout * L.hout;
-    g.bn = std::min(128, round_up(g.N, 16));
-    const int gx = (g.M + umma::BM - 1) / umma::BM, gy = (g.N + g.bn - 1) / g.bn;
-    const int chunks = (g.K + umma::BK - 1) / umma::BK;
-    int slices = std::min(kMaxSlices, std::min(chunks, std::max(1, (2 * 152 + gx * gy - 1) / (gx * gy))));
-    g.chunks_per_split = (chunks + slices - 1) / slices;
-    slices = (chunks + g.chunks_per_split - 1) / g.chunks_per_split;
-    g.a = dz;
-    g.x = in;
-    g.out = w->wpart;
-    cudaError_t e = launch_gemm(w, g, gx, gy, slices);
+    const int P = L.hout * L.hout, gs = L.cpo % 32 == 0 ? 4 : 2, per = kT / gs;     // pixels per block
+    const int bs = (int)std::min<long long>(kBiasSlices, ((long long)P * B + per - 1) / per);
+    mask_split_kernel<<<dim3(bs, L.cpo / 8 / gs), kT, 0, w->stream>>>(gz, mr, mp, w->zplanes, w->bpart, L.co, L.cpo, P,
+                                                                      B, gs);
+    cudaError_t e = cudaGetLastError();
+    Plan* p = nullptr;
+    if (e == cudaSuccess) e = gemm_plan(w, l, umma::BWD_WEIGHT, B, &p);
+    if (e == cudaSuccess) e = launch_gemm(w, *p, p->g);
+    if (e == cudaSuccess) e = sum_slices(w, L, L.cpi, p->g.splits, bs);
+    if (e == cudaSuccess) e = gemm_plan(w, l, umma::BWD_DATA, B, &p);
     if (e != cudaSuccess) return e;
-    const size_t nw = (size_t)L.co * L.ci * 9;
-    sum_slices_kernel<<<blocks_for(nw), kT, 0, w->stream>>>(w->wpart, w->g + L.woff, nw, slices);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    bias_grad_kernel<<<L.co, kT, 0, w->stream>>>(dz, w->g + L.boff, L.co, (size_t)L.hout * L.hout, B);
-    e = cudaGetLastError();
-    if (e != cudaSuccess || din == nullptr) return e;
-    // data gradient: D[input pixel][ci]
-    umma::ConvGemm d = gemm_base(L, umma::BWD_DATA, B);
-    d.M = B * L.hin * L.hin;
-    d.N = L.ci;
-    d.K = 9 * (L.up ? 4 : 1) * L.cpo;
-    d.cp = L.cpo;
-    d.bn = L.bnd;
-    e = split_planes(w, dz, B, L.co, L.hout, L.cpo, &d.plane_elems);
-    if (e != cudaSuccess) return e;
-    d.planes = w->planes;
-    d.w = L.wd;
-    d.wld = L.ldd;
+    umma::ConvGemm d = p->g;
     d.out = din;
     d.accumulate = accumulate;
-    return launch_gemm_split(w, d, L.rowsd / L.bnd);
+    return launch_gemm(w, *p, d);
 }
 
 // refresh the GEMMs' bf16 weight matrices from the master weights
 cudaError_t pack_weights(lgnk_ws* w) {
-    for (const Layer& L : w->L) {
+    for (int l = 1; l < 7; ++l) {
+        const Layer& L = w->L[l];
         const size_t n = (size_t)L.rowsf * L.ldf + (size_t)L.rowsd * L.ldd;
         pack_wmats_kernel<<<blocks_for(n), kT, 0, w->stream>>>(w->p, L);
         const cudaError_t e = cudaGetLastError();
@@ -347,17 +588,19 @@ cudaError_t pack_weights(lgnk_ws* w) {
     return cudaSuccess;
 }
 
-lgnk_status forward_pass(lgnk_ws* w, int B, const float* T, const float* R, float* v) {
-    const size_t n = (size_t)w->m * w->m;
-    stack_input_kernel<<<blocks_for(n * B), kT, 0, w->stream>>>(T, R, w->x, n, B);
+// The network; with train, also what only the backward pass reads (r4, r5).
+lgnk_status forward_pass(lgnk_ws* w, int B, const float* T, const float* R, float* v, bool train) {
+    const Layer& L0 = w->L[0];
+    const size_t n = (size_t)w->m * w->m * B;
+    conv_first_kernel<<<dim3(blocks_for(n), w->L[1].cpi / kFirstCh), kT, 0, w->stream>>>(
+        T, R, w->p + L0.woff, w->p + L0.boff, w->planes[1], L0.co, w->L[1].cpi, w->m, B);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = conv_fwd(w, 0, w->x, w->e0, nullptr, nullptr, 1, 1.0f, B);
-    if (e == cudaSuccess) e = conv_fwd(w, 1, w->e0, w->e1, nullptr, nullptr, 1, 1.0f, B);
-    if (e == cudaSuccess) e = conv_fwd(w, 2, w->e1, w->e2, nullptr, nullptr, 1, 1.0f, B);
-    if (e == cudaSuccess) e = conv_fwd(w, 3, w->e2, w->e3, nullptr, nullptr, 1, 1.0f, B);
-    if (e == cudaSuccess) e = conv_fwd(w, 4, w->e3, w->d2, w->r4, w->e2, 1, 1.0f, B);
-    if (e == cudaSuccess) e = conv_fwd(w, 5, w->d2, w->d1, w->r5, w->e1, 1, 1.0f, B);
-    if (e == cudaSuccess) e = conv_fwd(w, 6, w->d1, v, nullptr, nullptr, 0, w->scale, B);
+    if (e == cudaSuccess) e = conv_fwd(w, 1, w->e1, nullptr, nullptr, 1, 1.0f, B);
+    if (e == cudaSuccess) e = conv_fwd(w, 2, w->e2, nullptr, nullptr, 1, 1.0f, B);
+    if (e == cudaSuccess) e = conv_fwd(w, 3, nullptr, nullptr, nullptr, 1, 1.0f, B);
+    if (e == cudaSuccess) e = conv_fwd(w, 4, nullptr, train ? w->r4 : nullptr, w->e2, 1, 1.0f, B);
+    if (e == cudaSuccess) e = conv_fwd(w, 5, nullptr, train ? w->r5 : nullptr, w->e1, 1, 1.0f, B);
+    if (e == cudaSuccess) e = conv_fwd(w, 6, v, nullptr, nullptr, 0, w->scale, B);
     if (e != cudaSuccess) {
         snprintf(w->err, sizeof(w->err), "%s", cudaGetErrorString(e));
         return LGNK_ERR_CUDA;
@@ -429,56 +672,72 @@ lgnk_status lgnk_ws_create(int image_m, int base_channels, int max_batch, float 
         (s = ws_alloc_n(w, off, &w->as)) || (s = ws_alloc_n(w, 1, &w->derr)))
         return fail(s);
     // the GEMMs' bf16 weight matrices (N per CTA up to 256, rows and K padded)
-    size_t pmax = 0;
-    for (Layer& L : w->L) {
+    size_t zmax = 0;
+    for (int l = 0; l < 7; ++l) {
+        Layer& L = w->L[l];
         const int R = L.up ? 4 : 1;
-        L.cpi = round_up(L.ci, 8);
-        L.cpo = round_up(L.co, 8);
-        L.bnf = std::min(256, round_up(L.co, 16));
+        L.cpi = round_up(L.ci, 16);
+        L.cpo = round_up(L.co, 16);
+        if (l == 0) continue;             // the first layer has kernels of its own
+        L.bnf = std::min(256, L.cpo);
         L.rowsf = round_up(L.co, L.bnf);
         L.ldf = round_up(9 * L.cpi, umma::BK);
-        L.bnd = std::min(256, round_up(L.ci, 16));
+        L.bnd = std::min(256, L.cpi);
         L.rowsd = round_up(L.ci, L.bnd);
         L.ldd = round_up(9 * R * L.cpo, umma::BK);
-        pmax = std::max(pmax, (size_t)B * L.hin * L.hin * L.cpi);
-        pmax = std::max(pmax, (size_t)B * L.hout * L.hout * L.cpo);
-        if ((s = ws_alloc_n(w, (size_t)L.rowsf * L.ldf, &L.wf)) || (s = ws_alloc_n(w, (size_t)L.rowsd * L.ldd, &L.wd)))
+        zmax = std::max(zmax, (size_t)B * L.hout * L.hout * L.cpo);
+        if ((s = ws_alloc_n(w, (size_t)L.rowsf * L.ldf, &L.wf)) || (s = ws_alloc_n(w, (size_t)L.rowsd * L.ldd, &L.wd)) ||
+            (s = ws_alloc_n(w, (size_t)3 * B * L.hin * L.hin * L.cpi, &w->planes[l])))
             return fail(s);
     }
-    w->planes_cap = pmax;
-    if ((s = ws_alloc_n(w, 3 * pmax, &w->planes))) return fail(s);
+    if ((s = ws_alloc_n(w, 3 * zmax, &w->zplanes))) return fail(s);
     // split-K partials: the largest splits x M x N any batch size up to max_batch needs
     size_t gmax = 1;
     for (int b = 1; b <= B; ++b) {
-        for (const Layer& L : w->L) {
-            const int R = L.up ? 4 : 1;
-            const long long Mf = (long long)b * L.hout * L.hout, Md = (long long)b * L.hin * L.hin;
-            const int tf = (int)((Mf + umma::BM - 1) / umma::BM) * (L.rowsf / L.bnf);
-            const int td = (int)((Md + umma::BM - 1) / umma::BM) * (L.rowsd / L.bnd);
-            const int sf = split_slices(tf, (9 * L.cpi + umma::BK - 1) / umma::BK);
-            const int sd = split_slices(td, (9 * R * L.cpo + umma::BK - 1) / umma::BK);
-            if (sf > 1) gmax = std::max(gmax, (size_t)sf * (size_t)Mf * L.co);
-            if (sd > 1) gmax = std::max(gmax, (size_t)sd * (size_t)Md * L.ci);
+        for (int l = 1; l < 7; ++l) {
+            const Layer& L = w->L[l];
+            for (int kind : {umma::FWD, umma::BWD_DATA}) {
+                const umma::ConvGemm g = gemm_shape(L, kind, b);
+                if (g.splits > 1) gmax = std::max(gmax, (size_t)g.splits * (size_t)g.M * g.N);
+            }
         }
     }
     w->gpart_cap = gmax;
     if ((s = ws_alloc_n(w, gmax, &w->gpart))) return fail(s);
-    const size_t big = act_size(w, c, m, B);   // the largest activation: e0
-    if ((s = ws_alloc_n(w, act_size(w, 2, m, B), &w->x)) || (s = ws_alloc_n(w, big, &w->e0)) ||
-        (s = ws_alloc_n(w, act_size(w, 2 * c, m / 2, B), &w->e1)) ||
+    // gradients: ga of e1 and d1, gb of e2 and d2, gc the output's, e3's and e0's in turn
+    if ((s = ws_alloc_n(w, act_size(w, 2 * c, m / 2, B), &w->e1)) ||
         (s = ws_alloc_n(w, act_size(w, 4 * c, m / 4, B), &w->e2)) ||
-        (s = ws_alloc_n(w, act_size(w, 8 * c, m / 8, B), &w->e3)) ||
         (s = ws_alloc_n(w, act_size(w, 4 * c, m / 4, B), &w->r4)) ||
-        (s = ws_alloc_n(w, act_size(w, 4 * c, m / 4, B), &w->d2)) ||
         (s = ws_alloc_n(w, act_size(w, 2 * c, m / 2, B), &w->r5)) ||
-        (s = ws_alloc_n(w, act_size(w, 2 * c, m / 2, B), &w->d1)) ||
-        (s = ws_alloc_n(w, act_size(w, 2, m / 2, B), &w->z6)) || (s = ws_alloc_n(w, big, &w->ga)) ||
-        (s = ws_alloc_n(w, big, &w->gb)) || (s = ws_alloc_n(w, big, &w->gc)) ||
-        (s = ws_alloc_n(w, (size_t)4096, &w->partial)))
+        (s = ws_alloc_n(w, act_size(w, 2, m / 2, B), &w->z6)) ||
+        (s = ws_alloc_n(w, act_size(w, 2 * c, m / 2, B), &w->ga)) ||
+        (s = ws_alloc_n(w, act_size(w, 4 * c, m / 4, B), &w->gb)) ||
+        (s = ws_alloc_n(w, act_size(w, c, m, B), &w->gc)) || (s = ws_alloc_n(w, (size_t)4096, &w->partial)))
         return fail(s);
-    size_t wmax = 0;
-    for (const Layer& L : w->L) wmax = std::max(wmax, (size_t)L.co * L.ci * 9);
-    if ((s = ws_alloc_n(w, wmax * kMaxSlices, &w->wpart))) return fail(s);
+    size_t wmax = 0, bmax = 0;
+    for (const Layer& L : w->L) {
+        wmax = std::max(wmax, (size_t)L.co * L.cpi * 9);
+        bmax = std::max(bmax, (size_t)L.co);
+    }
+    if ((s = ws_alloc_n(w, wmax * kMaxSlices, &w->wpart)) || (s = ws_alloc_n(w, bmax * kBiasSlices, &w->bpart)))
+        return fail(s);
+    {
+        int dev = 0, optin = 0;
+        cudaFuncAttributes fa{};
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&w->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+            cudaFuncGetAttributes(&fa, umma::conv_gemm_kernel) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(LGNK_ERR_CUDA);
+        }
+        w->smem_max = optin - (int)fa.sharedSizeBytes;
+        if (cudaFuncSetAttribute(umma::conv_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, w->smem_max) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return fail(LGNK_ERR_CUDA);
+        }
+    }
     if (cudaMallocHost((void**)&w->hres, 8 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         w->hres = nullptr;
@@ -522,7 +781,7 @@ lgnk_status lgnk_ws_get_grads(lgnk_ws* w, float* grads) {
 lgnk_status lgnk_ws_predict(lgnk_ws* w, int batch, const float* T, const float* R, float* v) {
     if (w == nullptr || T == nullptr || R == nullptr || v == nullptr || batch < 1 || batch > w->max_batch)
         return LGNK_ERR_INVALID_ARG;
-    return forward_pass(w, batch, T, R, v);
+    return forward_pass(w, batch, T, R, v, false);
 }
 
 lgnk_status lgnk_ws_train_step(lgnk_ws* w, int batch, const float* T, const float* R, const float* target, float lr,
@@ -530,55 +789,37 @@ lgnk_status lgnk_ws_train_step(lgnk_ws* w, int batch, const float* T, const floa
     if (w == nullptr || T == nullptr || R == nullptr || target == nullptr || batch < 1 || batch > w->max_batch)
         return LGNK_ERR_INVALID_ARG;
     const int B = batch;
-    lgnk_status st = forward_pass(w, B, T, R, w->z6);
+    lgnk_status st = forward_pass(w, B, T, R, w->z6, true);
     if (st != LGNK_OK) return st;
-    const int c = w->c, m = w->m;
+    const int m = w->m;
     // loss and dz6 (gradient w.r.t. the unscaled output)
     const size_t nv = act_size(w, 2, m / 2, B);
     const int nb = blocks_for(nv) < 1024 ? blocks_for(nv) : 1024;
     float* dz6 = w->gc;
     mse_kernel<<<nb, kT, 0, w->stream>>>(w->z6, target, dz6, nv, w->scale, w->partial);
     WS_CHECK(cudaGetLastError());
-    // layer 6: d(d1) -> ga
-    float* dd1 = w->ga;
-    WS_CHECK(conv_bwd(w, 6, w->d1, dz6, dd1, 0, B));
-    // d1 = r5 + e1: d(e1) accumulates d(d1); dz5 = d(d1) * (r5 > 0)
-    float* de1 = w->gb;
-    const size_t n1 = act_size(w, 2 * c, m / 2, B);
-    WS_CHECK(cudaMemcpyAsync(de1, dd1, n1 * sizeof(float), cudaMemcpyDeviceToDevice, w->stream));
-    relu_mask_kernel<<<blocks_for(n1), kT, 0, w->stream>>>(dd1, w->r5, n1);
-    WS_CHECK(cudaGetLastError());
-    // layer 5 (input up2(d2)): d(d2) -> gc
-    float* dd2 = w->gc;
-    WS_CHECK(conv_bwd(w, 5, w->d2, dd1, dd2, 0, B));
-    // d2 = r4 + e2: d(e2) accumulates d(d2); dz4 = d(d2) * (r4 > 0)
-    const size_t n2 = act_size(w, 4 * c, m / 4, B);
-    float* de2 = w->ga;   // dd1 is no longer needed
-    WS_CHECK(cudaMemcpyAsync(de2, dd2, n2 * sizeof(float), cudaMemcpyDeviceToDevice, w->stream));
-    relu_mask_kernel<<<blocks_for(n2), kT, 0, w->stream>>>(dd2, w->r4, n2);
-    WS_CHECK(cudaGetLastError());
-    // layer 4 (input up2(e3)): d(e3) -> ga + n2 (free room after de2)
-    float* de3 = w->ga + n2;
-    WS_CHECK(conv_bwd(w, 4, w->e3, dd2, de3, 0, B));
-    const size_t n3 = act_size(w, 8 * c, m / 8, B);
-    relu_mask_kernel<<<blocks_for(n3), kT, 0, w->stream>>>(de3, w->e3, n3);
-    WS_CHECK(cudaGetLastError());
-    // layer 3: d(e2) += ...
-    WS_CHECK(conv_bwd(w, 3, w->e2, de3, de2, 1, B));
-    relu_mask_kernel<<<blocks_for(n2), kT, 0, w->stream>>>(de2, w->e2, n2);
-    WS_CHECK(cudaGetLastError());
+    // layer 6: d(d1) -> ga; d1 = r5 + e1, so ga is also the start of d(e1)
+    WS_CHECK(conv_bwd(w, 6, dz6, nullptr, nullptr, w->ga, 0, B));
+    // layer 5 (input up2(d2)): d(d2) -> gb, also the start of d(e2) (d2 = r4 + e2)
+    WS_CHECK(conv_bwd(w, 5, w->ga, w->r5, nullptr, w->gb, 0, B));
+    // layer 4 (input up2(e3)): d(e3) -> gc
+    WS_CHECK(conv_bwd(w, 4, w->gb, w->r4, nullptr, w->gc, 0, B));
+    // layer 3: d(e2) += ...; the masks of e3, e2, e1 are read from the planes
+    WS_CHECK(conv_bwd(w, 3, w->gc, nullptr, w->planes[4], w->gb, 1, B));
     // layer 2: d(e1) += ...
-    WS_CHECK(conv_bwd(w, 2, w->e1, de2, de1, 1, B));
-    relu_mask_kernel<<<blocks_for(n1), kT, 0, w->stream>>>(de1, w->e1, n1);
-    WS_CHECK(cudaGetLastError());
+    WS_CHECK(conv_bwd(w, 2, w->gb, nullptr, w->planes[3], w->ga, 1, B));
     // layer 1: d(e0) -> gc
-    float* de0 = w->gc;
-    WS_CHECK(conv_bwd(w, 1, w->e0, de1, de0, 0, B));
-    const size_t n0 = act_size(w, c, m, B);
-    relu_mask_kernel<<<blocks_for(n0), kT, 0, w->stream>>>(de0, w->e0, n0);
-    WS_CHECK(cudaGetLastError());
+    WS_CHECK(conv_bwd(w, 1, w->ga, nullptr, w->planes[2], w->gc, 0, B));
     // layer 0: weights only
-    WS_CHECK(conv_bwd(w, 0, w->x, de0, nullptr, 0, B));
+    {
+        const Layer& L = w->L[0];
+        const size_t n = (size_t)m * m * B;
+        const int bs = (int)std::min<size_t>(kBiasSlices, (n + kT - 1) / kT);
+        conv_first_wgrad_kernel<<<dim3(bs, (L.co + kFirstW - 1) / kFirstW), kT, 0, w->stream>>>(
+            T, R, w->gc, w->planes[1], w->wpart, w->bpart, L.co, w->L[1].cpi, m, B);
+        WS_CHECK(cudaGetLastError());
+        WS_CHECK(sum_slices(w, L, 2, bs, bs));
+    }
     // Adam
     w->steps++;
     const float c1 = 1.0f - powf(0.9f, (float)w->steps), c2 = 1.0f - powf(0.999f, (float)w->steps);

@@ -145,3 +145,28 @@ def test_pipeline_end_to_end_small():
     assert ev["pairs"] == 4
     assert ev["zero"]["converged"] >= 3 and ev["warm"]["converged"] >= ev["zero"]["converged"] - 1
     assert ev["final_J_ratio_warm_over_zero"] == pytest.approx(1.0, rel=5e-2)
+
+
+# operand rows of 64, 32 and 16 channels, more than 256 columns, sides that the
+# boxes of positions do not divide, boxes that span images, and one-pixel grids
+@pytest.mark.parametrize("c,m,B", [(32, 32, 2), (40, 24, 1), (12, 8, 5), (16, 72, 2), (20, 40, 7)])
+def test_gemm_tilings_match_oracle(c, m, B):
+    scale = 0.05
+    p, T, R, vt = _inputs(c, m, B, seed=5)
+    net = _net(c, m, B, scale, p)
+    Tg, Rg, vg = _cuda(T, R, vt)
+    v = net.predict(Tg, Rg).cpu().numpy()
+    assert _rel(v, W.forward(p.astype(np.float64), T.astype(np.float64), R.astype(np.float64), c, scale).numpy()) <= 1e-5
+    loss = net.train_step(Tg, Rg, vg, lr=0.0)
+    g = net.grads().cpu().numpy()
+    lref, gref, _ = W.loss_and_grad(p.astype(np.float64), T, R, vt, c, scale)
+    assert abs(loss - lref) <= 1e-5 * lref
+    o = 0
+    for ci, co, _, _ in W.layer_shapes(c):
+        for n in (co * ci * 9, co):
+            assert _rel(g[o:o + n], gref[o:o + n]) <= 1e-4, (ci, co, n)
+            o += n
+    # a smaller batch through the same network
+    if B > 1:
+        v1 = net.predict(Tg[:1].contiguous(), Rg[:1].contiguous()).cpu().numpy()
+        assert _rel(v1, v[:1]) <= 1e-5
