@@ -94,6 +94,13 @@ struct ConvGemm {
     int* err;                 // set to 1 when a wait runs out
 };
 
+// Every kernel of a network pass is launched as a programmatic dependent of the
+// one before it: it may start (barriers, tensor memory, constants) while that
+// one still runs, and touches global memory only after dependency_wait(), which
+// returns when that kernel (which waited the same way) has completed.
+__device__ __forceinline__ void dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Shared-memory matrix descriptor of a swizzled tile whose rows are 2 kb bytes
@@ -269,6 +276,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool bw = g.kind == BWD_WEIGHT;
     const uint32_t alloc_cols = 2u * (uint32_t)g.ncols;
+    dependency_trigger();
 
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
@@ -276,6 +284,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&amap) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&bmap) : "memory");
         dead = 0;
         for (int s = 0; s < kMaxStages; ++s) {
             mbar_init(&full[s], 1);
@@ -290,6 +300,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
+    dependency_wait();
     const uint32_t tmem = tmem_base;
     const uint32_t smem0 = smem_u32(smem);
     const int S = g.stages;
@@ -520,12 +531,15 @@ __global__ void finish_split_kernel(const ConvGemm g, int splits) {
     const size_t M = (size_t)g.M, total = M * ((g.N + 7) / 8);
     const int h = g.kind == FWD ? g.hout : g.hin, C = g.kind == FWD ? g.co : g.ci;
     const size_t P = (size_t)h * h;
+    dependency_trigger();
+    dependency_wait();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int n0 = (int)(i / M) * 8;
         const size_t row = i - (size_t)(n0 / 8) * M, b = row / P, o = row - b * P;
         float acc[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
+#pragma unroll 4
         for (int z = 0; z < splits; ++z) {
             const float* p = g.part + ((size_t)z * g.N + n0) * M + row;
 #pragma unroll

@@ -63,8 +63,34 @@ struct Plan {
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-// The GEMMs' weight matrices from the FP32 master weights (bf16, nearest).
-__global__ void pack_wmats_kernel(const float* __restrict__ p, Layer L) {
+// Launch as a programmatic dependent of the kernel before it on the stream
+// (umma::dependency_wait): a pass is 13 to 60 kernels of a few microseconds, and
+// each one's start-up overlaps the end of the one before.
+template <class... KArgs, class... Args>
+cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+struct Layers {
+    Layer l[7];
+};
+
+// The GEMMs' weight matrices from the FP32 master weights (bf16, nearest), layer
+// 1 + blockIdx.y.
+__global__ void pack_wmats_kernel(const float* __restrict__ p, const Layers all) {
+    umma::dependency_trigger();
+    umma::dependency_wait();
+    const Layer L = all.l[1 + blockIdx.y];
     const size_t nf = (size_t)L.rowsf * L.ldf, nd = (size_t)L.rowsd * L.ldd;
     const int R = L.up ? 4 : 1;
     const float* W = p + L.woff;
@@ -91,13 +117,17 @@ __global__ void pack_wmats_kernel(const float* __restrict__ p, Layer L) {
 __global__ void sum_slices_kernel(const float* __restrict__ part, const float* __restrict__ bpart, float* dW, int co,
                                   int ci, int cp, int slices, int bslices) {
     const int nw = co * ci * 9, rows = 9 * cp;
+    umma::dependency_trigger();
+    umma::dependency_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nw + co; i += gridDim.x * blockDim.x) {
         float s = 0.0f;
         if (i < nw) {
             const int n = i / (ci * 9), r = i - n * ci * 9, c = r / 9, t = r - c * 9;
             const float* p = part + (size_t)n * rows + t * cp + c;
+#pragma unroll 8
             for (int k = 0; k < slices; ++k) s += p[(size_t)k * co * rows];
         } else {
+#pragma unroll 8
             for (int k = 0; k < bslices; ++k) s += bpart[(size_t)k * co + i - nw];
         }
         dW[i] = s;
@@ -112,13 +142,15 @@ __global__ void sum_slices_kernel(const float* __restrict__ part, const float* _
 // channels of one pixel at a time; a warp covers 4 (2) neighbouring channel
 // groups of 8 (16) pixels, so that reads (channel rows) and writes (pixels)
 // both touch whole sectors.
-constexpr int kBiasSlices = 64;
+constexpr int kBiasSlices = 152;
 __global__ void __launch_bounds__(kT) mask_split_kernel(const float* __restrict__ g, const float* __restrict__ mr,
                                                         const __nv_bfloat16* __restrict__ mp, __nv_bfloat16* planes,
                                                         float* bpart, int C, int cp, int P, int B, int gs) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pw = 32 / gs;      // pixels per warp
     const int c0 = (blockIdx.y * gs + lane / pw) * 8;
     const size_t n = (size_t)P * B, pe = n * cp;
+    umma::dependency_trigger();
+    umma::dependency_wait();
     float sum[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) sum[j] = 0.0f;
@@ -129,9 +161,12 @@ __global__ void __launch_bounds__(kT) mask_split_kernel(const float* __restrict_
 #pragma unroll
         for (int j = 0; j < 8; ++j) v[j] = c0 + j < C ? __ldg(g + (b * C + c0 + j) * P + o) : 0.0f;
         if (mr != nullptr) {
+            float r[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) r[j] = c0 + j < C ? __ldg(mr + (b * C + c0 + j) * P + o) : 0.0f;
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-                if (c0 + j < C && !(__ldg(mr + (b * C + c0 + j) * P + o) > 0.0f)) v[j] = 0.0f;
+                if (!(r[j] > 0.0f)) v[j] = 0.0f;
         } else if (mp != nullptr) {
             __align__(16) __nv_bfloat16 m[8];
             *reinterpret_cast<uint4*>(m) = __ldg(reinterpret_cast<const uint4*>(mp + e));
@@ -169,11 +204,13 @@ constexpr int kFirstCh = 16;
 __global__ void __launch_bounds__(kT) conv_first_kernel(const float* __restrict__ T, const float* __restrict__ R,
                                                         const float* __restrict__ W, const float* __restrict__ bias,
                                                         __nv_bfloat16* planes, int C, int cp, int m, int B) {
-    __shared__ float w[kFirstCh][18], bs[kFirstCh];
+    __shared__ __align__(16) float w[kFirstCh][20], bs[kFirstCh];     // 16-byte rows: five loads a channel
     const int c0 = blockIdx.y * kFirstCh;
-    for (int i = threadIdx.x; i < kFirstCh * 18; i += kT) {
-        const int c = i / 18, k = i % 18, tap = k >> 1, ci = k & 1;       // order (tap, ci)
-        w[c][k] = c0 + c < C ? __bfloat162float(__float2bfloat16_rn(W[((size_t)(c0 + c) * 2 + ci) * 9 + tap])) : 0.0f;
+    umma::dependency_trigger();
+    umma::dependency_wait();
+    for (int i = threadIdx.x; i < kFirstCh * 20; i += kT) {
+        const int c = i / 20, k = i % 20, tap = k >> 1, ci = k & 1;       // order (tap, ci)
+        w[c][k] = c0 + c < C && k < 18 ? __bfloat162float(__float2bfloat16_rn(W[((size_t)(c0 + c) * 2 + ci) * 9 + tap])) : 0.0f;
     }
     if (threadIdx.x < kFirstCh) bs[threadIdx.x] = c0 + (int)threadIdx.x < C ? bias[c0 + threadIdx.x] : 0.0f;
     __syncthreads();
@@ -196,8 +233,18 @@ __global__ void __launch_bounds__(kT) conv_first_kernel(const float* __restrict_
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 float a = 0.0f;
+                const float4* wr = reinterpret_cast<const float4*>(w[q + j]);
 #pragma unroll
-                for (int k = 0; k < 18; ++k) a = fmaf(in[k], w[q + j][k], a);
+                for (int k = 0; k < 4; ++k) {
+                    const float4 t = wr[k];
+                    a = fmaf(in[4 * k], t.x, a);
+                    a = fmaf(in[4 * k + 1], t.y, a);
+                    a = fmaf(in[4 * k + 2], t.z, a);
+                    a = fmaf(in[4 * k + 3], t.w, a);
+                }
+                const float4 t = wr[4];
+                a = fmaf(in[16], t.x, a);
+                a = fmaf(in[17], t.y, a);
                 v[j] = c0 + q + j < C ? fmaxf(a + bs[q + j], 0.0f) : 0.0f;
             }
             umma::store_planes8(planes, n * cp, i * cp + c0 + q, v);
@@ -216,6 +263,8 @@ __global__ void __launch_bounds__(kT) conv_first_wgrad_kernel(const float* __res
                                                               float* bpart, int C, int cp, int m, int B) {
     const int c0 = blockIdx.y * kFirstW, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t P = (size_t)m * m, n = P * B;
+    umma::dependency_trigger();
+    umma::dependency_wait();
     float acc[kFirstW][19];
 #pragma unroll
     for (int j = 0; j < kFirstW; ++j)
@@ -271,6 +320,8 @@ __global__ void __launch_bounds__(kT) conv_first_wgrad_kernel(const float* __res
 // unscaled output z (v = scale z): dz = (v - t) / (scale N).
 __global__ void mse_kernel(const float* __restrict__ v, const float* __restrict__ t, float* dz, size_t n, float scale,
                            double* partial) {
+    umma::dependency_trigger();
+    umma::dependency_wait();
     double s = 0.0;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float e = v[i] - t[i];
@@ -289,6 +340,8 @@ __global__ void mse_kernel(const float* __restrict__ v, const float* __restrict_
 
 __global__ void adam_kernel(float* p, const float* __restrict__ g, float* m, float* s, size_t n, float lr, float c1,
                             float c2) {
+    umma::dependency_trigger();
+    umma::dependency_wait();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = 0.9f * m[i] + 0.1f * gi;
@@ -519,11 +572,10 @@ cudaError_t gemm_plan(lgnk_ws* w, int l, int kind, int B, Plan** out) {
 }
 
 cudaError_t launch_gemm(lgnk_ws* w, const Plan& p, const umma::ConvGemm& g) {
-    umma::conv_gemm_kernel<<<p.grid, umma::kThreads, p.smem, w->stream>>>(p.a, p.b, g);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch(umma::conv_gemm_kernel, dim3(p.grid), umma::kThreads, p.smem, w->stream, p.a, p.b, g);
     if (e != cudaSuccess || g.kind == umma::BWD_WEIGHT || g.splits == 1) return e;
-    umma::finish_split_kernel<<<blocks_for((size_t)g.M * g.N), kT, 0, w->stream>>>(g, g.splits);
-    return cudaGetLastError();
+    return launch(umma::finish_split_kernel, dim3(blocks_for((size_t)g.M * ((g.N + 7) / 8))), kT, 0, w->stream, g,
+                  g.splits);
 }
 
 // Layer l >= 1 from the planes of its input: out = scale (act(conv + b) + add)
@@ -548,9 +600,8 @@ cudaError_t conv_fwd(lgnk_ws* w, int l, float* out, float* r, const float* add, 
 
 cudaError_t sum_slices(lgnk_ws* w, const Layer& L, int cp, int slices, int bslices) {
     const size_t n = (size_t)L.co * L.ci * 9 + L.co;
-    sum_slices_kernel<<<blocks_for(n), kT, 0, w->stream>>>(w->wpart, w->bpart, w->g + L.woff, L.co, L.ci, cp, slices,
-                                                           bslices);
-    return cudaGetLastError();
+    return launch(sum_slices_kernel, dim3(blocks_for(n)), kT, 0, w->stream, w->wpart, w->bpart, w->g + L.woff, L.co,
+                  L.ci, cp, slices, bslices);
 }
 
 // Backward of layer l >= 1 from the gradient gz of its ReLU's output (masked by
@@ -561,9 +612,8 @@ cudaError_t conv_bwd(lgnk_ws* w, int l, const float* gz, const float* mr, const 
     const Layer& L = w->L[l];
     const int P = L.hout * L.hout, gs = L.cpo % 32 == 0 ? 4 : 2, per = kT / gs;     // pixels per block
     const int bs = (int)std::min<long long>(kBiasSlices, ((long long)P * B + per - 1) / per);
-    mask_split_kernel<<<dim3(bs, L.cpo / 8 / gs), kT, 0, w->stream>>>(gz, mr, mp, w->zplanes, w->bpart, L.co, L.cpo, P,
-                                                                      B, gs);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch(mask_split_kernel, dim3(bs, L.cpo / 8 / gs), kT, 0, w->stream, gz, mr, mp, w->zplanes,
+                           w->bpart, L.co, L.cpo, P, B, gs);
     Plan* p = nullptr;
     if (e == cudaSuccess) e = gemm_plan(w, l, umma::BWD_WEIGHT, B, &p);
     if (e == cudaSuccess) e = launch_gemm(w, *p, p->g);
@@ -578,23 +628,21 @@ cudaError_t conv_bwd(lgnk_ws* w, int l, const float* gz, const float* mr, const 
 
 // refresh the GEMMs' bf16 weight matrices from the master weights
 cudaError_t pack_weights(lgnk_ws* w) {
-    for (int l = 1; l < 7; ++l) {
-        const Layer& L = w->L[l];
-        const size_t n = (size_t)L.rowsf * L.ldf + (size_t)L.rowsd * L.ldd;
-        pack_wmats_kernel<<<blocks_for(n), kT, 0, w->stream>>>(w->p, L);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+    Layers all;
+    size_t n = 0;
+    for (int l = 0; l < 7; ++l) {
+        all.l[l] = w->L[l];
+        if (l > 0) n = std::max(n, (size_t)w->L[l].rowsf * w->L[l].ldf + (size_t)w->L[l].rowsd * w->L[l].ldd);
     }
-    return cudaSuccess;
+    return launch(pack_wmats_kernel, dim3(std::min(blocks_for(n), 608), 6), kT, 0, w->stream, w->p, all);
 }
 
 // The network; with train, also what only the backward pass reads (r4, r5).
 lgnk_status forward_pass(lgnk_ws* w, int B, const float* T, const float* R, float* v, bool train) {
     const Layer& L0 = w->L[0];
     const size_t n = (size_t)w->m * w->m * B;
-    conv_first_kernel<<<dim3(blocks_for(n), w->L[1].cpi / kFirstCh), kT, 0, w->stream>>>(
-        T, R, w->p + L0.woff, w->p + L0.boff, w->planes[1], L0.co, w->L[1].cpi, w->m, B);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch(conv_first_kernel, dim3(blocks_for(n), w->L[1].cpi / kFirstCh), kT, 0, w->stream, T, R,
+                           w->p + L0.woff, w->p + L0.boff, w->planes[1], L0.co, w->L[1].cpi, w->m, B);
     if (e == cudaSuccess) e = conv_fwd(w, 1, w->e1, nullptr, nullptr, 1, 1.0f, B);
     if (e == cudaSuccess) e = conv_fwd(w, 2, w->e2, nullptr, nullptr, 1, 1.0f, B);
     if (e == cudaSuccess) e = conv_fwd(w, 3, nullptr, nullptr, nullptr, 1, 1.0f, B);
@@ -796,8 +844,7 @@ lgnk_status lgnk_ws_train_step(lgnk_ws* w, int batch, const float* T, const floa
     const size_t nv = act_size(w, 2, m / 2, B);
     const int nb = blocks_for(nv) < 1024 ? blocks_for(nv) : 1024;
     float* dz6 = w->gc;
-    mse_kernel<<<nb, kT, 0, w->stream>>>(w->z6, target, dz6, nv, w->scale, w->partial);
-    WS_CHECK(cudaGetLastError());
+    WS_CHECK(launch(mse_kernel, dim3(nb), kT, 0, w->stream, w->z6, target, dz6, nv, w->scale, w->partial));
     // layer 6: d(d1) -> ga; d1 = r5 + e1, so ga is also the start of d(e1)
     WS_CHECK(conv_bwd(w, 6, dz6, nullptr, nullptr, w->ga, 0, B));
     // layer 5 (input up2(d2)): d(d2) -> gb, also the start of d(e2) (d2 = r4 + e2)
@@ -814,17 +861,18 @@ lgnk_status lgnk_ws_train_step(lgnk_ws* w, int batch, const float* T, const floa
     {
         const Layer& L = w->L[0];
         const size_t n = (size_t)m * m * B;
-        const int bs = (int)std::min<size_t>(kBiasSlices, (n + kT - 1) / kT);
-        conv_first_wgrad_kernel<<<dim3(bs, (L.co + kFirstW - 1) / kFirstW), kT, 0, w->stream>>>(
-            T, R, w->gc, w->planes[1], w->wpart, w->bpart, L.co, w->L[1].cpi, m, B);
-        WS_CHECK(cudaGetLastError());
+        // one wave of two blocks per SM
+        const int groups = (L.co + kFirstW - 1) / kFirstW, wave = std::max(1, 2 * w->sms / groups);
+        const int bs = (int)std::min<size_t>(std::min(kMaxSlices, wave), (n + kT - 1) / kT);
+        WS_CHECK(launch(conv_first_wgrad_kernel, dim3(bs, groups), kT, 0, w->stream, T, R, w->gc, w->planes[1], w->wpart,
+                        w->bpart, L.co, w->L[1].cpi, m, B));
         WS_CHECK(sum_slices(w, L, 2, bs, bs));
     }
     // Adam
     w->steps++;
     const float c1 = 1.0f - powf(0.9f, (float)w->steps), c2 = 1.0f - powf(0.999f, (float)w->steps);
-    adam_kernel<<<blocks_for(w->nparams), kT, 0, w->stream>>>(w->p, w->g, w->am, w->as, w->nparams, lr, c1, c2);
-    WS_CHECK(cudaGetLastError());
+    WS_CHECK(launch(adam_kernel, dim3(blocks_for(w->nparams)), kT, 0, w->stream, w->p, w->g, w->am, w->as, w->nparams, lr,
+                    c1, c2));
     WS_CHECK(pack_weights(w));
     if (loss != nullptr) {
         launch_reduce(w->partial, nb, w->partial + 2048, w->stream);
