@@ -103,15 +103,16 @@ __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Shared-memory matrix descriptor of a swizzled tile whose rows are 2 kb bytes
-// (leading byte offset: MN blocks of an MN-major tile; stride byte offset:
-// 8-row groups; swizzle of 128, 64 or 32 bytes).
+// Shared-memory matrix descriptor.  kb = 64, 32, 16: a swizzled tile whose rows
+// are 2 kb bytes (leading byte offset: MN blocks of an MN-major tile; stride byte
+// offset: 8-row groups).  kb = 0: core matrices of 8 rows x 16 bytes without
+// swizzle (K-major; leading byte offset: next along K, stride: next 8 rows).
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo, int kb) {
     uint64_t d = (uint64_t)((addr >> 4) & 0x3FFFu);
     d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
     d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
     d |= (uint64_t)1 << 46;   // descriptor version of this architecture
-    d |= (uint64_t)(kb == 64 ? 2 : (kb == 32 ? 4 : 6)) << 61;
+    d |= (uint64_t)(kb == 64 ? 2 : (kb == 32 ? 4 : (kb == 16 ? 6 : 0))) << 61;
     return d;
 }
 
@@ -367,6 +368,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         // ---- MMA: one elected thread
         if (lane == 0) {
             const uint32_t idesc = instr_desc(BM, g.bn, bw);
+            // descriptors of a stage at address zero; planes are aplane (zplane) x 16 bytes apart
+            const uint64_t adesc = bw ? smem_desc(0, 3u * BK * arow, 8 * arow, g.kb) : smem_desc(0, 16, 8 * arow, g.kb);
+            const uint64_t bdesc =
+                (bw ? smem_desc(0, 3u * BK * zrow, 8 * zrow, g.kz) : smem_desc(0, 16, 8 * arow, g.kb)) +
+                ((uint32_t)g.a_bytes >> 4);
+            const uint32_t aplane = (bw ? BK : BM) * arow / 16, zplane = BK * zrow / 16;
+            const int nkk = g.kb / 16;
             int n = 0, a = 0;                                   // stages consumed, tiles begun
             bool ok = true;
             for (int it = blockIdx.x; ok && it < g.items; it += gridDim.x, ++a) {
@@ -389,27 +397,30 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int s = n % S;
                     if (!(ok = mbar_wait(&full[s], (uint32_t)((n / S) & 1), &dead))) break;
                     asm volatile("tcgen05.fence::after_thread_sync;");
-                    const uint32_t sa = smem0 + (uint32_t)s * (uint32_t)g.stage_bytes, sb = sa + (uint32_t)g.a_bytes;
+                    // descriptors differ by their start addresses (in 16 bytes) only
+                    const uint32_t s4 = (smem0 + (uint32_t)s * (uint32_t)g.stage_bytes) >> 4;
+                    const uint64_t ad = adesc + s4, bd = bdesc + s4;
                     if (!bw) {
-                        for (int kk = 0; kk < g.kb / 16; ++kk) {
-                            const uint64_t bd = smem_desc(sb + kk * 32, 16, 8 * arow, g.kb);
 #pragma unroll
-                            for (int p = 0; p < 3; ++p) {
-                                mma_bf16(d, smem_desc(sa + p * BM * arow + kk * 32, 16, 8 * arow, g.kb), bd, idesc, issued);
-                                issued = 1;
+                        for (int kk = 0; kk < 4; ++kk) {
+                            if (kk < nkk) {
+#pragma unroll
+                                for (int p = 0; p < 3; ++p) {
+                                    mma_bf16(d, ad + (uint32_t)p * aplane + 2 * kk, bd + 2 * kk, idesc, issued);
+                                    issued = 1;
+                                }
                             }
                         }
                     } else {
                         // 16 pixels at a time; plane pairs (dz, x) with pz + px <= 2
+#pragma unroll
                         for (int kk = 0; kk < BK / 16; ++kk) {
 #pragma unroll
                             for (int pz = 0; pz < 3; ++pz) {
-                                const uint64_t bd =
-                                    smem_desc(sb + pz * BK * zrow + kk * 16 * zrow, 3u * BK * zrow, 8 * zrow, g.kz);
 #pragma unroll
                                 for (int px = 0; px + pz <= 2; ++px) {
-                                    mma_bf16(d, smem_desc(sa + px * BK * arow + kk * 16 * arow, 3u * BK * arow, 8 * arow, g.kb),
-                                             bd, idesc, issued);
+                                    mma_bf16(d, ad + (uint32_t)px * aplane + kk * arow, bd + (uint32_t)pz * zplane + kk * zrow,
+                                             idesc, issued);
                                     issued = 1;
                                 }
                             }

@@ -18,9 +18,10 @@
 //
 // The convolutions, their data gradients and their weight gradients run as
 // implicit GEMMs on the tensor cores (conv_umma.cuh), each reading the bf16
-// planes that the kernel before it wrote; the first layer (two input channels,
-// 18 products a value) and its weight gradient are direct FP32 kernels here, as
-// are the ReLU masks, the loss and Adam.
+// planes that the kernel before it wrote.  The first layer (two input channels,
+// 18 products a value) has kernels of its own here: its forward pass on the tensor
+// cores, its weight gradient in FP32; the ReLU masks, the loss and Adam are
+// elementwise kernels.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -196,60 +197,131 @@ __global__ void __launch_bounds__(kT) mask_split_kernel(const float* __restrict_
 }
 
 // The first layer, e0 = relu(conv(x = [T, R]) + b), written as the next layer's
-// planes.  Two input channels make K = 18: as an implicit GEMM its operand rows
-// are 32 bytes of mostly padding (0.19 ms at batch 32, 128^2, against 0.10 ms for
-// a gather kernel); here a thread holds the 18 inputs of a pixel and makes
-// kFirstCh channels, bound by the 6 bytes a value it writes.
-constexpr int kFirstCh = 16;
-__global__ void __launch_bounds__(kT) conv_first_kernel(const float* __restrict__ T, const float* __restrict__ R,
-                                                        const float* __restrict__ W, const float* __restrict__ bias,
-                                                        __nv_bfloat16* planes, int C, int cp, int m, int B) {
-    __shared__ __align__(16) float w[kFirstCh][20], bs[kFirstCh];     // 16-byte rows: five loads a channel
-    const int c0 = blockIdx.y * kFirstCh;
+// planes: M = 128 pixels, N = bn = C rounded up to 16, K = 9 taps x 8 channels (two
+// used) rounded up to 80.  A thread makes one row of A: it reads the 18 inputs of
+// its pixel and writes their planes to shared memory as 16-byte core-matrix rows
+// (no TMA form fits: through tensor maps the rows are 32 bytes of mostly padding,
+// 0.19 ms at batch 32, 128^2, against 0.10 ms for a generic gather); three CTAs of
+// 128 threads per SM overlap the gather, the 15 MMAs and the stores, and the
+// 6 bytes a value that it writes bound it.  K is summed as two taps per MMA step
+// with the plane products innermost; the rounding of e0 decides its ReLU, and
+// with it whole gradient entries.
+constexpr int kFirstK = 10;       // 16-byte groups of K
+__global__ void __launch_bounds__(128) conv_first_kernel(const float* __restrict__ T, const float* __restrict__ R,
+                                                         const float* __restrict__ W, const float* __restrict__ bias,
+                                                         __nv_bfloat16* planes, int C, int bn, int cp, int m, int B,
+                                                         int tiles, int ncols, int* err) {
+    extern __shared__ __align__(128) uint8_t sm[];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint32_t tmem_base;
+    __shared__ int dead;
+    uint8_t* sb = sm + 3 * kFirstK * 2048;      // B: [k group][row] x 16 bytes; A: [plane][k group][row] x 16 bytes
+    float* bs = reinterpret_cast<float*>(sb + kFirstK * bn * 16);
+    const int tid = threadIdx.x, warp = tid >> 5;
     umma::dependency_trigger();
-    umma::dependency_wait();
-    for (int i = threadIdx.x; i < kFirstCh * 20; i += kT) {
-        const int c = i / 20, k = i % 20, tap = k >> 1, ci = k & 1;       // order (tap, ci)
-        w[c][k] = c0 + c < C && k < 18 ? __bfloat162float(__float2bfloat16_rn(W[((size_t)(c0 + c) * 2 + ci) * 9 + tap])) : 0.0f;
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(umma::smem_u32(&tmem_base)),
+                     "r"(ncols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    if (threadIdx.x < kFirstCh) bs[threadIdx.x] = c0 + (int)threadIdx.x < C ? bias[c0 + threadIdx.x] : 0.0f;
+    if (tid == 0) {
+        dead = 0;
+        umma::mbar_init(&bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    umma::dependency_wait();
+    for (int i = tid; i < kFirstK * bn; i += 128) {
+        const int tap = i / bn, n = i - tap * bn;
+        __align__(16) __nv_bfloat16 w[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            w[c] = __float2bfloat16_rn(c < 2 && tap < 9 && n < C ? W[((size_t)n * 2 + c) * 9 + tap] : 0.0f);
+        *reinterpret_cast<uint4*>(sb + (size_t)i * 16) = *reinterpret_cast<const uint4*>(w);
+    }
+    for (int i = tid; i < bn; i += 128) bs[i] = i < C ? bias[i] : 0.0f;
+#pragma unroll
+    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint4*>(sm + ((p * kFirstK + 9) * 128 + tid) * 16) = make_uint4(0, 0, 0, 0);
+    asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = tmem_base, a0 = umma::smem_u32(sm), b0 = umma::smem_u32(sb);
+    const uint32_t idesc = umma::instr_desc(umma::BM, bn, false);
     const size_t P = (size_t)m * m, n = P * B;
-    for (size_t i = blockIdx.x * (size_t)kT + threadIdx.x; i < n; i += (size_t)gridDim.x * kT) {
+    bool ok = true;
+    uint32_t phase = 0;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, phase ^= 1u) {
+        const size_t i = (size_t)tile * umma::BM + tid;
+        const bool valid = i < n;
         const size_t b = i / P;
         const int o = (int)(i - b * P), y = o / m, x = o - y * m;
         float in[18];
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
             const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
-            const bool ok = yy >= 0 && yy < m && xx >= 0 && xx < m;
-            const size_t e = b * P + (size_t)(ok ? yy * m + xx : 0);
-            in[2 * t] = ok ? __ldg(T + e) : 0.0f;
-            in[2 * t + 1] = ok ? __ldg(R + e) : 0.0f;
+            const bool in_img = valid && yy >= 0 && yy < m && xx >= 0 && xx < m;
+            const size_t e = in_img ? b * P + (size_t)(yy * m + xx) : 0;
+            in[2 * t] = in_img ? __ldg(T + e) : 0.0f;
+            in[2 * t + 1] = in_img ? __ldg(R + e) : 0.0f;
         }
 #pragma unroll
-        for (int q = 0; q < kFirstCh; q += 8) {
-            float v[8];
+        for (int t = 0; t < 9; ++t) {
+            __nv_bfloat16 h[2], q[2], l[2];
+            umma::split3(in[2 * t], h[0], q[0], l[0]);
+            umma::split3(in[2 * t + 1], h[1], q[1], l[1]);
+            uint8_t* dst = sm + (t * 128 + tid) * 16;
+            *reinterpret_cast<uint4*>(dst) = make_uint4(*reinterpret_cast<const uint32_t*>(h), 0, 0, 0);
+            *reinterpret_cast<uint4*>(dst + kFirstK * 2048) = make_uint4(*reinterpret_cast<const uint32_t*>(q), 0, 0, 0);
+            *reinterpret_cast<uint4*>(dst + 2 * kFirstK * 2048) = make_uint4(*reinterpret_cast<const uint32_t*>(l), 0, 0, 0);
+        }
+        asm volatile("fence.proxy.async.shared::cta;");
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        __syncthreads();
+        if (tid == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                float a = 0.0f;
-                const float4* wr = reinterpret_cast<const float4*>(w[q + j]);
+            for (int kk = 0; kk < kFirstK / 2; ++kk) {
+                const uint64_t bd = umma::smem_desc(b0 + kk * 2 * bn * 16, (uint32_t)bn * 16, 128, 0);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float4 t = wr[k];
-                    a = fmaf(in[4 * k], t.x, a);
-                    a = fmaf(in[4 * k + 1], t.y, a);
-                    a = fmaf(in[4 * k + 2], t.z, a);
-                    a = fmaf(in[4 * k + 3], t.w, a);
-                }
-                const float4 t = wr[4];
-                a = fmaf(in[16], t.x, a);
-                a = fmaf(in[17], t.y, a);
-                v[j] = c0 + q + j < C ? fmaxf(a + bs[q + j], 0.0f) : 0.0f;
+                for (int p = 0; p < 3; ++p)
+                    umma::mma_bf16(tmem, umma::smem_desc(a0 + (p * kFirstK + kk * 2) * 2048, 2048, 128, 0), bd, idesc,
+                                   kk + p > 0 ? 1u : 0u);
             }
-            umma::store_planes8(planes, n * cp, i * cp + c0 + q, v);
+            umma::mma_commit(&bar);
+        }
+        ok = umma::mbar_wait(&bar, phase, &dead);
+        if (__syncthreads_or(!ok)) {
+            ok = false;
+            break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        for (int c0 = 0; c0 < bn; c0 += 16) {
+            uint32_t v[16];
+            asm volatile(
+                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+                : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
+            asm volatile("tcgen05.wait::ld.sync.aligned;");
+            if (!valid) continue;
+            float z[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                z[j] = c0 + j < C ? fmaxf(__uint_as_float(v[j]) + bs[c0 + j], 0.0f) : 0.0f;
+            umma::store_planes8(planes, n * cp, i * cp + c0, z);
+            umma::store_planes8(planes, n * cp, i * cp + c0 + 8, z + 8);
         }
     }
+    if (!ok) {            // once more, bounded, for the MMAs in flight
+        if (tid == 0) {
+            atomicExch(err, 1);
+            for (long k = 0; k < umma::kWaitLimit && !umma::mbar_try(&bar, phase); ++k) {
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
 }
 
 // Partial weight and bias gradients of the first layer from the gradient g of
@@ -637,12 +709,20 @@ cudaError_t pack_weights(lgnk_ws* w) {
     return launch(pack_wmats_kernel, dim3(std::min(blocks_for(n), 608), 6), kT, 0, w->stream, w->p, all);
 }
 
+// Shared memory of the first layer's kernel, and its CTAs per SM (bounded by
+// that and by the 512 columns of tensor memory).
+size_t first_smem(int bn) { return (size_t)3 * kFirstK * 2048 + (size_t)kFirstK * bn * 16 + (size_t)bn * 4; }
+int first_ctas(int bn) { return bn <= 64 ? 3 : 2; }
+
 // The network; with train, also what only the backward pass reads (r4, r5).
 lgnk_status forward_pass(lgnk_ws* w, int B, const float* T, const float* R, float* v, bool train) {
     const Layer& L0 = w->L[0];
     const size_t n = (size_t)w->m * w->m * B;
-    cudaError_t e = launch(conv_first_kernel, dim3(blocks_for(n), w->L[1].cpi / kFirstCh), kT, 0, w->stream, T, R,
-                           w->p + L0.woff, w->p + L0.boff, w->planes[1], L0.co, w->L[1].cpi, w->m, B);
+    const int bn = w->L[1].cpi, tiles = (int)((n + umma::BM - 1) / umma::BM);
+    const int ncols = bn <= 32 ? 32 : (bn <= 64 ? 64 : (bn <= 128 ? 128 : 256));
+    cudaError_t e = launch(conv_first_kernel, dim3(std::min(tiles, first_ctas(bn) * w->sms)), 128, first_smem(bn), w->stream,
+                           T, R, w->p + L0.woff, w->p + L0.boff, w->planes[1], L0.co, bn, bn, w->m, B, tiles, ncols,
+                           w->derr);
     if (e == cudaSuccess) e = conv_fwd(w, 1, w->e1, nullptr, nullptr, 1, 1.0f, B);
     if (e == cudaSuccess) e = conv_fwd(w, 2, w->e2, nullptr, nullptr, 1, 1.0f, B);
     if (e == cudaSuccess) e = conv_fwd(w, 3, nullptr, nullptr, nullptr, 1, 1.0f, B);
@@ -780,6 +860,11 @@ lgnk_status lgnk_ws_create(int image_m, int base_channels, int max_batch, float 
             return fail(LGNK_ERR_CUDA);
         }
         w->smem_max = optin - (int)fa.sharedSizeBytes;
+        if (cudaFuncSetAttribute(conv_first_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)first_smem(256)) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return fail(LGNK_ERR_CUDA);
+        }
         if (cudaFuncSetAttribute(umma::conv_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, w->smem_max) !=
             cudaSuccess) {
             cudaGetLastError();
