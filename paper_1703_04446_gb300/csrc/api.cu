@@ -95,9 +95,11 @@ struct lgnk_ctx {
     void *Vp = nullptr, *dVp = nullptr, *Gp = nullptr;
     float *Tp = nullptr, *acc = nullptr, *rp = nullptr, *itmp = nullptr, *rtmp = nullptr;
     float *pc0 = nullptr, *pc1 = nullptr, *Cm[3] = {nullptr, nullptr, nullptr}, *inv_eig = nullptr;
-    // the DCT matrices in the shared-memory layouts of the tiled kernels, rows
-    // padded to P = m rounded up to 4: forward Cf[q][k] = C[k][q], inverse Ci[q][k] = C[q][k]
+    // the DCT matrices in the shared-memory layouts of the kernels: half tables
+    // (half[a]), or rows padded to P = m rounded up to 4 for the tiled per-axis
+    // kernel, forward Cf[q][k] = C[k][q], inverse Ci[q][k] = C[q][k]
     float *Cf[3] = {nullptr, nullptr, nullptr}, *Ci[3] = {nullptr, nullptr, nullptr};
+    bool half[3] = {false, false, false};
     PcgGraph pcg_graphs[2];       // [0] matrix-free, [1] assembled products
     PcgLoopGraph pcg_loops[2];
     double* partial = nullptr;
@@ -641,47 +643,44 @@ lgnk_status hessvec_assembled_packed(lgnk_ctx* ctx, const float* dv, float* out)
 }
 
 lgnk_status precond_apply(lgnk_ctx* ctx, const float* r, float* z) {
-    const int kd = ctx->K * ctx->d;
+    const int kd = ctx->K * ctx->d, d = ctx->d;
     cudaStream_t s = ctx->stream;
-    if (ctx->vg.m[ctx->d - 1] <= 128) {
-        // the last axis's forward transform, scale and inverse transform in one pass
-        if (ctx->d == 3 && ctx->vg.m[0] <= 64 && ctx->vg.m[1] <= 64) {
-            // y and x of each xy plane in one pass each way: three launches
-            const long long planes = (long long)kd * ctx->vg.m[2];
-            KL(launch_dct_plane(r, ctx->pc0, ctx->Cf[0], ctx->Cf[1], ctx->vg, planes, s));
-            KL(launch_dct_last_fused(ctx->pc0, ctx->pc1, ctx->Cf[2], ctx->Ci[2], ctx->inv_eig, ctx->vg, 3, kd, s));
-            KL(launch_dct_plane(ctx->pc1, z, ctx->Ci[0], ctx->Ci[1], ctx->vg, planes, s));
-        } else if (ctx->d == 3) {
-            KL(launch_dct_axis(r, ctx->pc0, ctx->Cm[0], ctx->Cf[0], ctx->vg, 3, kd, 0, false, s));
-            KL(launch_dct_axis(ctx->pc0, ctx->pc1, ctx->Cm[1], ctx->Cf[1], ctx->vg, 3, kd, 1, false, s));
-            KL(launch_dct_last_fused(ctx->pc1, ctx->pc0, ctx->Cf[2], ctx->Ci[2], ctx->inv_eig, ctx->vg, 3, kd, s));
-            KL(launch_dct_axis(ctx->pc0, ctx->pc1, ctx->Cm[1], ctx->Ci[1], ctx->vg, 3, kd, 1, true, s));
-            KL(launch_dct_axis(ctx->pc1, z, ctx->Cm[0], ctx->Ci[0], ctx->vg, 3, kd, 0, true, s));
-        } else if (ctx->d == 2 && ctx->vg.m[0] <= 64 && ctx->vg.m[1] <= 64) {
-            // the whole transform of each plane in one CTA: one launch
-            KL(launch_dct_plane2d(r, z, ctx->Cf[0], ctx->Cf[1], ctx->Ci[0], ctx->Ci[1], ctx->inv_eig, ctx->vg, kd, s));
-        } else {
-            KL(launch_dct_axis(r, ctx->pc0, ctx->Cm[0], ctx->Cf[0], ctx->vg, 2, kd, 0, false, s));
-            KL(launch_dct_last_fused(ctx->pc0, ctx->pc1, ctx->Cf[1], ctx->Ci[1], ctx->inv_eig, ctx->vg, 2, kd, s));
-            KL(launch_dct_axis(ctx->pc1, z, ctx->Cm[0], ctx->Ci[0], ctx->vg, 2, kd, 0, true, s));
-        }
+    const float *in = r;
+    float *bufs[2] = {ctx->pc0, ctx->pc1}, *out = z;
+    if (d == 3 && ctx->half[0]) {
+        // y and x of each xy plane in one pass each way, the last axis both ways with
+        // the scale in between: three launches
+        const long long planes = (long long)kd * ctx->vg.m[2];
+        KL(launch_dct_plane(r, ctx->pc0, ctx->Cf[0], ctx->Cf[1], false, ctx->vg, planes, s));
+        KL(launch_dct_last_half(ctx->pc0, ctx->pc1, ctx->Cf[2], ctx->Ci[2], ctx->inv_eig, ctx->vg, 3, kd, s));
+        KL(launch_dct_plane(ctx->pc1, z, ctx->Ci[0], ctx->Ci[1], true, ctx->vg, planes, s));
         return LGNK_OK;
     }
-    if (ctx->d == 3) {
-        KL(launch_dct_axis(r, ctx->pc0, ctx->Cm[0], ctx->Cf[0], ctx->vg, 3, kd, 0, false, s));
-        KL(launch_dct_axis(ctx->pc0, ctx->pc1, ctx->Cm[1], ctx->Cf[1], ctx->vg, 3, kd, 1, false, s));
-        KL(launch_dct_axis(ctx->pc1, ctx->pc0, ctx->Cm[2], ctx->Cf[2], ctx->vg, 3, kd, 2, false, s));
-        KL(launch_scale_modes(ctx->pc0, ctx->inv_eig, ctx->Mv, ctx->n, s));
-        KL(launch_dct_axis(ctx->pc0, ctx->pc1, ctx->Cm[2], ctx->Ci[2], ctx->vg, 3, kd, 2, true, s));
-        KL(launch_dct_axis(ctx->pc1, ctx->pc0, ctx->Cm[1], ctx->Ci[1], ctx->vg, 3, kd, 1, true, s));
-        KL(launch_dct_axis(ctx->pc0, z, ctx->Cm[0], ctx->Ci[0], ctx->vg, 3, kd, 0, true, s));
-    } else {
-        KL(launch_dct_axis(r, ctx->pc0, ctx->Cm[0], ctx->Cf[0], ctx->vg, 2, kd, 0, false, s));
-        KL(launch_dct_axis(ctx->pc0, ctx->pc1, ctx->Cm[1], ctx->Cf[1], ctx->vg, 2, kd, 1, false, s));
-        KL(launch_scale_modes(ctx->pc1, ctx->inv_eig, ctx->Mv, ctx->n, s));
-        KL(launch_dct_axis(ctx->pc1, ctx->pc0, ctx->Cm[1], ctx->Ci[1], ctx->vg, 2, kd, 1, true, s));
-        KL(launch_dct_axis(ctx->pc0, z, ctx->Cm[0], ctx->Ci[0], ctx->vg, 2, kd, 0, true, s));
+    if (d == 2 && ctx->half[0]) {
+        // the whole transform of each plane in one CTA: one launch
+        KL(launch_dct_plane2d(r, z, ctx->Cf[0], ctx->Cf[1], ctx->Ci[0], ctx->Ci[1], ctx->inv_eig, ctx->vg, kd, s));
+        return LGNK_OK;
     }
+    // per axis: forward up to the last one, that one with the scale (fused when it
+    // has half tables), and back
+    int b = 0;
+    auto axis = [&](int a, bool inverse, float* dst) -> lgnk_status {
+        KL(launch_dct_axis(in, dst, ctx->Cm[a], inverse ? ctx->Ci[a] : ctx->Cf[a], ctx->vg, d, kd, a, inverse, s));
+        in = dst;
+        b ^= 1;
+        return LGNK_OK;
+    };
+    for (int a = 0; a < d - 1; ++a) TRY(axis(a, false, bufs[b]));
+    if (ctx->half[d - 1]) {
+        KL(launch_dct_last_half(in, bufs[b], ctx->Cf[d - 1], ctx->Ci[d - 1], ctx->inv_eig, ctx->vg, d, kd, s));
+        in = bufs[b];
+        b ^= 1;
+    } else {
+        TRY(axis(d - 1, false, bufs[b]));
+        KL(launch_scale_modes(bufs[b ^ 1], ctx->inv_eig, ctx->Mv, ctx->n, s));
+        TRY(axis(d - 1, true, bufs[b]));
+    }
+    for (int a = d - 2; a >= 0; --a) TRY(axis(a, true, a == 0 ? out : bufs[b]));
     return LGNK_OK;
 }
 
@@ -840,10 +839,22 @@ lgnk_status lgnk_create(const lgnk_problem* prob, void* stream, size_t mem_budge
     if ((s = dalloc(ctx, ctx->n, &ctx->pc0)) != LGNK_OK) return fail(s);
     if ((s = dalloc(ctx, ctx->n, &ctx->pc1)) != LGNK_OK) return fail(s);
     for (int a = 0; a < d; ++a) {
+        // one block: the padded tables and the plain matrix, or the two half tables
+        // (which are never larger: rows of about m floats, half as many)
         const size_t m = (size_t)ctx->vg.m[a], P = (m + 3) & ~(size_t)3;
-        if ((s = dalloc(ctx, m * m, &ctx->Cm[a])) != LGNK_OK) return fail(s);
-        if ((s = dalloc(ctx, m * P, &ctx->Cf[a])) != LGNK_OK) return fail(s);
-        if ((s = dalloc(ctx, m * P, &ctx->Ci[a])) != LGNK_OK) return fail(s);
+        if ((s = dalloc(ctx, m * m + 2 * m * P, &ctx->Cf[a])) != LGNK_OK) return fail(s);
+    }
+    {
+        // whole planes by halves when every axis allows it, else the last axis only;
+        // (the last axis of a 2D grid whose first is long runs on as many lines)
+        bool all = true;
+        for (int a = 0; a < d; ++a) all = all && dct_half_axis_ok(ctx->vg.m[a]);
+        for (int a = 0; a < d; ++a) {
+            const size_t m = (size_t)ctx->vg.m[a], P = (m + 3) & ~(size_t)3;
+            ctx->half[a] = all || (a == d - 1 && dct_half_axis_ok(ctx->vg.m[a]) && ctx->K * d <= 65535);
+            ctx->Ci[a] = ctx->Cf[a] + (ctx->half[a] ? dct_half_floats(ctx->vg.m[a]) : m * P);
+            ctx->Cm[a] = ctx->half[a] ? nullptr : ctx->Cf[a] + 2 * m * P;
+        }
     }
     if ((s = dalloc(ctx, ctx->Mv, &ctx->inv_eig)) != LGNK_OK) return fail(s);
     // per-block partials: a trace's blocks, or two per reduction block (two inner
@@ -880,15 +891,20 @@ lgnk_status lgnk_create(const lgnk_problem* prob, void* stream, size_t mem_budge
             for (int i = 0; i < m; ++i)
                 hostC[(size_t)k * m + i] =
                     (float)(std::sqrt((k == 0 ? 1.0 : 2.0) / m) * std::cos(M_PI * k * (2 * i + 1) / (2.0 * m)));
-        if (cudaMemcpy(ctx->Cm[a], hostC.data(), hostC.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
-            return fail(LGNK_ERR_CUDA);
         const size_t P = ((size_t)m + 3) & ~(size_t)3;
-        std::vector<float> hf((size_t)m * P, 0.0f), hi((size_t)m * P, 0.0f);
-        for (int q = 0; q < m; ++q)
-            for (int k = 0; k < m; ++k) {
-                hf[(size_t)q * P + k] = hostC[(size_t)k * m + q];
-                hi[(size_t)q * P + k] = hostC[(size_t)q * m + k];
-            }
+        const size_t nt = ctx->half[a] ? dct_half_floats(m) : (size_t)m * P;
+        std::vector<float> hf(nt, 0.0f), hi(nt, 0.0f);
+        if (ctx->half[a]) {
+            dct_half_tables(hostC.data(), m, hf.data(), hi.data());
+        } else {
+            for (int q = 0; q < m; ++q)
+                for (int k = 0; k < m; ++k) {
+                    hf[(size_t)q * P + k] = hostC[(size_t)k * m + q];
+                    hi[(size_t)q * P + k] = hostC[(size_t)q * m + k];
+                }
+            if (cudaMemcpy(ctx->Cm[a], hostC.data(), hostC.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
+                return fail(LGNK_ERR_CUDA);
+        }
         if (cudaMemcpy(ctx->Cf[a], hf.data(), hf.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(ctx->Ci[a], hi.data(), hi.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
             return fail(LGNK_ERR_CUDA);

@@ -528,6 +528,12 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 
+// the same for 4 bytes (rows that are not 16-byte aligned)
+__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+
 __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
@@ -642,291 +648,505 @@ __global__ void __launch_bounds__(kBlock) dct_tile_kernel(const float* __restric
     }
 }
 
-// The last axis of the preconditioner in one pass: forward DCT along the
-// axis, the spectral scale inv_eig (per mode, the same for every block), and
-// the inverse DCT, with the scaled modes kept in shared memory in between.
-// LINES lines per CTA of 4 LINES threads, with the register blocking of
-// dct_tile_kernel (strided form); every sum still runs in increasing index
-// order.
-constexpr int kDctFusedLines = 32;
+// ---- transforms by halves.  The DCT-II rows are even or odd about the middle of
+// the axis, C[k][m-1-q] = (-1)^k C[k][q], so with s_q = x_q + x_(m-1-q) and
+// d_q = x_q - x_(m-1-q) the even modes are sums over s and the odd modes over d of
+// half the length, and the inverse is x_q = E_q + O_q, x_(m-1-q) = E_q - O_q with
+// E (O) the sum over the even (odd) modes: half the FMAs and half the table.
+//
+// A table (dct_half_table) has a row of the even and the odd part, each padded
+// to P4 = ceil(m/2) rounded up to 4 floats; forward rows run over q, inverse rows
+// over the mode pairs.  The operand of either direction is a tile of lines in
+// shared memory, [index][LS], first folded into s and d (forward).  A task is 4 even
+// and 4 odd outputs (forward: 8 consecutive modes; inverse: 4 q and their mirrors)
+// of LT lines, done by one thread (LT = 8: 64 FMAs per 6 shared loads) or, where a
+// CTA would have few threads, by two neighbouring lanes (SPLIT, LT = 4), one for
+// the even and one for the odd part, which then exchange what the other stores.
+// Sums run in increasing index order.
 
-template <int LINES>
-__global__ void __launch_bounds__(4 * LINES) dct_last_fused_kernel(const float* __restrict__ in,
-                                                                   float* __restrict__ out,
-                                                                   const float* __restrict__ Cfg,
-                                                                   const float* __restrict__ Cig,
-                                                                   const float* __restrict__ inv_eig, int m,
-                                                                   long long inner, int vec_in) {
-    constexpr int NT = 4 * LINES, LS = LINES + 4;
-    extern __shared__ __align__(16) float sm[];
-    const int MP = (m + 3) & ~3;
-    float* Cf = sm;                   // forward: [q][k] = C[k][q]
-    float* Ci = sm + m * MP;          // inverse: [k][k'] = C[k][k']
-    float* tile = sm + 2 * m * MP;    // [q][LS], then the scaled modes [k][LS]
-    const int t = threadIdx.x;
-    for (int e = t; e < m * MP / 4; e += NT) {
-        cp_async16(Cf + 4 * e, Cfg + 4 * e);
-        cp_async16(Ci + 4 * e, Cig + 4 * e);
+// acc_e[i][l] = sum_r tab[r][j0 + i] E_r[l], acc_o = sum_r tab[r][P4 + j0 + i] O_r[l]
+// over the m/2 pairs and the unpaired even row of an odd m; row r of the even
+// (odd) operand is at even + r se (odd + r so).
+template <int LT>
+__device__ __forceinline__ void dct_half_product(const float* tab, int P4, int stride, int m, int j0, const float* even,
+                                                 int se, const float* odd, int so, float (&ae)[4][LT],
+                                                 float (&ao)[4][LT]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int l = 0; l < LT; ++l) ae[i][l] = ao[i][l] = 0.0f;
+    const int n = m / 2;
+    const float* te = tab + j0;
+#pragma unroll 2
+    for (int r = 0; r < n; ++r) {
+        const float4 a = *reinterpret_cast<const float4*>(te);
+        const float4 b = *reinterpret_cast<const float4*>(te + P4);
+        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+        float x[LT], y[LT];
+#pragma unroll
+        for (int l = 0; l < LT; l += 4) {
+            *reinterpret_cast<float4*>(x + l) = *reinterpret_cast<const float4*>(even + l);
+            *reinterpret_cast<float4*>(y + l) = *reinterpret_cast<const float4*>(odd + l);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int l = 0; l < LT; ++l) {
+                ae[i][l] = fmaf(av[i], x[l], ae[i][l]);
+                ao[i][l] = fmaf(bv[i], y[l], ao[i][l]);
+            }
+        te += stride;
+        even += se;
+        odd += so;
     }
+    if (m & 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int l = 0; l < LT; ++l) ae[i][l] = fmaf(te[i], even[l], ae[i][l]);
+    }
+}
+
+// The even (p = 0) or odd (p = 1) part of a task.
+__device__ __forceinline__ void dct_half_part(const float* tab, int P4, int stride, int m, bool inverse, const float* S,
+                                              int LS, int j0, int l0, int p, float (&a)[4][4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int l = 0; l < 4; ++l) a[i][l] = 0.0f;
+    const int n = m / 2, st = inverse ? 2 * LS : (p ? -LS : LS);
+    const float* t = tab + j0 + p * P4;
+    const float* x = S + l0 + (inverse ? p * LS : p * (m - 1) * LS);
+#pragma unroll 4
+    for (int r = 0; r < n; ++r) {
+        const float4 c = *reinterpret_cast<const float4*>(t);
+        const float4 v = *reinterpret_cast<const float4*>(x);
+        const float cv[4] = {c.x, c.y, c.z, c.w}, xv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int l = 0; l < 4; ++l) a[i][l] = fmaf(cv[i], xv[l], a[i][l]);
+        t += stride;
+        x += st;
+    }
+    if ((m & 1) && p == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int l = 0; l < 4; ++l) a[i][l] = fmaf(t[i], x[l], a[i][l]);
+    }
+}
+
+// Line l of a split task: the four outputs this lane stores, from position
+// `at` (dct_part_start) on.  Every lane of the warp calls it.
+__device__ __forceinline__ float4 dct_part_outputs(bool inverse, const float (&a)[4][4], int l, int p) {
+    float v[4];
+    if (inverse) {           // even lane E + O at j0 + i; odd lane E - O, mirrored
+        float w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float o = __shfl_xor_sync(0xffffffffu, a[i][l], 1);
+            w[i] = p ? o - a[i][l] : a[i][l] + o;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = p ? w[3 - i] : w[i];
+    } else {                 // modes e0 o0 e1 o1 (even lane), e2 o2 e3 o3 (odd lane)
+        const float r0 = __shfl_xor_sync(0xffffffffu, p ? a[0][l] : a[2][l], 1);
+        const float r1 = __shfl_xor_sync(0xffffffffu, p ? a[1][l] : a[3][l], 1);
+        v[0] = p ? r0 : a[0][l];
+        v[1] = p ? a[2][l] : r0;
+        v[2] = p ? r1 : a[1][l];
+        v[3] = p ? a[3][l] : r1;
+    }
+    return make_float4(v[0], v[1], v[2], v[3]);
+}
+
+__device__ __forceinline__ int dct_part_start(bool inverse, int m, int j0, int p) {
+    return inverse ? (p ? m - 4 - j0 : j0) : 2 * j0 + 4 * p;
+}
+
+// ... into a row of m values: positions below 0 or past m (forward), past the middle
+// (inverse) are no outputs of this lane.
+__device__ __forceinline__ void dct_store_part(float* dst, int m, int j0, int p, bool inverse, bool vec, float4 v) {
+    const int at = dct_part_start(inverse, m, j0, p), h = (m + 1) / 2;
+    if (vec && (inverse ? j0 + 4 <= m / 2 : at + 4 <= m)) {
+        *reinterpret_cast<float4*>(dst + at) = v;
+        return;
+    }
+    const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (inverse ? j0 + (p ? 3 - i : i) < h : at + i < m) dst[at + i] = x[i];
+}
+
+// x_q, x_(m-1-q) -> s_q, d_q in place (rows of a tile); every thread of the CTA.
+__device__ __forceinline__ void dct_fold(float* S, int LS, int m, int lines) {
+    const int c4 = (lines + 3) / 4, n = m / 2;
+    for (int e = threadIdx.x; e < n * c4; e += blockDim.x) {
+        const int q = e / c4, l = 4 * (e % c4);
+        float4* p = reinterpret_cast<float4*>(S + q * LS + l);
+        float4* r = reinterpret_cast<float4*>(S + (m - 1 - q) * LS + l);
+        const float4 a = *p, b = *r;
+        *p = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+        *r = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+    }
+}
+
+// One direction of an axis on the tile S: the product of this thread's task.
+template <int LT>
+__device__ __forceinline__ void dct_half_axis(const float* tab, int P4, int stride, int m, bool inverse, const float* S,
+                                              int LS, int j0, int l0, float (&ae)[4][LT], float (&ao)[4][LT]) {
+    if (inverse) dct_half_product<LT>(tab, P4, stride, m, j0, S + l0, 2 * LS, S + LS + l0, 2 * LS, ae, ao);
+    else dct_half_product<LT>(tab, P4, stride, m, j0, S + l0, LS, S + (m - 1) * LS + l0, -LS, ae, ao);
+}
+
+// The 8 outputs of line l of a task: forward, modes 2 j0 .. 2 j0 + 7 in v; inverse,
+// positions j0 .. j0 + 3 in v[0..3] and m - 1 - j0 - 3 .. m - 1 - j0 in v[4..7].
+template <int LT>
+__device__ __forceinline__ void dct_outputs(bool inverse, const float (&ae)[4][LT], const float (&ao)[4][LT], int l,
+                                            float* v) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (inverse) {
+            v[i] = ae[i][l] + ao[i][l];
+            v[7 - i] = ae[i][l] - ao[i][l];
+        } else {
+            v[2 * i] = ae[i][l];
+            v[2 * i + 1] = ao[i][l];
+        }
+    }
+}
+
+// Stores the 8 outputs of one line into a row of m values at dst.
+__device__ __forceinline__ void dct_store_line(float* dst, int m, int j0, bool inverse, bool vec, const float* v) {
+    const int h = (m + 1) / 2, a = inverse ? j0 : 2 * j0, b = inverse ? m - 4 - j0 : 2 * j0 + 4;
+    // whole groups: forward both halves inside m; inverse 4 positions below the middle, mirrors distinct
+    if (vec && (inverse ? j0 + 4 <= m / 2 : b + 4 <= m)) {
+        *reinterpret_cast<float4*>(dst + a) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4*>(dst + b) = make_float4(v[4], v[5], v[6], v[7]);
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (inverse) {
+            if (j0 + i < h) {
+                dst[j0 + i] = v[i];
+                dst[m - 1 - j0 - i] = v[7 - i];      // the middle of an odd m is written twice with the same value
+            }
+        } else {
+            if (a + i < m) dst[a + i] = v[i];
+            if (b + i < m) dst[b + i] = v[4 + i];
+        }
+    }
+}
+
+struct HalfTable {
+    const float* p;
+    int P4, stride, rows;     // padded length of a part; floats of a row; rows (ceil(m/2))
+};
+
+__device__ __forceinline__ void dct_stage_table(float* dst, const HalfTable& t) {
+    for (int e = threadIdx.x; e < t.rows * t.stride / 4; e += blockDim.x) cp_async16(dst + 4 * e, t.p + 4 * e);
+}
+
+// The last axis of the preconditioner in one pass: forward transform, the
+// spectral scale inv_eig (per mode, the same for every block) and the inverse,
+// with the scaled modes kept in shared memory in between.  A CTA takes
+// LINES lines (64, or 32 where that leaves SMs without a CTA), a thread 8 outputs
+// of 4 lines.
+constexpr int kDctFusedLines = 64;
+
+template <int LINES, bool SPLIT>
+__global__ void __launch_bounds__(kBlock) dct_last_half_kernel(const float* __restrict__ in, float* __restrict__ out,
+                                                               const HalfTable tf, const HalfTable ti,
+                                                               const float* __restrict__ inv_eig, int m,
+                                                               long long inner, int vec_in) {
+    constexpr int LS = LINES + 4, LT = 4;
+    extern __shared__ __align__(16) float sm[];
+    float* F = sm;
+    float* I = F + tf.rows * tf.stride;
+    float* tile = I + ti.rows * ti.stride;     // [q][LS], then the scaled modes [k][LS]
+    dct_stage_table(F, tf);
+    dct_stage_table(I, ti);
     const long long o = blockIdx.y, i0 = (long long)blockIdx.x * LINES;
+    const int t = threadIdx.x;
     if (vec_in) {                     // inner a multiple of 4, in 16-byte aligned: whole float4s in or out
-        for (int e = t; e < m * (LINES / 4); e += NT) {
+        for (int e = t; e < m * (LINES / 4); e += blockDim.x) {
             const int q = e / (LINES / 4), l = 4 * (e % (LINES / 4));
             if (i0 + l < inner) cp_async16(tile + q * LS + l, in + ((size_t)o * m + q) * inner + i0 + l);
             else *reinterpret_cast<float4*>(tile + q * LS + l) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
     } else {
-        for (int e = t; e < LINES * m; e += NT) {
+        for (int e = t; e < LINES * m; e += blockDim.x) {
             const int q = e / LINES, l = e % LINES;
-            tile[q * LS + l] = (i0 + l < inner) ? __ldg(in + ((size_t)o * m + q) * inner + i0 + l) : 0.0f;
+            if (i0 + l < inner) cp_async4(tile + q * LS + l, in + ((size_t)o * m + q) * inner + i0 + l);
+            else tile[q * LS + l] = 0.0f;
         }
     }
     cp_async_wait_all();
     __syncthreads();
-    const int ntask = (MP / 4) * (LINES / 4);
-    float acc[2][4][4];               // at most two tasks per thread (MP <= 128)
-    for (int pass = 0; pass < 2; ++pass) {
-        const float* Cm = pass == 0 ? Cf : Ci;
+    dct_fold(tile, LS, m, LINES);
+    __syncthreads();
+    const int p = SPLIT ? t & 1 : 0, task = SPLIT ? t >> 1 : t;
+    const int l0 = LT * (task % (LINES / LT)), j0 = 4 * (task / (LINES / LT));
+    const int h = (m + 1) / 2;
+    const bool act = j0 < h;
+    float ae[4][LT], ao[4][LT];
+    if (act) {
+        if (SPLIT) dct_half_part(F, tf.P4, tf.stride, m, false, tile, LS, j0, l0, p, ae);
+        else dct_half_axis<LT>(F, tf.P4, tf.stride, m, false, tile, LS, j0, l0, ae, ao);
+    }
+    __syncthreads();                  // every thread is done reading the tile
+    const bool vec = vec_in && i0 + l0 + LT <= inner;
+    if (act) {
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int task = t + r * NT;
-            if (task >= ntask) break;
-            const int kb = task / (LINES / 4), lb = task % (LINES / 4);
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[r][i][j] = 0.0f;
-            const float4* cp = reinterpret_cast<const float4*>(Cm) + kb;
-            const float4* xp = reinterpret_cast<const float4*>(tile) + lb;
-#pragma unroll 4
-            for (int q = 0; q < m; ++q) {
-                const float4 c = cp[q * (MP / 4)];
-                const float4 x = xp[q * (LS / 4)];
-                const float cv[4] = {c.x, c.y, c.z, c.w}, xv[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[r][i][j] = fmaf(cv[i], xv[j], acc[r][i][j]);
+            for (int q = 0; q < (SPLIT ? 1 : 2); ++q) {
+                const int k = 2 * (j0 + i) + (SPLIT ? p : q);
+                if (k >= m) continue;
+                const float4 v = q ? make_float4(ao[i][0], ao[i][1], ao[i][2], ao[i][3])
+                                   : make_float4(ae[i][0], ae[i][1], ae[i][2], ae[i][3]);
+                const float* e = inv_eig + (size_t)k * inner + i0 + l0;
+                float4 sc;
+                if (vec) {
+                    sc = __ldg(reinterpret_cast<const float4*>(e));
+                } else {
+                    sc.x = i0 + l0 < inner ? __ldg(e) : 0.0f;
+                    sc.y = i0 + l0 + 1 < inner ? __ldg(e + 1) : 0.0f;
+                    sc.z = i0 + l0 + 2 < inner ? __ldg(e + 2) : 0.0f;
+                    sc.w = i0 + l0 + 3 < inner ? __ldg(e + 3) : 0.0f;
+                }
+                *reinterpret_cast<float4*>(tile + k * LS + l0) =
+                    make_float4(v.x * sc.x, v.y * sc.y, v.z * sc.z, v.w * sc.w);
             }
-        }
-        __syncthreads();              // every thread is done reading the tile
+    }
+    __syncthreads();
+    if (act) {
+        if (SPLIT) dct_half_part(I, ti.P4, ti.stride, m, true, tile, LS, j0, l0, p, ae);
+        else dct_half_axis<LT>(I, ti.P4, ti.stride, m, true, tile, LS, j0, l0, ae, ao);
+    }
+    const bool vec_out = vec && reinterpret_cast<uintptr_t>(out) % 16 == 0;
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int task = t + r * NT;
-            if (task >= ntask) break;
-            const int kb = task / (LINES / 4), lb = task % (LINES / 4);
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int k = 4 * kb + i;
-                if (k >= m) break;
+        for (int c = 0; c < (SPLIT ? 1 : 2); ++c) {
+            const int mir = SPLIT ? p : c, q = mir ? m - 1 - j0 - i : j0 + i;
+            float v[LT];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const long long l = i0 + 4 * lb + j;
-                    if (pass == 0) {
-                        const float sc = l < inner ? __ldg(inv_eig + (size_t)k * inner + l) : 0.0f;
-                        tile[k * LS + 4 * lb + j] = acc[r][i][j] * sc;
-                    } else if (l < inner) {
-                        out[((size_t)o * m + k) * inner + l] = acc[r][i][j];
-                    }
+            for (int l = 0; l < LT; ++l) {
+                if (SPLIT) {
+                    const float o = __shfl_xor_sync(0xffffffffu, ae[i][l], 1);
+                    v[l] = p ? o - ae[i][l] : ae[i][l] + o;
+                } else {
+                    v[l] = c ? ae[i][l] - ao[i][l] : ae[i][l] + ao[i][l];
                 }
             }
+            if (!act || j0 + i >= h) continue;
+            float* d = out + ((size_t)o * m + q) * inner + i0 + l0;
+            if (vec_out) {
+                *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
+            } else {
+#pragma unroll
+                for (int l = 0; l < LT; ++l)
+                    if (i0 + l0 + l < inner) d[l] = v[l];
+            }
         }
-        __syncthreads();
-    }
 }
 
 // The y and x axes of the transform on whole xy planes (both at most
 // kDctPlaneMax cells): a CTA holds one plane of one (block, z) in shared
-// memory and applies the y axis and then the x axis, two small matrix products
-// chained through shared memory.  The y result goes back transposed, [x][k],
-// from registers, so that both products read float4 rows of shared memory and
-// the plane is loaded and stored row-major.  With Ay, Ax the padded tables of
-// the direction (forward Cf, inverse Ci):
-//   forward: modes = C_y X C_x^T      inverse: X = C_y^T modes C_x
-// The tables and the plane are staged with asynchronous 16-byte copies, all
-// issued before the first wait.  A thread computes a 4 x 4 block of each
-// product; every sum runs over its index in increasing order.  The two axes
-// commute, so this equals the per-axis passes up to rounding.
-constexpr int kDctPlaneMax = 64;
+// memory and applies the y axis and then the x axis, two products chained
+// through shared memory.  The y result goes back transposed, [x][k], so that both
+// products read float4 rows and the plane is loaded and stored row-major.  The
+// two axes commute, so one order serves both directions.
+constexpr int kDctPlaneMax = 128;
 
-// The chained products of one plane: the plane is in S as rows [y][LS]; the
-// y product with Ay ([q][PY]) goes back into S transposed, [x][LT], and the x
-// product with Ax ([q][PX]) is left in acc[i][j] = (x index 4 xb + i, y index
-// 4 kb + j) of this thread's block.  Every thread of the CTA calls it (two
-// barriers); act: the thread has a block.
-__device__ __forceinline__ void plane_yx(const float* Ay, const float* Ax, float* S, int mx, int my, int PX, int PY,
-                                         int LS, int LT, bool act, int kb, int xb, float (&acc)[4][4]) {
+// A thread's task in the plane kernels: LT = 8 lines, both parts; LT = 4 (split), one part.
+template <int LT>
+struct PlaneTask {
+    static constexpr bool SPLIT = LT == 4;
+    int j0, l0, p;
+    bool act;
+    float ae[4][LT], ao[SPLIT ? 1 : 4][SPLIT ? 1 : LT];
+
+    // consecutive threads take consecutive output groups of one line group: the
+    // transposed store and the store of the plane then write whole rows
+    __device__ __forceinline__ void place(int m, int lines) {
+        const int t = SPLIT ? threadIdx.x >> 1 : threadIdx.x, g = ((m + 1) / 2 + 3) / 4;
+        p = SPLIT ? threadIdx.x & 1 : 0;
+        j0 = 4 * (t % g);
+        l0 = LT * (t / g);
+        act = l0 < lines;
+    }
+    __device__ __forceinline__ void product(const float* tab, const HalfTable& t, int m, bool inverse, const float* S,
+                                            int LS) {
+        if (!act) return;
+        if constexpr (SPLIT) dct_half_part(tab, t.P4, t.stride, m, inverse, S, LS, j0, l0, p, ae);
+        else dct_half_axis<LT>(tab, t.P4, t.stride, m, inverse, S, LS, j0, l0, ae, ao);
+    }
+    // Stores the outputs of lines l0 .. as rows of m values, `row` floats apart;
+    // scale: NULL or factors of the same layout (rows of m).  Every thread calls it.
+    __device__ __forceinline__ void store(float* dst, size_t row, int m, int lines, bool inverse, bool vec,
+                                          const float* scale) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+        for (int l = 0; l < LT; ++l) {
+            const bool in = act && l0 + l < lines;
+            if constexpr (SPLIT) {
+                float4 v = dct_part_outputs(inverse, ae, l, p);
+                if (!in) continue;
+                if (scale != nullptr) {
+                    const int at = dct_part_start(inverse, m, j0, p);
+                    const float* sc = scale + (size_t)(l0 + l) * m + at;
+                    v.x *= at < m ? __ldg(sc) : 0.0f;
+                    v.y *= at + 1 < m ? __ldg(sc + 1) : 0.0f;
+                    v.z *= at + 2 < m ? __ldg(sc + 2) : 0.0f;
+                    v.w *= at + 3 < m ? __ldg(sc + 3) : 0.0f;
+                }
+                dct_store_part(dst + (l0 + l) * row, m, j0, p, inverse, vec, v);
+            } else {
+                if (!in) continue;
+                float v[8];
+                dct_outputs<LT>(inverse, ae, ao, l, v);
+                if (scale != nullptr) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;   // [k along y][x]
-    if (act) {
-        const float4* ap = reinterpret_cast<const float4*>(Ay) + kb;
-        const float4* sp = reinterpret_cast<const float4*>(S) + xb;
-#pragma unroll 4
-        for (int q = 0; q < my; ++q) {
-            const float4 a = ap[q * (PY / 4)];
-            const float4 x = sp[q * (LS / 4)];
-            const float av[4] = {a.x, a.y, a.z, a.w}, xv[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], xv[j], acc[i][j]);
+                    for (int i = 0; i < 8; ++i)
+                        v[i] *= 2 * j0 + i < m ? __ldg(scale + (size_t)(l0 + l) * m + 2 * j0 + i) : 0.0f;
+                }
+                dct_store_line(dst + (l0 + l) * row, m, j0, inverse, vec, v);
+            }
         }
     }
+};
+
+// Both products of the plane in S (rows [y][LS]), every thread of the CTA; the x
+// product's outputs (lines = ky) stay in the task.
+template <int LT>
+__device__ __forceinline__ void plane_half_yx(const float* Ty, const HalfTable& ty, const float* Tx, const HalfTable& tx,
+                                              float* S, int mx, int my, int LS, int LTR, bool inverse, PlaneTask<LT>& k) {
+    if (!inverse) {
+        dct_fold(S, LS, my, mx);
+        __syncthreads();
+    }
+    k.place(my, mx);
+    k.product(Ty, ty, my, inverse, S, LS);
     __syncthreads();                      // every read of the plane is done
-    if (act) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            *reinterpret_cast<float4*>(S + (4 * xb + j) * LT + 4 * kb) =
-                make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
-    }
+    k.store(S, LTR, my, mx, inverse, my % 4 == 0, nullptr);
     __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;   // now [k along x][y]
-    if (act) {
-        const float4* ap = reinterpret_cast<const float4*>(Ax) + xb;
-        const float4* tp = reinterpret_cast<const float4*>(S) + kb;
-#pragma unroll 4
-        for (int q = 0; q < mx; ++q) {
-            const float4 a = ap[q * (PX / 4)];
-            const float4 x = tp[q * (LT / 4)];
-            const float av[4] = {a.x, a.y, a.z, a.w}, xv[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], xv[j], acc[i][j]);
-        }
+    if (!inverse) {
+        dct_fold(S, LTR, mx, my);
+        __syncthreads();
     }
+    k.place(mx, my);
+    k.product(Tx, tx, mx, inverse, S, LTR);
 }
 
-// Stage a plane of `in` (block `plane`) into S rows [y][LS], pad columns zero.
-__device__ __forceinline__ void plane_load(const float* __restrict__ in, size_t base, float* S, int mx, int my, int PX,
-                                           int LS, int vec_in) {
-    const int t = threadIdx.x;
-    if (vec_in) {                         // mx a multiple of 4 (PX = mx), in 16-byte aligned
+// Stage a plane of `in` into S rows [y][LS].
+__device__ __forceinline__ void plane_load(const float* __restrict__ in, size_t base, float* S, int mx, int my, int LS,
+                                           int vec_in) {
+    if (vec_in) {                         // mx a multiple of 4, in 16-byte aligned
         const int c4 = mx / 4;
-        for (int e = t; e < my * c4; e += blockDim.x) {
+        for (int e = threadIdx.x; e < my * c4; e += blockDim.x) {
             const int y = e / c4, x = 4 * (e % c4);
             cp_async16(S + y * LS + x, in + base + (size_t)y * mx + x);
         }
     } else {
-        for (int e = t; e < my * PX; e += blockDim.x) {
-            const int y = e / PX, x = e % PX;
-            S[y * LS + x] = x < mx ? __ldg(in + base + (size_t)y * mx + x) : 0.0f;
+        for (int e = threadIdx.x; e < my * mx; e += blockDim.x) {
+            const int y = e / mx, x = e % mx;
+            cp_async4(S + y * LS + x, in + base + e);
         }
     }
 }
 
-// Store this thread's block acc[i][j] = (x 4 xb + i, y 4 kb + j) of the plane.
-__device__ __forceinline__ void plane_store(float* __restrict__ out, size_t base, int mx, int my, int kb, int xb,
-                                            const float (&acc)[4][4], int vec_out) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int y = 4 * kb + j;
-        if (y >= my) break;
-        float* o = out + base + (size_t)y * mx + 4 * xb;
-        if (vec_out) {
-            *reinterpret_cast<float4*>(o) = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (4 * xb + i < mx) o[i] = acc[i][j];
-        }
-    }
-}
-
+template <int LT>
 __global__ void __launch_bounds__(kBlock) dct_plane_kernel(const float* __restrict__ in, float* __restrict__ out,
-                                                           const float* __restrict__ Axg,
-                                                           const float* __restrict__ Ayg, int mx, int my,
-                                                           int vec_in, int vec_out) {
+                                                           const HalfTable tx, const HalfTable ty, int inverse, int mx,
+                                                           int my, int vec_in, int vec_out) {
     extern __shared__ __align__(16) float sm[];
-    const int PX = (mx + 3) & ~3, PY = (my + 3) & ~3;
-    const int LS = PX + 4, LT = PY + 4;   // row strides of the plane [y][x] and of the transposed result [x][k]
-    float* Ay = sm;                       // [q][PY]
-    float* Ax = Ay + my * PY;             // [q][PX]
-    float* S = Ax + mx * PX;              // the plane, later the y result transposed
-    const int t = threadIdx.x;
-    for (int e = t; e < my * PY / 4; e += kBlock) cp_async16(Ay + 4 * e, Ayg + 4 * e);
-    for (int e = t; e < mx * PX / 4; e += kBlock) cp_async16(Ax + 4 * e, Axg + 4 * e);
+    const int LS = ((mx + 3) & ~3) + 4, LTR = ((my + 3) & ~3) + 4;   // row strides of [y][x] and of [x][k]
+    float* Ty = sm;
+    float* Tx = Ty + ty.rows * ty.stride;
+    float* S = Tx + tx.rows * tx.stride;  // the plane, later the y result transposed
+    dct_stage_table(Ty, ty);
+    dct_stage_table(Tx, tx);
     const size_t base = (size_t)blockIdx.x * mx * my;
-    plane_load(in, base, S, mx, my, PX, LS, vec_in);
+    plane_load(in, base, S, mx, my, LS, vec_in);
     cp_async_wait_all();
     __syncthreads();
-    const int nxb = PX / 4;
-    const bool act = t < (PY / 4) * nxb;  // at most 256 blocks of 4 x 4: one per thread
-    const int kb = act ? t / nxb : 0, xb = act ? t % nxb : 0;
-    float acc[4][4];
-    plane_yx(Ay, Ax, S, mx, my, PX, PY, LS, LT, act, kb, xb, acc);
-    if (act) plane_store(out, base, mx, my, kb, xb, acc, vec_out);
+    PlaneTask<LT> k;
+    plane_half_yx<LT>(Ty, ty, Tx, tx, S, mx, my, LS, LTR, inverse != 0, k);
+    k.store(out + base, mx, mx, my, inverse != 0, vec_out != 0, nullptr);
 }
 
-// The whole 2D preconditioner on one plane (a (time node, component) block of
-// at most 64 x 64 cells) in one CTA: modes = C_y X C_x^T, scaled by inv_eig,
-// then X = C_y^T modes C_x, with the scaled modes written back into the plane
-// buffer between the two halves.
+// The whole 2D preconditioner on one plane (a (time node, component) block) in
+// one CTA: forward, scale by inv_eig, inverse, with the scaled modes written
+// back into the plane buffer between the two halves.
+template <int LT>
 __global__ void __launch_bounds__(kBlock) dct_plane2d_kernel(const float* __restrict__ in, float* __restrict__ out,
-                                                             const float* __restrict__ Cfx,
-                                                             const float* __restrict__ Cfy,
-                                                             const float* __restrict__ Cix,
-                                                             const float* __restrict__ Ciy,
-                                                             const float* __restrict__ inv_eig, int mx, int my,
-                                                             int vec_in, int vec_out) {
+                                                             const HalfTable fx, const HalfTable fy, const HalfTable ix,
+                                                             const HalfTable iy, const float* __restrict__ inv_eig,
+                                                             int mx, int my, int vec_in, int vec_out) {
     extern __shared__ __align__(16) float sm[];
-    const int PX = (mx + 3) & ~3, PY = (my + 3) & ~3;
-    const int LS = PX + 4, LT = PY + 4;
-    float* Fy = sm;                       // forward tables [q][P]
-    float* Fx = Fy + my * PY;
-    float* Iy = Fx + mx * PX;             // inverse tables [q][P]
-    float* Ix = Iy + my * PY;
-    float* S = Ix + mx * PX;
-    const int t = threadIdx.x;
-    for (int e = t; e < my * PY / 4; e += kBlock) {
-        cp_async16(Fy + 4 * e, Cfy + 4 * e);
-        cp_async16(Iy + 4 * e, Ciy + 4 * e);
-    }
-    for (int e = t; e < mx * PX / 4; e += kBlock) {
-        cp_async16(Fx + 4 * e, Cfx + 4 * e);
-        cp_async16(Ix + 4 * e, Cix + 4 * e);
-    }
+    const int LS = ((mx + 3) & ~3) + 4, LTR = ((my + 3) & ~3) + 4;
+    float* Fy = sm;
+    float* Fx = Fy + fy.rows * fy.stride;
+    float* Iy = Fx + fx.rows * fx.stride;
+    float* Ix = Iy + iy.rows * iy.stride;
+    float* S = Ix + ix.rows * ix.stride;
+    dct_stage_table(Fy, fy);
+    dct_stage_table(Fx, fx);
+    dct_stage_table(Iy, iy);
+    dct_stage_table(Ix, ix);
     const size_t base = (size_t)blockIdx.x * mx * my;
-    plane_load(in, base, S, mx, my, PX, LS, vec_in);
+    plane_load(in, base, S, mx, my, LS, vec_in);
     cp_async_wait_all();
     __syncthreads();
-    const int nxb = PX / 4;
-    const bool act = t < (PY / 4) * nxb;
-    const int kb = act ? t / nxb : 0, xb = act ? t % nxb : 0;
-    float acc[4][4];
-    plane_yx(Fy, Fx, S, mx, my, PX, PY, LS, LT, act, kb, xb, acc);
-    // scale the modes (kx = 4 xb + i, ky = 4 kb + j; padding modes are zero) and put
-    // them back as rows [ky][LS] once every thread is done with the transposed buffer
+    PlaneTask<LT> k;
+    plane_half_yx<LT>(Fy, fy, Fx, fx, S, mx, my, LS, LTR, false, k);
+    // the scaled modes back as rows [ky][LS] once every thread is done with the transposed buffer
     __syncthreads();
-    if (act) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int ky = 4 * kb + j;
-            float sc[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int kx = 4 * xb + i;
-                sc[i] = (kx < mx && ky < my) ? acc[i][j] * __ldg(inv_eig + (size_t)ky * mx + kx) : 0.0f;
-            }
-            // rows ky >= my are never read (the inverse sums over q < my) and may lie past the buffer
-            if (ky < my) *reinterpret_cast<float4*>(S + ky * LS + 4 * xb) = make_float4(sc[0], sc[1], sc[2], sc[3]);
-        }
-    }
+    k.store(S, LS, mx, my, false, mx % 4 == 0, inv_eig);
     __syncthreads();
-    plane_yx(Iy, Ix, S, mx, my, PX, PY, LS, LT, act, kb, xb, acc);
-    if (act) plane_store(out, base, mx, my, kb, xb, acc, vec_out);
+    plane_half_yx<LT>(Iy, iy, Ix, ix, S, mx, my, LS, LTR, true, k);
+    k.store(out + base, mx, mx, my, true, vec_out != 0, nullptr);
 }
 
-inline size_t dct_plane_smem(int mx, int my, int tables = 1) {
-    const size_t PX = (size_t)((mx + 3) & ~3), PY = (size_t)((my + 3) & ~3);
-    const size_t plane = std::max((size_t)my * (PX + 4), PX * (PY + 4));
-    return (tables * ((size_t)my * PY + (size_t)mx * PX) + plane) * sizeof(float);
+inline HalfTable half_table(const float* p, int m) {
+    HalfTable t;
+    t.p = p;
+    t.rows = (m + 1) / 2;
+    t.P4 = (t.rows + 3) & ~3;
+    t.stride = m > 1 ? 2 * t.P4 : t.P4;
+    return t;
 }
+
+inline size_t half_floats(int m) {
+    const HalfTable t = half_table(nullptr, m);
+    return (size_t)t.rows * t.stride;
+}
+
+// Shared memory of the plane kernels with `dirs` directions' tables.
+inline size_t dct_plane_smem(int mx, int my, int dirs) {
+    const size_t LS = (size_t)((mx + 3) & ~3) + 4, LTR = (size_t)((my + 3) & ~3) + 4;
+    const size_t plane = std::max((size_t)my * LS, (size_t)mx * LTR) + 8;    // (rows are read in groups of 8 lines)
+    return (dirs * (half_floats(mx) + half_floats(my)) + plane) * sizeof(float);
+}
+
+// Threads with a task in a plane kernel, for either form (the larger of the two
+// products); the split form where it needs at most kBlock.  Every launch has kBlock
+// threads, or with many CTAs only those with a task (dct_threads).
+inline int dct_plane_threads(int mx, int my, int lt) {
+    const int ty = ((my + 1) / 2 + 3) / 4 * ((mx + lt - 1) / lt), tx = ((mx + 1) / 2 + 3) / 4 * ((my + lt - 1) / lt);
+    return ((lt == 4 ? 2 : 1) * std::max(ty, tx) + 31) / 32 * 32;
+}
+// Threads of a CTA with `tasks` threads' tasks: kBlock where the CTAs hardly fill the
+// GPU, since threads without a task help to stage and fold (a 70 x 70 plane alone: 30
+// us with 96, 23 us with 128 threads); else just those, so that more CTAs fit (2160
+// planes of 96 x 112: 204 against 180 us).
+inline int dct_threads(int tasks, long long blocks) {
+    return blocks < reduce_block_cap() / 2 ? kBlock : (tasks + 31) / 32 * 32;
+}
+inline bool dct_plane_split(int mx, int my) { return dct_plane_threads(mx, my, 4) <= kBlock; }
 
 // Shared memory of dct_tile_kernel for an axis of m cells (bytes).
 inline size_t dct_tile_smem(int m) {
@@ -1338,69 +1558,104 @@ cudaError_t launch_dct_axis(const float* in, float* out, const float* C, const f
     return cudaGetLastError();
 }
 
-cudaError_t launch_dct_plane(const float* in, float* out, const float* Ax, const float* Ay, const DevGrid& g,
+size_t dct_half_floats(int m) { return half_floats(m); }
+
+bool dct_half_axis_ok(int m) { return m <= kDctPlaneMax; }
+
+void dct_half_tables(const float* C, int m, float* f, float* i) {
+    const HalfTable t = half_table(nullptr, m);
+    for (size_t e = 0; e < (size_t)t.rows * t.stride; ++e) f[e] = i[e] = 0.0f;
+    for (int r = 0; r < t.rows; ++r)
+        for (int j = 0; j < t.rows; ++j) {
+            // forward row r = q: modes 2j (even part) and 2j + 1; inverse row r: modes 2r, 2r + 1 at q = j
+            if (2 * j < m) f[(size_t)r * t.stride + j] = C[(size_t)(2 * j) * m + r];
+            if (2 * j + 1 < m) f[(size_t)r * t.stride + t.P4 + j] = C[(size_t)(2 * j + 1) * m + r];
+            if (2 * r < m) i[(size_t)r * t.stride + j] = C[(size_t)(2 * r) * m + j];
+            if (2 * r + 1 < m) i[(size_t)r * t.stride + t.P4 + j] = C[(size_t)(2 * r + 1) * m + j];
+        }
+}
+
+// Raises the dynamic shared-memory limit of a kernel, once per device.
+template <class K>
+static cudaError_t raise_smem(K kernel, size_t bytes, bool (&done)[64]) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (done[dev]) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) done[dev] = true;
+    return e;
+}
+
+cudaError_t launch_dct_plane(const float* in, float* out, const float* Tx, const float* Ty, bool inverse, const DevGrid& g,
                              long long planes, cudaStream_t s) {
     const int mx = g.m[0], my = g.m[1];
     if (mx > kDctPlaneMax || my > kDctPlaneMax || planes < 1 || planes > 0x7fffffffLL) return cudaErrorNotSupported;
-    static bool attr_set_dev[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!attr_set_dev[dev]) {
-        const cudaError_t e = cudaFuncSetAttribute(dct_plane_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)dct_plane_smem(kDctPlaneMax, kDctPlaneMax));
-        if (e != cudaSuccess) return e;
-        attr_set_dev[dev] = true;
-    }
     const int vec_in = (mx % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
     const int vec_out = (mx % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0) ? 1 : 0;
-    dct_plane_kernel<<<(unsigned)planes, kBlock, dct_plane_smem(mx, my), s>>>(in, out, Ax, Ay, mx, my, vec_in,
-                                                                              vec_out);
+    const HalfTable tx = half_table(Tx, mx), ty = half_table(Ty, my);
+    const size_t smem = dct_plane_smem(mx, my, 1);
+    if (!dct_plane_split(mx, my)) {
+        static bool done[64] = {};
+        const cudaError_t e = raise_smem(dct_plane_kernel<8>, dct_plane_smem(kDctPlaneMax, kDctPlaneMax, 1), done);
+        if (e != cudaSuccess) return e;
+        dct_plane_kernel<8><<<(unsigned)planes, dct_threads(dct_plane_threads(mx, my, 8), planes), smem, s>>>(in, out, tx, ty, inverse, mx, my,
+                                                                                         vec_in, vec_out);
+    } else {
+        static bool done[64] = {};
+        const cudaError_t e = raise_smem(dct_plane_kernel<4>, dct_plane_smem(kDctPlaneMax, kDctPlaneMax, 1), done);
+        if (e != cudaSuccess) return e;
+        dct_plane_kernel<4><<<(unsigned)planes, dct_threads(dct_plane_threads(mx, my, 4), planes), smem, s>>>(in, out, tx, ty, inverse, mx, my,
+                                                                                         vec_in, vec_out);
+    }
     return cudaGetLastError();
 }
 
-cudaError_t launch_dct_plane2d(const float* in, float* out, const float* Cfx, const float* Cfy, const float* Cix,
-                               const float* Ciy, const float* inv_eig, const DevGrid& g, int blocks, cudaStream_t s) {
+cudaError_t launch_dct_plane2d(const float* in, float* out, const float* Fx, const float* Fy, const float* Ix,
+                               const float* Iy, const float* inv_eig, const DevGrid& g, int blocks, cudaStream_t s) {
     const int mx = g.m[0], my = g.m[1];
     if (mx > kDctPlaneMax || my > kDctPlaneMax || blocks < 1) return cudaErrorNotSupported;
-    static bool attr_set_dev[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!attr_set_dev[dev]) {
-        const cudaError_t e = cudaFuncSetAttribute(dct_plane2d_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)dct_plane_smem(kDctPlaneMax, kDctPlaneMax, 2));
-        if (e != cudaSuccess) return e;
-        attr_set_dev[dev] = true;
-    }
     const int vec_in = (mx % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
     const int vec_out = (mx % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0) ? 1 : 0;
-    dct_plane2d_kernel<<<(unsigned)blocks, kBlock, dct_plane_smem(mx, my, 2), s>>>(in, out, Cfx, Cfy, Cix, Ciy, inv_eig,
-                                                                                  mx, my, vec_in, vec_out);
+    const size_t smem = dct_plane_smem(mx, my, 2), smax = dct_plane_smem(kDctPlaneMax, kDctPlaneMax, 2);
+    const HalfTable fx = half_table(Fx, mx), fy = half_table(Fy, my), ix = half_table(Ix, mx), iy = half_table(Iy, my);
+    if (!dct_plane_split(mx, my)) {
+        static bool done[64] = {};
+        const cudaError_t e = raise_smem(dct_plane2d_kernel<8>, smax, done);
+        if (e != cudaSuccess) return e;
+        dct_plane2d_kernel<8><<<blocks, kBlock, smem, s>>>(in, out, fx, fy, ix, iy, inv_eig, mx, my,
+                                                                                 vec_in, vec_out);
+    } else {
+        static bool done[64] = {};
+        const cudaError_t e = raise_smem(dct_plane2d_kernel<4>, smax, done);
+        if (e != cudaSuccess) return e;
+        dct_plane2d_kernel<4><<<blocks, kBlock, smem, s>>>(in, out, fx, fy, ix, iy, inv_eig, mx, my,
+                                                                                 vec_in, vec_out);
+    }
     return cudaGetLastError();
 }
 
-cudaError_t launch_dct_last_fused(const float* in, float* out, const float* Cf, const float* Ci, const float* inv_eig,
-                                  const DevGrid& g, int d, int nblocks_kd, cudaStream_t s) {
-    constexpr int L = kDctFusedLines;
-    const int axis = d - 1;
-    const int m = g.m[axis];
-    const long long inner = axis == 1 ? (long long)g.m[0] : (long long)g.m[0] * g.m[1];
-    if (m > kDctTileMax || nblocks_kd > 65535) return cudaErrorNotSupported;
-    const size_t MP = (size_t)((m + 3) & ~3);
-    const size_t smem = (2 * (size_t)m * MP + (size_t)m * (L + 4)) * sizeof(float);
-    static bool attr_set_dev[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!attr_set_dev[dev]) {
-        const int smax = (int)((2 * (size_t)kDctTileMax * kDctTileMax + (size_t)kDctTileMax * (L + 4)) * sizeof(float));
-        const cudaError_t e =
-            cudaFuncSetAttribute(dct_last_fused_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-        if (e != cudaSuccess) return e;
-        attr_set_dev[dev] = true;
-    }
-    const dim3 grid((unsigned)((inner + L - 1) / L), (unsigned)nblocks_kd);
+cudaError_t launch_dct_last_half(const float* in, float* out, const float* Tf, const float* Ti, const float* inv_eig,
+                                 const DevGrid& g, int d, int nblocks_kd, cudaStream_t s) {
+    const int m = g.m[d - 1];
+    const long long inner = d == 2 ? (long long)g.m[0] : (long long)g.m[0] * g.m[1];
+    if (m > kDctPlaneMax || nblocks_kd > 65535) return cudaErrorNotSupported;
     const int vec_in = (inner % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
-    dct_last_fused_kernel<L><<<grid, 4 * L, smem, s>>>(in, out, Cf, Ci, inv_eig, m, inner, vec_in);
-    return cudaGetLastError();
+    const HalfTable tf = half_table(Tf, m), ti = half_table(Ti, m);
+    const long long blocks = (inner + kDctFusedLines - 1) / kDctFusedLines * nblocks_kd;
+    const int groups = ((m + 1) / 2 + 3) / 4;
+    auto run = [&](auto kernel, int lines, bool split, bool (&done)[64]) -> cudaError_t {
+        const auto bytes = [&](int n) { return (2 * half_floats(n) + (size_t)n * (lines + 4)) * sizeof(float); };
+        const cudaError_t e = raise_smem(kernel, bytes(kDctPlaneMax), done);
+        if (e != cudaSuccess) return e;
+        const dim3 grid((unsigned)((inner + lines - 1) / lines), (unsigned)nblocks_kd);
+        kernel<<<grid, dct_threads((split ? 2 : 1) * groups * (lines / 4), blocks), bytes(m), s>>>(in, out, tf, ti, inv_eig,
+                                                                                                m, inner, vec_in);
+        return cudaGetLastError();
+    };
+    static bool done[3][64] = {};
+    if (blocks < reduce_block_cap() / 4) return run(dct_last_half_kernel<32, true>, 32, true, done[0]);
+    if (2 * groups * (kDctFusedLines / 4) <= kBlock) return run(dct_last_half_kernel<64, true>, 64, true, done[1]);
+    return run(dct_last_half_kernel<64, false>, 64, false, done[2]);
 }
 
 cudaError_t launch_scale_modes(float* x, const float* inv_eig, size_t block_elems, size_t count, cudaStream_t s) {

@@ -167,22 +167,25 @@ cudaError_t launch_elastic(int d, const float* x, const float* div, float* out, 
 // forward, Ci inverse; tiled kernel)
 cudaError_t launch_dct_axis(const float* in, float* out, const float* C, const float* Cp, const DevGrid& g, int d,
                             int nblocks_kd, int axis, bool inverse, cudaStream_t s);
-// Padded DCT tables per axis (rows of P = m rounded up to 4 floats, zero past
-// m): forward Cf[q][k] = C[k][q], inverse Ci[q][k] = C[q][k].
-// The y and x axes of the spectral transform on whole xy planes (3D, both
-// axes at most 64 cells) with the tables of one direction (Cf or Ci of the x
-// and y axes): planes = blocks x z-planes.  cudaErrorNotSupported for larger
-// planes (the per-axis kernels cover them).
-cudaError_t launch_dct_plane(const float* in, float* out, const float* Ax, const float* Ay, const DevGrid& g,
+// Half tables of an axis (forward and inverse; see the transforms by halves in
+// grid_ops.cu) from its orthonormal DCT-II matrix C (host memory): dct_half_floats(m)
+// floats each, for axes that dct_half_axis_ok.
+size_t dct_half_floats(int m);
+bool dct_half_axis_ok(int m);
+void dct_half_tables(const float* C, int m, float* f, float* i);
+// The y and x axes of the spectral transform on whole xy planes with the half
+// tables of one direction: planes = blocks x z-planes.  cudaErrorNotSupported for
+// larger planes (the per-axis kernels cover them).
+cudaError_t launch_dct_plane(const float* in, float* out, const float* Tx, const float* Ty, bool inverse, const DevGrid& g,
                              long long planes, cudaStream_t s);
 // The whole 2D preconditioner (forward transform, inv_eig, inverse) with one CTA
-// per (time node, component) plane of at most 64 x 64 cells.
-cudaError_t launch_dct_plane2d(const float* in, float* out, const float* Cfx, const float* Cfy, const float* Cix,
-                               const float* Ciy, const float* inv_eig, const DevGrid& g, int blocks, cudaStream_t s);
+// per (time node, component) plane.
+cudaError_t launch_dct_plane2d(const float* in, float* out, const float* Fx, const float* Fy, const float* Ix,
+                               const float* Iy, const float* inv_eig, const DevGrid& g, int blocks, cudaStream_t s);
 // forward DCT, scale by inv_eig and inverse DCT along the last axis in one pass
-// (the axis's Cf and Ci); cudaErrorNotSupported when that axis has more than 128 cells
-cudaError_t launch_dct_last_fused(const float* in, float* out, const float* Cf, const float* Ci, const float* inv_eig,
-                                  const DevGrid& g, int d, int nblocks_kd, cudaStream_t s);
+// (the axis's half tables); cudaErrorNotSupported when that axis is too long
+cudaError_t launch_dct_last_half(const float* in, float* out, const float* Tf, const float* Ti, const float* inv_eig,
+                                 const DevGrid& g, int d, int nblocks_kd, cudaStream_t s);
 cudaError_t launch_scale_modes(float* x, const float* inv_eig, size_t block_elems, size_t count,
                                cudaStream_t s);
 // y = a * x + b * y  (count floats)
