@@ -54,7 +54,7 @@ struct PcgGraph {
 };
 
 // The whole PCG loop of one GN step as one graph: a while node whose body is
-// one iteration followed by launch_pcg_control, which ends the loop on the
+// one iteration whose last inner product ends with pcg_control, which ends the loop on the
 // stopping test, non-positive curvature or the iteration cap.  The host reads
 // the loop state once per GN step instead of once per iteration.
 struct PcgLoopGraph {
@@ -109,7 +109,7 @@ struct lgnk_ctx {
     double* hres = nullptr;       // pinned host mirror of dres
     float* fsc = nullptr;         // PCG step lengths on the device (alpha, -alpha, beta)
     unsigned* dcounter = nullptr; // completion counter of launch_dot_fused (zero between launches)
-    int* dctl = nullptr;          // device-side PCG loop state (launch_pcg_control)
+    int* dctl = nullptr;          // device-side PCG loop state (pcg_control)
     unsigned char* hpin = nullptr; // pinned: the loop state's host copy (4 ints) and its tolerance (a double)
     // lgnk_solve runs on a stream of its own (capturable, unlike the legacy
     // default stream), ordered after and before the caller's stream by events
@@ -1190,7 +1190,9 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
         // the device work of one iteration; ends with p.Hp and r.r in hres[2], hres[3]
         // with the diffusion regularizer, the end of the product, p.Hp and alpha are one kernel
         const bool fused_finish = ctx->prob.regularizer == LGNK_DIFFUSION;
-        auto body = [&](bool readback) -> lgnk_status {
+        // loop: the handle of the device-side loop the iteration is a body of (its control runs in
+        // the last inner product), 0 when the host makes the tests
+        auto body = [&](bool readback, cudaGraphConditionalHandle loop) -> lgnk_status {
             TRY(use_asm ? hessvec_assembled_accumulate(ctx, p) : hessvec_accumulate(ctx, T, p));
             if (fused_finish) {
                 KL(launch_hess_finish(ctx->d, ctx->Gp, p, Hp, ctx->vg, ctx->K, use_asm ? ctx->slices : ctx->grads, 1.0f,
@@ -1204,7 +1206,8 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
             KL(launch_pcg_update_xr(x, p, r, Hp, ctx->fsc, n, s));
             if (o.precond) TRY(precond_apply(ctx, r, z));
             else CK(cudaMemcpyAsync(z, r, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
-            KL(launch_dot_fused(r, r, z, n, ctx->partial, nb, ctx->dcounter, ctx->dres, 3, 4, 1, ctx->fsc, s));
+            KL(launch_dot_fused(r, r, z, n, ctx->partial, nb, ctx->dcounter, ctx->dres, 3, 4, 1, ctx->fsc, s,
+                                readback ? nullptr : ctx->dctl, loop));
             KL(launch_axpby_dev(1.0f, nullptr, z, 0.0f, ctx->fsc + 2, p, n, s));
             if (readback) CK(cudaMemcpyAsync(ctx->hres, ctx->dres, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
             return LGNK_OK;
@@ -1240,11 +1243,7 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
                 ok = cudaStreamBeginCaptureToGraph(s, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                                    cudaStreamCaptureModeThreadLocal) == cudaSuccess;
                 if (ok) {
-                    bool bok = body(false) == LGNK_OK;
-                    if (bok) {
-                        ctx->launches++;
-                        bok = launch_pcg_control(ctx->dres, ctx->dctl, handle, s) == cudaSuccess;
-                    }
+                    const bool bok = body(false, handle) == LGNK_OK;
                     cudaGraph_t captured = nullptr;
                     ok = (cudaStreamEndCapture(s, &captured) == cudaSuccess) && bok;
                 }
@@ -1285,7 +1284,7 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
                 cudaGraph_t graph = nullptr;
                 bool ok = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
                 if (ok) {
-                    ok = body(true) == LGNK_OK;
+                    ok = body(true, 0) == LGNK_OK;
                     ok = (cudaStreamEndCapture(s, &graph) == cudaSuccess) && ok && graph != nullptr;
                 }
                 if (ok) ok = cudaGraphInstantiate(&gr.exec, graph, 0) == cudaSuccess;
@@ -1307,7 +1306,7 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
                 ctx->launches += gr.launches;
                 ctx->trace_launches += gr.trace_launches;
             } else {
-                TRY(body(true));
+                TRY(body(true, 0));
             }
             CK(cudaStreamSynchronize(s));
             rep.hessvecs++;

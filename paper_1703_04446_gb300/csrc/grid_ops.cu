@@ -229,13 +229,37 @@ __device__ __forceinline__ void pcg_step_lengths(double* sc, float* f, int mode)
     }
 }
 
+// End of one PCG iteration inside a device-side loop (a CUDA-graph while
+// node): the same tests the host loop makes, on sc[2] = p.Hp, sc[3] = r.r and
+// the tolerance sc[6] = pcg_rtol |g|.  ctl: [0] iterations run, [1] accepted
+// iterations, [2] 1 = non-positive curvature, 2 = non-finite, [3] the cap.
+// The loop continues while the handle is non-zero; the cap ends it.  Part of
+// the iteration's last inner product (a kernel of its own took 2.3 us of a 2D
+// iteration of 45 us).
+__device__ __forceinline__ void pcg_control(const double* sc, int* ctl, cudaGraphConditionalHandle handle) {
+    const int it = ctl[0] + 1;
+    ctl[0] = it;
+    const double php = sc[2], rr = sc[3];
+    unsigned go = 0;
+    if (!isfinite(php) || !isfinite(rr)) {
+        ctl[2] = 2;
+    } else if (!(php > 0.0)) {
+        ctl[2] = 1;
+    } else {
+        ctl[1] = it;
+        go = (sqrt(rr) <= sc[6] || it >= ctl[3]) ? 0u : 1u;
+    }
+    cudaGraphSetConditional(handle, go);
+}
+
 // Second half of the fused inner products: block sums of the per-thread
 // accumulators s (a.b) and, when `two`, t (a.c); every block writes its
 // partials (FP64) and the last block to finish adds them in a fixed order
 // (FP64, deterministic) into sc[slot_b] (sc[slot_c]) and applies
 // pcg_step_lengths(mode).  Every thread of every block calls it.
 __device__ __forceinline__ void dot_blocks_finish(lsum s, lsum t, bool two, double* partial, unsigned* counter,
-                                                  double* sc, int slot_b, int slot_c, int mode, float* f) {
+                                                  double* sc, int slot_b, int slot_c, int mode, float* f,
+                                                  int* ctl = nullptr, cudaGraphConditionalHandle handle = 0) {
     s = lsum_block_sum(s);
     if (two) {
         __syncthreads();      // lsum_block_sum's shared slots are reused
@@ -268,19 +292,21 @@ __device__ __forceinline__ void dot_blocks_finish(lsum s, lsum t, bool two, doub
         if (two) sc[slot_c] = w;
         pcg_step_lengths(sc, f, mode);
         *counter = 0u;
+        if (ctl != nullptr) pcg_control(sc, ctl, handle);
     }
 }
 
 __global__ void dot_fused_kernel(const float* __restrict__ a, const float* __restrict__ b,
                                  const float* __restrict__ c, size_t count, double* partial, unsigned* counter,
-                                 double* sc, int slot_b, int slot_c, int mode, float* f) {
+                                 double* sc, int slot_b, int slot_c, int mode, float* f, int* ctl,
+                                 cudaGraphConditionalHandle handle) {
     lsum s = lsum_zero(), t = lsum_zero();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
         const float ai = a[i];
         lsum_add_prod(s, ai, b[i]);
         if (c != nullptr) lsum_add_prod(t, ai, c[i]);
     }
-    dot_blocks_finish(s, t, c != nullptr, partial, counter, sc, slot_b, slot_c, mode, f);
+    dot_blocks_finish(s, t, c != nullptr, partial, counter, sc, slot_b, slot_c, mode, f, ctl, handle);
 }
 
 // The end of a Gauss-Newton product inside PCG with the diffusion
@@ -353,28 +379,6 @@ __global__ void pcg_update_xr_kernel(float* x, const float* __restrict__ p, floa
     }
 }
 
-// End of one PCG iteration inside a device-side loop (a CUDA-graph while
-// node): the same tests the host loop makes, on sc[2] = p.Hp, sc[3] = r.r and
-// the tolerance sc[6] = pcg_rtol |g|.  ctl: [0] iterations run, [1] accepted
-// iterations, [2] 1 = non-positive curvature, 2 = non-finite, [3] the cap.
-// The loop continues while the handle is non-zero; the cap ends it.
-__global__ void pcg_control_kernel(const double* sc, int* ctl, cudaGraphConditionalHandle handle) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int it = ctl[0] + 1;
-    ctl[0] = it;
-    const double php = sc[2], rr = sc[3];
-    unsigned go = 0;
-    if (!isfinite(php) || !isfinite(rr)) {
-        ctl[2] = 2;
-    } else if (!(php > 0.0)) {
-        ctl[2] = 1;
-    } else {
-        ctl[1] = it;
-        go = (sqrt(rr) <= sc[6] || it >= ctl[3]) ? 0u : 1u;
-    }
-    cudaGraphSetConditional(handle, go);
-}
-
 // After the device-side PCG loop: when its first iteration met non-positive
 // curvature (ctl[2] = 1 with no accepted iteration), the step is the
 // preconditioned steepest-descent direction, x = z.
@@ -393,12 +397,30 @@ __global__ void axpby_dev_kernel(float a, const float* __restrict__ ap, const fl
         y[i] = fmaf(ea, x[i], eb * y[i]);
 }
 
-// Deterministic final sum of the per-block partials (one block).
-__global__ void reduce_kernel(const double* __restrict__ partial, int count, double* out) {
+// Deterministic final sum of the per-block partials, in one block: eight
+// loads of a thread in flight at a time (8192 partials of a 128^3 trace took 7 to
+// 16 us one by one in 256 threads).
+constexpr int kReduceBlock = 1024;
+__global__ void __launch_bounds__(kReduceBlock) reduce_kernel(const double* __restrict__ partial, int count, double* out) {
     double s = 0.0;
-    for (int i = threadIdx.x; i < count; i += blockDim.x) s += partial[i];
-    s = block_reduce(s);
-    if (threadIdx.x == 0) out[0] = s;
+    for (int i = threadIdx.x; i < count; i += 8 * kReduceBlock) {
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = i + k * kReduceBlock < count ? __ldg(partial + i + k * kReduceBlock) : 0.0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += v[k];
+    }
+    __shared__ double red[kReduceBlock / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        s = red[threadIdx.x];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) out[0] = s;
+    }
 }
 
 // ----------------------------------------------------------- regularizers --
@@ -1414,7 +1436,7 @@ cudaError_t launch_residual(const float* u1, const float* R, float* rp, const De
 }
 
 cudaError_t launch_reduce(const double* partial, int count, double* out, cudaStream_t s) {
-    reduce_kernel<<<1, kBlock, 0, s>>>(partial, count, out);
+    reduce_kernel<<<1, kReduceBlock, 0, s>>>(partial, count, out);
     return cudaGetLastError();
 }
 
@@ -1426,8 +1448,9 @@ int dot_blocks(size_t count) {
 
 cudaError_t launch_dot_fused(const float* a, const float* b, const float* c, size_t count, double* partial,
                              int nblocks, unsigned* counter, double* sc, int slot_b, int slot_c, int mode, float* f,
-                             cudaStream_t s) {
-    dot_fused_kernel<<<nblocks, kBlock, 0, s>>>(a, b, c, count, partial, counter, sc, slot_b, slot_c, mode, f);
+                             cudaStream_t s, int* ctl, cudaGraphConditionalHandle handle) {
+    dot_fused_kernel<<<nblocks, kBlock, 0, s>>>(a, b, c, count, partial, counter, sc, slot_b, slot_c, mode, f, ctl,
+                                                handle);
     return cudaGetLastError();
 }
 
@@ -1461,11 +1484,6 @@ cudaError_t launch_pcg_curvature_fix(float* x, const float* z, const int* ctl, s
     const int cap = reduce_block_cap();
     const int blocks = (int)(want < (size_t)cap ? (want > 0 ? want : 1) : (size_t)cap);
     pcg_curvature_fix_kernel<<<blocks, kBlock, 0, s>>>(x, z, ctl, count);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pcg_control(const double* sc, int* ctl, cudaGraphConditionalHandle handle, cudaStream_t s) {
-    pcg_control_kernel<<<1, 32, 0, s>>>(sc, ctl, handle);
     return cudaGetLastError();
 }
 

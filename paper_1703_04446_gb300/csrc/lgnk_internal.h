@@ -132,10 +132,11 @@ cudaError_t launch_dot(const float* a, const float* b, size_t count, double* par
                        cudaStream_t s);
 int dot_blocks(size_t count);
 // a.b (and a.c) reduced to sc[slot_b] (sc[slot_c]) in one launch, then the PCG
-// step `mode` (-1 none, 0 alpha, 1 beta); counter: a zeroed device word
+// step `mode` (-1 none, 0 alpha, 1 beta); counter: a zeroed device word; with ctl,
+// then the loop test of a device-side PCG loop (see pcg_control in grid_ops.cu)
 cudaError_t launch_dot_fused(const float* a, const float* b, const float* c, size_t count, double* partial,
                              int nblocks, unsigned* counter, double* sc, int slot_b, int slot_c, int mode, float* f,
-                             cudaStream_t s);
+                             cudaStream_t s, int* ctl = nullptr, cudaGraphConditionalHandle handle = 0);
 // Hp = gscale * distributed slice gradients + rscale * B^T B p + gamma * p (diffusion
 // regularizer), then p.Hp into sc[2] and alpha (fused inner-product step, mode 0)
 cudaError_t launch_hess_finish(int d, const void* Gp, const float* p, float* Hp, const DevGrid& g, int K,
@@ -144,8 +145,6 @@ cudaError_t launch_hess_finish(int d, const void* Gp, const float* p, float* Hp,
 // x += f[0] p, r += f[1] Hp
 cudaError_t launch_pcg_update_xr(float* x, const float* p, float* r, const float* Hp, const float* f, size_t count,
                                  cudaStream_t s);
-// PCG loop test at the end of an iteration of a device-side while loop (see grid_ops.cu)
-cudaError_t launch_pcg_control(const double* sc, int* ctl, cudaGraphConditionalHandle handle, cudaStream_t s);
 // x = z when the device-side PCG loop's first iteration met non-positive curvature (ctl as above)
 cudaError_t launch_pcg_curvature_fix(float* x, const float* z, const int* ctl, size_t count, cudaStream_t s);
 cudaError_t launch_axpby_dev(float a, const float* ap, const float* x, float b, const float* bp, float* y,
