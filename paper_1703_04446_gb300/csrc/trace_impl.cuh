@@ -135,16 +135,17 @@ template <int D> struct TileShape;
 template <> struct TileShape<2> { static constexpr int X = 16, Y = 16, Z = 1; };
 template <> struct TileShape<3> { static constexpr int X = 8, Y = 8, Z = 4; };
 
-// Voxel handled by this thread.
+// Voxel handled by this thread, of the tile that LGNK_BLOCK / threads CTAs share.
 template <int D>
-__device__ __forceinline__ void voxel_index(const TraceArgs& A, int* idx) {
+__device__ __forceinline__ void voxel_index(const TraceArgs& A, int threads, int* idx) {
     using TS = TileShape<D>;
-    int b = blockIdx.x;
+    const int per = LGNK_BLOCK / threads;
+    int b = blockIdx.x / per;
     const int bx = b % A.tiles[0];
     b /= A.tiles[0];
     const int by = b % A.tiles[1];
     const int bz = b / A.tiles[1];
-    const int t = threadIdx.x;
+    const int t = threadIdx.x + (blockIdx.x % per) * threads;
     idx[0] = bx * TS::X + t % TS::X;
     idx[1] = by * TS::Y + (t / TS::X) % TS::Y;
     idx[2] = bz * TS::Z + t / (TS::X * TS::Y);
@@ -1463,17 +1464,25 @@ static cudaError_t launch_ell_dim(int mode, const EllArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// CTAs per SM the register budget of a kernel is set for (256 threads).  The
-// 3D kernels hold a cell's coefficients and a pending block (24 registers each,
+// Threads of a CTA (a tile of voxels, whose partial sums are one, or half of one
+// where nothing is summed: 465 -> 454 us for the 128^3 product by rows, 6.29 -> 6.10
+// ms for the brain-scale J^T, from the shorter wait for a CTA's last warp) and CTAs
+// per SM the register budget is set for.  The 3D kernels hold a cell's coefficients and a pending block (24 registers each,
 // 48 for the two nodes of a time cell) and run at 128 registers; the forward
-// sweep holds the coefficients only and runs at 80.
+// sweep holds the coefficients only and runs at 80.  More CTAs at 96 registers
+// spill (the brain-scale J^T 8.2 ms); three of 128 threads at 168 are too few (7.0 ms).
 template <int D, int TM, int MODEL, int MODE>
 struct TraceOccupancy {
-    static constexpr int value = D == 3 ? (MODE == MODE_FWD ? 3 : 2) : (MODE == MODE_FWD ? 4 : 3);
+    static constexpr int threads =
+        MODE == MODE_JTVP || MODE == MODE_HESS || MODE == MODE_HROW ? LGNK_BLOCK / 2 : LGNK_BLOCK;
+    static constexpr int ctas = D == 3 ? (MODE == MODE_FWD ? 3 : 2) : (MODE == MODE_FWD ? 4 : 3);
+    static constexpr int value = ctas * (LGNK_BLOCK / threads);
 };
 
 template <int D, int TM, int MODEL, int MODE>
-__global__ void __launch_bounds__(LGNK_BLOCK, (TraceOccupancy<D, TM, MODEL, MODE>::value)) trace_kernel(const TraceArgs A) {
+__global__ void __launch_bounds__((TraceOccupancy<D, TM, MODEL, MODE>::threads), (TraceOccupancy<D, TM, MODEL, MODE>::value))
+    trace_kernel(const TraceArgs A) {
+    constexpr int THREADS = TraceOccupancy<D, TM, MODEL, MODE>::threads;
     constexpr bool TRANSPORT = MODEL == LGNK_TRANSPORT;
     constexpr int FORM = TRANSPORT ? POLY : CORNERS;
     constexpr bool ROWS = MODE == MODE_HROW;
@@ -1488,7 +1497,7 @@ __global__ void __launch_bounds__(LGNK_BLOCK, (TraceOccupancy<D, TM, MODEL, MODE
     int entries = 0;         // MODE_ASM: blocks of this thread's row
 
     int idx[3];
-    voxel_index<D>(A, idx);
+    voxel_index<D>(A, THREADS, idx);
     const bool active = idx[0] < A.ig.m[0] && idx[1] < A.ig.m[1] && (D == 2 || idx[2] < A.ig.m[2]);
     int sp[D];                // continuity FWD / JVP: the end cell, offsets, mass and dy of the splat
     float sf[D], sdy[D], smass = 0.0f;
@@ -1641,7 +1650,8 @@ static cudaError_t launch_one(const TraceArgs& a0, cudaStream_t s) {
     trace_tile_shape(D, ts);
     for (int i = 0; i < 3; ++i) a.tiles[i] = (a.ig.m[i] + ts[i] - 1) / ts[i];
     const int blocks = a.tiles[0] * a.tiles[1] * a.tiles[2];
-    trace_kernel<D, TM, MODEL, MODE><<<blocks, LGNK_BLOCK, 0, s>>>(a);
+    constexpr int threads = TraceOccupancy<D, TM, MODEL, MODE>::threads;
+    trace_kernel<D, TM, MODEL, MODE><<<blocks * (LGNK_BLOCK / threads), threads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
