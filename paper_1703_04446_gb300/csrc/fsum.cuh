@@ -28,6 +28,8 @@
 
 #include <cuda_runtime.h>
 
+#include "lgnk_internal.h"
+
 #ifndef LGNK_SUMS
 #define LGNK_SUMS 2
 #endif
@@ -145,20 +147,21 @@ __device__ __forceinline__ lsum lsum_warp_sum(lsum a) {
     return a;
 }
 
-// Sum over the block (at most 32 warps, blockDim.x a multiple of 32; every
-// thread calls it); the result is valid in thread 0.  Uses one shared array,
-// so two calls in a row need a __syncthreads() between them.
+// Sum over the block (at most LGNK_BLOCK threads, blockDim.x a multiple of 32;
+// every thread calls it); the result is valid in thread 0.  Warp 0 adds the
+// other warps' lanes column by column and then its own lanes: 12 FP64
+// additions of a warp for 256 threads, where a shuffle tree in every warp is
+// 45, and at 16 cycles each on this GPU's FP64 pipe these were most of a small
+// inner product's time (and 465 -> 456 us for the 128^3 assembly trace).  Uses one shared array a SLOT, so two calls of one slot
+// need a __syncthreads() between them.
+template <int SLOT = 0>
 __device__ __forceinline__ lsum lsum_block_sum(lsum a) {
-    __shared__ lsum red[32];
-    const int nw = (int)(blockDim.x >> 5);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    a = lsum_warp_sum(a);
-    if (lane == 0) red[warp] = a;
+    __shared__ lsum red[LGNK_BLOCK];
+    red[threadIdx.x] = a;
     __syncthreads();
-    lsum s = lsum_zero();
-    if (warp == 0) {
-        if (lane < nw) s = red[lane];
-        s = lsum_warp_sum(s);
+    if (threadIdx.x < 32) {
+        for (int i = threadIdx.x + 32; i < (int)blockDim.x; i += 32) lsum_add(a, red[i]);
+        a = lsum_warp_sum(a);
     }
-    return s;
+    return a;
 }

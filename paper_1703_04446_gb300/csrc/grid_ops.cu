@@ -210,62 +210,37 @@ __global__ void dot_kernel(const float* __restrict__ a, const float* __restrict_
 
 // One or two inner products sharing the first operand, finished in the same
 // launch: every block writes its partial sums (FP64, in the partial buffer's
-// slots), and the last block to finish (a counter, reset by
-// that block) adds the partials in a fixed order (deterministic) into
-// sc[slot_b] (a.b) and sc[slot_c] (a.c, when c is given), then the PCG step
-// lengths of step `mode` (-1: none), in FP64, from the inner products in sc
-// ([2] p.Hp, [3] r.r, [4] r.z new, [5] r.z current):
-//   mode 0: alpha = rz / pHp, or 0 when pHp is not positive; f[0] = alpha, f[1] = -alpha
-//   mode 1: beta = rz_new / rz, then rz = rz_new;             f[2] = beta
-__device__ __forceinline__ void pcg_step_lengths(double* sc, float* f, int mode) {
-    if (mode == 0) {
-        const double php = sc[2];
-        const double a = php > 0.0 ? sc[5] / php : 0.0;
-        f[0] = (float)a;
-        f[1] = (float)-a;
-    } else if (mode == 1) {
-        f[2] = (float)(sc[4] / sc[5]);
-        sc[5] = sc[4];
-    }
-}
-
+// slots), and the last block to finish (a counter, reset by that block) adds
+// the partials in a fixed order (deterministic) into sc[slot_b] (a.b) and
+// sc[slot_c] (a.c, when c is given), then the PCG step lengths of step `mode`,
+// in FP64, from the inner products in sc ([2] p.Hp, [3] r.r, [4] r.z new,
+// [5] r.z current):
+//   mode 0 (slot_b = 2): alpha = rz / pHp, or 0 when pHp is not positive; f[0] = alpha, f[1] = -alpha
+//   mode 1 (slot_c = 4): beta = rz_new / rz, then rz = rz_new;             f[2] = beta
+//
 // End of one PCG iteration inside a device-side loop (a CUDA-graph while
-// node): the same tests the host loop makes, on sc[2] = p.Hp, sc[3] = r.r and
-// the tolerance sc[6] = pcg_rtol |g|.  ctl: [0] iterations run, [1] accepted
-// iterations, [2] 1 = non-positive curvature, 2 = non-finite, [3] the cap.
-// The loop continues while the handle is non-zero; the cap ends it.  Part of
-// the iteration's last inner product (a kernel of its own took 2.3 us of a 2D
-// iteration of 45 us).
-__device__ __forceinline__ void pcg_control(const double* sc, int* ctl, cudaGraphConditionalHandle handle) {
-    const int it = ctl[0] + 1;
-    ctl[0] = it;
-    const double php = sc[2], rr = sc[3];
-    unsigned go = 0;
-    if (!isfinite(php) || !isfinite(rr)) {
-        ctl[2] = 2;
-    } else if (!(php > 0.0)) {
-        ctl[2] = 1;
-    } else {
-        ctl[1] = it;
-        go = (sqrt(rr) <= sc[6] || it >= ctl[3]) ? 0u : 1u;
-    }
-    cudaGraphSetConditional(handle, go);
-}
-
-// Second half of the fused inner products: block sums of the per-thread
-// accumulators s (a.b) and, when `two`, t (a.c); every block writes its
-// partials (FP64) and the last block to finish adds them in a fixed order
-// (FP64, deterministic) into sc[slot_b] (sc[slot_c]) and applies
-// pcg_step_lengths(mode).  Every thread of every block calls it.
+// node; ctl given, slot_b = 3): the same tests the host loop makes, on
+// sc[2] = p.Hp, sc[3] = r.r and the tolerance sc[6] = pcg_rtol |g|.  ctl: [0]
+// iterations run, [1] accepted iterations, [2] 1 = non-positive curvature,
+// 2 = non-finite, [3] the cap.  The loop continues while the handle is
+// non-zero; the cap ends it.  Part of the iteration's last inner product (a
+// kernel of its own took 2.3 us of a 2D iteration of 45 us).
+//
+// What bounds it is the FP64 rate of the sums and the chain of latencies after
+// the loads (block sum, fence, counter, partials, final sum, scalars, divide,
+// test), so the scalars are read while the partials are, a warp of its own
+// makes the loop test, and up to 32 partials are summed by one warp.  With the
+// block sums of fsum.cuh and half the blocks: r.r and r.z of 64 x 64 x 2 values
+// 7.4 -> 5.8 us, of 64^3 x 3 values 14.7 -> 11.3 us (192 blocks of 1024 threads,
+// whose FP64 additions of empty slots count too: 35 us).
 __device__ __forceinline__ void dot_blocks_finish(lsum s, lsum t, bool two, double* partial, unsigned* counter,
                                                   double* sc, int slot_b, int slot_c, int mode, float* f,
                                                   int* ctl = nullptr, cudaGraphConditionalHandle handle = 0) {
-    s = lsum_block_sum(s);
-    if (two) {
-        __syncthreads();      // lsum_block_sum's shared slots are reused
-        t = lsum_block_sum(t);
-    }
+    __shared__ double dred[2][32];
     __shared__ bool last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+    s = lsum_block_sum<0>(s);
+    if (two) t = lsum_block_sum<1>(t);
     if (threadIdx.x == 0) {
         partial[blockIdx.x] = lsum_value(s);
         if (two) partial[gridDim.x + blockIdx.x] = lsum_value(t);
@@ -275,36 +250,108 @@ __device__ __forceinline__ void dot_blocks_finish(lsum s, lsum t, bool two, doub
     __syncthreads();
     if (!last) return;
     __threadfence();
-    const volatile double* vp = partial;
-    double u = 0.0, w = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
-        u += vp[i];
-        if (two) w += vp[gridDim.x + i];
+    double u = 0.0, w = 0.0;              // the totals, in thread 0
+    double rz = 0.0, php = 0.0, tol = 0.0;
+    int it = 0, cap = 0;
+    if (threadIdx.x == 0 && mode >= 0) rz = sc[5];
+    if (threadIdx.x == 32 && ctl != nullptr) {
+        php = sc[2];
+        tol = sc[6];
+        it = ctl[0] + 1;
+        cap = ctl[3];
     }
-    __syncthreads();          // the first block sums' shared slots are reused
-    u = block_reduce(u);
-    if (two) {
+    const volatile double* vp = partial;
+    const int n = (int)gridDim.x;
+    if (n <= 32) {
+        if (lane < n && warp == 0) {
+            u = vp[lane];
+            if (two) w = vp[n + lane];
+        }
+    } else {
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            u += vp[i];
+            if (two) w += vp[n + i];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            u += __shfl_down_sync(0xffffffffu, u, o);
+            if (two) w += __shfl_down_sync(0xffffffffu, w, o);
+        }
+        if (lane == 0) {
+            dred[0][warp] = u;
+            dred[1][warp] = w;
+        }
         __syncthreads();
-        w = block_reduce(w);
+        u = lane < nw ? dred[0][lane] : 0.0;
+        w = lane < nw ? dred[1][lane] : 0.0;
+    }
+    if (warp == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            u += __shfl_down_sync(0xffffffffu, u, o);
+            if (two) w += __shfl_down_sync(0xffffffffu, w, o);
+        }
+    }
+    if (ctl != nullptr) {                 // r.r to the thread of the loop test
+        __syncthreads();
+        if (threadIdx.x == 0) dred[0][0] = u;
+        __syncthreads();
     }
     if (threadIdx.x == 0) {
         sc[slot_b] = u;
         if (two) sc[slot_c] = w;
-        pcg_step_lengths(sc, f, mode);
+        if (mode == 0) {
+            const double a = u > 0.0 ? rz / u : 0.0;
+            f[0] = (float)a;
+            f[1] = (float)-a;
+        } else if (mode == 1) {
+            f[2] = (float)(w / rz);
+            sc[5] = w;
+        }
         *counter = 0u;
-        if (ctl != nullptr) pcg_control(sc, ctl, handle);
+    }
+    if (threadIdx.x == 32 && ctl != nullptr) {
+        const double rr = dred[0][0];
+        ctl[0] = it;
+        unsigned go = 0;
+        if (!isfinite(php) || !isfinite(rr)) {
+            ctl[2] = 2;
+        } else if (!(php > 0.0)) {
+            ctl[2] = 1;
+        } else {
+            ctl[1] = it;
+            go = (sqrt(rr) <= tol || it >= cap) ? 0u : 1u;
+        }
+        cudaGraphSetConditional(handle, go);
     }
 }
+
+// kDotElems elements of a thread are loaded before the first is added.
+constexpr int kDotElems = 4;
 
 __global__ void dot_fused_kernel(const float* __restrict__ a, const float* __restrict__ b,
                                  const float* __restrict__ c, size_t count, double* partial, unsigned* counter,
                                  double* sc, int slot_b, int slot_c, int mode, float* f, int* ctl,
                                  cudaGraphConditionalHandle handle) {
     lsum s = lsum_zero(), t = lsum_zero();
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
-        const float ai = a[i];
-        lsum_add_prod(s, ai, b[i]);
-        if (c != nullptr) lsum_add_prod(t, ai, c[i]);
+    const size_t step = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += kDotElems * step) {
+        float x[kDotElems], y[kDotElems], z[kDotElems];
+#pragma unroll
+        for (int k = 0; k < kDotElems; ++k) {
+            const size_t e = i + k * step;
+            const bool in = e < count;
+            x[k] = in ? a[e] : 0.0f;
+            y[k] = in ? b[e] : 0.0f;
+            z[k] = in && c != nullptr ? c[e] : 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < kDotElems; ++k) {
+            if (i + k * step < count) {
+                lsum_add_prod(s, x[k], y[k]);
+                if (c != nullptr) lsum_add_prod(t, x[k], z[k]);
+            }
+        }
     }
     dot_blocks_finish(s, t, c != nullptr, partial, counter, sc, slot_b, slot_c, mode, f, ctl, handle);
 }
@@ -1449,8 +1496,10 @@ int dot_blocks(size_t count) {
 cudaError_t launch_dot_fused(const float* a, const float* b, const float* c, size_t count, double* partial,
                              int nblocks, unsigned* counter, double* sc, int slot_b, int slot_c, int mode, float* f,
                              cudaStream_t s, int* ctl, cudaGraphConditionalHandle handle) {
-    dot_fused_kernel<<<nblocks, kBlock, 0, s>>>(a, b, c, count, partial, counter, sc, slot_b, slot_c, mode, f, ctl,
-                                                handle);
+    // two blocks an SM at most: 11.3 us for 64^3 x 3 values, 12.9 with one, 11.6 with four
+    const int blocks = nblocks < reduce_block_cap() / 2 ? nblocks : reduce_block_cap() / 2;
+    dot_fused_kernel<<<blocks, kBlock, 0, s>>>(a, b, c, count, partial, counter, sc, slot_b, slot_c, mode, f, ctl,
+                                                  handle);
     return cudaGetLastError();
 }
 

@@ -1464,13 +1464,14 @@ static cudaError_t launch_ell_dim(int mode, const EllArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Threads of a CTA (a tile of voxels, whose partial sums are one, or half of one
-// where nothing is summed: 465 -> 454 us for the 128^3 product by rows, 6.29 -> 6.10
-// ms for the brain-scale J^T, from the shorter wait for a CTA's last warp) and CTAs
-// per SM the register budget is set for.  The 3D kernels hold a cell's coefficients and a pending block (24 registers each,
-// 48 for the two nodes of a time cell) and run at 128 registers; the forward
-// sweep holds the coefficients only and runs at 80.  More CTAs at 96 registers
-// spill (the brain-scale J^T 8.2 ms); three of 128 threads at 168 are too few (7.0 ms).
+// Threads of a CTA and CTAs per SM that the register budget is set for.  A CTA
+// covers a tile of voxels where it writes the tile's partial sums and half a
+// tile where nothing is summed: 465 -> 454 us for the 128^3 product by rows, 6.29
+// -> 6.10 ms for the brain-scale J^T, from the shorter wait for a CTA's last
+// warp.  The 3D kernels hold a cell's coefficients and a pending block (24
+// registers each, 48 for the two nodes of a time cell) and run at 128
+// registers: at 96 they spill (the brain-scale J^T 8.2 ms), at 168 too few warps
+// run (7.0 ms).  The forward sweep holds the coefficients only and runs at 80.
 template <int D, int TM, int MODEL, int MODE>
 struct TraceOccupancy {
     static constexpr int threads =
@@ -1634,11 +1635,16 @@ __global__ void __launch_bounds__((TraceOccupancy<D, TM, MODEL, MODE>::threads),
     }
     if constexpr (MODE == MODE_ASM) {
         if (A.cpartial != nullptr) {
-            __syncthreads();      // lsum_block_sum's shared slots are reused
-            lsum c = lsum_zero();
-            lsum_add(c, (float)entries);
-            c = lsum_block_sum(c);   // exact: at most 256 x 16 blocks
-            if (threadIdx.x == 0) A.cpartial[blockIdx.x] = lsum_value(c);
+            __shared__ int rowsum[THREADS / 32];
+            const int w = __reduce_add_sync(0xffffffffu, entries);
+            if ((threadIdx.x & 31) == 0) rowsum[threadIdx.x >> 5] = w;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                int c = 0;
+#pragma unroll
+                for (int i = 0; i < THREADS / 32; ++i) c += rowsum[i];
+                A.cpartial[blockIdx.x] = (double)c;
+            }
         }
     }
 }
