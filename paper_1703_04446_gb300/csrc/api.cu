@@ -327,14 +327,40 @@ lgnk_status trace(lgnk_ctx* ctx, int mode, const TraceArgs& a) {
     return LGNK_OK;
 }
 
-lgnk_status pack_v(lgnk_ctx* ctx, const float* v, void* dst) {
-    KL(launch_pack_velocity(ctx->d, v, dst, ctx->vg, ctx->K, ctx->slices, ctx->stream));
+// The layouts of a call in one launch (each null or false: left out): v into
+// Vp, dv into dVp, an image into Tp (or imagep), gradients (as many slices as
+// *gz has) and the push-forward's sums to zero.
+lgnk_status pack(lgnk_ctx* ctx, const float* v, const float* dv, const float* image, const SliceTable* gz, bool acc,
+                 float* imagep = nullptr) {
+    PackArgs a{};
+    a.vg = ctx->vg;
+    a.ig = ctx->ig;
+    a.tab = ctx->slices;
+    int k = 0;
+    if (v != nullptr) {
+        a.v[k] = v;
+        a.vp[k++] = static_cast<float*>(ctx->Vp);
+    }
+    if (dv != nullptr) {
+        a.v[k] = dv;
+        a.vp[k] = static_cast<float*>(ctx->dVp);
+    }
+    if (gz != nullptr) {
+        a.Gz = ctx->Gp;
+        a.nz = gz->n;
+    }
+    a.image = image;
+    a.imagep = imagep != nullptr ? imagep : ctx->Tp;
+    if (acc) a.zero = ctx->acc;
+    KL(launch_pack(ctx->d, a, ctx->stream));
     return LGNK_OK;
 }
 
-lgnk_status pack_T(lgnk_ctx* ctx, const float* T) {
-    KL(launch_pack_image(T, ctx->Tp, ctx->ig, ctx->d, 1.0f, ctx->stream));
-    return LGNK_OK;
+lgnk_status pack_v(lgnk_ctx* ctx, const float* v) { return pack(ctx, v, nullptr, nullptr, nullptr, false); }
+
+// v and, for the transport model, the template.
+lgnk_status pack_vT(lgnk_ctx* ctx, const float* v, const float* T) {
+    return pack(ctx, v, nullptr, ctx->prob.model == LGNK_TRANSPORT ? T : nullptr, nullptr, false);
 }
 
 lgnk_status zero_G(lgnk_ctx* ctx, const SliceTable& tab) {
@@ -399,14 +425,14 @@ lgnk_status dot_host(lgnk_ctx* ctx, const float* a, const float* b, size_t count
 
 // ---- internal operations: velocity already packed in Vp (and template in Tp) ----
 
-lgnk_status forward_packed(lgnk_ctx* ctx, const float* T, float* u1, float* y) {
+lgnk_status forward_packed(lgnk_ctx* ctx, const float* T, float* u1, float* y, bool zeroed) {
     TraceArgs a = base_args(ctx);
     a.yout = y;
     if (ctx->prob.model == LGNK_TRANSPORT) {
         a.u1 = u1;
         return trace(ctx, MODE_FWD, a);
     }
-    TRY(zero_acc(ctx));
+    if (!zeroed) TRY(zero_acc(ctx));
     a.T = T;
     a.acc = ctx->acc;
     TRY(trace(ctx, MODE_FWD, a));
@@ -418,21 +444,22 @@ lgnk_status forward_packed(lgnk_ctx* ctx, const float* T, float* u1, float* y) {
 // objective_packed in two halves: the device work with the copy of its sums
 // to hres[0..1] (no wait), and, once the stream has been synchronized, the
 // objective from them.
-lgnk_status objective_enqueue(lgnk_ctx* ctx, const float* v, const float* T, const float* R, float* grad) {
+lgnk_status objective_enqueue(lgnk_ctx* ctx, const float* v, const float* T, const float* R, float* grad,
+                              bool zeroed = false) {
     TraceArgs a = base_args(ctx);
     a.R = R;
     a.partial = ctx->partial;
     int nred = trace_blocks_for(ctx, grad != nullptr ? MODE_OBJGRAD : MODE_FWD);
     if (ctx->prob.model == LGNK_TRANSPORT) {
         if (grad != nullptr) {
-            TRY(zero_G(ctx, ctx->grads));
+            if (!zeroed) TRY(zero_G(ctx, ctx->grads));
             TRY(trace(ctx, MODE_OBJGRAD, a));
         } else {
             a.u1 = ctx->itmp;
             TRY(trace(ctx, MODE_FWD, a));
         }
     } else {
-        TRY(zero_acc(ctx));
+        if (!zeroed) TRY(zero_acc(ctx));
         TraceArgs f = base_args(ctx);
         f.T = T;
         f.acc = ctx->acc;
@@ -442,7 +469,7 @@ lgnk_status objective_enqueue(lgnk_ctx* ctx, const float* v, const float* T, con
         KL(launch_residual(ctx->itmp, R, ctx->rp, ctx->ig, ctx->d, (float)ctx->cellvol, ctx->partial, nred,
                            ctx->stream));
         if (grad != nullptr) {
-            TRY(zero_G(ctx, ctx->grads));
+            if (!zeroed) TRY(zero_G(ctx, ctx->grads));
             TraceArgs b = base_args(ctx);
             b.T = T;
             b.r = ctx->rp;
@@ -476,23 +503,23 @@ lgnk_status objective_collect(lgnk_ctx* ctx, double* J, double* D, double* S) {
 
 // J, D, S (and with grad the gradient, Eq. 9) at the packed velocity.
 lgnk_status objective_packed(lgnk_ctx* ctx, const float* v, const float* T, const float* R, float* grad,
-                             double* J, double* D, double* S) {
-    TRY(objective_enqueue(ctx, v, T, R, grad));
+                             double* J, double* D, double* S, bool zeroed = false) {
+    TRY(objective_enqueue(ctx, v, T, R, grad, zeroed));
     CK(cudaStreamSynchronize(ctx->stream));
     return objective_collect(ctx, J, D, S);
 }
 
 // out = J^T h^d J dv + alpha dt h_v^d A dv + gamma dv at the packed velocity.
 // The data term of the Gauss-Newton product into the slice gradients Gp
-// (the first half of hessvec_packed).
-lgnk_status hessvec_accumulate(lgnk_ctx* ctx, const float* T, const float* dv) {
-    // packs the direction and zeroes the gradients in one pass
-    KL(launch_pack_velocity(ctx->d, dv, ctx->dVp, ctx->vg, ctx->K, ctx->slices, ctx->stream, ctx->Gp, ctx->grads.n));
-    if (ctx->prob.model == LGNK_TRANSPORT) {
+// (hessvec_finish is the second half).
+// With v (and the template, for the transport model) they are packed too.
+lgnk_status hessvec_accumulate(lgnk_ctx* ctx, const float* T, const float* dv, const float* v = nullptr) {
+    const bool transport = ctx->prob.model == LGNK_TRANSPORT;
+    TRY(pack(ctx, v, dv, v != nullptr && transport ? T : nullptr, &ctx->grads, !transport));
+    if (transport) {
         TraceArgs a = base_args(ctx);
         TRY(trace(ctx, ctx->gn_rows ? MODE_HROW : MODE_HESS, a));
     } else {
-        TRY(zero_acc(ctx));
         TraceArgs a = base_args(ctx);
         a.T = T;
         a.acc = ctx->acc;
@@ -517,11 +544,6 @@ lgnk_status hessvec_finish(lgnk_ctx* ctx, const SliceTable& tab, const float* dv
     }
     KL(launch_distribute_gradient(ctx->d, ctx->Gp, out, ctx->vg, ctx->K, tab, 1.0f, ctx->stream));
     return reg_apply(ctx, dv, out, ctx->prob.alpha * ctx->wreg, ctx->prob.gamma, out);
-}
-
-lgnk_status hessvec_packed(lgnk_ctx* ctx, const float* T, const float* dv, float* out) {
-    TRY(hessvec_accumulate(ctx, T, dv));
-    return hessvec_finish(ctx, ctx->grads, dv, out);
 }
 
 EllArgs ell_args(const lgnk_ctx* ctx) {
@@ -632,8 +654,7 @@ lgnk_status assemble_packed(lgnk_ctx* ctx, const float* v = nullptr, const float
 }
 
 lgnk_status hessvec_assembled_accumulate(lgnk_ctx* ctx, const float* dv) {
-    KL(launch_pack_velocity(ctx->d, dv, ctx->dVp, ctx->vg, ctx->K, ctx->slices, ctx->stream, ctx->Gp,
-                            ctx->slices.n));
+    TRY(pack(ctx, nullptr, dv, nullptr, &ctx->slices, false));
     return ell(ctx, ELL_HESS, ell_args(ctx));
 }
 
@@ -944,24 +965,22 @@ lgnk_status lgnk_forward(lgnk_ctx* ctx, const float* v, const float* T, float* u
     CHECK_CTX();
     REQUIRE(v && T && u1, "v, T and u1 must be non-NULL");
     REQUIRE(distinct(u1, {v, T}) && distinct(y, {v, T, u1}), "outputs must not alias inputs");
-    TRY(pack_v(ctx, v, ctx->Vp));
-    if (ctx->prob.model == LGNK_TRANSPORT) TRY(pack_T(ctx, T));
-    return forward_packed(ctx, T, u1, y);
+    const bool transport = ctx->prob.model == LGNK_TRANSPORT;
+    TRY(pack(ctx, v, nullptr, transport ? T : nullptr, nullptr, !transport));
+    return forward_packed(ctx, T, u1, y, true);
 }
 
 lgnk_status lgnk_jvp(lgnk_ctx* ctx, const float* v, const float* T, const float* dv, float* du) {
     CHECK_CTX();
     REQUIRE(v && T && dv && du, "v, T, dv and du must be non-NULL");
     REQUIRE(distinct(du, {v, T, dv}), "outputs must not alias inputs");
-    TRY(pack_v(ctx, v, ctx->Vp));
-    TRY(pack_v(ctx, dv, ctx->dVp));
+    const bool transport = ctx->prob.model == LGNK_TRANSPORT;
+    TRY(pack(ctx, v, dv, transport ? T : nullptr, nullptr, !transport));
     TraceArgs a = base_args(ctx);
-    if (ctx->prob.model == LGNK_TRANSPORT) {
-        TRY(pack_T(ctx, T));
+    if (transport) {
         a.u1 = du;
         return trace(ctx, MODE_JVP, a);
     }
-    TRY(zero_acc(ctx));
     a.T = T;
     a.acc = ctx->acc;
     TRY(trace(ctx, MODE_JVP, a));
@@ -973,14 +992,12 @@ lgnk_status lgnk_jtvp(lgnk_ctx* ctx, const float* v, const float* T, const float
     CHECK_CTX();
     REQUIRE(v && T && r && gv, "v, T, r and gv must be non-NULL");
     REQUIRE(distinct(gv, {v, T, r}), "outputs must not alias inputs");
-    TRY(pack_v(ctx, v, ctx->Vp));
-    TRY(zero_G(ctx, ctx->grads));
     TraceArgs a = base_args(ctx);
     if (ctx->prob.model == LGNK_TRANSPORT) {
-        TRY(pack_T(ctx, T));
+        TRY(pack(ctx, v, nullptr, T, &ctx->grads, false));
         a.r = r;
     } else {
-        KL(launch_pack_image(r, ctx->rp, ctx->ig, ctx->d, 1.0f, ctx->stream));
+        TRY(pack(ctx, v, nullptr, r, &ctx->grads, false, ctx->rp));
         a.T = T;
         a.r = ctx->rp;
     }
@@ -994,18 +1011,17 @@ lgnk_status lgnk_objective(lgnk_ctx* ctx, const float* v, const float* T, const 
     CHECK_CTX();
     REQUIRE(v && T && R, "v, T and R must be non-NULL");
     REQUIRE(distinct(grad, {v, T, R}), "outputs must not alias inputs");
-    TRY(pack_v(ctx, v, ctx->Vp));
-    if (ctx->prob.model == LGNK_TRANSPORT) TRY(pack_T(ctx, T));
-    return objective_packed(ctx, v, T, R, grad, J, D, S);
+    const bool transport = ctx->prob.model == LGNK_TRANSPORT;
+    TRY(pack(ctx, v, nullptr, transport ? T : nullptr, grad != nullptr ? &ctx->grads : nullptr, !transport));
+    return objective_packed(ctx, v, T, R, grad, J, D, S, true);
 }
 
 lgnk_status lgnk_hessvec(lgnk_ctx* ctx, const float* v, const float* T, const float* dv, float* Hdv) {
     CHECK_CTX();
     REQUIRE(v && T && dv && Hdv, "v, T, dv and Hdv must be non-NULL");
     REQUIRE(distinct(Hdv, {v, T, dv}), "outputs must not alias inputs");
-    TRY(pack_v(ctx, v, ctx->Vp));
-    if (ctx->prob.model == LGNK_TRANSPORT) TRY(pack_T(ctx, T));
-    return hessvec_packed(ctx, T, dv, Hdv);
+    TRY(hessvec_accumulate(ctx, T, dv, v));
+    return hessvec_finish(ctx, ctx->grads, dv, Hdv);
 }
 
 lgnk_status lgnk_assemble(lgnk_ctx* ctx, const float* v, const float* T, size_t* blocks) {
@@ -1013,8 +1029,7 @@ lgnk_status lgnk_assemble(lgnk_ctx* ctx, const float* v, const float* T, size_t*
     ctx->asm_valid = false;
     REQUIRE(v && T, "v and T must be non-NULL");
     REQUIRE(ctx->prob.model == LGNK_TRANSPORT, "J is assembled for the transport model only");
-    TRY(pack_v(ctx, v, ctx->Vp));
-    TRY(pack_T(ctx, T));
+    TRY(pack_vT(ctx, v, T));
     TRY(assemble_packed(ctx));
     if (blocks) *blocks = ctx->asm_entries;
     return LGNK_OK;
@@ -1024,7 +1039,7 @@ lgnk_status lgnk_jvp_assembled(lgnk_ctx* ctx, const float* dv, float* du) {
     CHECK_CTX();
     REQUIRE(dv && du && (const void*)dv != (const void*)du, "dv and du must be non-NULL and distinct");
     REQUIRE(ctx->asm_valid, "no assembled J on this context (call lgnk_assemble)");
-    TRY(pack_v(ctx, dv, ctx->dVp));
+    TRY(pack(ctx, nullptr, dv, nullptr, nullptr, false));
     EllArgs e = ell_args(ctx);
     e.out = du;
     return ell(ctx, ELL_JVP, e);
@@ -1055,9 +1070,8 @@ lgnk_status lgnk_jacobian_determinant(lgnk_ctx* ctx, const float* v, const float
     REQUIRE(v && T, "v and T must be non-NULL");
     REQUIRE(distinct(det, {v, T}), "det must not alias the inputs");
     if (ctx->ybuf == nullptr) TRY(dalloc(ctx, ctx->M * ctx->d, &ctx->ybuf));
-    TRY(pack_v(ctx, v, ctx->Vp));
-    if (ctx->prob.model == LGNK_TRANSPORT) TRY(pack_T(ctx, T));
-    TRY(forward_packed(ctx, T, ctx->itmp, ctx->ybuf));
+    TRY(pack_vT(ctx, v, T));
+    TRY(forward_packed(ctx, T, ctx->itmp, ctx->ybuf, false));
     KL(launch_jacobian_det(ctx->d, ctx->ybuf, det, ctx->ig, ctx->partial, ctx->dres + 4, ctx->stream));
     CK(cudaMemcpyAsync(ctx->hres + 4, ctx->dres + 4, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
@@ -1135,8 +1149,7 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
     lgnk_solve_report rep;
     memset(&rep, 0, sizeof(rep));
 
-    if (ctx->prob.model == LGNK_TRANSPORT) TRY(pack_T(ctx, T));
-    TRY(pack_v(ctx, v, ctx->Vp));
+    TRY(pack_vT(ctx, v, T));
     double J, D, S;
     // With the assembled J (transport), one trace per accepted iterate yields
     // the objective, the rows of J and, through them, the gradient; the PCG
@@ -1332,7 +1345,7 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
         // evaluated at the accepted point.
         TRY(dot_dev(ctx, g, x, n, 8));
         KL(launch_add_scaled(vt, v, 1.0f, x, 1.0f, n, s));
-        TRY(pack_v(ctx, vt, ctx->Vp));
+        TRY(pack_v(ctx, vt));
         bool spec_asm = false;
         if (!asm_off) {
             const lgnk_status es = assemble_enqueue(ctx, vt, R, g);
@@ -1378,14 +1391,14 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
         for (int ls = 1; !accepted && ls < o.max_ls; ++ls) {
             mu *= 0.5;
             KL(launch_add_scaled(vt, v, 1.0f, x, (float)mu, n, s));
-            TRY(pack_v(ctx, vt, ctx->Vp));
+            TRY(pack_v(ctx, vt));
             TRY(objective_packed(ctx, vt, T, R, nullptr, &Jt, nullptr, nullptr));
             rep.objective_evals++;
             accepted = Jt <= J + o.armijo_c * mu * slope;
         }
         rep.gn_iters = it + 1;
         if (!accepted) {
-            TRY(pack_v(ctx, v, ctx->Vp));
+            TRY(pack_v(ctx, v));
             ctx->asm_valid = false;     // rows (if any) of the rejected full step
             status = LGNK_LS_FAILED;
             break;

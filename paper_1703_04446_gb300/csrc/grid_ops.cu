@@ -44,14 +44,14 @@ __device__ __forceinline__ void split_xyz(unsigned i, unsigned nx, unsigned ny, 
 // the gradients, which share the [slice][padded node] index, are zeroed in the
 // same pass.
 template <int D>
-__global__ void pack_velocity_kernel(const float* __restrict__ v, float* __restrict__ Vp, DevGrid g, SliceTable tab,
-                                     void* Gz, int nz) {
+__device__ __forceinline__ void pack_velocity(const float* __restrict__ v, float* __restrict__ Vp, const DevGrid& g,
+                                              const SliceTable& tab, void* Gz, int nz, unsigned block, unsigned blocks) {
     const size_t nodes = padded_size(g);
     const size_t total = nodes * tab.n;
     const size_t zero = Gz != nullptr ? nodes * nz : 0;
     const size_t Mv = (size_t)g.m[0] * g.m[1] * g.m[2];
     constexpr int PS = (D == 3) ? 8 : 4;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+    for (size_t i = block * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)blocks * blockDim.x) {
         if (i < zero) {
             if (D == 3) reinterpret_cast<float4*>(Gz)[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             else reinterpret_cast<float2*>(Gz)[i] = make_float2(0.0f, 0.0f);
@@ -130,15 +130,44 @@ __global__ void distribute_gradient_kernel(const float* __restrict__ Gp, float* 
     }
 }
 
-__global__ void pack_image_kernel(const float* __restrict__ T, float* __restrict__ Tp, DevGrid g, int d, float scale) {
+__device__ __forceinline__ void pack_image(const float* __restrict__ T, float* __restrict__ Tp, const DevGrid& g, int d,
+                                           unsigned block, unsigned blocks) {
     const size_t total = padded_size(g);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+    for (size_t i = block * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)blocks * blockDim.x) {
         int px, py, pz;
         split_xyz((unsigned)i, (unsigned)g.mp[0], (unsigned)g.mp[1], px, py, pz);
         const int x = px - LGNK_PAD, y = py - LGNK_PAD, z = (d == 3) ? pz - LGNK_PAD : 0;
         const bool in = x >= 0 && x < g.m[0] && y >= 0 && y < g.m[1] && z >= 0 && z < g.m[2];
-        Tp[i] = in ? scale * T[((size_t)z * g.m[1] + y) * g.m[0] + x] : 0.0f;
+        Tp[i] = in ? T[((size_t)z * g.m[1] + y) * g.m[0] + x] : 0.0f;
     }
+}
+
+// Everything a call lays out before its trace: the parts take consecutive
+// blocks.  The parts are bound by memory at large sizes (the brain-scale product's
+// 492 us are what its two packings and its clearing took) and by their launches
+// at small ones, each about 4 us of the host and 2 us of the GPU: the 64 x 64
+// forward 21.1 -> 18.1 us with one launch for two, the 256 x 256 mass-preserving
+// product 103 -> 95 us with one for three and a clearing.
+template <int D>
+__global__ void __launch_bounds__(kBlock) pack_kernel(const PackArgs A) {
+    unsigned b = blockIdx.x;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const unsigned n = (unsigned)A.blocks[k];
+        if (b < n) {
+            const bool last = k == 1 || A.v[1] == nullptr;
+            pack_velocity<D>(A.v[k], A.vp[k], A.vg, A.tab, last ? A.Gz : nullptr, A.nz, b, n);
+            return;
+        }
+        b -= n;
+    }
+    if (b < (unsigned)A.blocks[2]) {
+        pack_image(A.image, A.imagep, A.ig, D, b, (unsigned)A.blocks[2]);
+        return;
+    }
+    b -= (unsigned)A.blocks[2];
+    const size_t total = padded_size(A.ig);
+    for (size_t i = b * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)A.blocks[3] * blockDim.x) A.zero[i] = 0.0f;
 }
 
 __global__ void unpack_image_kernel(const float* __restrict__ acc, float* __restrict__ out, DevGrid g, int d) {
@@ -163,22 +192,6 @@ __global__ void repad_image_kernel(float* acc, DevGrid g, int d, float scale) {
 }
 
 // ------------------------------------------------------------- reductions --
-
-__device__ __forceinline__ double block_reduce(double x) {
-    __shared__ double red[kBlock / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) red[warp] = x;
-    __syncthreads();
-    double s = 0.0;
-    if (warp == 0) {
-        s = (lane < kBlock / 32) ? red[lane] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    }
-    return s;
-}
 
 // res = u1 - R (Eq. 10): partial sums of res^2 per block (FP64); rp (padded) = scale * res.
 __global__ void residual_kernel(const float* __restrict__ u1, const float* __restrict__ R, float* __restrict__ rp,
@@ -1385,13 +1398,17 @@ inline int grid_for(size_t count) {
 
 }  // namespace
 
-cudaError_t launch_pack_velocity(int d, const float* v, void* Vp, const DevGrid& g, int K, const SliceTable& t,
-                                 cudaStream_t s, void* Gz, int nz) {
-    (void)K;
-    if (nz > t.n) return cudaErrorInvalidValue;
-    const size_t total = (size_t)g.mp[0] * g.mp[1] * g.mp[2] * t.n;
-    if (d == 3) pack_velocity_kernel<3><<<grid_for(total), kBlock, 0, s>>>(v, (float*)Vp, g, t, Gz, nz);
-    else pack_velocity_kernel<2><<<grid_for(total), kBlock, 0, s>>>(v, (float*)Vp, g, t, Gz, nz);
+cudaError_t launch_pack(int d, PackArgs a, cudaStream_t s) {
+    if (a.nz > a.tab.n || (a.v[0] == nullptr && a.v[1] != nullptr)) return cudaErrorInvalidValue;
+    const size_t vn = (size_t)a.vg.mp[0] * a.vg.mp[1] * a.vg.mp[2] * a.tab.n;
+    const size_t in = (size_t)a.ig.mp[0] * a.ig.mp[1] * a.ig.mp[2];
+    for (int k = 0; k < 2; ++k) a.blocks[k] = a.v[k] != nullptr ? grid_for(vn) : 0;
+    a.blocks[2] = a.image != nullptr ? grid_for(in) : 0;
+    a.blocks[3] = a.zero != nullptr ? grid_for(in) : 0;
+    const int blocks = a.blocks[0] + a.blocks[1] + a.blocks[2] + a.blocks[3];
+    if (blocks == 0) return cudaSuccess;
+    if (d == 3) pack_kernel<3><<<blocks, kBlock, 0, s>>>(a);
+    else pack_kernel<2><<<blocks, kBlock, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1428,12 +1445,6 @@ void make_slice_table(int K, int N, double t0, double dt, SliceTable* t) {
         t->j[m] = j;
         t->th[m] = (float)(sv - j);
     }
-}
-
-cudaError_t launch_pack_image(const float* T, float* Tp, const DevGrid& g, int d, float scale, cudaStream_t s) {
-    const size_t total = (size_t)g.mp[0] * g.mp[1] * g.mp[2];
-    pack_image_kernel<<<grid_for(total), kBlock, 0, s>>>(T, Tp, g, d, scale);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_unpack_image(const float* acc, float* out, const DevGrid& g, int d, cudaStream_t s) {

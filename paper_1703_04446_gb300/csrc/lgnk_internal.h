@@ -106,11 +106,24 @@ cudaError_t launch_ell(int d, int mode, const EllArgs& a, cudaStream_t s);
 cudaError_t launch_trace(int d, TimeMode tm, int model, int mode, const TraceArgs& a, cudaStream_t s);
 
 // grid utilities (grid_ops.cu)
-// ABI velocity [K][d][z][y][x] -> pair-packed padded time slices
-// (velocity_pair_bytes(d) bytes per node and slice)
-// (and, when Gz is given, zero nz gradient slices, at most as many as t has)
-cudaError_t launch_pack_velocity(int d, const float* v, void* Vp, const DevGrid& g, int K, const SliceTable& t,
-                                 cudaStream_t s, void* Gz = nullptr, int nz = 0);
+// What a call lays out before it traces, in one launch (null: left out): up to two
+// ABI velocities [K][d][z][y][x] as pair-packed padded time slices
+// (velocity_pair_bytes(d) bytes per node and slice), with the first nz gradient
+// slices, at most as many as tab has, zeroed beside the last of them; an image
+// into its padded grid; a padded image grid to zero.
+struct PackArgs {
+    DevGrid vg, ig;
+    SliceTable tab;
+    const float* v[2];
+    float* vp[2];
+    void* Gz;
+    int nz;
+    const float* image;
+    float* imagep;
+    float* zero;
+    int blocks[4];            // of each part, set by launch_pack
+};
+cudaError_t launch_pack(int d, PackArgs a, cudaStream_t s);
 inline size_t velocity_pair_bytes(int d) { return d == 3 ? 32 : 16; }
 // slice gradients [m][padded nodes] -> ABI [K][d][z][y][x], out = scale * sum_m w_j(m) G_m
 cudaError_t launch_distribute_gradient(int d, const void* Gp, float* out, const DevGrid& g, int K,
@@ -119,7 +132,6 @@ cudaError_t launch_distribute_gradient(int d, const void* Gp, float* out, const 
 void make_node_table(int K, SliceTable* t);
 // stage-time slices of a trace with N steps from t0 in steps dt, over K time nodes
 void make_slice_table(int K, int N, double t0, double dt, SliceTable* t);
-cudaError_t launch_pack_image(const float* T, float* Tp, const DevGrid& g, int d, float scale, cudaStream_t s);
 cudaError_t launch_unpack_image(const float* acc, float* out, const DevGrid& g, int d, cudaStream_t s);
 cudaError_t launch_repad_image(float* acc, const DevGrid& g, int d, float scale, cudaStream_t s);
 cudaError_t launch_residual(const float* u1, const float* R, float* rp, const DevGrid& g, int d,

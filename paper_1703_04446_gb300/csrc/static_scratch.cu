@@ -125,8 +125,15 @@ extern "C" lgnk_status lgnk_forward_transport_static(const lgnk_problem* prob, c
     // Every scratch byte a launch reads is written earlier in the same call
     // (packing writes pads and interiors, each block writes its partial), so
     // nothing left by a previous call needs clearing.
-    cudaError_t e = launch_pack_velocity(d, v, Vp, vg, K, slices, s);
-    if (e == cudaSuccess) e = launch_pack_image(T, Tp, ig, d, 1.0f, s);
+    PackArgs pk{};
+    pk.vg = vg;
+    pk.ig = ig;
+    pk.tab = slices;
+    pk.v[0] = v;
+    pk.vp[0] = static_cast<float*>(Vp);
+    pk.image = T;
+    pk.imagep = Tp;
+    cudaError_t e = launch_pack(d, pk, s);
     TraceArgs a{};
     a.ig = ig;
     a.vg = vg;
