@@ -175,21 +175,22 @@ def algorithmic_bytes_hess(wl):
 
 
 # FP32 FLOPs (FMA = 2) of one voxel-step of the fused matvec in 3D for a
-# stationary velocity, counted from the kernel's formulation (the cell's
-# multilinear interpolant held as polynomial coefficients):
-#   tangent step: 4 stages x (locate 3 FFMA + 3 FADD, q / h 3 FMUL, per
-#     component value and gradient 11 FFMA, J q 1 FMUL + 2 FFMA, dv value
-#     7 FFMA) = 4 x 135, plus the RK4 state updates 18 FADD + 36 FFMA = 90 -> 630;
+# stationary velocity and N >= 4, counted from the kernel's formulation (the
+# row of J by one adjoint sweep, the cell's multilinear interpolant held as
+# polynomial coefficients):
+#   value step: 4 stages x (locate 3 FFMA + 3 FADD, value 7 FFMA a component)
+#     = 4 x 51, plus the RK4 state updates 18 FFMA + 3 FADD = 39 -> 243;
 #   adjoint step: 4 stages x (the stage's cell and offsets read from the
-#     tangent sweep's record, no locate; coefficients of v . mu 7 FMUL +
+#     value sweep's record, no locate; coefficients of v . mu 7 FMUL +
 #     14 FFMA, its gradient 8 FFMA, nu 3 FMUL, the pending block in moment
 #     form: offset products 4 FMUL, 3 FADD + 21 FFMA) = 4 x 103, plus
 #     bookkeeping 12 FMUL + 9 FFMA + 12 FADD = 42 -> 454.
 # The coefficients themselves (13 FADD per component when a stage enters a
-# new cell) and the block's conversion from moments to corners (12 FADD per
-# component when the cell changes) depend on the data and are not counted;
-# ncu's executed counts are in the committed profile.
-HESS_FLOPS_PER_VOXEL_STEP = 1084
+# new cell) and, per block of the row, its conversion from moments to corners
+# (12 FADD per component), its product with dv and its scaling (24 FFMA, 24 FMUL)
+# depend on the data and are not counted; ncu's executed counts are in the
+# committed profile.
+HESS_FLOPS_PER_VOXEL_STEP = 697
 
 
 def algorithmic_flops_hess(wl):
@@ -704,7 +705,7 @@ def run_gpu(args):
         "e2e": {"value": job_throughput(e2e_ms, world), "unit": UNIT, "h2d_bytes_per_step": 4 * (2 * n + M),
                 "d2h_bytes_per_step": 4 * n},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                     "frac": achieved / peak, "traffic": traffic, "kernel": "trace_kernel<3,stat,transport,HESS>",
+                     "frac": achieved / peak, "traffic": traffic, "kernel": "trace_kernel<3,stat,transport,HROW>",
                      "kernel_ms": kern_avg_ms, "flops_per_launch": flops,
                      "peak_kind": f"FP32 from {sms} SMs (device count) x 128 lanes x 2 x max SM clock "
                                   f"{peak_mhz:.0f} MHz", "sms": sms,
@@ -742,7 +743,7 @@ def profile_case(args):
     from paper_1703_04446_gb300 import lgnk, synth
     if args.profile_case == "ws":
         # the warm-start network (c = 32) on a batch of 32 pairs of S^2 images: `launches`
-        # predictions (each 7 convolution GEMMs), then `launches` training steps
+        # predictions (each the first layer and 6 convolution GEMMs), then `launches` training steps
         S, c, B = args.size, 32, 32
         net = lgnk.WarmStart(S, c, B, 0.05)
         net.set_params(torch.from_numpy(synth.warmstart_init(c, 0)))

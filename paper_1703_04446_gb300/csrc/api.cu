@@ -54,7 +54,7 @@ struct PcgGraph {
 };
 
 // The whole PCG loop of one GN step as one graph: a while node whose body is
-// one iteration whose last inner product ends with pcg_control, which ends the loop on the
+// one iteration whose last inner product ends with the loop test (dot_blocks_finish), which ends the loop on the
 // stopping test, non-positive curvature or the iteration cap.  The host reads
 // the loop state once per GN step instead of once per iteration.
 struct PcgLoopGraph {
@@ -109,7 +109,7 @@ struct lgnk_ctx {
     double* hres = nullptr;       // pinned host mirror of dres
     float* fsc = nullptr;         // PCG step lengths on the device (alpha, -alpha, beta)
     unsigned* dcounter = nullptr; // completion counter of launch_dot_fused (zero between launches)
-    int* dctl = nullptr;          // device-side PCG loop state (pcg_control)
+    int* dctl = nullptr;          // device-side PCG loop state (dot_blocks_finish)
     unsigned char* hpin = nullptr; // pinned: the loop state's host copy (4 ints) and its tolerance (a double)
     // lgnk_solve runs on a stream of its own (capturable, unlike the legacy
     // default stream), ordered after and before the caller's stream by events

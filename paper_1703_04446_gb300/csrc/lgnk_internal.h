@@ -145,7 +145,7 @@ cudaError_t launch_dot(const float* a, const float* b, size_t count, double* par
 int dot_blocks(size_t count);
 // a.b (and a.c) reduced to sc[slot_b] (sc[slot_c]) in one launch, then the PCG
 // step `mode` (-1 none, 0 alpha, 1 beta); counter: a zeroed device word; with ctl,
-// then the loop test of a device-side PCG loop (see pcg_control in grid_ops.cu)
+// then the loop test of a device-side PCG loop (see dot_blocks_finish in grid_ops.cu)
 cudaError_t launch_dot_fused(const float* a, const float* b, const float* c, size_t count, double* partial,
                              int nblocks, unsigned* counter, double* sc, int slot_b, int slot_c, int mode, float* f,
                              cudaStream_t s, int* ctl = nullptr, cudaGraphConditionalHandle handle = 0);

@@ -45,7 +45,7 @@
 // What bounds these kernels: first the issue slots, now latency.  Paired FP32
 // instructions, the row form of the Gauss-Newton product and the floor without
 // conversions took the 128^3 product from 495M to 336M warp instructions (issue
-// slots 0.70 -> 0.58 busy) and from 554 to 466 us; what the warps wait for is
+// slots 0.70 -> 0.58 busy) and from 554 to 454 us; what the warps wait for is
 // the cell's corners after a change (long scoreboard, at 16 warps per SM).
 //
 // Time slices.  Every RK4 stage time is t0 + m dt/2 (m = 0..2N), so the host
