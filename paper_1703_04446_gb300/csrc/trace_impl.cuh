@@ -693,7 +693,9 @@ __device__ __forceinline__ float row_value(pair2 row, const float* f) {
 }
 
 // Derivatives along the fractional offsets (per cell width); the constant
-// coefficient is not read.
+// coefficient is not read.  The order of the sums is fixed (3D: f_z first for
+// the x and y derivatives, f_x first for the z derivative): the rows of J, and
+// with them a solve's iterates, keep their rounding whatever the pairing.
 template <int D>
 __device__ __forceinline__ void poly_grad(const pair2* a, const float* f, const pair2* fd, float* gr) {
     constexpr int NP = 1 << (D - 1);
@@ -707,8 +709,10 @@ __device__ __forceinline__ void poly_grad(const pair2* a, const float* f, const 
     unpk(fma2(fd[D - 2], a[NP - 1], a[1]), t0, t1);
     gr[0] = fmaf(f[D - 1], hi2(a[NP / 2]), fmaf(f[1], t1, hi2(a[0])));
     gr[1] = fmaf(f[0], t1, t0);
-    unpk(fma2(fd[0], a[NP - 1], a[NP / 2]), t0, t1);
-    gr[D - 1] = fmaf(f[0], t1, t0);
+    unpk(a[NP / 2], t0, t1);
+    float u0, u1;
+    unpk(a[NP - 1], u0, u1);
+    gr[D - 1] = fmaf(f[1], fmaf(f[0], u1, u0), fmaf(f[0], t1, t0));
 }
 
 // The same interpolant as nested linear interpolations (x, then y, then z) of
