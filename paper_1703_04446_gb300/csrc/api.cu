@@ -94,12 +94,8 @@ struct lgnk_ctx {
     double wreg = 0.0;            // dt * h_v^d of the regularizer (Sec. 3.2)
     void *Vp = nullptr, *dVp = nullptr, *Gp = nullptr;
     float *Tp = nullptr, *acc = nullptr, *rp = nullptr, *itmp = nullptr, *rtmp = nullptr;
-    float *pc0 = nullptr, *pc1 = nullptr, *Cm[3] = {nullptr, nullptr, nullptr}, *inv_eig = nullptr;
-    // the DCT matrices in the shared-memory layouts of the kernels: half tables
-    // (half[a]), or rows padded to P = m rounded up to 4 for the tiled per-axis
-    // kernel, forward Cf[q][k] = C[k][q], inverse Ci[q][k] = C[q][k]
-    float *Cf[3] = {nullptr, nullptr, nullptr}, *Ci[3] = {nullptr, nullptr, nullptr};
-    bool half[3] = {false, false, false};
+    float *pc0 = nullptr, *pc1 = nullptr, *inv_eig = nullptr;
+    float *Cf[3] = {nullptr, nullptr, nullptr}, *Ci[3] = {nullptr, nullptr, nullptr};   // DCT tables, or C in both
     PcgGraph pcg_graphs[2];       // [0] matrix-free, [1] assembled products
     PcgLoopGraph pcg_loops[2];
     double* partial = nullptr;
@@ -663,37 +659,47 @@ lgnk_status hessvec_assembled_packed(lgnk_ctx* ctx, const float* dv, float* out)
     return hessvec_finish(ctx, ctx->slices, dv, out);
 }
 
-lgnk_status precond_apply(lgnk_ctx* ctx, const float* r, float* z) {
+// z = the spectral preconditioner of r.  full: the transforms as direct sums (grid_ops.cu),
+// else by even and odd modes, half the operations and the smaller error (precond at brain
+// scale 491 us, 1084 us as direct sums).  The PCG of a 3D solve uses the direct sums: by
+// halves the velocity of the first Gauss-Newton step moved by 1.07e-6 of its norm (128^3 image,
+// 8 iterations; two runs differ by 5.1e-7 through the order of the atomic additions), enough to
+// put another of the 2 million end points of the second step on the other side of an image
+// node, where grad T jumps.  A 2D image has a hundredth of the voxels, and its planes
+// take 11 us by halves against 15 us.
+lgnk_status precond_apply(lgnk_ctx* ctx, const float* r, float* z, bool full) {
     const int kd = ctx->K * ctx->d, d = ctx->d;
     cudaStream_t s = ctx->stream;
     const float *in = r;
     float *bufs[2] = {ctx->pc0, ctx->pc1}, *out = z;
-    if (d == 3 && ctx->half[0]) {
+    const int* m = ctx->vg.m;
+    const bool last = dct_table_ok(m[d - 1]);
+    if (last && d == 3 && dct_plane_ok(m[0], m[1], full)) {
         // y and x of each xy plane in one pass each way, the last axis both ways with
         // the scale in between: three launches
-        const long long planes = (long long)kd * ctx->vg.m[2];
-        KL(launch_dct_plane(r, ctx->pc0, ctx->Cf[0], ctx->Cf[1], false, ctx->vg, planes, s));
-        KL(launch_dct_last_half(ctx->pc0, ctx->pc1, ctx->Cf[2], ctx->Ci[2], ctx->inv_eig, ctx->vg, 3, kd, s));
-        KL(launch_dct_plane(ctx->pc1, z, ctx->Ci[0], ctx->Ci[1], true, ctx->vg, planes, s));
+        const long long planes = (long long)kd * m[2];
+        KL(launch_dct_plane(r, ctx->pc0, ctx->Cf[0], ctx->Cf[1], false, full, ctx->vg, planes, s));
+        KL(launch_dct_last(ctx->pc0, ctx->pc1, ctx->Cf[2], ctx->Ci[2], ctx->inv_eig, full, ctx->vg, 3, kd, s));
+        KL(launch_dct_plane(ctx->pc1, z, ctx->Ci[0], ctx->Ci[1], true, full, ctx->vg, planes, s));
         return LGNK_OK;
     }
-    if (d == 2 && ctx->half[0]) {
+    if (d == 2 && !full && dct_plane_ok(m[0], m[1], false)) {
         // the whole transform of each plane in one CTA: one launch
         KL(launch_dct_plane2d(r, z, ctx->Cf[0], ctx->Cf[1], ctx->Ci[0], ctx->Ci[1], ctx->inv_eig, ctx->vg, kd, s));
         return LGNK_OK;
     }
     // per axis: forward up to the last one, that one with the scale (fused when it
-    // has half tables), and back
+    // has tables), and back
     int b = 0;
     auto axis = [&](int a, bool inverse, float* dst) -> lgnk_status {
-        KL(launch_dct_axis(in, dst, ctx->Cm[a], inverse ? ctx->Ci[a] : ctx->Cf[a], ctx->vg, d, kd, a, inverse, s));
+        KL(launch_dct_axis(in, dst, inverse ? ctx->Ci[a] : ctx->Cf[a], ctx->vg, kd, a, inverse, s));
         in = dst;
         b ^= 1;
         return LGNK_OK;
     };
     for (int a = 0; a < d - 1; ++a) TRY(axis(a, false, bufs[b]));
-    if (ctx->half[d - 1]) {
-        KL(launch_dct_last_half(in, bufs[b], ctx->Cf[d - 1], ctx->Ci[d - 1], ctx->inv_eig, ctx->vg, d, kd, s));
+    if (last) {
+        KL(launch_dct_last(in, bufs[b], ctx->Cf[d - 1], ctx->Ci[d - 1], ctx->inv_eig, full, ctx->vg, d, kd, s));
         in = bufs[b];
         b ^= 1;
     } else {
@@ -860,22 +866,10 @@ lgnk_status lgnk_create(const lgnk_problem* prob, void* stream, size_t mem_budge
     if ((s = dalloc(ctx, ctx->n, &ctx->pc0)) != LGNK_OK) return fail(s);
     if ((s = dalloc(ctx, ctx->n, &ctx->pc1)) != LGNK_OK) return fail(s);
     for (int a = 0; a < d; ++a) {
-        // one block: the padded tables and the plain matrix, or the two half tables
-        // (which are never larger: rows of about m floats, half as many)
-        const size_t m = (size_t)ctx->vg.m[a], P = (m + 3) & ~(size_t)3;
-        if ((s = dalloc(ctx, m * m + 2 * m * P, &ctx->Cf[a])) != LGNK_OK) return fail(s);
-    }
-    {
-        // whole planes by halves when every axis allows it, else the last axis only;
-        // (the last axis of a 2D grid whose first is long runs on as many lines)
-        bool all = true;
-        for (int a = 0; a < d; ++a) all = all && dct_half_axis_ok(ctx->vg.m[a]);
-        for (int a = 0; a < d; ++a) {
-            const size_t m = (size_t)ctx->vg.m[a], P = (m + 3) & ~(size_t)3;
-            ctx->half[a] = all || (a == d - 1 && dct_half_axis_ok(ctx->vg.m[a]) && ctx->K * d <= 65535);
-            ctx->Ci[a] = ctx->Cf[a] + (ctx->half[a] ? dct_half_floats(ctx->vg.m[a]) : m * P);
-            ctx->Cm[a] = ctx->half[a] ? nullptr : ctx->Cf[a] + 2 * m * P;
-        }
+        const int m = ctx->vg.m[a];
+        const size_t nt = dct_table_ok(m) ? dct_table_floats(m) : 0;
+        if ((s = dalloc(ctx, nt != 0 ? 2 * nt : (size_t)m * m, &ctx->Cf[a])) != LGNK_OK) return fail(s);
+        ctx->Ci[a] = ctx->Cf[a] + nt;
     }
     if ((s = dalloc(ctx, ctx->Mv, &ctx->inv_eig)) != LGNK_OK) return fail(s);
     // per-block partials: a trace's blocks, or two per reduction block (two inner
@@ -912,22 +906,12 @@ lgnk_status lgnk_create(const lgnk_problem* prob, void* stream, size_t mem_budge
             for (int i = 0; i < m; ++i)
                 hostC[(size_t)k * m + i] =
                     (float)(std::sqrt((k == 0 ? 1.0 : 2.0) / m) * std::cos(M_PI * k * (2 * i + 1) / (2.0 * m)));
-        const size_t P = ((size_t)m + 3) & ~(size_t)3;
-        const size_t nt = ctx->half[a] ? dct_half_floats(m) : (size_t)m * P;
-        std::vector<float> hf(nt, 0.0f), hi(nt, 0.0f);
-        if (ctx->half[a]) {
-            dct_half_tables(hostC.data(), m, hf.data(), hi.data());
-        } else {
-            for (int q = 0; q < m; ++q)
-                for (int k = 0; k < m; ++k) {
-                    hf[(size_t)q * P + k] = hostC[(size_t)k * m + q];
-                    hi[(size_t)q * P + k] = hostC[(size_t)q * m + k];
-                }
-            if (cudaMemcpy(ctx->Cm[a], hostC.data(), hostC.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
-                return fail(LGNK_ERR_CUDA);
-        }
+        const bool tables = dct_table_ok(m);
+        std::vector<float> hf(tables ? dct_table_floats(m) : 0), hi(hf.size());
+        if (tables) dct_tables(hostC.data(), m, hf.data(), hi.data());
+        else hf = hostC;
         if (cudaMemcpy(ctx->Cf[a], hf.data(), hf.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(ctx->Ci[a], hi.data(), hi.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
+            (tables && cudaMemcpy(ctx->Ci[a], hi.data(), hi.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess))
             return fail(LGNK_ERR_CUDA);
     }
     std::vector<double> pv(ctx->Mv);
@@ -1083,7 +1067,7 @@ lgnk_status lgnk_jacobian_determinant(lgnk_ctx* ctx, const float* v, const float
 lgnk_status lgnk_precond(lgnk_ctx* ctx, const float* r, float* z) {
     CHECK_CTX();
     REQUIRE(r && z, "r and z must be non-NULL");
-    return precond_apply(ctx, r, z);
+    return precond_apply(ctx, r, z, false);
 }
 
 lgnk_status lgnk_dot(lgnk_ctx* ctx, const float* a, const float* b, size_t count, double* out) {
@@ -1189,7 +1173,7 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
         // PCG on H x = -g from x = 0 (Eq. 11)
         CK(cudaMemsetAsync(x, 0, n * sizeof(float), s));
         KL(launch_add_scaled(r, g, -1.0f, g, 0.0f, n, s));
-        if (o.precond) TRY(precond_apply(ctx, r, z));
+        if (o.precond) TRY(precond_apply(ctx, r, z, ctx->d == 3));
         else CK(cudaMemcpyAsync(z, r, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
         CK(cudaMemcpyAsync(p, z, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
         // The step lengths stay on the device (dres[5] = r.z, fsc = alpha,
@@ -1217,7 +1201,7 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
                                     s));
             }
             KL(launch_pcg_update_xr(x, p, r, Hp, ctx->fsc, n, s));
-            if (o.precond) TRY(precond_apply(ctx, r, z));
+            if (o.precond) TRY(precond_apply(ctx, r, z, ctx->d == 3));
             else CK(cudaMemcpyAsync(z, r, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
             KL(launch_dot_fused(r, r, z, n, ctx->partial, nb, ctx->dcounter, ctx->dres, 3, 4, 1, ctx->fsc, s,
                                 readback ? nullptr : ctx->dctl, loop));

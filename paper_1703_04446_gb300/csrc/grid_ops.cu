@@ -634,16 +634,50 @@ constexpr int kDctTileMax = 128;
 constexpr int kDctLines = 64;
 constexpr int kDctLS = kDctLines + 4;        // tile row stride (float4-aligned)
 
+// The two tables of an axis of m <= kDctTileMax cells (C its orthonormal DCT-II
+// matrix), read by every tiled transform, each 2 h rows (h = ceil(m/2)) of two parts of
+// P4 = h rounded up to 4 floats, zero padded (m = 1: of one part).
+//   forward row q: C[2j][q] | C[2j+1][q]
+//   inverse row r < h: C[2r][j] | C[2r+1][j], row h + r: C[2r][m-1-j] | C[2r+1][m-1-j]
+// The first h rows are what the transforms by halves need.  The direct sums read the
+// inverse table as rows k of P4 floats, C[k][j], and the same mirrored h rows further on.
+struct DctTable {
+    const float* p;
+    int m, h, P4, stride;     // cells; ceil(m/2); floats of a part and of a row
+    __host__ __device__ __forceinline__ int step(bool full, bool inverse) const { return full && inverse ? P4 : stride; }
+    __host__ __device__ __forceinline__ int part(bool full, bool inverse) const {     // offset of the second part
+        return full && inverse ? h * stride : (m > 1 ? P4 : 0);
+    }
+};
+
+inline DctTable dct_table(const float* p, int m) {
+    DctTable t;
+    t.p = p;
+    t.m = m;
+    t.h = (m + 1) / 2;
+    t.P4 = (t.h + 3) & ~3;
+    t.stride = m > 1 ? 2 * t.P4 : t.P4;
+    return t;
+}
+
+// Output index (forward: mode, inverse: position) of column c of a table, -1 for padding.
+__device__ __forceinline__ int dct_column(int c, int P4, int m, bool inverse) {
+    const int j = c < P4 ? c : c - P4, h = (m + 1) / 2;
+    if (inverse) return c < P4 ? (j < h ? j : -1) : (j < m - h ? m - 1 - j : -1);
+    const int k = 2 * j + (c < P4 ? 0 : 1);
+    return k < m ? k : -1;
+}
+
 template <bool XAXIS>
 __global__ void __launch_bounds__(kBlock) dct_tile_kernel(const float* __restrict__ in, float* __restrict__ out,
-                                                          const float* __restrict__ Ctg, int m, long long inner,
+                                                          const DctTable tab, int inverse, long long inner,
                                                           long long lines, int vec_in) {
     extern __shared__ __align__(16) float sm[];
-    const int MP = (m + 3) & ~3;                 // k padded to whole float4s
-    float* Ct = sm;                              // [q][MP]: the padded table of the direction (Cf or Ci)
-    float* tile = sm + m * MP;                   // [q][kDctLS], later the output stage of axis 0
-    const int t = threadIdx.x;
-    for (int e = t; e < m * MP / 4; e += kBlock) cp_async16(Ct + 4 * e, Ctg + 4 * e);
+    const int m = tab.m, MP = tab.stride;        // columns, whole float4s
+    float* Ct = sm;                              // the table of the direction
+    float* tile = sm + 2 * tab.h * MP;           // [q][kDctLS], later the output stage of axis 0
+    const int t = threadIdx.x, step = tab.step(true, inverse), part = tab.part(true, inverse);
+    for (int e = t; e < 2 * tab.h * MP / 4; e += kBlock) cp_async16(Ct + 4 * e, tab.p + 4 * e);
     long long o = 0, i0 = 0, r0 = 0;
     if (XAXIS) {                                 // lines are rows: loaded transposed, element by element
         r0 = (long long)blockIdx.x * kDctLines;
@@ -652,8 +686,9 @@ __global__ void __launch_bounds__(kBlock) dct_tile_kernel(const float* __restric
             tile[q * kDctLS + l] = (r0 + l < lines) ? __ldg(in + (size_t)(r0 + l) * m + q) : 0.0f;
         }
     } else {
-        o = blockIdx.y;
-        i0 = (long long)blockIdx.x * kDctLines;
+        const long long tiles = (inner + kDctLines - 1) / kDctLines;
+        o = blockIdx.x / tiles;
+        i0 = (blockIdx.x - o * tiles) * kDctLines;
         if (vec_in) {                            // inner a multiple of 4, in 16-byte aligned
             for (int e = t; e < m * (kDctLines / 4); e += kBlock) {
                 const int q = e / (kDctLines / 4), l = 4 * (e % (kDctLines / 4));
@@ -681,11 +716,12 @@ __global__ void __launch_bounds__(kBlock) dct_tile_kernel(const float* __restric
         for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc[r][i][j] = 0.0f;
-        const float4* cp = reinterpret_cast<const float4*>(Ct) + kb;
+        const float4* cp =
+            reinterpret_cast<const float4*>(Ct + (4 * kb < tab.P4 ? 4 * kb : part + 4 * kb - tab.P4));
         const float4* xp = reinterpret_cast<const float4*>(tile) + lb;
 #pragma unroll 4
         for (int q = 0; q < m; ++q) {
-            const float4 c = cp[q * (MP / 4)];
+            const float4 c = cp[q * (step / 4)];
             const float4 x = xp[q * (kDctLS / 4)];
             const float cv[4] = {c.x, c.y, c.z, c.w}, xv[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
@@ -696,8 +732,8 @@ __global__ void __launch_bounds__(kBlock) dct_tile_kernel(const float* __restric
         if (!XAXIS) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const int k = 4 * kb + i;
-                if (k >= m) break;
+                const int k = dct_column(4 * kb + i, tab.P4, m, inverse != 0);
+                if (k < 0) continue;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const long long l = i0 + 4 * lb + j;
@@ -716,8 +752,8 @@ __global__ void __launch_bounds__(kBlock) dct_tile_kernel(const float* __restric
             const int kb = task / (kDctLines / 4), lb = task % (kDctLines / 4);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const int k = 4 * kb + i;
-                if (k >= m) break;
+                const int k = dct_column(4 * kb + i, tab.P4, m, inverse != 0);
+                if (k < 0) continue;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) stage[(4 * lb + j) * SS + k] = acc[r][i][j];
             }
@@ -736,52 +772,55 @@ __global__ void __launch_bounds__(kBlock) dct_tile_kernel(const float* __restric
 // half the length, and the inverse is x_q = E_q + O_q, x_(m-1-q) = E_q - O_q with
 // E (O) the sum over the even (odd) modes: half the FMAs and half the table.
 //
-// A table (dct_half_table) has a row of the even and the odd part, each padded
-// to P4 = ceil(m/2) rounded up to 4 floats; forward rows run over q, inverse rows
-// over the mode pairs.  The operand of either direction is a tile of lines in
-// shared memory, [index][LS], first folded into s and d (forward).  A task is 4 even
-// and 4 odd outputs (forward: 8 consecutive modes; inverse: 4 q and their mirrors)
-// of LT lines, done by one thread (LT = 8: 64 FMAs per 6 shared loads) or, where a
-// CTA would have few threads, by two neighbouring lanes (SPLIT, LT = 4), one for
-// the even and one for the odd part, which then exchange what the other stores.
-// Sums run in increasing index order.
+// The operand of either direction is a tile of lines in shared
+// memory, [index][LS], first folded into s and d (forward).  A task is 4 even and 4
+// odd outputs (forward: 8 consecutive modes; inverse: 4 q and their mirrors) of LT
+// lines, done by one thread (LT = 8: 64 FMAs per 6 shared loads) or, where a CTA
+// would have few threads, by two neighbouring lanes (SPLIT, LT = 4), one for the
+// even and one for the odd part, which then exchange what the other stores.
+//
+// With FULL the same tasks sum over the whole axis in increasing index order.  The
+// PCG of a 3D solve uses these (precond_apply): its iterates then keep the rounding of
+// the direct sums.  The second Gauss-Newton step takes
+// grad T, which jumps at image nodes, at end points of the first step's velocity, so
+// a change of that velocity by a rounding can move a voxel's row of J by O(1).
 
-// acc_e[i][l] = sum_r tab[r][j0 + i] E_r[l], acc_o = sum_r tab[r][P4 + j0 + i] O_r[l]
+// acc_e[i][l] = sum_r tab[r][j0 + i] E_r[l], acc_o = sum_r tab[r][po + j0 + i] O_r[l]
 // over the m/2 pairs and the unpaired even row of an odd m; row r of the even
-// (odd) operand is at even + r se (odd + r so).
-template <int LT>
-__device__ __forceinline__ void dct_half_product(const float* tab, int P4, int stride, int m, int j0, const float* even,
+// (odd) operand is at even + r se (odd + r so).  FULL: over m rows of one operand.
+template <int LT, bool FULL>
+__device__ __forceinline__ void dct_half_product(const float* tab, int po, int stride, int m, int j0, const float* even,
                                                  int se, const float* odd, int so, float (&ae)[4][LT],
                                                  float (&ao)[4][LT]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int l = 0; l < LT; ++l) ae[i][l] = ao[i][l] = 0.0f;
-    const int n = m / 2;
+    const int n = FULL ? m : m / 2;
     const float* te = tab + j0;
 #pragma unroll 2
     for (int r = 0; r < n; ++r) {
         const float4 a = *reinterpret_cast<const float4*>(te);
-        const float4 b = *reinterpret_cast<const float4*>(te + P4);
+        const float4 b = *reinterpret_cast<const float4*>(te + po);
         const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-        float x[LT], y[LT];
+        float x[LT], y[FULL ? 1 : LT];
 #pragma unroll
         for (int l = 0; l < LT; l += 4) {
             *reinterpret_cast<float4*>(x + l) = *reinterpret_cast<const float4*>(even + l);
-            *reinterpret_cast<float4*>(y + l) = *reinterpret_cast<const float4*>(odd + l);
+            if constexpr (!FULL) *reinterpret_cast<float4*>(y + l) = *reinterpret_cast<const float4*>(odd + l);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int l = 0; l < LT; ++l) {
                 ae[i][l] = fmaf(av[i], x[l], ae[i][l]);
-                ao[i][l] = fmaf(bv[i], y[l], ao[i][l]);
+                ao[i][l] = fmaf(bv[i], FULL ? x[l] : y[FULL ? 0 : l], ao[i][l]);
             }
         te += stride;
         even += se;
         odd += so;
     }
-    if (m & 1) {
+    if (!FULL && (m & 1)) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -789,16 +828,33 @@ __device__ __forceinline__ void dct_half_product(const float* tab, int P4, int s
     }
 }
 
-// The even (p = 0) or odd (p = 1) part of a task.
-__device__ __forceinline__ void dct_half_part(const float* tab, int P4, int stride, int m, bool inverse, const float* S,
+// The even (p = 0) or odd (p = 1) part of a task (FULL, forward: its first or last four modes).
+template <bool FULL>
+__device__ __forceinline__ void dct_half_part(const float* tab, int po, int stride, int m, bool inverse, const float* S,
                                               int LS, int j0, int l0, int p, float (&a)[4][4]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int l = 0; l < 4; ++l) a[i][l] = 0.0f;
-    const int n = m / 2, st = inverse ? 2 * LS : (p ? -LS : LS);
-    const float* t = tab + j0 + p * P4;
-    const float* x = S + l0 + (inverse ? p * LS : p * (m - 1) * LS);
+    const int n = FULL ? m : m / 2, st = FULL ? LS : (inverse ? 2 * LS : (p ? -LS : LS));
+    const float* t = tab + j0 + p * po;
+    const float* x = S + l0 + (FULL ? 0 : (inverse ? p * LS : p * (m - 1) * LS));
+    if (FULL && !inverse) {
+        t = tab + j0 + 2 * p;
+#pragma unroll 4
+        for (int r = 0; r < n; ++r) {
+            const float2 e = *reinterpret_cast<const float2*>(t), o = *reinterpret_cast<const float2*>(t + po);
+            const float4 v = *reinterpret_cast<const float4*>(x);
+            const float cv[4] = {e.x, o.x, e.y, o.y}, xv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int l = 0; l < 4; ++l) a[i][l] = fmaf(cv[i], xv[l], a[i][l]);
+            t += stride;
+            x += LS;
+        }
+        return;
+    }
 #pragma unroll 4
     for (int r = 0; r < n; ++r) {
         const float4 c = *reinterpret_cast<const float4*>(t);
@@ -811,7 +867,7 @@ __device__ __forceinline__ void dct_half_part(const float* tab, int P4, int stri
         t += stride;
         x += st;
     }
-    if ((m & 1) && p == 0) {
+    if (!FULL && (m & 1) && p == 0) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -821,17 +877,25 @@ __device__ __forceinline__ void dct_half_part(const float* tab, int P4, int stri
 
 // Line l of a split task: the four outputs this lane stores, from position
 // `at` (dct_part_start) on.  Every lane of the warp calls it.
+template <bool FULL>
 __device__ __forceinline__ float4 dct_part_outputs(bool inverse, const float (&a)[4][4], int l, int p) {
     float v[4];
-    if (inverse) {           // even lane E + O at j0 + i; odd lane E - O, mirrored
+    if (inverse) {           // even lane E + O at j0 + i; odd lane E - O, mirrored (FULL: the sums themselves)
         float w[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const float o = __shfl_xor_sync(0xffffffffu, a[i][l], 1);
-            w[i] = p ? o - a[i][l] : a[i][l] + o;
+            if constexpr (FULL) {
+                w[i] = a[i][l];
+            } else {
+                const float o = __shfl_xor_sync(0xffffffffu, a[i][l], 1);
+                w[i] = p ? o - a[i][l] : a[i][l] + o;
+            }
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) v[i] = p ? w[3 - i] : w[i];
+    } else if (FULL) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = a[i][l];
     } else {                 // modes e0 o0 e1 o1 (even lane), e2 o2 e3 o3 (odd lane)
         const float r0 = __shfl_xor_sync(0xffffffffu, p ? a[0][l] : a[2][l], 1);
         const float r1 = __shfl_xor_sync(0xffffffffu, p ? a[1][l] : a[3][l], 1);
@@ -875,23 +939,24 @@ __device__ __forceinline__ void dct_fold(float* S, int LS, int m, int lines) {
 }
 
 // One direction of an axis on the tile S: the product of this thread's task.
-template <int LT>
-__device__ __forceinline__ void dct_half_axis(const float* tab, int P4, int stride, int m, bool inverse, const float* S,
+template <int LT, bool FULL>
+__device__ __forceinline__ void dct_half_axis(const float* tab, int po, int stride, int m, bool inverse, const float* S,
                                               int LS, int j0, int l0, float (&ae)[4][LT], float (&ao)[4][LT]) {
-    if (inverse) dct_half_product<LT>(tab, P4, stride, m, j0, S + l0, 2 * LS, S + LS + l0, 2 * LS, ae, ao);
-    else dct_half_product<LT>(tab, P4, stride, m, j0, S + l0, LS, S + (m - 1) * LS + l0, -LS, ae, ao);
+    if (FULL) dct_half_product<LT, true>(tab, po, stride, m, j0, S + l0, LS, S + l0, LS, ae, ao);
+    else if (inverse) dct_half_product<LT, false>(tab, po, stride, m, j0, S + l0, 2 * LS, S + LS + l0, 2 * LS, ae, ao);
+    else dct_half_product<LT, false>(tab, po, stride, m, j0, S + l0, LS, S + (m - 1) * LS + l0, -LS, ae, ao);
 }
 
 // The 8 outputs of line l of a task: forward, modes 2 j0 .. 2 j0 + 7 in v; inverse,
 // positions j0 .. j0 + 3 in v[0..3] and m - 1 - j0 - 3 .. m - 1 - j0 in v[4..7].
-template <int LT>
+template <int LT, bool FULL>
 __device__ __forceinline__ void dct_outputs(bool inverse, const float (&ae)[4][LT], const float (&ao)[4][LT], int l,
                                             float* v) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         if (inverse) {
-            v[i] = ae[i][l] + ao[i][l];
-            v[7 - i] = ae[i][l] - ao[i][l];
+            v[i] = FULL ? ae[i][l] : ae[i][l] + ao[i][l];
+            v[7 - i] = FULL ? ao[i][l] : ae[i][l] - ao[i][l];
         } else {
             v[2 * i] = ae[i][l];
             v[2 * i + 1] = ao[i][l];
@@ -922,13 +987,15 @@ __device__ __forceinline__ void dct_store_line(float* dst, int m, int j0, bool i
     }
 }
 
-struct HalfTable {
-    const float* p;
-    int P4, stride, rows;     // padded length of a part; floats of a row; rows (ceil(m/2))
-};
+// Rows of a table that a transform stages.
+template <bool FULL>
+__host__ __device__ inline int dct_rows(int m) {
+    return (FULL ? 2 : 1) * ((m + 1) / 2);
+}
 
-__device__ __forceinline__ void dct_stage_table(float* dst, const HalfTable& t) {
-    for (int e = threadIdx.x; e < t.rows * t.stride / 4; e += blockDim.x) cp_async16(dst + 4 * e, t.p + 4 * e);
+template <bool FULL>
+__device__ __forceinline__ void dct_stage_table(float* dst, const DctTable& t) {
+    for (int e = threadIdx.x; e < dct_rows<FULL>(t.m) * t.stride / 4; e += blockDim.x) cp_async16(dst + 4 * e, t.p + 4 * e);
 }
 
 // The last axis of the preconditioner in one pass: forward transform, the
@@ -938,18 +1005,18 @@ __device__ __forceinline__ void dct_stage_table(float* dst, const HalfTable& t) 
 // of 4 lines.
 constexpr int kDctFusedLines = 64;
 
-template <int LINES, bool SPLIT>
+template <int LINES, bool SPLIT, bool FULL>
 __global__ void __launch_bounds__(kBlock) dct_last_half_kernel(const float* __restrict__ in, float* __restrict__ out,
-                                                               const HalfTable tf, const HalfTable ti,
+                                                               const DctTable tf, const DctTable ti,
                                                                const float* __restrict__ inv_eig, int m,
                                                                long long inner, int vec_in) {
     constexpr int LS = LINES + 4, LT = 4;
     extern __shared__ __align__(16) float sm[];
     float* F = sm;
-    float* I = F + tf.rows * tf.stride;
-    float* tile = I + ti.rows * ti.stride;     // [q][LS], then the scaled modes [k][LS]
-    dct_stage_table(F, tf);
-    dct_stage_table(I, ti);
+    float* I = F + dct_rows<FULL>(m) * tf.stride;
+    float* tile = I + dct_rows<FULL>(m) * ti.stride;     // [q][LS], then the scaled modes [k][LS]
+    dct_stage_table<FULL>(F, tf);
+    dct_stage_table<FULL>(I, ti);
     const long long o = blockIdx.y, i0 = (long long)blockIdx.x * LINES;
     const int t = threadIdx.x;
     if (vec_in) {                     // inner a multiple of 4, in 16-byte aligned: whole float4s in or out
@@ -967,16 +1034,18 @@ __global__ void __launch_bounds__(kBlock) dct_last_half_kernel(const float* __re
     }
     cp_async_wait_all();
     __syncthreads();
-    dct_fold(tile, LS, m, LINES);
-    __syncthreads();
+    if (!FULL) {
+        dct_fold(tile, LS, m, LINES);
+        __syncthreads();
+    }
     const int p = SPLIT ? t & 1 : 0, task = SPLIT ? t >> 1 : t;
     const int l0 = LT * (task % (LINES / LT)), j0 = 4 * (task / (LINES / LT));
     const int h = (m + 1) / 2;
     const bool act = j0 < h;
     float ae[4][LT], ao[4][LT];
     if (act) {
-        if (SPLIT) dct_half_part(F, tf.P4, tf.stride, m, false, tile, LS, j0, l0, p, ae);
-        else dct_half_axis<LT>(F, tf.P4, tf.stride, m, false, tile, LS, j0, l0, ae, ao);
+        if (SPLIT) dct_half_part<FULL>(F, tf.part(FULL, false), tf.step(FULL, false), m, false, tile, LS, j0, l0, p, ae);
+        else dct_half_axis<LT, FULL>(F, tf.part(FULL, false), tf.step(FULL, false), m, false, tile, LS, j0, l0, ae, ao);
     }
     __syncthreads();                  // every thread is done reading the tile
     const bool vec = vec_in && i0 + l0 + LT <= inner;
@@ -985,7 +1054,7 @@ __global__ void __launch_bounds__(kBlock) dct_last_half_kernel(const float* __re
         for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int q = 0; q < (SPLIT ? 1 : 2); ++q) {
-                const int k = 2 * (j0 + i) + (SPLIT ? p : q);
+                const int k = SPLIT && FULL ? 2 * j0 + 4 * p + i : 2 * (j0 + i) + (SPLIT ? p : q);
                 if (k >= m) continue;
                 const float4 v = q ? make_float4(ao[i][0], ao[i][1], ao[i][2], ao[i][3])
                                    : make_float4(ae[i][0], ae[i][1], ae[i][2], ae[i][3]);
@@ -1005,8 +1074,8 @@ __global__ void __launch_bounds__(kBlock) dct_last_half_kernel(const float* __re
     }
     __syncthreads();
     if (act) {
-        if (SPLIT) dct_half_part(I, ti.P4, ti.stride, m, true, tile, LS, j0, l0, p, ae);
-        else dct_half_axis<LT>(I, ti.P4, ti.stride, m, true, tile, LS, j0, l0, ae, ao);
+        if (SPLIT) dct_half_part<FULL>(I, ti.part(FULL, true), ti.step(FULL, true), m, true, tile, LS, j0, l0, p, ae);
+        else dct_half_axis<LT, FULL>(I, ti.part(FULL, true), ti.step(FULL, true), m, true, tile, LS, j0, l0, ae, ao);
     }
     const bool vec_out = vec && reinterpret_cast<uintptr_t>(out) % 16 == 0;
 #pragma unroll
@@ -1017,7 +1086,9 @@ __global__ void __launch_bounds__(kBlock) dct_last_half_kernel(const float* __re
             float v[LT];
 #pragma unroll
             for (int l = 0; l < LT; ++l) {
-                if (SPLIT) {
+                if constexpr (FULL) {
+                    v[l] = !SPLIT && c ? ao[i][l] : ae[i][l];
+                } else if (SPLIT) {
                     const float o = __shfl_xor_sync(0xffffffffu, ae[i][l], 1);
                     v[l] = p ? o - ae[i][l] : ae[i][l] + o;
                 } else {
@@ -1043,9 +1114,10 @@ __global__ void __launch_bounds__(kBlock) dct_last_half_kernel(const float* __re
 // products read float4 rows and the plane is loaded and stored row-major.  The
 // two axes commute, so one order serves both directions.
 constexpr int kDctPlaneMax = 128;
+constexpr int kDctFullPlaneMax = 64;         // of the direct sums (their tables are twice as long)
 
 // A thread's task in the plane kernels: LT = 8 lines, both parts; LT = 4 (split), one part.
-template <int LT>
+template <int LT, bool FULL>
 struct PlaneTask {
     static constexpr bool SPLIT = LT == 4;
     int j0, l0, p;
@@ -1061,11 +1133,11 @@ struct PlaneTask {
         l0 = LT * (t / g);
         act = l0 < lines;
     }
-    __device__ __forceinline__ void product(const float* tab, const HalfTable& t, int m, bool inverse, const float* S,
+    __device__ __forceinline__ void product(const float* tab, const DctTable& t, int m, bool inverse, const float* S,
                                             int LS) {
         if (!act) return;
-        if constexpr (SPLIT) dct_half_part(tab, t.P4, t.stride, m, inverse, S, LS, j0, l0, p, ae);
-        else dct_half_axis<LT>(tab, t.P4, t.stride, m, inverse, S, LS, j0, l0, ae, ao);
+        if constexpr (SPLIT) dct_half_part<FULL>(tab, t.part(FULL, inverse), t.step(FULL, inverse), m, inverse, S, LS, j0, l0, p, ae);
+        else dct_half_axis<LT, FULL>(tab, t.part(FULL, inverse), t.step(FULL, inverse), m, inverse, S, LS, j0, l0, ae, ao);
     }
     // Stores the outputs of lines l0 .. as rows of m values, `row` floats apart;
     // scale: NULL or factors of the same layout (rows of m).  Every thread calls it.
@@ -1075,7 +1147,7 @@ struct PlaneTask {
         for (int l = 0; l < LT; ++l) {
             const bool in = act && l0 + l < lines;
             if constexpr (SPLIT) {
-                float4 v = dct_part_outputs(inverse, ae, l, p);
+                float4 v = dct_part_outputs<FULL>(inverse, ae, l, p);
                 if (!in) continue;
                 if (scale != nullptr) {
                     const int at = dct_part_start(inverse, m, j0, p);
@@ -1089,7 +1161,7 @@ struct PlaneTask {
             } else {
                 if (!in) continue;
                 float v[8];
-                dct_outputs<LT>(inverse, ae, ao, l, v);
+                dct_outputs<LT, FULL>(inverse, ae, ao, l, v);
                 if (scale != nullptr) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
@@ -1103,10 +1175,11 @@ struct PlaneTask {
 
 // Both products of the plane in S (rows [y][LS]), every thread of the CTA; the x
 // product's outputs (lines = ky) stay in the task.
-template <int LT>
-__device__ __forceinline__ void plane_half_yx(const float* Ty, const HalfTable& ty, const float* Tx, const HalfTable& tx,
-                                              float* S, int mx, int my, int LS, int LTR, bool inverse, PlaneTask<LT>& k) {
-    if (!inverse) {
+template <int LT, bool FULL>
+__device__ __forceinline__ void plane_half_yx(const float* Ty, const DctTable& ty, const float* Tx, const DctTable& tx,
+                                              float* S, int mx, int my, int LS, int LTR, bool inverse,
+                                              PlaneTask<LT, FULL>& k) {
+    if (!FULL && !inverse) {
         dct_fold(S, LS, my, mx);
         __syncthreads();
     }
@@ -1115,7 +1188,7 @@ __device__ __forceinline__ void plane_half_yx(const float* Ty, const HalfTable& 
     __syncthreads();                      // every read of the plane is done
     k.store(S, LTR, my, mx, inverse, my % 4 == 0, nullptr);
     __syncthreads();
-    if (!inverse) {
+    if (!FULL && !inverse) {
         dct_fold(S, LTR, mx, my);
         __syncthreads();
     }
@@ -1140,78 +1213,73 @@ __device__ __forceinline__ void plane_load(const float* __restrict__ in, size_t 
     }
 }
 
-template <int LT>
+template <int LT, bool FULL>
 __global__ void __launch_bounds__(kBlock) dct_plane_kernel(const float* __restrict__ in, float* __restrict__ out,
-                                                           const HalfTable tx, const HalfTable ty, int inverse, int mx,
+                                                           const DctTable tx, const DctTable ty, int inverse, int mx,
                                                            int my, int vec_in, int vec_out) {
     extern __shared__ __align__(16) float sm[];
     const int LS = ((mx + 3) & ~3) + 4, LTR = ((my + 3) & ~3) + 4;   // row strides of [y][x] and of [x][k]
     float* Ty = sm;
-    float* Tx = Ty + ty.rows * ty.stride;
-    float* S = Tx + tx.rows * tx.stride;  // the plane, later the y result transposed
-    dct_stage_table(Ty, ty);
-    dct_stage_table(Tx, tx);
+    float* Tx = Ty + dct_rows<FULL>(my) * ty.stride;
+    float* S = Tx + dct_rows<FULL>(mx) * tx.stride;  // the plane, later the y result transposed
+    dct_stage_table<FULL>(Ty, ty);
+    dct_stage_table<FULL>(Tx, tx);
     const size_t base = (size_t)blockIdx.x * mx * my;
     plane_load(in, base, S, mx, my, LS, vec_in);
     cp_async_wait_all();
     __syncthreads();
-    PlaneTask<LT> k;
-    plane_half_yx<LT>(Ty, ty, Tx, tx, S, mx, my, LS, LTR, inverse != 0, k);
+    PlaneTask<LT, FULL> k;
+    plane_half_yx<LT, FULL>(Ty, ty, Tx, tx, S, mx, my, LS, LTR, inverse != 0, k);
     k.store(out + base, mx, mx, my, inverse != 0, vec_out != 0, nullptr);
 }
 
 // The whole 2D preconditioner on one plane (a (time node, component) block) in
 // one CTA: forward, scale by inv_eig, inverse, with the scaled modes written
-// back into the plane buffer between the two halves.
+// back into the plane buffer between the two halves.  Few planes leave most SMs idle, but
+// up to 128 x 128 the three launches of the per-axis path cost more: two planes of
+// 65 x 65 33 -> 21 us, of 128 x 16 41 -> 11, of 128 x 128 51 -> 43, of 127 x 125 56 -> 51.
 template <int LT>
 __global__ void __launch_bounds__(kBlock) dct_plane2d_kernel(const float* __restrict__ in, float* __restrict__ out,
-                                                             const HalfTable fx, const HalfTable fy, const HalfTable ix,
-                                                             const HalfTable iy, const float* __restrict__ inv_eig,
+                                                             const DctTable fx, const DctTable fy, const DctTable ix,
+                                                             const DctTable iy, const float* __restrict__ inv_eig,
                                                              int mx, int my, int vec_in, int vec_out) {
     extern __shared__ __align__(16) float sm[];
     const int LS = ((mx + 3) & ~3) + 4, LTR = ((my + 3) & ~3) + 4;
     float* Fy = sm;
-    float* Fx = Fy + fy.rows * fy.stride;
-    float* Iy = Fx + fx.rows * fx.stride;
-    float* Ix = Iy + iy.rows * iy.stride;
-    float* S = Ix + ix.rows * ix.stride;
-    dct_stage_table(Fy, fy);
-    dct_stage_table(Fx, fx);
-    dct_stage_table(Iy, iy);
-    dct_stage_table(Ix, ix);
+    float* Fx = Fy + dct_rows<false>(my) * fy.stride;
+    float* Iy = Fx + dct_rows<false>(mx) * fx.stride;
+    float* Ix = Iy + dct_rows<false>(my) * iy.stride;
+    float* S = Ix + dct_rows<false>(mx) * ix.stride;
+    dct_stage_table<false>(Fy, fy);
+    dct_stage_table<false>(Fx, fx);
+    dct_stage_table<false>(Iy, iy);
+    dct_stage_table<false>(Ix, ix);
     const size_t base = (size_t)blockIdx.x * mx * my;
     plane_load(in, base, S, mx, my, LS, vec_in);
     cp_async_wait_all();
     __syncthreads();
-    PlaneTask<LT> k;
-    plane_half_yx<LT>(Fy, fy, Fx, fx, S, mx, my, LS, LTR, false, k);
+    PlaneTask<LT, false> k;
+    plane_half_yx<LT, false>(Fy, fy, Fx, fx, S, mx, my, LS, LTR, false, k);
     // the scaled modes back as rows [ky][LS] once every thread is done with the transposed buffer
     __syncthreads();
     k.store(S, LS, mx, my, false, mx % 4 == 0, inv_eig);
     __syncthreads();
-    plane_half_yx<LT>(Iy, iy, Ix, ix, S, mx, my, LS, LTR, true, k);
+    plane_half_yx<LT, false>(Iy, iy, Ix, ix, S, mx, my, LS, LTR, true, k);
     k.store(out + base, mx, mx, my, true, vec_out != 0, nullptr);
 }
 
-inline HalfTable half_table(const float* p, int m) {
-    HalfTable t;
-    t.p = p;
-    t.rows = (m + 1) / 2;
-    t.P4 = (t.rows + 3) & ~3;
-    t.stride = m > 1 ? 2 * t.P4 : t.P4;
-    return t;
-}
-
-inline size_t half_floats(int m) {
-    const HalfTable t = half_table(nullptr, m);
-    return (size_t)t.rows * t.stride;
+// Floats of an axis's staged table
+template <bool FULL>
+inline size_t staged_floats(int m) {
+    return (size_t)dct_rows<FULL>(m) * dct_table(nullptr, m).stride;
 }
 
 // Shared memory of the plane kernels with `dirs` directions' tables.
+template <bool FULL>
 inline size_t dct_plane_smem(int mx, int my, int dirs) {
     const size_t LS = (size_t)((mx + 3) & ~3) + 4, LTR = (size_t)((my + 3) & ~3) + 4;
     const size_t plane = std::max((size_t)my * LS, (size_t)mx * LTR) + 8;    // (rows are read in groups of 8 lines)
-    return (dirs * (half_floats(mx) + half_floats(my)) + plane) * sizeof(float);
+    return (dirs * (staged_floats<FULL>(mx) + staged_floats<FULL>(my)) + plane) * sizeof(float);
 }
 
 // Threads with a task in a plane kernel, for either form (the larger of the two
@@ -1232,9 +1300,8 @@ inline bool dct_plane_split(int mx, int my) { return dct_plane_threads(mx, my, 4
 
 // Shared memory of dct_tile_kernel for an axis of m cells (bytes).
 inline size_t dct_tile_smem(int m) {
-    const size_t MP = (size_t)((m + 3) & ~3);
     const size_t tile = std::max((size_t)m * kDctLS, (size_t)kDctLines * (kDctTileMax + 1));
-    return ((size_t)m * MP + tile) * sizeof(float);
+    return (dct_table_floats(m) + tile) * sizeof(float);
 }
 
 __global__ void scale_modes_kernel(float* x, const float* __restrict__ inv_eig, size_t block_elems, size_t count) {
@@ -1590,69 +1657,6 @@ cudaError_t launch_elastic(int d, const float* x, const float* div, float* out, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_dct_axis(const float* in, float* out, const float* C, const float* Cp, const DevGrid& g, int d,
-                            int nblocks_kd, int axis, bool inverse, cudaStream_t s) {
-    (void)d;
-    const size_t total = (size_t)g.m[0] * g.m[1] * g.m[2] * nblocks_kd;
-    const int m = g.m[axis];
-    if (m > kDctTileMax) {
-        dct_axis_kernel<<<grid_for(total), kBlock, 0, s>>>(in, out, C, g, nblocks_kd, axis, inverse ? 1 : 0);
-        return cudaGetLastError();
-    }
-    const size_t smem = dct_tile_smem(m);
-    // the dynamic shared-memory limit is raised once per device and kernel
-    static bool attr_set_dev[64][2] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    bool* attr_set = attr_set_dev[dev];
-    const int smem_max = (int)dct_tile_smem(kDctTileMax);
-    const long long inner = axis == 0 ? 1 : (axis == 1 ? (long long)g.m[0] : (long long)g.m[0] * g.m[1]);
-    const long long outer = (long long)(total / ((size_t)m * inner));
-    if (axis == 0) {
-        if (!attr_set[0]) {
-            const cudaError_t e =
-                cudaFuncSetAttribute(dct_tile_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-            if (e != cudaSuccess) return e;
-            attr_set[0] = true;
-        }
-        const long long rows = outer;   // inner = 1: every (y, z, block) is one line
-        dct_tile_kernel<true><<<(unsigned)((rows + kDctLines - 1) / kDctLines), kBlock, smem, s>>>(
-            in, out, Cp, m, 1, rows, 0);
-    } else {
-        if (!attr_set[1]) {
-            const cudaError_t e =
-                cudaFuncSetAttribute(dct_tile_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-            if (e != cudaSuccess) return e;
-            attr_set[1] = true;
-        }
-        if (outer > 65535) {
-            dct_axis_kernel<<<grid_for(total), kBlock, 0, s>>>(in, out, C, g, nblocks_kd, axis, inverse ? 1 : 0);
-            return cudaGetLastError();
-        }
-        const dim3 grid((unsigned)((inner + kDctLines - 1) / kDctLines), (unsigned)outer);
-        const int vec_in = (inner % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
-        dct_tile_kernel<false><<<grid, kBlock, smem, s>>>(in, out, Cp, m, inner, inner * m * outer, vec_in);
-    }
-    return cudaGetLastError();
-}
-
-size_t dct_half_floats(int m) { return half_floats(m); }
-
-bool dct_half_axis_ok(int m) { return m <= kDctPlaneMax; }
-
-void dct_half_tables(const float* C, int m, float* f, float* i) {
-    const HalfTable t = half_table(nullptr, m);
-    for (size_t e = 0; e < (size_t)t.rows * t.stride; ++e) f[e] = i[e] = 0.0f;
-    for (int r = 0; r < t.rows; ++r)
-        for (int j = 0; j < t.rows; ++j) {
-            // forward row r = q: modes 2j (even part) and 2j + 1; inverse row r: modes 2r, 2r + 1 at q = j
-            if (2 * j < m) f[(size_t)r * t.stride + j] = C[(size_t)(2 * j) * m + r];
-            if (2 * j + 1 < m) f[(size_t)r * t.stride + t.P4 + j] = C[(size_t)(2 * j + 1) * m + r];
-            if (2 * r < m) i[(size_t)r * t.stride + j] = C[(size_t)(2 * r) * m + j];
-            if (2 * r + 1 < m) i[(size_t)r * t.stride + t.P4 + j] = C[(size_t)(2 * r + 1) * m + j];
-        }
-}
-
 // Raises the dynamic shared-memory limit of a kernel, once per device.
 template <class K>
 static cudaError_t raise_smem(K kernel, size_t bytes, bool (&done)[64]) {
@@ -1664,76 +1668,131 @@ static cudaError_t raise_smem(K kernel, size_t bytes, bool (&done)[64]) {
     return e;
 }
 
-cudaError_t launch_dct_plane(const float* in, float* out, const float* Tx, const float* Ty, bool inverse, const DevGrid& g,
+cudaError_t launch_dct_axis(const float* in, float* out, const float* C, const DevGrid& g, int nblocks_kd, int axis,
+                            bool inverse, cudaStream_t s) {
+    const size_t total = (size_t)g.m[0] * g.m[1] * g.m[2] * nblocks_kd;
+    const int m = g.m[axis];
+    if (m > kDctTileMax) {
+        dct_axis_kernel<<<grid_for(total), kBlock, 0, s>>>(in, out, C, g, nblocks_kd, axis, inverse ? 1 : 0);
+        return cudaGetLastError();
+    }
+    const long long inner = axis == 0 ? 1 : (axis == 1 ? (long long)g.m[0] : (long long)g.m[0] * g.m[1]);
+    const long long outer = (long long)(total / ((size_t)m * inner));
+    const long long blocks = axis == 0 ? (outer + kDctLines - 1) / kDctLines    // inner = 1: every (y, z, block) is one line
+                                       : (inner + kDctLines - 1) / kDctLines * outer;
+    const int vec_in = (inner % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
+    static bool done[2][64] = {};
+    auto run = [&](auto kernel, long long lines, bool (&d)[64]) -> cudaError_t {
+        const cudaError_t e = raise_smem(kernel, dct_tile_smem(kDctTileMax), d);
+        if (e != cudaSuccess) return e;
+        kernel<<<(unsigned)blocks, kBlock, dct_tile_smem(m), s>>>(in, out, dct_table(C, m), inverse, inner, lines, vec_in);
+        return cudaGetLastError();
+    };
+    return axis == 0 ? run(dct_tile_kernel<true>, outer, done[0]) : run(dct_tile_kernel<false>, inner * m * outer, done[1]);
+}
+
+bool dct_table_ok(int m) { return m <= kDctTileMax; }
+
+size_t dct_table_floats(int m) { return (size_t)2 * dct_table(nullptr, m).h * dct_table(nullptr, m).stride; }
+
+void dct_tables(const float* C, int m, float* f, float* i) {
+    const DctTable t = dct_table(nullptr, m);
+    for (size_t e = 0; e < dct_table_floats(m); ++e) f[e] = i[e] = 0.0f;
+    for (int r = 0; r < m; ++r)
+        for (int j = 0; j < t.h; ++j) {
+            float* fr = f + (size_t)r * t.stride + j;
+            fr[0] = C[(size_t)(2 * j) * m + r];
+            if (2 * j + 1 < m) fr[t.P4] = C[(size_t)(2 * j + 1) * m + r];
+            float* ir = i + (size_t)r * t.P4 + j;
+            ir[0] = C[(size_t)r * m + j];
+            ir[t.h * t.stride] = C[(size_t)r * m + m - 1 - j];
+        }
+}
+
+bool dct_plane_ok(int mx, int my, bool full) {
+    const int most = full ? kDctFullPlaneMax : kDctPlaneMax;
+    return mx <= most && my <= most;
+}
+
+template <int LT, bool FULL>
+static cudaError_t run_plane(const float* in, float* out, const float* Tx, const float* Ty, bool inverse, int mx, int my,
                              long long planes, cudaStream_t s) {
-    const int mx = g.m[0], my = g.m[1];
-    if (mx > kDctPlaneMax || my > kDctPlaneMax || planes < 1 || planes > 0x7fffffffLL) return cudaErrorNotSupported;
+    constexpr int most = FULL ? kDctFullPlaneMax : kDctPlaneMax;
+    static bool done[64] = {};
+    const cudaError_t e = raise_smem(dct_plane_kernel<LT, FULL>, dct_plane_smem<FULL>(most, most, 1), done);
+    if (e != cudaSuccess) return e;
     const int vec_in = (mx % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
     const int vec_out = (mx % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0) ? 1 : 0;
-    const HalfTable tx = half_table(Tx, mx), ty = half_table(Ty, my);
-    const size_t smem = dct_plane_smem(mx, my, 1);
-    if (!dct_plane_split(mx, my)) {
-        static bool done[64] = {};
-        const cudaError_t e = raise_smem(dct_plane_kernel<8>, dct_plane_smem(kDctPlaneMax, kDctPlaneMax, 1), done);
-        if (e != cudaSuccess) return e;
-        dct_plane_kernel<8><<<(unsigned)planes, dct_threads(dct_plane_threads(mx, my, 8), planes), smem, s>>>(in, out, tx, ty, inverse, mx, my,
-                                                                                         vec_in, vec_out);
-    } else {
-        static bool done[64] = {};
-        const cudaError_t e = raise_smem(dct_plane_kernel<4>, dct_plane_smem(kDctPlaneMax, kDctPlaneMax, 1), done);
-        if (e != cudaSuccess) return e;
-        dct_plane_kernel<4><<<(unsigned)planes, dct_threads(dct_plane_threads(mx, my, 4), planes), smem, s>>>(in, out, tx, ty, inverse, mx, my,
-                                                                                         vec_in, vec_out);
-    }
+    dct_plane_kernel<LT, FULL><<<(unsigned)planes, dct_threads(dct_plane_threads(mx, my, LT), planes),
+                                 dct_plane_smem<FULL>(mx, my, 1), s>>>(in, out, dct_table(Tx, mx), dct_table(Ty, my),
+                                                                       inverse, mx, my, vec_in, vec_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dct_plane(const float* in, float* out, const float* Tx, const float* Ty, bool inverse, bool full,
+                             const DevGrid& g, long long planes, cudaStream_t s) {
+    const int mx = g.m[0], my = g.m[1];
+    if (!dct_plane_ok(mx, my, full) || planes < 1 || planes > 0x7fffffffLL) return cudaErrorNotSupported;
+    if (dct_plane_split(mx, my))
+        return full ? run_plane<4, true>(in, out, Tx, Ty, inverse, mx, my, planes, s)
+                    : run_plane<4, false>(in, out, Tx, Ty, inverse, mx, my, planes, s);
+    return full ? run_plane<8, true>(in, out, Tx, Ty, inverse, mx, my, planes, s)
+                : run_plane<8, false>(in, out, Tx, Ty, inverse, mx, my, planes, s);
+}
+
+template <int LT>
+static cudaError_t run_plane2d(const float* in, float* out, const float* Fx, const float* Fy, const float* Ix,
+                               const float* Iy, const float* inv_eig, int mx, int my, int blocks, cudaStream_t s) {
+    static bool done[64] = {};
+    const cudaError_t e =
+        raise_smem(dct_plane2d_kernel<LT>, dct_plane_smem<false>(kDctPlaneMax, kDctPlaneMax, 2), done);
+    if (e != cudaSuccess) return e;
+    const int vec_in = (mx % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
+    const int vec_out = (mx % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0) ? 1 : 0;
+    dct_plane2d_kernel<LT><<<blocks, kBlock, dct_plane_smem<false>(mx, my, 2), s>>>(
+        in, out, dct_table(Fx, mx), dct_table(Fy, my), dct_table(Ix, mx), dct_table(Iy, my), inv_eig, mx, my, vec_in,
+        vec_out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_dct_plane2d(const float* in, float* out, const float* Fx, const float* Fy, const float* Ix,
                                const float* Iy, const float* inv_eig, const DevGrid& g, int blocks, cudaStream_t s) {
     const int mx = g.m[0], my = g.m[1];
-    if (mx > kDctPlaneMax || my > kDctPlaneMax || blocks < 1) return cudaErrorNotSupported;
-    const int vec_in = (mx % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
-    const int vec_out = (mx % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0) ? 1 : 0;
-    const size_t smem = dct_plane_smem(mx, my, 2), smax = dct_plane_smem(kDctPlaneMax, kDctPlaneMax, 2);
-    const HalfTable fx = half_table(Fx, mx), fy = half_table(Fy, my), ix = half_table(Ix, mx), iy = half_table(Iy, my);
-    if (!dct_plane_split(mx, my)) {
-        static bool done[64] = {};
-        const cudaError_t e = raise_smem(dct_plane2d_kernel<8>, smax, done);
-        if (e != cudaSuccess) return e;
-        dct_plane2d_kernel<8><<<blocks, kBlock, smem, s>>>(in, out, fx, fy, ix, iy, inv_eig, mx, my,
-                                                                                 vec_in, vec_out);
-    } else {
-        static bool done[64] = {};
-        const cudaError_t e = raise_smem(dct_plane2d_kernel<4>, smax, done);
-        if (e != cudaSuccess) return e;
-        dct_plane2d_kernel<4><<<blocks, kBlock, smem, s>>>(in, out, fx, fy, ix, iy, inv_eig, mx, my,
-                                                                                 vec_in, vec_out);
-    }
+    if (!dct_plane_ok(mx, my, false) || blocks < 1) return cudaErrorNotSupported;
+    return dct_plane_split(mx, my) ? run_plane2d<4>(in, out, Fx, Fy, Ix, Iy, inv_eig, mx, my, blocks, s)
+                                   : run_plane2d<8>(in, out, Fx, Fy, Ix, Iy, inv_eig, mx, my, blocks, s);
+}
+
+template <int LINES, bool SPLIT, bool FULL>
+static cudaError_t run_last(const float* in, float* out, const float* Tf, const float* Ti, const float* inv_eig, int m,
+                            long long inner, int nblocks_kd, long long blocks, cudaStream_t s) {
+    const auto bytes = [](int n) { return (2 * staged_floats<FULL>(n) + (size_t)n * (LINES + 4)) * sizeof(float); };
+    static bool done[64] = {};
+    const cudaError_t e = raise_smem(dct_last_half_kernel<LINES, SPLIT, FULL>, bytes(kDctTileMax), done);
+    if (e != cudaSuccess) return e;
+    const int groups = ((m + 1) / 2 + 3) / 4;
+    const int vec_in = (inner % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
+    const dim3 grid((unsigned)((inner + LINES - 1) / LINES), (unsigned)nblocks_kd);
+    dct_last_half_kernel<LINES, SPLIT, FULL><<<grid, dct_threads((SPLIT ? 2 : 1) * groups * (LINES / 4), blocks), bytes(m),
+                                               s>>>(in, out, dct_table(Tf, m), dct_table(Ti, m), inv_eig, m, inner, vec_in);
     return cudaGetLastError();
 }
 
-cudaError_t launch_dct_last_half(const float* in, float* out, const float* Tf, const float* Ti, const float* inv_eig,
-                                 const DevGrid& g, int d, int nblocks_kd, cudaStream_t s) {
+cudaError_t launch_dct_last(const float* in, float* out, const float* Tf, const float* Ti, const float* inv_eig,
+                            bool full, const DevGrid& g, int d, int nblocks_kd, cudaStream_t s) {
     const int m = g.m[d - 1];
     const long long inner = d == 2 ? (long long)g.m[0] : (long long)g.m[0] * g.m[1];
-    if (m > kDctPlaneMax || nblocks_kd > 65535) return cudaErrorNotSupported;
-    const int vec_in = (inner % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
-    const HalfTable tf = half_table(Tf, m), ti = half_table(Ti, m);
+    if (m > kDctTileMax || nblocks_kd > 65535) return cudaErrorNotSupported;
     const long long blocks = (inner + kDctFusedLines - 1) / kDctFusedLines * nblocks_kd;
     const int groups = ((m + 1) / 2 + 3) / 4;
-    auto run = [&](auto kernel, int lines, bool split, bool (&done)[64]) -> cudaError_t {
-        const auto bytes = [&](int n) { return (2 * half_floats(n) + (size_t)n * (lines + 4)) * sizeof(float); };
-        const cudaError_t e = raise_smem(kernel, bytes(kDctPlaneMax), done);
-        if (e != cudaSuccess) return e;
-        const dim3 grid((unsigned)((inner + lines - 1) / lines), (unsigned)nblocks_kd);
-        kernel<<<grid, dct_threads((split ? 2 : 1) * groups * (lines / 4), blocks), bytes(m), s>>>(in, out, tf, ti, inv_eig,
-                                                                                                m, inner, vec_in);
-        return cudaGetLastError();
-    };
-    static bool done[3][64] = {};
-    if (blocks < reduce_block_cap() / 4) return run(dct_last_half_kernel<32, true>, 32, true, done[0]);
-    if (2 * groups * (kDctFusedLines / 4) <= kBlock) return run(dct_last_half_kernel<64, true>, 64, true, done[1]);
-    return run(dct_last_half_kernel<64, false>, 64, false, done[2]);
+    if (blocks < reduce_block_cap() / 4)
+        return full ? run_last<32, true, true>(in, out, Tf, Ti, inv_eig, m, inner, nblocks_kd, blocks, s)
+                    : run_last<32, true, false>(in, out, Tf, Ti, inv_eig, m, inner, nblocks_kd, blocks, s);
+    if (2 * groups * (kDctFusedLines / 4) <= kBlock)
+        return full ? run_last<64, true, true>(in, out, Tf, Ti, inv_eig, m, inner, nblocks_kd, blocks, s)
+                    : run_last<64, true, false>(in, out, Tf, Ti, inv_eig, m, inner, nblocks_kd, blocks, s);
+    return full ? run_last<64, false, true>(in, out, Tf, Ti, inv_eig, m, inner, nblocks_kd, blocks, s)
+                : run_last<64, false, false>(in, out, Tf, Ti, inv_eig, m, inner, nblocks_kd, blocks, s);
 }
 
 cudaError_t launch_scale_modes(float* x, const float* inv_eig, size_t block_elems, size_t count, cudaStream_t s) {

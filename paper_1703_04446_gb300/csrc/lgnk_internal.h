@@ -173,30 +173,29 @@ cudaError_t launch_divergence(int d, const float* x, float* div, const DevGrid& 
 // out_c = addsrc + smu * A x_c + slm * D_c^T div + gamma * x_c (elastic operator)
 cudaError_t launch_elastic(int d, const float* x, const float* div, float* out, const DevGrid& g, int K,
                            float smu, float slm, float gamma, const float* addsrc, cudaStream_t s);
-// one axis of the spectral transform: C the m x m matrix (untiled kernel,
-// axes of more than 128 cells), Cp its padded table of the direction (Cf
-// forward, Ci inverse; tiled kernel)
-cudaError_t launch_dct_axis(const float* in, float* out, const float* C, const float* Cp, const DevGrid& g, int d,
-                            int nblocks_kd, int axis, bool inverse, cudaStream_t s);
-// Half tables of an axis (forward and inverse; see the transforms by halves in
-// grid_ops.cu) from its orthonormal DCT-II matrix C (host memory): dct_half_floats(m)
-// floats each, for axes that dct_half_axis_ok.
-size_t dct_half_floats(int m);
-bool dct_half_axis_ok(int m);
-void dct_half_tables(const float* C, int m, float* f, float* i);
-// The y and x axes of the spectral transform on whole xy planes with the half
-// tables of one direction: planes = blocks x z-planes.  cudaErrorNotSupported for
-// larger planes (the per-axis kernels cover them).
-cudaError_t launch_dct_plane(const float* in, float* out, const float* Tx, const float* Ty, bool inverse, const DevGrid& g,
-                             long long planes, cudaStream_t s);
+// The spectral transforms.  An axis of at most 128 cells (dct_table_ok) has two
+// tables, forward and inverse, of dct_table_floats(m) floats each, made on the host from
+// its orthonormal DCT-II matrix C (see DctTable in grid_ops.cu); a longer axis has C
+// itself.  full: every sum over the whole axis in increasing order; else by even and
+// odd halves, half the operations, where the kernel has that form.
+bool dct_table_ok(int m);
+size_t dct_table_floats(int m);
+void dct_tables(const float* C, int m, float* f, float* i);
+bool dct_plane_ok(int mx, int my, bool full);
+// one axis (C: the axis's table of the direction, or its matrix); always full sums
+cudaError_t launch_dct_axis(const float* in, float* out, const float* C, const DevGrid& g, int nblocks_kd, int axis,
+                            bool inverse, cudaStream_t s);
+// The y and x axes on whole xy planes (dct_plane_ok) with the tables of one direction:
+// planes = blocks x z-planes
+cudaError_t launch_dct_plane(const float* in, float* out, const float* Tx, const float* Ty, bool inverse, bool full,
+                             const DevGrid& g, long long planes, cudaStream_t s);
 // The whole 2D preconditioner (forward transform, inv_eig, inverse) with one CTA
-// per (time node, component) plane.
+// per (time node, component) plane (dct_plane_ok); by halves only
 cudaError_t launch_dct_plane2d(const float* in, float* out, const float* Fx, const float* Fy, const float* Ix,
                                const float* Iy, const float* inv_eig, const DevGrid& g, int blocks, cudaStream_t s);
-// forward DCT, scale by inv_eig and inverse DCT along the last axis in one pass
-// (the axis's half tables); cudaErrorNotSupported when that axis is too long
-cudaError_t launch_dct_last_half(const float* in, float* out, const float* Tf, const float* Ti, const float* inv_eig,
-                                 const DevGrid& g, int d, int nblocks_kd, cudaStream_t s);
+// forward DCT, scale by inv_eig and inverse DCT along the last axis (dct_table_ok) in one pass
+cudaError_t launch_dct_last(const float* in, float* out, const float* Tf, const float* Ti, const float* inv_eig,
+                            bool full, const DevGrid& g, int d, int nblocks_kd, cudaStream_t s);
 cudaError_t launch_scale_modes(float* x, const float* inv_eig, size_t block_elems, size_t count,
                                cudaStream_t s);
 // y = a * x + b * y  (count floats)
