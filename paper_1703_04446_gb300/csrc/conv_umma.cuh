@@ -98,6 +98,13 @@ struct ConvGemm {
 // one before it: it may start (barriers, tensor memory, constants) while that
 // one still runs, and touches global memory only after dependency_wait(), which
 // returns when that kernel (which waited the same way) has completed.
+//
+// A kernel that allocates tensor memory triggers after the allocation, past the
+// barrier that publishes its address.  tcgen05.alloc waits without a bound until the
+// columns are free; a dependent that took them first would hold them in its
+// dependency_wait(), for the very kernel that waits for the columns.  Since a
+// dependent starts only when every CTA before it has triggered, every holder of
+// columns waits for kernels that have theirs, so each allocation ends.
 __device__ __forceinline__ void dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -277,7 +284,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool bw = g.kind == BWD_WEIGHT;
     const uint32_t alloc_cols = 2u * (uint32_t)g.ncols;
-    dependency_trigger();
 
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
@@ -301,6 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
+    dependency_trigger();                 // the CTA has its tensor memory (see dependency_trigger)
     dependency_wait();
     const uint32_t tmem = tmem_base;
     const uint32_t smem0 = smem_u32(smem);

@@ -218,7 +218,6 @@ __global__ void __launch_bounds__(128) conv_first_kernel(const float* __restrict
     uint8_t* sb = sm + 3 * kFirstK * 2048;      // B: [k group][row] x 16 bytes; A: [plane][k group][row] x 16 bytes
     float* bs = reinterpret_cast<float*>(sb + kFirstK * bn * 16);
     const int tid = threadIdx.x, warp = tid >> 5;
-    umma::dependency_trigger();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(umma::smem_u32(&tmem_base)),
                      "r"(ncols));
@@ -229,6 +228,8 @@ __global__ void __launch_bounds__(128) conv_first_kernel(const float* __restrict
         umma::mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
+    __syncthreads();
+    umma::dependency_trigger();           // the CTA has its tensor memory (see dependency_trigger)
     umma::dependency_wait();
     for (int i = tid; i < kFirstK * bn; i += 128) {
         const int tap = i / bn, n = i - tap * bn;

@@ -1,0 +1,54 @@
+"""What the warm-start kernels' overlap rests on, read from their source (the
+faults these rules keep out would hang or fault a GPU, so nothing here runs).
+
+Every kernel of a network pass is a programmatic dependent of the one before:
+it may be resident while that one runs, until its dependency_wait() returns."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1703_04446_gb300", "csrc")
+
+
+def _kernels():
+    """{name: (parameters, body)} of the __global__ functions of the network, comments removed."""
+    out = {}
+    for name in ("conv_umma.cuh", "warmstart.cu"):
+        src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        for m in re.finditer(r"__global__ void (?:__launch_bounds__\([^()]*\)\s*)?(\w+)\(", src):
+            i, depth = m.end(), 1
+            while depth:
+                depth += {"(": 1, ")": -1}.get(src[i], 0)
+                i += 1
+            params = src[m.end():i - 1]
+            i = j = src.index("{", i)
+            depth = 0
+            while True:
+                depth += {"{": 1, "}": -1}.get(src[j], 0)
+                j += 1
+                if depth == 0:
+                    break
+            out[m.group(1)] = (params, src[i:j])
+    return out
+
+
+KERNELS = _kernels()
+
+
+def test_the_kernels_were_found():
+    assert {"conv_gemm_kernel", "finish_split_kernel", "conv_first_kernel", "conv_first_wgrad_kernel",
+            "mask_split_kernel", "sum_slices_kernel", "pack_wmats_kernel", "mse_kernel", "adam_kernel"} <= set(KERNELS)
+
+
+@pytest.mark.parametrize("name", sorted(KERNELS))
+def test_every_kernel_triggers_and_waits_once(name):
+    body = KERNELS[name][1]
+    assert body.count("dependency_trigger()") == 1 and body.count("dependency_wait()") == 1
+
+
+@pytest.mark.parametrize("name", sorted(k for k in KERNELS if "tcgen05.alloc" in KERNELS[k][1]))
+def test_dependents_start_after_the_tensor_memory_is_allocated(name):
+    body = KERNELS[name][1]
+    alloc, trigger = body.index("tcgen05.alloc"), body.index("dependency_trigger()")
+    assert alloc < trigger and "__syncthreads()" in body[alloc:trigger]
