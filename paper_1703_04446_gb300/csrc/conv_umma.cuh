@@ -43,8 +43,9 @@
 // gradient, which split FP32 elements on the fly, 1.7 ms.
 //
 // Every mbarrier wait is bounded; a wait that runs out sets an error flag and
-// a flag that ends the CTA's other roles, the CTA then waits (bounded) for its
-// copies and MMAs in flight and frees the tensor memory.
+// a flag that ends the CTA's other roles.  The TMA and the MMA role always end with a
+// bounded wait for their copies and MMAs in flight (mbar_drain), and only then the
+// CTA frees the tensor memory.
 #pragma once
 
 #include <cuda.h>
@@ -171,6 +172,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     }
     *dead = 1;
     return false;
+}
+
+// Bounded wait that no other role's giving up cuts short: a role ends with it on the
+// copies (MMAs) that it has issued, whichever role gave up, so that they land before
+// the CTA frees its memory.  Without a give-up they have landed, or the epilogue waits for
+// them anyway.
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity, volatile int* dead) {
+    for (long i = 0; i < kWaitLimit; ++i)
+        if (mbar_try(bar, parity)) return;
+    *dead = 1;
 }
 
 __device__ __forceinline__ void tma_5d(uint32_t dst, const CUtensorMap* map, uint64_t* bar, int c, int x, int y, int b) {
@@ -365,11 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
             }
-            // the copies still in flight land before the CTA may end (bounded)
-            for (int k = max(0, n - S); !ok && k < n; ++k) {
-                for (long i = 0; i < kWaitLimit && !mbar_try(&full[k % S], (uint32_t)((k / S) & 1)); ++i) {
-                }
-            }
+            for (int k = max(0, n - S); k < n; ++k) mbar_drain(&full[k % S], (uint32_t)((k / S) & 1), &dead);
         }
     } else if (warp == 1) {
         // ---- MMA: one elected thread
@@ -440,11 +447,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (issued) mma_commit(&accf[ab]);
                 else mbar_arrive(&accf[ab]);                    // an empty slice of K
             }
-            // bounded wait for the MMAs still in flight
-            if (!ok && n > 0) {
-                for (long i = 0; i < kWaitLimit && !mbar_try(&empty[(n - 1) % S], (uint32_t)(((n - 1) / S) & 1)); ++i) {
-                }
-            }
+            if (n > 0) mbar_drain(&empty[(n - 1) % S], (uint32_t)(((n - 1) / S) & 1), &dead);
         }
     } else {
         // ---- epilogue: warp w reads the tensor-memory lanes 32 (w mod 4) ..

@@ -52,3 +52,15 @@ def test_dependents_start_after_the_tensor_memory_is_allocated(name):
     body = KERNELS[name][1]
     alloc, trigger = body.index("tcgen05.alloc"), body.index("dependency_trigger()")
     assert alloc < trigger and "__syncthreads()" in body[alloc:trigger]
+
+
+def test_both_issuing_roles_drain_whatever_role_gave_up():
+    """The last copies (full barriers) and the last MMAs (empty barrier) are waited for
+    without a look at whether this role's own waits succeeded."""
+    body = KERNELS["conv_gemm_kernel"][1]
+    loops = body.index("if (warp == 0)")
+    for bar in ("full", "empty"):
+        waits = [m.start() for m in re.finditer(r"mbar_drain\(&%s\[" % bar, body)]
+        assert len(waits) == 1 and waits[0] > loops
+        statement = body[max(body.rfind(c, 0, waits[0]) for c in "{}"):waits[0]]
+        assert "ok" not in statement
