@@ -109,6 +109,27 @@ struct ConvGemm {
 __device__ __forceinline__ void dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Loads of global memory in these kernels.  A kernel may be resident while an earlier
+// one (or the caller's own kernel before the pass) still writes what it reads, so its data is
+// not read-only for the kernel's lifetime, which is what the non-coherent path (__ldg,
+// const __restrict__) asks for: plain loads, volatile so that none moves above
+// dependency_wait().
+__device__ __forceinline__ float ld(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ld(const uint2* p) {
+    uint2 v;
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 ld(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Shared-memory matrix descriptor.  kb = 64, 32, 16: a swizzled tile whose rows
@@ -507,11 +528,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                     float z[16];
                     const size_t oi = ((size_t)b * g.co + n0) * P + o;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) z[j] = g.add != nullptr && n0 + j < g.N ? __ldg(g.add + oi + j * P) : 0.0f;
+                    for (int j = 0; j < 16; ++j) z[j] = g.add != nullptr && n0 + j < g.N ? ld(g.add + oi + j * P) : 0.0f;
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const bool in = n0 + j < g.N;
-                        float t1 = __uint_as_float(v[j]) + (in ? __ldg(g.bias + n0 + j) : 0.0f);
+                        float t1 = __uint_as_float(v[j]) + (in ? ld(g.bias + n0 + j) : 0.0f);
                         if (g.relu) t1 = fmaxf(t1, 0.0f);
                         if (g.r != nullptr && in) g.r[oi + j * P] = t1;
                         if (g.add != nullptr) t1 += z[j];
@@ -527,7 +548,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     float* p = g.out + ((size_t)b * g.ci + n0) * P + o;
                     float z[16];
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) z[j] = g.accumulate && n0 + j < g.N ? p[j * P] : 0.0f;
+                    for (int j = 0; j < 16; ++j) z[j] = g.accumulate && n0 + j < g.N ? ld(p + j * P) : 0.0f;
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
                         if (n0 + j < g.N) p[j * P] = z[j] + __uint_as_float(v[j]);
@@ -565,17 +586,17 @@ __global__ void finish_split_kernel(const ConvGemm g, int splits) {
             const float* p = g.part + ((size_t)z * g.N + n0) * M + row;
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-                if (n0 + j < g.N) acc[j] += p[j * M];
+                if (n0 + j < g.N) acc[j] += ld(p + j * M);
         }
         const size_t oi = (b * C + n0) * P + o;
         if (g.kind == FWD) {
             float z[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) z[j] = g.add != nullptr && n0 + j < g.N ? __ldg(g.add + oi + j * P) : 0.0f;
+            for (int j = 0; j < 8; ++j) z[j] = g.add != nullptr && n0 + j < g.N ? ld(g.add + oi + j * P) : 0.0f;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const bool in = n0 + j < g.N;
-                float t = acc[j] + (in ? __ldg(g.bias + n0 + j) : 0.0f);
+                float t = acc[j] + (in ? ld(g.bias + n0 + j) : 0.0f);
                 if (g.relu) t = fmaxf(t, 0.0f);
                 if (g.r != nullptr && in) g.r[oi + j * P] = t;
                 if (g.add != nullptr) t += z[j];
@@ -586,7 +607,7 @@ __global__ void finish_split_kernel(const ConvGemm g, int splits) {
         } else {
             float z[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) z[j] = g.accumulate && n0 + j < g.N ? g.out[oi + j * P] : 0.0f;
+            for (int j = 0; j < 8; ++j) z[j] = g.accumulate && n0 + j < g.N ? ld(g.out + oi + j * P) : 0.0f;
 #pragma unroll
             for (int j = 0; j < 8; ++j)
                 if (n0 + j < g.N) g.out[oi + j * P] = z[j] + acc[j];

@@ -88,7 +88,7 @@ struct Layers {
 
 // The GEMMs' weight matrices from the FP32 master weights (bf16, nearest), layer
 // 1 + blockIdx.y.
-__global__ void pack_wmats_kernel(const float* __restrict__ p, const Layers all) {
+__global__ void pack_wmats_kernel(const float* p, const Layers all) {
     umma::dependency_trigger();
     umma::dependency_wait();
     const Layer L = all.l[1 + blockIdx.y];
@@ -100,13 +100,13 @@ __global__ void pack_wmats_kernel(const float* __restrict__ p, const Layers all)
         if (i < nf) {
             const int n = (int)(i / L.ldf), k = (int)(i % L.ldf);
             const int t = k / L.cpi, c = k - t * L.cpi;
-            if (n < L.co && t < 9 && c < L.ci) v = W[((size_t)n * L.ci + c) * 9 + t];
+            if (n < L.co && t < 9 && c < L.ci) v = umma::ld(W + ((size_t)n * L.ci + c) * 9 + t);
             L.wf[i] = __float2bfloat16_rn(v);
         } else {
             const size_t j = i - nf;
             const int n = (int)(j / L.ldd), k = (int)(j % L.ldd);
             const int pos = k / L.cpo, cc = k - pos * L.cpo, t = pos / R;
-            if (n < L.ci && t < 9 && cc < L.co) v = W[((size_t)cc * L.ci + n) * 9 + t];
+            if (n < L.ci && t < 9 && cc < L.co) v = umma::ld(W + ((size_t)cc * L.ci + n) * 9 + t);
             L.wd[j] = __float2bfloat16_rn(v);
         }
     }
@@ -115,7 +115,7 @@ __global__ void pack_wmats_kernel(const float* __restrict__ p, const Layers all)
 // The end of a layer's weight and bias gradients, partials summed in increasing
 // order: dW[co][ci][tap] = sum_s part[s][co][tap cp + ci], and behind it
 // db[co] = sum_s bpart[s][co].
-__global__ void sum_slices_kernel(const float* __restrict__ part, const float* __restrict__ bpart, float* dW, int co,
+__global__ void sum_slices_kernel(const float* part, const float* bpart, float* dW, int co,
                                   int ci, int cp, int slices, int bslices) {
     const int nw = co * ci * 9, rows = 9 * cp;
     umma::dependency_trigger();
@@ -126,10 +126,10 @@ __global__ void sum_slices_kernel(const float* __restrict__ part, const float* _
             const int n = i / (ci * 9), r = i - n * ci * 9, c = r / 9, t = r - c * 9;
             const float* p = part + (size_t)n * rows + t * cp + c;
 #pragma unroll 8
-            for (int k = 0; k < slices; ++k) s += p[(size_t)k * co * rows];
+            for (int k = 0; k < slices; ++k) s += umma::ld(p + (size_t)k * co * rows);
         } else {
 #pragma unroll 8
-            for (int k = 0; k < bslices; ++k) s += bpart[(size_t)k * co + i - nw];
+            for (int k = 0; k < bslices; ++k) s += umma::ld(bpart + (size_t)k * co + i - nw);
         }
         dW[i] = s;
     }
@@ -144,8 +144,8 @@ __global__ void sum_slices_kernel(const float* __restrict__ part, const float* _
 // groups of 8 (16) pixels, so that reads (channel rows) and writes (pixels)
 // both touch whole sectors.
 constexpr int kBiasSlices = 152;
-__global__ void __launch_bounds__(kT) mask_split_kernel(const float* __restrict__ g, const float* __restrict__ mr,
-                                                        const __nv_bfloat16* __restrict__ mp, __nv_bfloat16* planes,
+__global__ void __launch_bounds__(kT) mask_split_kernel(const float* g, const float* mr,
+                                                        const __nv_bfloat16* mp, __nv_bfloat16* planes,
                                                         float* bpart, int C, int cp, int P, int B, int gs) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pw = 32 / gs;      // pixels per warp
     const int c0 = (blockIdx.y * gs + lane / pw) * 8;
@@ -160,17 +160,17 @@ __global__ void __launch_bounds__(kT) mask_split_kernel(const float* __restrict_
         const size_t b = pix / P, o = pix - b * P, e = pix * cp + c0;
         float v[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = c0 + j < C ? __ldg(g + (b * C + c0 + j) * P + o) : 0.0f;
+        for (int j = 0; j < 8; ++j) v[j] = c0 + j < C ? umma::ld(g + (b * C + c0 + j) * P + o) : 0.0f;
         if (mr != nullptr) {
             float r[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) r[j] = c0 + j < C ? __ldg(mr + (b * C + c0 + j) * P + o) : 0.0f;
+            for (int j = 0; j < 8; ++j) r[j] = c0 + j < C ? umma::ld(mr + (b * C + c0 + j) * P + o) : 0.0f;
 #pragma unroll
             for (int j = 0; j < 8; ++j)
                 if (!(r[j] > 0.0f)) v[j] = 0.0f;
         } else if (mp != nullptr) {
             __align__(16) __nv_bfloat16 m[8];
-            *reinterpret_cast<uint4*>(m) = __ldg(reinterpret_cast<const uint4*>(mp + e));
+            *reinterpret_cast<uint4*>(m) = umma::ld(reinterpret_cast<const uint4*>(mp + e));
 #pragma unroll
             for (int j = 0; j < 8; ++j)
                 if (!(__bfloat162float(m[j]) > 0.0f)) v[j] = 0.0f;
@@ -207,8 +207,8 @@ __global__ void __launch_bounds__(kT) mask_split_kernel(const float* __restrict_
 // with the plane products innermost; the rounding of e0 decides its ReLU, and
 // with it whole gradient entries.
 constexpr int kFirstK = 10;       // 16-byte groups of K
-__global__ void __launch_bounds__(128) conv_first_kernel(const float* __restrict__ T, const float* __restrict__ R,
-                                                         const float* __restrict__ W, const float* __restrict__ bias,
+__global__ void __launch_bounds__(128) conv_first_kernel(const float* T, const float* R,
+                                                         const float* W, const float* bias,
                                                          __nv_bfloat16* planes, int C, int bn, int cp, int m, int B,
                                                          int tiles, int ncols, int* err) {
     extern __shared__ __align__(128) uint8_t sm[];
@@ -236,10 +236,10 @@ __global__ void __launch_bounds__(128) conv_first_kernel(const float* __restrict
         __align__(16) __nv_bfloat16 w[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c)
-            w[c] = __float2bfloat16_rn(c < 2 && tap < 9 && n < C ? W[((size_t)n * 2 + c) * 9 + tap] : 0.0f);
+            w[c] = __float2bfloat16_rn(c < 2 && tap < 9 && n < C ? umma::ld(W + ((size_t)n * 2 + c) * 9 + tap) : 0.0f);
         *reinterpret_cast<uint4*>(sb + (size_t)i * 16) = *reinterpret_cast<const uint4*>(w);
     }
-    for (int i = tid; i < bn; i += 128) bs[i] = i < C ? bias[i] : 0.0f;
+    for (int i = tid; i < bn; i += 128) bs[i] = i < C ? umma::ld(bias + i) : 0.0f;
 #pragma unroll
     for (int p = 0; p < 3; ++p) *reinterpret_cast<uint4*>(sm + ((p * kFirstK + 9) * 128 + tid) * 16) = make_uint4(0, 0, 0, 0);
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -261,8 +261,8 @@ __global__ void __launch_bounds__(128) conv_first_kernel(const float* __restrict
             const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
             const bool in_img = valid && yy >= 0 && yy < m && xx >= 0 && xx < m;
             const size_t e = in_img ? b * P + (size_t)(yy * m + xx) : 0;
-            in[2 * t] = in_img ? __ldg(T + e) : 0.0f;
-            in[2 * t + 1] = in_img ? __ldg(R + e) : 0.0f;
+            in[2 * t] = in_img ? umma::ld(T + e) : 0.0f;
+            in[2 * t + 1] = in_img ? umma::ld(R + e) : 0.0f;
         }
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
@@ -330,9 +330,9 @@ __global__ void __launch_bounds__(128) conv_first_kernel(const float* __restrict
 // over the pixels of block column s.  A thread accumulates 18 x kFirstW products
 // over its pixels; a block sums them once.
 constexpr int kFirstW = 4;
-__global__ void __launch_bounds__(kT) conv_first_wgrad_kernel(const float* __restrict__ T, const float* __restrict__ R,
-                                                              const float* __restrict__ g,
-                                                              const __nv_bfloat16* __restrict__ e0, float* part,
+__global__ void __launch_bounds__(kT) conv_first_wgrad_kernel(const float* T, const float* R,
+                                                              const float* g,
+                                                              const __nv_bfloat16* e0, float* part,
                                                               float* bpart, int C, int cp, int m, int B) {
     const int c0 = blockIdx.y * kFirstW, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t P = (size_t)m * m, n = P * B;
@@ -347,11 +347,11 @@ __global__ void __launch_bounds__(kT) conv_first_wgrad_kernel(const float* __res
         const size_t b = i / P;
         const int o = (int)(i - b * P), y = o / m, x = o - y * m;
         __align__(8) __nv_bfloat16 h[kFirstW];
-        *reinterpret_cast<uint2*>(h) = __ldg(reinterpret_cast<const uint2*>(e0 + i * cp + c0));
+        *reinterpret_cast<uint2*>(h) = umma::ld(reinterpret_cast<const uint2*>(e0 + i * cp + c0));
         float z[kFirstW];
 #pragma unroll
         for (int j = 0; j < kFirstW; ++j) {
-            z[j] = c0 + j < C ? __ldg(g + (b * C + c0 + j) * P + o) : 0.0f;
+            z[j] = c0 + j < C ? umma::ld(g + (b * C + c0 + j) * P + o) : 0.0f;
             if (!(__bfloat162float(h[j]) > 0.0f)) z[j] = 0.0f;
             acc[j][18] += z[j];
         }
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(kT) conv_first_wgrad_kernel(const float* __res
             const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
             const bool ok = yy >= 0 && yy < m && xx >= 0 && xx < m;
             const size_t e = b * P + (size_t)(ok ? yy * m + xx : 0);
-            const float a = ok ? __ldg(T + e) : 0.0f, r = ok ? __ldg(R + e) : 0.0f;
+            const float a = ok ? umma::ld(T + e) : 0.0f, r = ok ? umma::ld(R + e) : 0.0f;
 #pragma unroll
             for (int j = 0; j < kFirstW; ++j) {
                 acc[j][2 * t] = fmaf(a, z[j], acc[j][2 * t]);
@@ -391,13 +391,13 @@ __global__ void __launch_bounds__(kT) conv_first_wgrad_kernel(const float* __res
 
 // loss partials (FP64) and the gradient of the loss with respect to the
 // unscaled output z (v = scale z): dz = (v - t) / (scale N).
-__global__ void mse_kernel(const float* __restrict__ v, const float* __restrict__ t, float* dz, size_t n, float scale,
+__global__ void mse_kernel(const float* v, const float* t, float* dz, size_t n, float scale,
                            double* partial) {
     umma::dependency_trigger();
     umma::dependency_wait();
     double s = 0.0;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float e = v[i] - t[i];
+        const float e = umma::ld(v + i) - umma::ld(t + i);
         s += (double)e * (double)e;
         dz[i] = e / (scale * (float)n);
     }
@@ -411,17 +411,17 @@ __global__ void mse_kernel(const float* __restrict__ v, const float* __restrict_
     if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
 
-__global__ void adam_kernel(float* p, const float* __restrict__ g, float* m, float* s, size_t n, float lr, float c1,
+__global__ void adam_kernel(float* p, const float* g, float* m, float* s, size_t n, float lr, float c1,
                             float c2) {
     umma::dependency_trigger();
     umma::dependency_wait();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = 0.9f * m[i] + 0.1f * gi;
-        const float si = 0.999f * s[i] + 0.001f * gi * gi;
+        const float gi = umma::ld(g + i);
+        const float mi = 0.9f * umma::ld(m + i) + 0.1f * gi;
+        const float si = 0.999f * umma::ld(s + i) + 0.001f * gi * gi;
         m[i] = mi;
         s[i] = si;
-        p[i] = p[i] - lr * (mi / c1) / (sqrtf(si / c2) + 1e-8f);
+        p[i] = umma::ld(p + i) - lr * (mi / c1) / (sqrtf(si / c2) + 1e-8f);
     }
 }
 

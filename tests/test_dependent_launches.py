@@ -64,3 +64,15 @@ def test_both_issuing_roles_drain_whatever_role_gave_up():
         assert len(waits) == 1 and waits[0] > loops
         statement = body[max(body.rfind(c, 0, waits[0]) for c in "{}"):waits[0]]
         assert "ok" not in statement
+
+
+@pytest.mark.parametrize("name", sorted(KERNELS))
+def test_no_load_takes_the_non_coherent_path(name):
+    """A buffer that an earlier kernel of the pass may still write is not read-only for the
+    reading kernel's lifetime: no __ldg, no const __restrict__ parameter, no plain
+    dereference that a compiler could turn into either (umma::ld is volatile)."""
+    params, body = KERNELS[name]
+    assert "__ldg" not in body and "__restrict__" not in params
+    pointers = re.findall(r"const (?:float|__nv_bfloat16)\s*\*\s*(\w+)", params)
+    for p in pointers:
+        assert not re.search(r"\b%s\[" % p, body), p
