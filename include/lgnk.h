@@ -313,7 +313,10 @@ lgnk_status lgnk_forward_transport_static(const lgnk_problem* prob, const float*
  * forward, backward and one Adam step with learning rate lr; loss: NULL or a
  * host double receiving the loss before the step (then the call synchronises
  * the stream).  lgnk_ws_get_grads copies the gradient of the last train step.
- * Errors: the status, with detail from lgnk_ws_last_error. */
+ * Errors: the status, with detail from lgnk_ws_last_error.  Should a wait inside a
+ * convolution run out (its waits are bounded), the weights are not updated from the
+ * unfinished results, and the call itself, if it synchronises, or else the next call on the
+ * network once the GPU has got there (set_params excepted) returns LGNK_ERR_INTERNAL, once. */
 typedef struct lgnk_ws lgnk_ws;
 lgnk_status lgnk_ws_create(int image_m, int base_channels, int max_batch, float scale, void* stream,
                            lgnk_ws** out);

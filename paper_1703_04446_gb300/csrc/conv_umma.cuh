@@ -92,8 +92,15 @@ struct ConvGemm {
     int relu;
     float scale;
     int accumulate;           // BWD_DATA: out += instead of out =
-    int* err;                 // set to 1 when a wait runs out
+    int *err, *herr;          // give_up when a wait runs out
 };
+
+// A wait ran out: err (device memory) keeps the weights from being updated with what is
+// unfinished, herr (pinned host memory) is what the network's next call reports.
+__device__ __forceinline__ void give_up(int* err, int* herr) {
+    atomicExch(err, 1);
+    *reinterpret_cast<volatile int*>(herr) = 1;
+}
 
 // Every kernel of a network pass is launched as a programmatic dependent of the
 // one before it: it may start (barriers, tensor memory, constants) while that
@@ -117,6 +124,11 @@ __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol
 __device__ __forceinline__ float ld(const float* p) {
     float v;
     asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int ld(const int* p) {
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
 __device__ __forceinline__ uint2 ld(const uint2* p) {
@@ -561,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (tid == 0 && dead) atomicExch(g.err, 1);
+    if (tid == 0 && dead) give_up(g.err, g.herr);
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(alloc_cols));
 }

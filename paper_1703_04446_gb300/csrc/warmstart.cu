@@ -87,10 +87,11 @@ struct Layers {
 };
 
 // The GEMMs' weight matrices from the FP32 master weights (bf16, nearest), layer
-// 1 + blockIdx.y.
-__global__ void pack_wmats_kernel(const float* p, const Layers all) {
+// 1 + blockIdx.y (left as they are when a wait ran out, as the master weights are).
+__global__ void pack_wmats_kernel(const float* p, const Layers all, const int* err) {
     umma::dependency_trigger();
     umma::dependency_wait();
+    if (umma::ld(err) != 0) return;
     const Layer L = all.l[1 + blockIdx.y];
     const size_t nf = (size_t)L.rowsf * L.ldf, nd = (size_t)L.rowsd * L.ldd;
     const int R = L.up ? 4 : 1;
@@ -210,7 +211,7 @@ constexpr int kFirstK = 10;       // 16-byte groups of K
 __global__ void __launch_bounds__(128) conv_first_kernel(const float* T, const float* R,
                                                          const float* W, const float* bias,
                                                          __nv_bfloat16* planes, int C, int bn, int cp, int m, int B,
-                                                         int tiles, int ncols, int* err) {
+                                                         int tiles, int ncols, int* err, int* herr) {
     extern __shared__ __align__(128) uint8_t sm[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tmem_base;
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(128) conv_first_kernel(const float* T, const f
     }
     if (!ok) {            // once more, bounded, for the MMAs in flight
         if (tid == 0) {
-            atomicExch(err, 1);
+            umma::give_up(err, herr);
             for (long k = 0; k < umma::kWaitLimit && !umma::mbar_try(&bar, phase); ++k) {
             }
         }
@@ -411,10 +412,12 @@ __global__ void mse_kernel(const float* v, const float* t, float* dz, size_t n, 
     if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
 
-__global__ void adam_kernel(float* p, const float* g, float* m, float* s, size_t n, float lr, float c1,
-                            float c2) {
+// No update from a step in which a wait ran out.
+__global__ void adam_kernel(float* p, const float* g, float* m, float* s, size_t n, float lr, float c1, float c2,
+                            const int* err) {
     umma::dependency_trigger();
     umma::dependency_wait();
+    if (umma::ld(err) != 0) return;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float gi = umma::ld(g + i);
         const float mi = 0.9f * umma::ld(m + i) + 0.1f * gi;
@@ -423,6 +426,12 @@ __global__ void adam_kernel(float* p, const float* g, float* m, float* s, size_t
         s[i] = si;
         p[i] = umma::ld(p + i) - lr * (mi / c1) / (sqrtf(si / c2) + 1e-8f);
     }
+}
+
+__global__ void give_up_kernel(int* err, int* herr) {
+    umma::dependency_trigger();
+    umma::dependency_wait();
+    umma::give_up(err, herr);
 }
 
 inline int blocks_for(size_t n) {
@@ -449,7 +458,7 @@ struct lgnk_ws {
     int sms, smem_max;          // of the device: SMs, dynamic shared memory of the GEMM kernel
     float* gpart;               // split-K partial tiles of the FWD and BWD_DATA GEMMs
     size_t gpart_cap;           // floats it holds
-    int* derr;                  // set by a tensor-core kernel whose wait ran out
+    int *derr, *herr;           // set by a tensor-core kernel whose wait ran out (umma::give_up)
     double* partial;
     double* hres;
     long long steps;
@@ -635,6 +644,7 @@ cudaError_t gemm_plan(lgnk_ws* w, int l, int kind, int B, Plan** out) {
     p.smem = (size_t)g.stages * g.stage_bytes + 1024;
     p.grid = std::min(g.items, w->sms);
     g.err = w->derr;
+    g.herr = w->herr;
     if (kind == umma::BWD_WEIGHT) g.part = w->wpart;
     else {
         g.part = w->gpart;
@@ -707,7 +717,7 @@ cudaError_t pack_weights(lgnk_ws* w) {
         all.l[l] = w->L[l];
         if (l > 0) n = std::max(n, (size_t)w->L[l].rowsf * w->L[l].ldf + (size_t)w->L[l].rowsd * w->L[l].ldd);
     }
-    return launch(pack_wmats_kernel, dim3(std::min(blocks_for(n), 608), 6), kT, 0, w->stream, w->p, all);
+    return launch(pack_wmats_kernel, dim3(std::min(blocks_for(n), 608), 6), kT, 0, w->stream, w->p, all, w->derr);
 }
 
 // Shared memory of the first layer's kernel, and its CTAs per SM (bounded by
@@ -723,7 +733,7 @@ lgnk_status forward_pass(lgnk_ws* w, int B, const float* T, const float* R, floa
     const int ncols = bn <= 32 ? 32 : (bn <= 64 ? 64 : (bn <= 128 ? 128 : 256));
     cudaError_t e = launch(conv_first_kernel, dim3(std::min(tiles, first_ctas(bn) * w->sms)), 128, first_smem(bn), w->stream,
                            T, R, w->p + L0.woff, w->p + L0.boff, w->planes[1], L0.co, bn, bn, w->m, B, tiles, ncols,
-                           w->derr);
+                           w->derr, w->herr);
     if (e == cudaSuccess) e = conv_fwd(w, 1, w->e1, nullptr, nullptr, 1, 1.0f, B);
     if (e == cudaSuccess) e = conv_fwd(w, 2, w->e2, nullptr, nullptr, 1, 1.0f, B);
     if (e == cudaSuccess) e = conv_fwd(w, 3, nullptr, nullptr, nullptr, 1, 1.0f, B);
@@ -735,6 +745,17 @@ lgnk_status forward_pass(lgnk_ws* w, int B, const float* T, const float* R, floa
         return LGNK_ERR_CUDA;
     }
     return LGNK_OK;
+}
+
+// What a call on the network begins with (and a synchronising one ends with): an error if an
+// earlier one's wait ran out, cleared as it is reported.
+lgnk_status report_give_up(lgnk_ws* w) {
+    if (*static_cast<volatile int*>(w->herr) == 0) return LGNK_OK;
+    *static_cast<volatile int*>(w->herr) = 0;
+    snprintf(w->err, sizeof(w->err), "a tensor-core convolution of an earlier call gave up waiting: its results are "
+             "unfinished (the weights were not updated from them)");
+    if (cudaMemsetAsync(w->derr, 0, sizeof(int), w->stream) != cudaSuccess) return LGNK_ERR_CUDA;
+    return LGNK_ERR_INTERNAL;
 }
 
 }  // namespace
@@ -877,6 +898,8 @@ lgnk_status lgnk_ws_create(int image_m, int base_channels, int max_batch, float 
         w->hres = nullptr;
         return fail(LGNK_ERR_OOM);
     }
+    w->herr = reinterpret_cast<int*>(w->hres + 7);
+    *w->herr = 0;
     if (cudaMemsetAsync(w->p, 0, off * sizeof(float), w->stream) != cudaSuccess ||
         cudaMemsetAsync(w->am, 0, off * sizeof(float), w->stream) != cudaSuccess ||
         cudaMemsetAsync(w->as, 0, off * sizeof(float), w->stream) != cudaSuccess ||
@@ -892,6 +915,7 @@ const char* lgnk_ws_last_error(const lgnk_ws* w) { return w ? w->err : "null net
 
 lgnk_status lgnk_ws_set_params(lgnk_ws* w, const float* params) {
     if (w == nullptr || params == nullptr) return LGNK_ERR_INVALID_ARG;
+    WS_CHECK(cudaMemsetAsync(w->derr, 0, sizeof(int), w->stream));      // new weights, new start
     WS_CHECK(cudaMemcpyAsync(w->p, params, w->nparams * sizeof(float), cudaMemcpyDeviceToDevice, w->stream));
     WS_CHECK(pack_weights(w));
     WS_CHECK(cudaMemsetAsync(w->am, 0, w->nparams * sizeof(float), w->stream));
@@ -902,12 +926,14 @@ lgnk_status lgnk_ws_set_params(lgnk_ws* w, const float* params) {
 
 lgnk_status lgnk_ws_get_params(lgnk_ws* w, float* params) {
     if (w == nullptr || params == nullptr) return LGNK_ERR_INVALID_ARG;
+    if (const lgnk_status st = report_give_up(w)) return st;
     WS_CHECK(cudaMemcpyAsync(params, w->p, w->nparams * sizeof(float), cudaMemcpyDeviceToDevice, w->stream));
     return LGNK_OK;
 }
 
 lgnk_status lgnk_ws_get_grads(lgnk_ws* w, float* grads) {
     if (w == nullptr || grads == nullptr) return LGNK_ERR_INVALID_ARG;
+    if (const lgnk_status st = report_give_up(w)) return st;
     WS_CHECK(cudaMemcpyAsync(grads, w->g, w->nparams * sizeof(float), cudaMemcpyDeviceToDevice, w->stream));
     return LGNK_OK;
 }
@@ -915,6 +941,7 @@ lgnk_status lgnk_ws_get_grads(lgnk_ws* w, float* grads) {
 lgnk_status lgnk_ws_predict(lgnk_ws* w, int batch, const float* T, const float* R, float* v) {
     if (w == nullptr || T == nullptr || R == nullptr || v == nullptr || batch < 1 || batch > w->max_batch)
         return LGNK_ERR_INVALID_ARG;
+    if (const lgnk_status st = report_give_up(w)) return st;
     return forward_pass(w, batch, T, R, v, false);
 }
 
@@ -923,7 +950,8 @@ lgnk_status lgnk_ws_train_step(lgnk_ws* w, int batch, const float* T, const floa
     if (w == nullptr || T == nullptr || R == nullptr || target == nullptr || batch < 1 || batch > w->max_batch)
         return LGNK_ERR_INVALID_ARG;
     const int B = batch;
-    lgnk_status st = forward_pass(w, B, T, R, w->z6, true);
+    lgnk_status st = report_give_up(w);
+    if (st == LGNK_OK) st = forward_pass(w, B, T, R, w->z6, true);
     if (st != LGNK_OK) return st;
     const int m = w->m;
     // loss and dz6 (gradient w.r.t. the unscaled output)
@@ -958,23 +986,20 @@ lgnk_status lgnk_ws_train_step(lgnk_ws* w, int batch, const float* T, const floa
     w->steps++;
     const float c1 = 1.0f - powf(0.9f, (float)w->steps), c2 = 1.0f - powf(0.999f, (float)w->steps);
     WS_CHECK(launch(adam_kernel, dim3(blocks_for(w->nparams)), kT, 0, w->stream, w->p, w->g, w->am, w->as, w->nparams, lr,
-                    c1, c2));
+                    c1, c2, w->derr));
     WS_CHECK(pack_weights(w));
     if (loss != nullptr) {
         launch_reduce(w->partial, nb, w->partial + 2048, w->stream);
         WS_CHECK(cudaGetLastError());
         WS_CHECK(cudaMemcpyAsync(w->hres, w->partial + 2048, sizeof(double), cudaMemcpyDeviceToHost, w->stream));
-        WS_CHECK(cudaMemcpyAsync(w->hres + 1, w->derr, sizeof(int), cudaMemcpyDeviceToHost, w->stream));
         WS_CHECK(cudaStreamSynchronize(w->stream));
-        int bad = 0;
-        memcpy(&bad, w->hres + 1, sizeof(int));
-        if (bad != 0) {
-            snprintf(w->err, sizeof(w->err), "a tensor-core convolution gave up waiting for its MMAs");
-            return LGNK_ERR_INTERNAL;
-        }
+        if ((st = report_give_up(w)) != LGNK_OK) return st;
         *loss = 0.5 * w->hres[0] / (double)nv / ((double)w->scale * w->scale);
     }
     return LGNK_OK;
 }
+
+// For the tests: enqueues what a kernel whose wait ran out does.
+void lgnk_internal_ws_give_up(lgnk_ws* w) { give_up_kernel<<<1, 1, 0, w->stream>>>(w->derr, w->herr); }
 
 }  // extern "C"
