@@ -144,7 +144,7 @@ __global__ void sum_slices_kernel(const float* part, const float* bpart, float* 
 // channels of one pixel at a time; a warp covers 4 (2) neighbouring channel
 // groups of 8 (16) pixels, so that reads (channel rows) and writes (pixels)
 // both touch whole sectors.
-constexpr int kBiasSlices = 152;
+constexpr int kBiasSlices = 152;     // at most: about one block a SM; also sizes the partials
 __global__ void __launch_bounds__(kT) mask_split_kernel(const float* g, const float* mr,
                                                         const __nv_bfloat16* mp, __nv_bfloat16* planes,
                                                         float* bpart, int C, int cp, int P, int B, int gs) {
@@ -488,15 +488,12 @@ lgnk_status ws_alloc_n(lgnk_ws* w, size_t n, T** out) {
 
 size_t act_size(const lgnk_ws* w, int layer_out_c, int side, int B) { return (size_t)B * layer_out_c * side * side; }
 
-// Tiles a split GEMM should reach: two per SM
-constexpr int kGemmCtas = 2 * 152;
-
 // K slices of a FWD / BWD_DATA GEMM with `tiles` output tiles and `chunks` K
-// chunks: enough slices to give about two tiles per SM, each at least two
-// chunks (1 when the tiles alone fill the GPU)
-inline int split_slices(int tiles, int chunks) {
-    if (tiles >= kGemmCtas) return 1;
-    const int s = std::min((kGemmCtas + tiles - 1) / tiles, std::max(1, chunks / 2));
+// chunks: enough slices to give about two tiles to each of the device's SMs, each at
+// least two chunks (1 when the tiles alone fill the GPU)
+inline int split_slices(int tiles, int chunks, int sms) {
+    if (tiles >= 2 * sms) return 1;
+    const int s = std::min((2 * sms + tiles - 1) / tiles, std::max(1, chunks / 2));
     const int cps = (chunks + s - 1) / s;
     return (chunks + cps - 1) / cps;
 }
@@ -525,7 +522,7 @@ void choose_box(int side, int batch, int total, umma::ConvGemm* g) {
 }
 
 // Everything of a layer's GEMM but its tensors, maps and stages.
-umma::ConvGemm gemm_shape(const Layer& L, int kind, int B) {
+umma::ConvGemm gemm_shape(const Layer& L, int kind, int B, int sms) {
     umma::ConvGemm g{};
     g.kind = kind;
     g.ci = L.ci;
@@ -549,7 +546,7 @@ umma::ConvGemm gemm_shape(const Layer& L, int kind, int B) {
         g.mtiles = (9 * g.cp + umma::BM - 1) / umma::BM;
         g.chunks = g.phases * g.tx * g.ty * g.tb;
         const int tiles = g.mtiles * g.ntn;
-        const int s = std::min(kMaxSlices, std::min(g.chunks, std::max(1, (kGemmCtas + tiles - 1) / tiles)));
+        const int s = std::min(kMaxSlices, std::min(g.chunks, std::max(1, (2 * sms + tiles - 1) / tiles)));
         g.chunks_per_split = (g.chunks + s - 1) / s;
         g.splits = (g.chunks + g.chunks_per_split - 1) / g.chunks_per_split;
         g.items = tiles * g.splits;
@@ -565,7 +562,7 @@ umma::ConvGemm gemm_shape(const Layer& L, int kind, int B) {
         choose_box(g.grid, B, umma::BM, &g);
         const int tiles = g.phases * g.tx * g.ty * g.tb * g.ntn;
         g.chunks = (9 * (!f && L.up ? 4 : 1) * g.cp + umma::BK - 1) / umma::BK;
-        const int s = split_slices(tiles, g.chunks);
+        const int s = split_slices(tiles, g.chunks, sms);
         g.chunks_per_split = (g.chunks + s - 1) / s;
         g.splits = (g.chunks + g.chunks_per_split - 1) / g.chunks_per_split;
         g.items = tiles * g.splits;
@@ -623,7 +620,7 @@ cudaError_t gemm_plan(lgnk_ws* w, int l, int kind, int B, Plan** out) {
     if (p.batch == B) return cudaSuccess;
     p.batch = 0;
     const Layer& L = w->L[l];
-    p.g = gemm_shape(L, kind, B);
+    p.g = gemm_shape(L, kind, B, w->sms);
     umma::ConvGemm& g = p.g;
     const EncodeTiled enc = encode_tiled();
     if (enc == nullptr) return cudaErrorNotSupported;
@@ -821,6 +818,28 @@ lgnk_status lgnk_ws_create(int image_m, int base_channels, int max_batch, float 
     if ((s = ws_alloc_n(w, off, &w->p)) || (s = ws_alloc_n(w, off, &w->g)) || (s = ws_alloc_n(w, off, &w->am)) ||
         (s = ws_alloc_n(w, off, &w->as)) || (s = ws_alloc_n(w, 1, &w->derr)))
         return fail(s);
+    {
+        int dev = 0, optin = 0;
+        cudaFuncAttributes fa{};
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&w->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+            cudaFuncGetAttributes(&fa, umma::conv_gemm_kernel) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(LGNK_ERR_CUDA);
+        }
+        w->smem_max = optin - (int)fa.sharedSizeBytes;
+        if (cudaFuncSetAttribute(conv_first_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)first_smem(256)) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return fail(LGNK_ERR_CUDA);
+        }
+        if (cudaFuncSetAttribute(umma::conv_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, w->smem_max) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return fail(LGNK_ERR_CUDA);
+        }
+    }
     // the GEMMs' bf16 weight matrices (N per CTA up to 256, rows and K padded)
     size_t zmax = 0;
     for (int l = 0; l < 7; ++l) {
@@ -847,7 +866,7 @@ lgnk_status lgnk_ws_create(int image_m, int base_channels, int max_batch, float 
         for (int l = 1; l < 7; ++l) {
             const Layer& L = w->L[l];
             for (int kind : {umma::FWD, umma::BWD_DATA}) {
-                const umma::ConvGemm g = gemm_shape(L, kind, b);
+                const umma::ConvGemm g = gemm_shape(L, kind, b, w->sms);
                 if (g.splits > 1) gmax = std::max(gmax, (size_t)g.splits * (size_t)g.M * g.N);
             }
         }
@@ -871,28 +890,6 @@ lgnk_status lgnk_ws_create(int image_m, int base_channels, int max_batch, float 
     }
     if ((s = ws_alloc_n(w, wmax * kMaxSlices, &w->wpart)) || (s = ws_alloc_n(w, bmax * kBiasSlices, &w->bpart)))
         return fail(s);
-    {
-        int dev = 0, optin = 0;
-        cudaFuncAttributes fa{};
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&w->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-            cudaFuncGetAttributes(&fa, umma::conv_gemm_kernel) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(LGNK_ERR_CUDA);
-        }
-        w->smem_max = optin - (int)fa.sharedSizeBytes;
-        if (cudaFuncSetAttribute(conv_first_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)first_smem(256)) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            return fail(LGNK_ERR_CUDA);
-        }
-        if (cudaFuncSetAttribute(umma::conv_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, w->smem_max) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            return fail(LGNK_ERR_CUDA);
-        }
-    }
     if (cudaMallocHost((void**)&w->hres, 8 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         w->hres = nullptr;

@@ -76,3 +76,10 @@ def test_no_load_takes_the_non_coherent_path(name):
     pointers = re.findall(r"const (?:float|__nv_bfloat16)\s*\*\s*(\w+)", params)
     for p in pointers:
         assert not re.search(r"\b%s\[" % p, body), p
+
+
+def test_gemm_splits_follow_the_device():
+    """How many K slices a GEMM gets depends on the SMs that its persistent CTAs run on,
+    which are read from the device: no SM count in the rule."""
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "warmstart.cu")).read())
+    assert re.findall(r"[^\n]*\b152\b[^\n]*", src) == ["constexpr int kBiasSlices = 152;     "]
