@@ -562,7 +562,10 @@ umma::ConvGemm gemm_shape(const Layer& L, int kind, int B, int sms) {
         choose_box(g.grid, B, umma::BM, &g);
         const int tiles = g.phases * g.tx * g.ty * g.tb * g.ntn;
         g.chunks = (9 * (!f && L.up ? 4 : 1) * g.cp + umma::BK - 1) / umma::BK;
-        const int s = split_slices(tiles, g.chunks, sms);
+        // the slices of K by the rows of D in tiles of 128, not by the boxes that cover them: they
+        // set the rounding of the sums, and a ReLU's sign with it (a gradient's entries jump there)
+        const int rows = (int)(((long long)B * ho * ho + umma::BM - 1) / umma::BM);
+        const int s = split_slices(rows * g.ntn, g.chunks, sms);
         g.chunks_per_split = (g.chunks + s - 1) / s;
         g.splits = (g.chunks + g.chunks_per_split - 1) / g.chunks_per_split;
         g.items = tiles * g.splits;
