@@ -54,9 +54,10 @@ struct PcgGraph {
 };
 
 // The whole PCG loop of one GN step as one graph: a while node whose body is
-// one iteration whose last inner product ends with the loop test (dot_blocks_finish), which ends the loop on the
-// stopping test, non-positive curvature or the iteration cap.  The host reads
-// the loop state once per GN step instead of once per iteration.
+// one iteration whose last inner product ends with the loop test
+// (dot_blocks_finish), which ends the loop on the stopping test, non-positive
+// curvature or the iteration cap.  The host reads the loop state once per GN step
+// instead of once per iteration.
 struct PcgLoopGraph {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -268,15 +269,11 @@ TraceArgs base_args(const lgnk_ctx* ctx) {
             const lgnk_grid& gi = ctx->prob.image;
             const lgnk_grid& gv = ctx->prob.velocity;
             const double hi = (gi.hi[i] - gi.lo[i]) / gi.m[i], hv = (gv.hi[i] - gv.lo[i]) / gv.m[i];
-            a.vxi_a[i] = (gi.lo[i] - gv.lo[i]) / hv - 0.5;
-            a.vxi_b[i] = hi / hv;
-            a.vxi_af[i] = (float)a.vxi_a[i];
-            a.vxi_bf[i] = (float)a.vxi_b[i];
+            a.vxi_a[i] = (float)((gi.lo[i] - gv.lo[i]) / hv - 0.5);
+            a.vxi_b[i] = (float)(hi / hv);
         } else {
-            a.vxi_a[i] = 0.0;
-            a.vxi_b[i] = 0.0;
-            a.vxi_af[i] = 0.0f;
-            a.vxi_bf[i] = 0.0f;
+            a.vxi_a[i] = 0.0f;
+            a.vxi_b[i] = 0.0f;
         }
     }
     for (int i = 0; i < 3; ++i)
@@ -911,7 +908,8 @@ lgnk_status lgnk_create(const lgnk_problem* prob, void* stream, size_t mem_budge
         if (tables) dct_tables(hostC.data(), m, hf.data(), hi.data());
         else hf = hostC;
         if (cudaMemcpy(ctx->Cf[a], hf.data(), hf.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
-            (tables && cudaMemcpy(ctx->Ci[a], hi.data(), hi.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess))
+            (tables &&
+             cudaMemcpy(ctx->Ci[a], hi.data(), hi.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess))
             return fail(LGNK_ERR_CUDA);
     }
     std::vector<double> pv(ctx->Mv);
@@ -1229,7 +1227,8 @@ lgnk_status solve_impl(lgnk_ctx* ctx, const float* T, const float* R, float* v, 
             const long long l0 = ctx->launches, t0 = ctx->trace_launches;
             cudaGraphConditionalHandle handle = 0;
             bool ok = cudaGraphCreate(&lg.graph, 0) == cudaSuccess;
-            ok = ok && cudaGraphConditionalHandleCreate(&handle, lg.graph, 1, cudaGraphCondAssignDefault) == cudaSuccess;
+            ok = ok &&
+                 cudaGraphConditionalHandleCreate(&handle, lg.graph, 1, cudaGraphCondAssignDefault) == cudaSuccess;
             cudaGraphNodeParams np = {cudaGraphNodeTypeConditional};   // the rest zero
             np.conditional.handle = handle;
             np.conditional.type = cudaGraphCondTypeWhile;

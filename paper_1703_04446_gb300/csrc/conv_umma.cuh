@@ -217,20 +217,31 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity, volat
     *dead = 1;
 }
 
-__device__ __forceinline__ void tma_5d(uint32_t dst, const CUtensorMap* map, uint64_t* bar, int c, int x, int y, int b) {
+__device__ __forceinline__ void tma_5d(uint32_t dst, const CUtensorMap* map, uint64_t* bar, int c, int x, int y,
+                                       int b) {
     asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], "
-        "[%2];" ::"r"(dst),
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(dst),
         "l"(map), "r"(smem_u32(bar)), "r"(c), "r"(x), "r"(y), "r"(b), "r"(0)
         : "memory");
 }
 
 __device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap* map, uint64_t* bar, int k, int row) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
-            dst),
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
         "l"(map), "r"(smem_u32(bar)), "r"(k), "r"(row)
         : "memory");
+}
+
+// 16 columns of this thread's tensor-memory lane
+__device__ __forceinline__ void tmem_ld16(uint32_t (&v)[16], uint32_t addr) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(addr));
 }
 
 // x = hi + mid + lo exactly (see the file comment)
@@ -466,8 +477,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                             for (int pz = 0; pz < 3; ++pz) {
 #pragma unroll
                                 for (int px = 0; px + pz <= 2; ++px) {
-                                    mma_bf16(d, ad + (uint32_t)px * aplane + kk * arow, bd + (uint32_t)pz * zplane + kk * zrow,
-                                             idesc, issued);
+                                    mma_bf16(d, ad + (uint32_t)px * aplane + kk * arow,
+                                             bd + (uint32_t)pz * zplane + kk * zrow, idesc, issued);
                                     issued = 1;
                                 }
                             }
@@ -521,11 +532,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int c0 = 0; c0 < g.bn; c0 += 16) {
                 uint32_t v[16];
                 const uint32_t ta = tmem + (uint32_t)(ab * g.ncols) + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                    : "r"(ta));
+                tmem_ld16(v, ta);
                 asm volatile("tcgen05.wait::ld.sync.aligned;");
                 if (!valid) continue;
                 const int n0 = t.nt * g.bn + c0;
@@ -540,7 +547,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     float z[16];
                     const size_t oi = ((size_t)b * g.co + n0) * P + o;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) z[j] = g.add != nullptr && n0 + j < g.N ? ld(g.add + oi + j * P) : 0.0f;
+                    for (int j = 0; j < 16; ++j)
+                        z[j] = g.add != nullptr && n0 + j < g.N ? ld(g.add + oi + j * P) : 0.0f;
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const bool in = n0 + j < g.N;

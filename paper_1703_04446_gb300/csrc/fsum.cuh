@@ -152,8 +152,8 @@ __device__ __forceinline__ lsum lsum_warp_sum(lsum a) {
 // other warps' lanes column by column and then its own lanes: 12 FP64
 // additions of a warp for 256 threads, where a shuffle tree in every warp is
 // 45, and at 16 cycles each on this GPU's FP64 pipe these were most of a small
-// inner product's time (and 465 -> 456 us for the 128^3 assembly trace).  Uses one shared array a SLOT, so two calls of one slot
-// need a __syncthreads() between them.
+// inner product's time (and 465 -> 456 us for the 128^3 assembly trace).  Uses one
+// shared array a SLOT, so two calls of one slot need a __syncthreads() between them.
 template <int SLOT = 0>
 __device__ __forceinline__ lsum lsum_block_sum(lsum a) {
     __shared__ lsum red[LGNK_BLOCK];

@@ -45,7 +45,8 @@ __device__ __forceinline__ void split_xyz(unsigned i, unsigned nx, unsigned ny, 
 // same pass.
 template <int D>
 __device__ __forceinline__ void pack_velocity(const float* __restrict__ v, float* __restrict__ Vp, const DevGrid& g,
-                                              const SliceTable& tab, void* Gz, int nz, unsigned block, unsigned blocks) {
+                                              const SliceTable& tab, void* Gz, int nz, unsigned block,
+                                              unsigned blocks) {
     const size_t nodes = padded_size(g);
     const size_t total = nodes * tab.n;
     const size_t zero = Gz != nullptr ? nodes * nz : 0;
@@ -109,7 +110,8 @@ __global__ void distribute_gradient_kernel(const float* __restrict__ Gp, float* 
         const size_t s = (unsigned)i - (unsigned)j * (unsigned)Mv;
         int x, y, z;
         split_xyz((unsigned)s, (unsigned)g.m[0], (unsigned)g.m[1], x, y, z);
-        const size_t node = ((size_t)(z + (D == 3 ? LGNK_PAD : 0)) * g.mp[1] + (y + LGNK_PAD)) * g.mp[0] + (x + LGNK_PAD);
+        const size_t node =
+            ((size_t)(z + (D == 3 ? LGNK_PAD : 0)) * g.mp[1] + (y + LGNK_PAD)) * g.mp[0] + (x + LGNK_PAD);
         float acc[3] = {0.0f, 0.0f, 0.0f};
         for (int m = 0; m < tab.n; ++m) {
             float w = 0.0f;
@@ -167,7 +169,8 @@ __global__ void __launch_bounds__(kBlock) pack_kernel(const PackArgs A) {
     }
     b -= (unsigned)A.blocks[2];
     const size_t total = padded_size(A.ig);
-    for (size_t i = b * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)A.blocks[3] * blockDim.x) A.zero[i] = 0.0f;
+    for (size_t i = b * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)A.blocks[3] * blockDim.x)
+        A.zero[i] = 0.0f;
 }
 
 __global__ void unpack_image_kernel(const float* __restrict__ acc, float* __restrict__ out, DevGrid g, int d) {
@@ -205,7 +208,8 @@ __global__ void residual_kernel(const float* __restrict__ u1, const float* __res
         if (rp != nullptr) {
             int x, y, z;
             split_xyz((unsigned)i, (unsigned)g.m[0], (unsigned)g.m[1], x, y, z);
-            const size_t p = ((size_t)(z + (d == 3 ? LGNK_PAD : 0)) * g.mp[1] + (y + LGNK_PAD)) * g.mp[0] + (x + LGNK_PAD);
+            const size_t p =
+                ((size_t)(z + (d == 3 ? LGNK_PAD : 0)) * g.mp[1] + (y + LGNK_PAD)) * g.mp[0] + (x + LGNK_PAD);
             rp[p] = scale * r;
         }
     }
@@ -461,7 +465,8 @@ __global__ void axpby_dev_kernel(float a, const float* __restrict__ ap, const fl
 // loads of a thread in flight at a time (8192 partials of a 128^3 trace took 7 to
 // 16 us one by one in 256 threads).
 constexpr int kReduceBlock = 1024;
-__global__ void __launch_bounds__(kReduceBlock) reduce_kernel(const double* __restrict__ partial, int count, double* out) {
+__global__ void __launch_bounds__(kReduceBlock)
+    reduce_kernel(const double* __restrict__ partial, int count, double* out) {
     double s = 0.0;
     for (int i = threadIdx.x; i < count; i += 8 * kReduceBlock) {
         double v[8];
@@ -644,7 +649,9 @@ constexpr int kDctLS = kDctLines + 4;        // tile row stride (float4-aligned)
 struct DctTable {
     const float* p;
     int m, h, P4, stride;     // cells; ceil(m/2); floats of a part and of a row
-    __host__ __device__ __forceinline__ int step(bool full, bool inverse) const { return full && inverse ? P4 : stride; }
+    __host__ __device__ __forceinline__ int step(bool full, bool inverse) const {     // from row to row
+        return full && inverse ? P4 : stride;
+    }
     __host__ __device__ __forceinline__ int part(bool full, bool inverse) const {     // offset of the second part
         return full && inverse ? h * stride : (m > 1 ? P4 : 0);
     }
@@ -995,7 +1002,8 @@ __host__ __device__ inline int dct_rows(int m) {
 
 template <bool FULL>
 __device__ __forceinline__ void dct_stage_table(float* dst, const DctTable& t) {
-    for (int e = threadIdx.x; e < dct_rows<FULL>(t.m) * t.stride / 4; e += blockDim.x) cp_async16(dst + 4 * e, t.p + 4 * e);
+    const int n = dct_rows<FULL>(t.m) * t.stride / 4;
+    for (int e = threadIdx.x; e < n; e += blockDim.x) cp_async16(dst + 4 * e, t.p + 4 * e);
 }
 
 // The last axis of the preconditioner in one pass: forward transform, the
@@ -1044,8 +1052,9 @@ __global__ void __launch_bounds__(kBlock) dct_last_half_kernel(const float* __re
     const bool act = j0 < h;
     float ae[4][LT], ao[4][LT];
     if (act) {
-        if (SPLIT) dct_half_part<FULL>(F, tf.part(FULL, false), tf.step(FULL, false), m, false, tile, LS, j0, l0, p, ae);
-        else dct_half_axis<LT, FULL>(F, tf.part(FULL, false), tf.step(FULL, false), m, false, tile, LS, j0, l0, ae, ao);
+        const int po = tf.part(FULL, false), st = tf.step(FULL, false);
+        if (SPLIT) dct_half_part<FULL>(F, po, st, m, false, tile, LS, j0, l0, p, ae);
+        else dct_half_axis<LT, FULL>(F, po, st, m, false, tile, LS, j0, l0, ae, ao);
     }
     __syncthreads();                  // every thread is done reading the tile
     const bool vec = vec_in && i0 + l0 + LT <= inner;
@@ -1074,8 +1083,9 @@ __global__ void __launch_bounds__(kBlock) dct_last_half_kernel(const float* __re
     }
     __syncthreads();
     if (act) {
-        if (SPLIT) dct_half_part<FULL>(I, ti.part(FULL, true), ti.step(FULL, true), m, true, tile, LS, j0, l0, p, ae);
-        else dct_half_axis<LT, FULL>(I, ti.part(FULL, true), ti.step(FULL, true), m, true, tile, LS, j0, l0, ae, ao);
+        const int po = ti.part(FULL, true), st = ti.step(FULL, true);
+        if (SPLIT) dct_half_part<FULL>(I, po, st, m, true, tile, LS, j0, l0, p, ae);
+        else dct_half_axis<LT, FULL>(I, po, st, m, true, tile, LS, j0, l0, ae, ao);
     }
     const bool vec_out = vec && reinterpret_cast<uintptr_t>(out) % 16 == 0;
 #pragma unroll
@@ -1136,8 +1146,9 @@ struct PlaneTask {
     __device__ __forceinline__ void product(const float* tab, const DctTable& t, int m, bool inverse, const float* S,
                                             int LS) {
         if (!act) return;
-        if constexpr (SPLIT) dct_half_part<FULL>(tab, t.part(FULL, inverse), t.step(FULL, inverse), m, inverse, S, LS, j0, l0, p, ae);
-        else dct_half_axis<LT, FULL>(tab, t.part(FULL, inverse), t.step(FULL, inverse), m, inverse, S, LS, j0, l0, ae, ao);
+        const int po = t.part(FULL, inverse), st = t.step(FULL, inverse);
+        if constexpr (SPLIT) dct_half_part<FULL>(tab, po, st, m, inverse, S, LS, j0, l0, p, ae);
+        else dct_half_axis<LT, FULL>(tab, po, st, m, inverse, S, LS, j0, l0, ae, ao);
     }
     // Stores the outputs of lines l0 .. as rows of m values, `row` floats apart;
     // scale: NULL or factors of the same layout (rows of m).  Every thread calls it.
@@ -1307,11 +1318,6 @@ inline size_t dct_tile_smem(int m) {
 __global__ void scale_modes_kernel(float* x, const float* __restrict__ inv_eig, size_t block_elems, size_t count) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
         x[i] *= inv_eig[i % block_elems];
-}
-
-__global__ void axpby_kernel(float a, const float* __restrict__ x, float b, float* y, size_t count) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
-        y[i] = fmaf(a, x[i], b * y[i]);
 }
 
 __global__ void add_scaled_kernel(float* out, const float* x, float ax, const float* y, float ay, size_t count) {
@@ -1627,18 +1633,15 @@ cudaError_t launch_dot(const float* a, const float* b, size_t count, double* par
 
 cudaError_t launch_laplacian(int d, const float* x, float* out, const DevGrid& g, int blocks_kd, float scale,
                              float gamma, const float* addsrc, cudaStream_t s) {
-    const size_t total = (size_t)g.m[0] * g.m[1] * g.m[2] * blocks_kd;
-    const float* gsrc = gamma != 0.0f ? x : nullptr;
-    if (d == 3) laplacian_kernel<3><<<grid_for(total), kBlock, 0, s>>>(x, out, g, blocks_kd, scale, gamma, gsrc, addsrc);
-    else laplacian_kernel<2><<<grid_for(total), kBlock, 0, s>>>(x, out, g, blocks_kd, scale, gamma, gsrc, addsrc);
-    return cudaGetLastError();
+    return launch_laplacian_ext(d, x, out, g, blocks_kd, scale, gamma, gamma != 0.0f ? x : nullptr, addsrc, s);
 }
 
 cudaError_t launch_laplacian_ext(int d, const float* x, float* out, const DevGrid& g, int blocks_kd, float scale,
                                  float gamma, const float* gsrc, const float* addsrc, cudaStream_t s) {
     const size_t total = (size_t)g.m[0] * g.m[1] * g.m[2] * blocks_kd;
-    if (d == 3) laplacian_kernel<3><<<grid_for(total), kBlock, 0, s>>>(x, out, g, blocks_kd, scale, gamma, gsrc, addsrc);
-    else laplacian_kernel<2><<<grid_for(total), kBlock, 0, s>>>(x, out, g, blocks_kd, scale, gamma, gsrc, addsrc);
+    const int grid = grid_for(total);
+    if (d == 3) laplacian_kernel<3><<<grid, kBlock, 0, s>>>(x, out, g, blocks_kd, scale, gamma, gsrc, addsrc);
+    else laplacian_kernel<2><<<grid, kBlock, 0, s>>>(x, out, g, blocks_kd, scale, gamma, gsrc, addsrc);
     return cudaGetLastError();
 }
 
@@ -1678,17 +1681,20 @@ cudaError_t launch_dct_axis(const float* in, float* out, const float* C, const D
     }
     const long long inner = axis == 0 ? 1 : (axis == 1 ? (long long)g.m[0] : (long long)g.m[0] * g.m[1]);
     const long long outer = (long long)(total / ((size_t)m * inner));
-    const long long blocks = axis == 0 ? (outer + kDctLines - 1) / kDctLines    // inner = 1: every (y, z, block) is one line
-                                       : (inner + kDctLines - 1) / kDctLines * outer;
+    // inner = 1: every (y, z, block) is one line
+    const long long blocks =
+        axis == 0 ? (outer + kDctLines - 1) / kDctLines : (inner + kDctLines - 1) / kDctLines * outer;
     const int vec_in = (inner % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
     static bool done[2][64] = {};
     auto run = [&](auto kernel, long long lines, bool (&d)[64]) -> cudaError_t {
         const cudaError_t e = raise_smem(kernel, dct_tile_smem(kDctTileMax), d);
         if (e != cudaSuccess) return e;
-        kernel<<<(unsigned)blocks, kBlock, dct_tile_smem(m), s>>>(in, out, dct_table(C, m), inverse, inner, lines, vec_in);
+        kernel<<<(unsigned)blocks, kBlock, dct_tile_smem(m), s>>>(in, out, dct_table(C, m), inverse, inner, lines,
+                                                                  vec_in);
         return cudaGetLastError();
     };
-    return axis == 0 ? run(dct_tile_kernel<true>, outer, done[0]) : run(dct_tile_kernel<false>, inner * m * outer, done[1]);
+    if (axis == 0) return run(dct_tile_kernel<true>, outer, done[0]);
+    return run(dct_tile_kernel<false>, inner * m * outer, done[1]);
 }
 
 bool dct_table_ok(int m) { return m <= kDctTileMax; }
@@ -1715,8 +1721,8 @@ bool dct_plane_ok(int mx, int my, bool full) {
 }
 
 template <int LT, bool FULL>
-static cudaError_t run_plane(const float* in, float* out, const float* Tx, const float* Ty, bool inverse, int mx, int my,
-                             long long planes, cudaStream_t s) {
+static cudaError_t run_plane(const float* in, float* out, const float* Tx, const float* Ty, bool inverse, int mx,
+                             int my, long long planes, cudaStream_t s) {
     constexpr int most = FULL ? kDctFullPlaneMax : kDctPlaneMax;
     static bool done[64] = {};
     const cudaError_t e = raise_smem(dct_plane_kernel<LT, FULL>, dct_plane_smem<FULL>(most, most, 1), done);
@@ -1773,8 +1779,9 @@ static cudaError_t run_last(const float* in, float* out, const float* Tf, const 
     const int groups = ((m + 1) / 2 + 3) / 4;
     const int vec_in = (inner % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0) ? 1 : 0;
     const dim3 grid((unsigned)((inner + LINES - 1) / LINES), (unsigned)nblocks_kd);
-    dct_last_half_kernel<LINES, SPLIT, FULL><<<grid, dct_threads((SPLIT ? 2 : 1) * groups * (LINES / 4), blocks), bytes(m),
-                                               s>>>(in, out, dct_table(Tf, m), dct_table(Ti, m), inv_eig, m, inner, vec_in);
+    const int threads = dct_threads((SPLIT ? 2 : 1) * groups * (LINES / 4), blocks);
+    dct_last_half_kernel<LINES, SPLIT, FULL><<<grid, threads, bytes(m), s>>>(
+        in, out, dct_table(Tf, m), dct_table(Ti, m), inv_eig, m, inner, vec_in);
     return cudaGetLastError();
 }
 
@@ -1797,11 +1804,6 @@ cudaError_t launch_dct_last(const float* in, float* out, const float* Tf, const 
 
 cudaError_t launch_scale_modes(float* x, const float* inv_eig, size_t block_elems, size_t count, cudaStream_t s) {
     scale_modes_kernel<<<grid_for(count), kBlock, 0, s>>>(x, inv_eig, block_elems, count);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_axpby(float a, const float* x, float b, float* y, size_t count, cudaStream_t s) {
-    axpby_kernel<<<grid_for(count), kBlock, 0, s>>>(a, x, b, y, count);
     return cudaGetLastError();
 }
 

@@ -25,7 +25,15 @@ struct DevGrid {
     float inv_h[3];
 };
 
-enum TraceMode { MODE_FWD = 0, MODE_JVP = 1, MODE_JTVP = 2, MODE_HESS = 3, MODE_OBJGRAD = 4, MODE_ASM = 5, MODE_HROW = 6 };
+enum TraceMode {
+    MODE_FWD = 0,
+    MODE_JVP = 1,
+    MODE_JTVP = 2,
+    MODE_HESS = 3,
+    MODE_OBJGRAD = 4,
+    MODE_ASM = 5,
+    MODE_HROW = 6
+};
 
 // Time dependence of a traced velocity.  TM_STEADY: one slice (K = 1).
 // TM_SLICES, TM_NODES: gathers read the velocity at the 2N + 1 stage times.
@@ -56,9 +64,8 @@ struct TraceArgs {
     float cellvol;            // image cell volume h^d (SSD weight)
     int tiles[3];             // voxel tiles per axis (grid = product), set per launch
     // continuous velocity-grid index of the start point of voxel i along axis a:
-    // vxi_a[a] + (i + 1/2) * vxi_b[a]  (exact in FP64: (x_c - lo_v) / h_v - 1/2)
-    double vxi_a[3], vxi_b[3];
-    float vxi_af[3], vxi_bf[3];  // the same in FP32 (per-stage recomputation)
+    // (x_c - lo_v) / h_v - 1/2 = vxi_a[a] + (i + 1/2) * vxi_b[a]
+    float vxi_a[3], vxi_b[3];
     float pic_rho[3];         // continuity PIC half-width in image cells per axis (0: width = cell)
     long long slice_nodes;    // padded velocity nodes per time slice
     int tj[LGNK_MAX_SLICES];  // TM_NODES: time cell of stage time m, and the offset in it
@@ -72,7 +79,8 @@ struct TraceArgs {
     float* u1;                // transport FWD output (ABI layout)
     float* yout;              // optional end points [d][M]
     float* acc;               // continuity splat accumulator (padded image)
-    void* G;                  // gradient accumulator slices (TM_NODES: nodes) [m][zp][yp][xp] of float4 (3D) / float2 (2D)
+    void* G;                  // gradient accumulator slices (TM_NODES: nodes) [m][zp][yp][xp] of float4 (3D) /
+                              // float2 (2D)
     double* partial;          // per-block partial sums of res^2 (FP64)
     // MODE_ASM (transport): rows of the assembled J, entry-major [e][voxel]
     long long* ekey;          // element of the lower corner of the entry's cell in the slice gradient space
@@ -198,8 +206,6 @@ cudaError_t launch_dct_last(const float* in, float* out, const float* Tf, const 
                             bool full, const DevGrid& g, int d, int nblocks_kd, cudaStream_t s);
 cudaError_t launch_scale_modes(float* x, const float* inv_eig, size_t block_elems, size_t count,
                                cudaStream_t s);
-// y = a * x + b * y  (count floats)
-cudaError_t launch_axpby(float a, const float* x, float b, float* y, size_t count, cudaStream_t s);
 cudaError_t launch_add_scaled(float* out, const float* x, float ax, const float* y, float ay, size_t count,
                               cudaStream_t s);
 

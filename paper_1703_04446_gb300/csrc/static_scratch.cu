@@ -149,10 +149,8 @@ extern "C" lgnk_status lgnk_forward_transport_static(const lgnk_problem* prob, c
             const double hi = (prob->image.hi[i] - prob->image.lo[i]) / prob->image.m[i];
             const double hv = (prob->velocity.hi[i] - prob->velocity.lo[i]) / prob->velocity.m[i];
             cellvol *= hi;
-            a.vxi_a[i] = (prob->image.lo[i] - prob->velocity.lo[i]) / hv - 0.5;
-            a.vxi_b[i] = hi / hv;
-            a.vxi_af[i] = (float)a.vxi_a[i];
-            a.vxi_bf[i] = (float)a.vxi_b[i];
+            a.vxi_a[i] = (float)((prob->image.lo[i] - prob->velocity.lo[i]) / hv - 0.5);
+            a.vxi_b[i] = (float)(hi / hv);
         }
     }
     a.cellvol = (float)cellvol;

@@ -27,7 +27,8 @@
 // Position representation.  A characteristic starts at a cell centre x_c and
 // its state is the FP32 displacement u = y - x_c.  Looking a point up on a grid
 // uses the start's continuous grid index split into an integer I0 and a
-// fraction F0 (computed once in FP64): the cell is I0 + floor(F0 + u / h).  A
+// fraction F0 (on the image exact; on the velocity grid one FP32 FMA, see
+// start_on_velocity): the cell is I0 + floor(F0 + u / h).  A
 // characteristic that barely moves off a grid node therefore keeps the sign of
 // its displacement (an absolute FP32 coordinate would round it away), and the
 // cell choice at the kinks of the piecewise-linear interpolant agrees with an
@@ -186,15 +187,17 @@ struct VelocityStart {
     unsigned c;
 };
 
-// (x_c - lo_v) / h_v - 1/2 = vxi_a + (i + 1/2) vxi_b, evaluated in FP32 (one
-// rounding, below 1e-5 cells for grids up to 2^7 cells).
+// (x_c - lo_v) / h_v - 1/2 = vxi_a + (i + 1/2) vxi_b, evaluated in FP32: exact where the
+// grids' extents and cell counts make both constants short binary fractions (a velocity of a
+// half or a quarter of the image's cells), else off by the constants' roundings and the
+// FMA's, up to 1.2e-7 of the index: 1e-5 cells at 2^7 cells, 0.1 at the 2^20 that an axis may have.
 template <int D>
 __device__ __forceinline__ void start_on_velocity(const TraceArgs& A, const int* idx, VelocityStart<D>& s) {
     unsigned st = 1;
     s.c = 0;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        const float xi = fmaf((float)idx[a] + 0.5f, A.vxi_bf[a], A.vxi_af[a]);
+        const float xi = fmaf((float)idx[a] + 0.5f, A.vxi_b[a], A.vxi_a[a]);
         const int i0 = min(max((int)floorf(xi), -2), A.vg.m[a]);
         s.F0[a] = xi - (float)i0;
         s.lo[a] = (float)(-2 - i0);
@@ -1054,7 +1057,8 @@ __device__ __noinline__ void pic_hat(const DevGrid& g, const int* I0, const floa
     w[2][0] = 1.0f;
     dw[2][0] = 0.0f;
 #pragma unroll
-    for (int a = 0; a < D; ++a) hat_axis(u[a] * g.inv_h[a], rho[a], I0[a], g.m[a], g.inv_h[a], c0[a], n[a], w[a], dw[a]);
+    for (int a = 0; a < D; ++a)
+        hat_axis(u[a] * g.inv_h[a], rho[a], I0[a], g.m[a], g.inv_h[a], c0[a], n[a], w[a], dw[a]);
     float gsum[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll 1
     for (int kz = 0; kz < n[2]; ++kz) {
@@ -1135,7 +1139,8 @@ __device__ __forceinline__ void value_sweep(const TraceArgs& A, const VelocitySt
             else dup_offsets<D>(f, fd);
 #pragma unroll
             for (int q = 0; q < D; ++q) {
-                const float v = FORM == CORNERS ? lerp_value<D>(C.e[q], f, fd) : row_value<D>(poly_row<D>(C.e[q], fd), f);
+                const float v =
+                    FORM == CORNERS ? lerp_value<D>(C.e[q], f, fd) : row_value<D>(poly_row<D>(C.e[q], fd), f);
                 acc[q] = st == 0 ? v : (st == 3 ? acc[q] + v : fmaf(2.0f, v, acc[q]));
                 if (st < 3) us[q] = fmaf(st == 2 ? dt : hdt, v, u[q]);
             }
@@ -1414,7 +1419,8 @@ __device__ __forceinline__ void ell_load(const EllArgs& A, long long i, int j, l
 }
 
 template <int D>
-__device__ __forceinline__ float ell_dot(const EllArgs& A, const float* __restrict__ dV, long long key, const float* b) {
+__device__ __forceinline__ float ell_dot(const EllArgs& A, const float* __restrict__ dV, long long key,
+                                         const float* b) {
     float s = 0.0f;
 #pragma unroll
     for (int r = 0; r < (1 << (D - 1)); ++r) {     // rows of x-pairs (cy, cz); corner (0, cy, cz) is 2 r
@@ -1571,7 +1577,8 @@ struct TraceOccupancy {
 };
 
 template <int D, int TM, int MODEL, int MODE>
-__global__ void __launch_bounds__((TraceOccupancy<D, TM, MODEL, MODE>::threads), (TraceOccupancy<D, TM, MODEL, MODE>::value))
+__global__ void
+__launch_bounds__((TraceOccupancy<D, TM, MODEL, MODE>::threads), (TraceOccupancy<D, TM, MODEL, MODE>::value))
     trace_kernel(const TraceArgs A) {
     constexpr int THREADS = TraceOccupancy<D, TM, MODEL, MODE>::threads;
     constexpr bool TRANSPORT = MODEL == LGNK_TRANSPORT;

@@ -220,8 +220,9 @@ __global__ void __launch_bounds__(128) conv_first_kernel(const float* T, const f
     float* bs = reinterpret_cast<float*>(sb + kFirstK * bn * 16);
     const int tid = threadIdx.x, warp = tid >> 5;
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(umma::smem_u32(&tmem_base)),
-                     "r"(ncols));
+        asm volatile(
+            "tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(umma::smem_u32(&tmem_base)),
+            "r"(ncols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
@@ -242,7 +243,8 @@ __global__ void __launch_bounds__(128) conv_first_kernel(const float* T, const f
     }
     for (int i = tid; i < bn; i += 128) bs[i] = i < C ? umma::ld(bias + i) : 0.0f;
 #pragma unroll
-    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint4*>(sm + ((p * kFirstK + 9) * 128 + tid) * 16) = make_uint4(0, 0, 0, 0);
+    for (int p = 0; p < 3; ++p)
+        *reinterpret_cast<uint4*>(sm + ((p * kFirstK + 9) * 128 + tid) * 16) = make_uint4(0, 0, 0, 0);
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
@@ -270,10 +272,10 @@ __global__ void __launch_bounds__(128) conv_first_kernel(const float* T, const f
             __nv_bfloat16 h[2], q[2], l[2];
             umma::split3(in[2 * t], h[0], q[0], l[0]);
             umma::split3(in[2 * t + 1], h[1], q[1], l[1]);
-            uint8_t* dst = sm + (t * 128 + tid) * 16;
-            *reinterpret_cast<uint4*>(dst) = make_uint4(*reinterpret_cast<const uint32_t*>(h), 0, 0, 0);
-            *reinterpret_cast<uint4*>(dst + kFirstK * 2048) = make_uint4(*reinterpret_cast<const uint32_t*>(q), 0, 0, 0);
-            *reinterpret_cast<uint4*>(dst + 2 * kFirstK * 2048) = make_uint4(*reinterpret_cast<const uint32_t*>(l), 0, 0, 0);
+            uint4* dst = reinterpret_cast<uint4*>(sm + (t * 128 + tid) * 16);      // planes kFirstK x 128 rows apart
+            dst[0] = make_uint4(*reinterpret_cast<const uint32_t*>(h), 0, 0, 0);
+            dst[kFirstK * 128] = make_uint4(*reinterpret_cast<const uint32_t*>(q), 0, 0, 0);
+            dst[2 * kFirstK * 128] = make_uint4(*reinterpret_cast<const uint32_t*>(l), 0, 0, 0);
         }
         asm volatile("fence.proxy.async.shared::cta;");
         asm volatile("tcgen05.fence::before_thread_sync;");
@@ -298,11 +300,7 @@ __global__ void __launch_bounds__(128) conv_first_kernel(const float* T, const f
         asm volatile("tcgen05.fence::after_thread_sync;");
         for (int c0 = 0; c0 < bn; c0 += 16) {
             uint32_t v[16];
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
+            umma::tmem_ld16(v, tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0);
             asm volatile("tcgen05.wait::ld.sync.aligned;");
             if (!valid) continue;
             float z[16];
@@ -602,7 +600,8 @@ bool planes_map(EncodeTiled enc, CUtensorMap* m, __nv_bfloat16* p, int cp, int h
                 const umma::ConvGemm& g, int step) {
     const cuuint64_t row = 2ull * cp, dims[5] = {(cuuint64_t)cp, (cuuint64_t)h, (cuuint64_t)h, (cuuint64_t)B, 3};
     const cuuint64_t strides[4] = {row, row * h, row * h * h, row * h * h * B};
-    const cuuint32_t box[5] = {(cuuint32_t)kb, (cuuint32_t)(g.bx * step), (cuuint32_t)(g.by * step), (cuuint32_t)g.bb, 3};
+    const cuuint32_t box[5] = {(cuuint32_t)kb, (cuuint32_t)(g.bx * step), (cuuint32_t)(g.by * step), (cuuint32_t)g.bb,
+                               3};
     const cuuint32_t steps[5] = {1, (cuuint32_t)step, (cuuint32_t)step, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, p, dims, strides, box, steps, CU_TENSOR_MAP_INTERLEAVE_NONE,
                swizzle_of(kb), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -731,9 +730,9 @@ lgnk_status forward_pass(lgnk_ws* w, int B, const float* T, const float* R, floa
     const size_t n = (size_t)w->m * w->m * B;
     const int bn = w->L[1].cpi, tiles = (int)((n + umma::BM - 1) / umma::BM);
     const int ncols = bn <= 32 ? 32 : (bn <= 64 ? 64 : (bn <= 128 ? 128 : 256));
-    cudaError_t e = launch(conv_first_kernel, dim3(std::min(tiles, first_ctas(bn) * w->sms)), 128, first_smem(bn), w->stream,
-                           T, R, w->p + L0.woff, w->p + L0.boff, w->planes[1], L0.co, bn, bn, w->m, B, tiles, ncols,
-                           w->derr, w->herr);
+    const dim3 grid(std::min(tiles, first_ctas(bn) * w->sms));
+    cudaError_t e = launch(conv_first_kernel, grid, 128, first_smem(bn), w->stream, T, R, w->p + L0.woff,
+                           w->p + L0.boff, w->planes[1], L0.co, bn, bn, w->m, B, tiles, ncols, w->derr, w->herr);
     if (e == cudaSuccess) e = conv_fwd(w, 1, w->e1, nullptr, nullptr, 1, 1.0f, B);
     if (e == cudaSuccess) e = conv_fwd(w, 2, w->e2, nullptr, nullptr, 1, 1.0f, B);
     if (e == cudaSuccess) e = conv_fwd(w, 3, nullptr, nullptr, nullptr, 1, 1.0f, B);
@@ -832,8 +831,8 @@ lgnk_status lgnk_ws_create(int image_m, int base_channels, int max_batch, float 
             return fail(LGNK_ERR_CUDA);
         }
         w->smem_max = optin - (int)fa.sharedSizeBytes;
-        if (cudaFuncSetAttribute(conv_first_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)first_smem(256)) !=
-            cudaSuccess) {
+        if (cudaFuncSetAttribute(conv_first_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)first_smem(256)) != cudaSuccess) {
             cudaGetLastError();
             return fail(LGNK_ERR_CUDA);
         }
@@ -858,7 +857,8 @@ lgnk_status lgnk_ws_create(int image_m, int base_channels, int max_batch, float 
         L.rowsd = round_up(L.ci, L.bnd);
         L.ldd = round_up(9 * R * L.cpo, umma::BK);
         zmax = std::max(zmax, (size_t)B * L.hout * L.hout * L.cpo);
-        if ((s = ws_alloc_n(w, (size_t)L.rowsf * L.ldf, &L.wf)) || (s = ws_alloc_n(w, (size_t)L.rowsd * L.ldd, &L.wd)) ||
+        if ((s = ws_alloc_n(w, (size_t)L.rowsf * L.ldf, &L.wf)) ||
+            (s = ws_alloc_n(w, (size_t)L.rowsd * L.ldd, &L.wd)) ||
             (s = ws_alloc_n(w, (size_t)3 * B * L.hin * L.hin * L.cpi, &w->planes[l])))
             return fail(s);
     }
@@ -978,15 +978,15 @@ lgnk_status lgnk_ws_train_step(lgnk_ws* w, int batch, const float* T, const floa
         // one wave of two blocks per SM
         const int groups = (L.co + kFirstW - 1) / kFirstW, wave = std::max(1, 2 * w->sms / groups);
         const int bs = (int)std::min<size_t>(std::min(kMaxSlices, wave), (n + kT - 1) / kT);
-        WS_CHECK(launch(conv_first_wgrad_kernel, dim3(bs, groups), kT, 0, w->stream, T, R, w->gc, w->planes[1], w->wpart,
-                        w->bpart, L.co, w->L[1].cpi, m, B));
+        WS_CHECK(launch(conv_first_wgrad_kernel, dim3(bs, groups), kT, 0, w->stream, T, R, w->gc, w->planes[1],
+                        w->wpart, w->bpart, L.co, w->L[1].cpi, m, B));
         WS_CHECK(sum_slices(w, L, 2, bs, bs));
     }
     // Adam
     w->steps++;
     const float c1 = 1.0f - powf(0.9f, (float)w->steps), c2 = 1.0f - powf(0.999f, (float)w->steps);
-    WS_CHECK(launch(adam_kernel, dim3(blocks_for(w->nparams)), kT, 0, w->stream, w->p, w->g, w->am, w->as, w->nparams, lr,
-                    c1, c2, w->derr));
+    WS_CHECK(launch(adam_kernel, dim3(blocks_for(w->nparams)), kT, 0, w->stream, w->p, w->g, w->am, w->as, w->nparams,
+                    lr, c1, c2, w->derr));
     WS_CHECK(pack_weights(w));
     if (loss != nullptr) {
         launch_reduce(w->partial, nb, w->partial + 2048, w->stream);

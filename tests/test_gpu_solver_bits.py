@@ -27,8 +27,8 @@ ROWS = [((20, 18, 16), (10, 9, 8), 1, 4), ((16, 16, 16), (16, 16, 16), 1, 8), ((
         ((40, 36), (20, 18), 1, 4), ((32, 32), (32, 32), 2, 8)]
 # one step of a 3D solve: cells of both grids; planes of at most and of more than 64 x 64
 # cells, a last axis of more than 64 and of more than 128 cells, odd sizes, small axes
-STEPS = [(16, 12, 10), (64, 64, 8), (13, 9, 11), (72, 10, 12), (8, 9, 72), (6, 5, 130), (130, 4, 6), (4, 67, 5), (3, 2, 1),
-         (48, 40, 56)]
+STEPS = [(16, 12, 10), (64, 64, 8), (13, 9, 11), (72, 10, 12), (8, 9, 72), (6, 5, 130), (130, 4, 6), (4, 67, 5),
+         (3, 2, 1), (48, 40, 56)]
 
 
 def _values(shape, seed, scale):
