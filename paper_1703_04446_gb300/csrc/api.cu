@@ -107,6 +107,7 @@ struct lgnk_ctx {
     float* fsc = nullptr;         // PCG step lengths on the device (alpha, -alpha, beta)
     unsigned* dcounter = nullptr; // completion counter of launch_dot_fused (zero between launches)
     int* dctl = nullptr;          // device-side PCG loop state (dot_blocks_finish)
+    int* dmany = nullptr;         // of the velocity in Vp: pack_many_cells (with gn_rows)
     unsigned char* hpin = nullptr; // pinned: the loop state's host copy (4 ints) and its tolerance (a double)
     // lgnk_solve runs on a stream of its own (capturable, unlike the legacy
     // default stream), ordered after and before the caller's stream by events
@@ -287,6 +288,7 @@ TraceArgs base_args(const lgnk_ctx* ctx) {
     }
     a.V = ctx->Vp;
     a.dV = ctx->dVp;
+    a.many = ctx->dmany;
     a.Tp = ctx->Tp;
     a.G = ctx->Gp;
     return a;
@@ -331,6 +333,10 @@ lgnk_status pack(lgnk_ctx* ctx, const float* v, const float* dv, const float* im
     a.tab = ctx->slices;
     int k = 0;
     if (v != nullptr) {
+        if (ctx->gn_rows) {
+            a.many = ctx->dmany;
+            a.many_faces = std::min(0.12f * (float)ctx->N, 1.1f);
+        }
         a.v[k] = v;
         a.vp[k++] = static_cast<float*>(ctx->Vp);
     }
@@ -875,6 +881,7 @@ lgnk_status lgnk_create(const lgnk_problem* prob, void* stream, size_t mem_budge
     if ((s = dalloc(ctx, (size_t)ctx->npartial, &ctx->partial)) != LGNK_OK) return fail(s);
     if ((s = dalloc(ctx, (size_t)ctx->trace_blocks, &ctx->cpartial)) != LGNK_OK) return fail(s);
     if ((s = dalloc(ctx, 16, &ctx->dres)) != LGNK_OK) return fail(s);
+    ctx->dmany = reinterpret_cast<int*>(ctx->dres + 15);
     if ((s = dalloc(ctx, 4, &ctx->fsc)) != LGNK_OK) return fail(s);
     if ((s = dalloc(ctx, 1, &ctx->dcounter)) != LGNK_OK) return fail(s);
     if ((s = dalloc(ctx, 4, &ctx->dctl)) != LGNK_OK) return fail(s);

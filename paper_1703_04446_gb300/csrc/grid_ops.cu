@@ -144,6 +144,37 @@ __device__ __forceinline__ void pack_image(const float* __restrict__ T, float* _
     }
 }
 
+// Whether a Gauss-Newton product with the stationary velocity v is cheaper by tangent sweeps than
+// by rows (trace_impl.cuh): a row costs a block for every cell its characteristic enters, and
+// a second sweep past the blocks that a thread keeps.  At the speed of a node a
+// characteristic crosses sum_a |v_a| / h_a cell faces; a warp takes the mean of 64 nodes
+// spread evenly.  Rows win up to about 0.12 N faces, 1.1 at most (the limit, from the caller).
+// Products on 128^3 voxels by rows / by the kernel before the rows / by this choice, us: velocity
+// of 64^3 cells, N = 4, displacements up to 25 voxels 503 / 417 / 394; velocity of
+// 128^3 cells, N = 8, 25 voxels 952 / 794 / 748, 8 voxels 654 / 690 / 639.  Taken in the
+// packing, the sample costs the trace one load; taken by each of its warps it cost 2% with N = 8.
+template <int D>
+__device__ __forceinline__ void pack_many_cells(const float* __restrict__ v, const DevGrid& g, float limit, int* many) {
+    constexpr int kNodes = 64;
+    constexpr float step[3] = {0.8191725f, 0.6710436f, 0.5497005f};      // evenly spread points of the unit cube
+    if (threadIdx.x >= 32) return;
+    const size_t Mv = (size_t)g.m[0] * g.m[1] * g.m[2];
+    float faces = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kNodes / 32; ++k) {
+        size_t e = 0;
+#pragma unroll
+        for (int a = D - 1; a >= 0; --a) {
+            const float x = ((float)(threadIdx.x + 32 * k) + 0.5f) * step[a];
+            e = e * (size_t)g.m[a] + (size_t)min((int)((x - floorf(x)) * (float)g.m[a]), g.m[a] - 1);
+        }
+#pragma unroll
+        for (int a = 0; a < D; ++a) faces = fmaf(fabsf(v[a * Mv + e]), g.inv_h[a], faces);
+    }
+    const int total = __reduce_add_sync(0xffffffffu, (int)(fminf(faces, 4096.0f) * 1024.0f));
+    if (threadIdx.x == 0) *many = (float)total > limit * (1024.0f * kNodes) ? 1 : 0;
+}
+
 // Everything a call lays out before its trace: the parts take consecutive
 // blocks.  The parts are bound by memory at large sizes (the brain-scale product's
 // 492 us are what its two packings and its clearing took) and by their launches
@@ -168,6 +199,10 @@ __global__ void __launch_bounds__(kBlock) pack_kernel(const PackArgs A) {
         return;
     }
     b -= (unsigned)A.blocks[2];
+    if (b >= (unsigned)A.blocks[3]) {
+        pack_many_cells<D>(A.v[0], A.vg, A.many_faces, A.many);
+        return;
+    }
     const size_t total = padded_size(A.ig);
     for (size_t i = b * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)A.blocks[3] * blockDim.x)
         A.zero[i] = 0.0f;
@@ -1478,7 +1513,8 @@ cudaError_t launch_pack(int d, PackArgs a, cudaStream_t s) {
     for (int k = 0; k < 2; ++k) a.blocks[k] = a.v[k] != nullptr ? grid_for(vn) : 0;
     a.blocks[2] = a.image != nullptr ? grid_for(in) : 0;
     a.blocks[3] = a.zero != nullptr ? grid_for(in) : 0;
-    const int blocks = a.blocks[0] + a.blocks[1] + a.blocks[2] + a.blocks[3];
+    if (a.many != nullptr && a.v[0] == nullptr) return cudaErrorInvalidValue;
+    const int blocks = a.blocks[0] + a.blocks[1] + a.blocks[2] + a.blocks[3] + (a.many != nullptr ? 1 : 0);
     if (blocks == 0) return cudaSuccess;
     if (d == 3) pack_kernel<3><<<blocks, kBlock, 0, s>>>(a);
     else pack_kernel<2><<<blocks, kBlock, 0, s>>>(a);

@@ -72,6 +72,7 @@ struct TraceArgs {
     float tth[LGNK_MAX_SLICES];
     const void* V;            // pair-packed velocity slices [m][zp][yp][xp] x [v(node) | v(node+1)]
     const void* dV;           // pair-packed direction slices (JVP, HESS, HROW)
+    const int* many;          // HROW: whether the velocity crosses many cells (PackArgs)
     const float* Tp;          // padded template (gathers)
     const float* T;           // template, ABI layout (continuity particle masses)
     const float* R;           // reference, ABI layout (OBJGRAD, FWD with residual)
@@ -118,7 +119,8 @@ cudaError_t launch_trace(int d, TimeMode tm, int model, int mode, const TraceArg
 // ABI velocities [K][d][z][y][x] as pair-packed padded time slices
 // (velocity_pair_bytes(d) bytes per node and slice), with the first nz gradient
 // slices, at most as many as tab has, zeroed beside the last of them; an image
-// into its padded grid; a padded image grid to zero.
+// into its padded grid; a padded image grid to zero; a word that says how many cells the
+// first velocity's characteristics cross.
 struct PackArgs {
     DevGrid vg, ig;
     SliceTable tab;
@@ -129,6 +131,8 @@ struct PackArgs {
     const float* image;
     float* imagep;
     float* zero;
+    int* many;                // set to 1 or 0: a stationary v[0] crosses more than many_faces cells (pack_many_cells)
+    float many_faces;
     int blocks[4];            // of each part, set by launch_pack
 };
 cudaError_t launch_pack(int d, PackArgs a, cudaStream_t s);

@@ -1283,40 +1283,6 @@ __device__ __forceinline__ void adjoint_sweep(const TraceArgs& A, const float* V
     }
 }
 
-// Whether a product is cheaper by tangent sweeps than by rows: a row costs a block for every
-// cell its characteristic enters, and a second sweep past RowScatter::CAP of them.  Decided for
-// the whole launch, by a sample of the velocity that every warp takes alike: at the speed of its
-// node a characteristic crosses sum_a |v_a| / h_a cell faces.  Rows win up to about 0.12 N faces
-// on average, 1.1 at most.  Products on 128^3 voxels by rows / by the kernel before the rows /
-// by this choice, us: velocity of 64^3 cells, N = 4, displacements up to 25 voxels
-// 503 / 417 / 415; velocity of 128^3 cells, N = 8, 25 voxels 952 / 794 / 764, 8 voxels 654 / 690 / 652.
-// What is paid for the choice where rows win: 240 -> 250 us with N = 4, 404 -> 407 with N = 8.
-// A launch-wide choice, since CTAs of both kinds together evict each other's instructions
-// (chosen per warp 778 us where rows alone took 710), and inline, since the function apart
-// reads its arguments through memory (522 us for the 415).
-constexpr int kManyCellsSample = 64;
-template <int D>
-__device__ __forceinline__ bool many_cells(const TraceArgs& A, const float* V) {
-    constexpr float step[3] = {0.8191725f, 0.6710436f, 0.5497005f};      // evenly spread points of the unit cube
-    float faces = 0.0f;
-#pragma unroll
-    for (int k = 0; k < kManyCellsSample / 32; ++k) {
-        size_t e = 0;
-#pragma unroll
-        for (int a = D - 1; a >= 0; --a) {
-            const float x = ((float)((threadIdx.x & 31) + 32 * k) + 0.5f) * step[a];
-            const int c = min((int)((x - floorf(x)) * (float)A.vg.m[a]), A.vg.m[a] - 1);
-            e = e * (size_t)A.vg.mp[a] + (size_t)(c + LGNK_PAD);
-        }
-        float v[3], next[3];
-        pair_value<D>(V, e, v, next);
-#pragma unroll
-        for (int a = 0; a < D; ++a) faces = fmaf(fabsf(v[a]), A.vg.inv_h[a], faces);
-    }
-    const int total = __reduce_add_sync(0xffffffffu, (int)(fminf(faces, 4096.0f) * 1024.0f));
-    return (float)total > fminf(0.12f * (float)A.N, 1.1f) * (1024.0f * kManyCellsSample);
-}
-
 // The fused Gauss-Newton product of one voxel (RowScatter): the row's sweep,
 // then its blocks dotted with the direction and, scaled by h^d J_i dv, into
 // the gradients; a row whose blocks did not fit is swept again with the scaled
@@ -1371,6 +1337,32 @@ __device__ __forceinline__ void gauss_newton_row(const TraceArgs& A, const float
 #pragma unroll
         for (int a = 0; a < D; ++a) lam[a] = s * gT[a];
     }
+}
+
+// The same product of one voxel by a tangent sweep, where the rule of pack_many_cells says so (A.many):
+// a launch-wide choice, since CTAs of both kinds together evict each other's instructions
+// (chosen per warp 778 us where rows alone took 710).
+template <int D, int TM, int FORM, int NB>
+__device__ __forceinline__ void gauss_newton_tangent(const TraceArgs& A, const int* idx, const VelocityStart<D>& sv,
+                                                     float4* rec) {
+    const float* V = static_cast<const float*>(A.V);
+    float u[D], dy[D], lam[D], du = 0.0f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) u[a] = dy[a] = 0.0f;
+    tangent_sweep<D, TM, FORM, true>(A, sv, V, static_cast<const float*>(A.dV), u, dy, rec);
+    Start<D> si;
+    start_on_image<D>(idx, si);
+    sample_image<D, true>(A.ig, si, A.Tp, u, lam);
+#pragma unroll
+    for (int a = 0; a < D; ++a) du = fmaf(lam[a], dy[a], du);
+#pragma unroll
+    for (int a = 0; a < D; ++a) lam[a] *= A.cellvol * du;
+    Cell<D, POLY> C;
+    C.key = -1;
+    BlockScatter<D, NB> S;
+    scatter_init(S, A.G, (int)A.slice_nodes);
+    adjoint_sweep<D, TM>(A, V, S, rec, lam, C);
+    scatter_finish(A.vg, S);
 }
 
 // Finish one assembled row: its keys at [e][voxel] (the blocks are already
@@ -1596,7 +1588,7 @@ __launch_bounds__((TraceOccupancy<D, TM, MODEL, MODE>::threads), (TraceOccupancy
     int entries = 0;         // MODE_ASM: blocks of this thread's row
 
     bool far = false;         // MODE_HROW: by tangent sweeps after all
-    if constexpr (ROWS) far = many_cells<D>(A, V);
+    if constexpr (ROWS) far = *A.many != 0;
     int idx[3];
     voxel_index<D>(A, THREADS, idx);
     const bool active = idx[0] < A.ig.m[0] && idx[1] < A.ig.m[1] && (D == 2 || idx[2] < A.ig.m[2]);
@@ -1624,9 +1616,12 @@ __launch_bounds__((TraceOccupancy<D, TM, MODEL, MODE>::threads), (TraceOccupancy
         // for an earlier 128^3 product).
         float4 rec[ADJOINT ? 4 * LGNK_MAX_STEPS : 1];
         if constexpr (ROWS) {
-            if (far) tangent_sweep<D, TM, FORM, true>(A, sv, V, dV, u, dy, rec);
-            else value_sweep<D, TM, FORM, true>(A, sv, V, u, rec);
-        } else if constexpr (TANGENT) tangent_sweep<D, TM, FORM, ADJOINT>(A, sv, V, dV, u, dy, rec);
+            if (far) {
+                gauss_newton_tangent<D, TM, FORM, NB>(A, idx, sv, rec);
+                return;
+            }
+        }
+        if constexpr (TANGENT) tangent_sweep<D, TM, FORM, ADJOINT>(A, sv, V, dV, u, dy, rec);
         else value_sweep<D, TM, FORM, ADJOINT>(A, sv, V, u, rec);
         if (A.yout != nullptr) {
             const int M = A.ig.m[0] * A.ig.m[1] * (D == 3 ? A.ig.m[2] : 1);
@@ -1699,20 +1694,6 @@ __launch_bounds__((TraceOccupancy<D, TM, MODEL, MODE>::threads), (TraceOccupancy
         if constexpr (ADJOINT) {
             Cell<D, POLY> C;
             C.key = -1;
-            if constexpr (ROWS) {
-                if (far) {
-                    float du = 0.0f;
-#pragma unroll
-                    for (int a = 0; a < D; ++a) du = fmaf(lam[a], dy[a], du);
-#pragma unroll
-                    for (int a = 0; a < D; ++a) lam[a] *= A.cellvol * du;
-                    BlockScatter<D, NB> S;
-                    scatter_init(S, A.G, (int)A.slice_nodes);
-                    adjoint_sweep<D, TM>(A, V, S, rec, lam, C);
-                    scatter_finish(A.vg, S);
-                    return;
-                }
-            }
             SC S;
             scatter_init(S, A.G, (int)A.slice_nodes);
             if constexpr (ROWS) {
