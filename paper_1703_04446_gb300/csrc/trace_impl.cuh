@@ -16,7 +16,8 @@
 //   HROW     the same product by rows (3D, stationary velocity): the adjoint
 //            sweep seeded with grad T(y_i) yields the row J_i as a few blocks of
 //            corner vectors; they are dotted with dv and scattered scaled by
-//            h^d J_i dv (RowScatter).
+//            h^d J_i dv (RowScatter).  Where the velocity crosses many cells, by
+//            tangent sweeps as HESS (gauss_newton_tangent).
 //   OBJGRAD  transport only: u1, SSD partials and the JTVP of h^d res fused.
 //   ASM      transport only: the adjoint sweep seeded with grad T(y) yields
 //            row i of J = d_v u1 (Sec. 3.3 assembles J as a sparse matrix);
@@ -45,8 +46,8 @@
 //
 // What bounds these kernels: first the issue slots, now latency.  Paired FP32
 // instructions, the row form of the Gauss-Newton product and the floor without
-// conversions took the 128^3 product from 495M to 336M warp instructions (issue
-// slots 0.70 -> 0.58 busy) and from 554 to 454 us; what the warps wait for is
+// conversions took the 128^3 product from 495M to 349M warp instructions (issue
+// slots 0.70 -> 0.61 busy) and from 554 to 458 us; what the warps wait for is
 // the cell's corners after a change (long scoreboard, at 16 warps per SM).
 //
 // Time slices.  Every RK4 stage time is t0 + m dt/2 (m = 0..2N), so the host
@@ -64,7 +65,10 @@
 // reduced once per cell.  Per stage time (TM_SLICES) it would be reduced at
 // every second stage; measured on the brain-scale J^T (K = 9, N = 16) 7.8 ms
 // with slices against 6.2 ms with nodes, and on the 128 x 150 x 128 product
-// with K = 2, N = 5 1058 against 870 us (both with the other changes here).
+// with K = 2, N = 5 1058 against 870 us (both with the other changes here).  A node's
+// FP32 accumulator then takes all the stages that a slice each took before: errors
+// against 64 bits 2.3e-7 -> 2.6e-7 (mass-preserving product, 96 x 112 x 80, K = 9),
+// 1.1e-7 -> 1.6e-7 (objective's gradient, 80 x 70 x 60, K = 3).
 // With shorter time cells (K - 1 > N) every stage time has two nodes of its own
 // and the slices take half the reductions; a streaming kernel then distributes
 // them onto the time nodes with the transposed time weights.  A shared-memory
@@ -475,7 +479,7 @@ __device__ __forceinline__ void scatter_emit(const DevGrid& g, CornerScatter<D, 
 // Against a tangent sweep for J dv (MODE_HESS) this drops the direction's
 // interpolation and the products d_y I q at every stage, 390 instead of 615
 // FP32 operations per voxel-step, and adds the blocks' way through local
-// memory once per row: at 128^3 0.447 against 0.513 ms with N = 8, 0.279 against
+// memory once per row and cell: at 128^3 0.447 against 0.513 ms with N = 8, 0.279 against
 // 0.293 ms with N = 4, but 0.200 against 0.190 ms with N = 2 (64 x 60 x 62:
 // 61 / 70, 39 / 43, 30.5 / 28.6 us).  It stays with the tangent sweep in 2D (cheap
 // stages: 10 to 20% slower by rows) and for K > 1 (a block per time node and
